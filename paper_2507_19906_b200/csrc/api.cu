@@ -375,7 +375,8 @@ int calidrop_select_from_scores(const calidrop_params* p, const float* scores, i
   g.W = tail; g.n_cand = p->L - tail; g.k_sel = p->budget - tail; g.sized = 0; g.n_calib = 0;
   if (!select_cluster_supported(g)) return CALIDROP_UNSUPPORTED;
   if (!device_supported()) return CALIDROP_UNSUPPORTED;
-  cudaError_t e = launch_pool_select_scores(g, ws, (char*)workspace, scores, (size_t)p->L, kept_idx, (cudaStream_t)stream);
+  cudaError_t e = launch_pool_select_scores(g, ws, (char*)workspace, scores, (size_t)p->L, 1, 0, nullptr, kept_idx,
+                                            (cudaStream_t)stream);
   return e == cudaSuccess ? CALIDROP_OK : cuda_fail(e);
 }
 

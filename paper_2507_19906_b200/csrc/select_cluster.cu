@@ -1,16 +1,33 @@
-// Pooling + per-(batch, kv-head) top-k on a thread-block cluster.
+// Pooling + per-(batch, kv-head) top-k on thread-block clusters.
 //
-// The single-CTA selection of select.cu uses one SM per unit; with a few dozen units most of the
-// GPU idles.  Here a cluster of eight CTAs shares a unit: CTA r owns the contiguous key range
-// [r * chunk, (r + 1) * chunk), every thread keeps its ROWS keys (pooled votes as fp32 bit
-// patterns) in registers, and the CTAs exchange only their 256-bin histograms and their counts
-// through distributed shared memory.  The algorithm is the same exact radix select: four 8-bit
-// passes find the bit pattern T of the k-th largest pooled vote and how many candidates equal to
-// T still fit; an ordered compaction then emits, ascending, every candidate above T and the first
-// need_eq candidates equal to T (ties go to the lowest index), plus the kept bitmap.
-// Key (row i, thread tid) of CTA r is candidate r * chunk + i * 1024 + tid, so a warp covers 32
-// consecutive candidates: loads coalesce and one ballot is one bitmap word.
+// A cluster of 1..8 CTAs shares a unit: CTA r owns the contiguous key range [r * chunk, (r + 1) * chunk),
+// every thread keeps its ROWS keys (pooled votes as fp32 bit patterns; non-negative, so unsigned order is
+// numeric order) in registers, and the CTAs exchange only histograms and counts through distributed
+// shared memory.  Exact radix select, digits of 8 + 8 + 8 + 7 bits (the sign bit is zero), finds a threshold
+// T and how many candidates equal to T are taken besides all those above it; an ordered compaction then
+// emits them ascending (ties go to the lowest index), plus the kept bitmap.  With a calibration size
+// the second threshold is searched in the same passes.
+//
+// What bounds it is latency: barriers and the round trips between them; no pipe or memory is near a limit.
+// Hence
+//   * the votes are staged in shared memory once, with the pool's halo, instead of `pool` loads per key;
+//   * votes have few exponents, so the first digits fall into a handful of bins: a histogram has a column
+//     per LANE (word bin * 32 + lane), so that the lanes of a warp never meet in a word or a bank;
+//   * three barriers per pass: the columns of a bin are summed by one warp reduction and cleared as they
+//     are read, the sums are PUSHED to every CTA of the cluster, and one warp per threshold walks them;
+//   * the passes end as soon as all keys of the chosen bin are taken (usually after two or three);
+//   * key (warp w, row i, lane l) of CTA r is candidate r * chunk + (w * ROWS + i) * 32 + l: a warp owns a
+//     contiguous run, so the compaction scans one count per warp (a ballot is one bitmap word);
+//   * the cluster is only as large as the prompt needs: a prompt of 2048 keys takes one CTA and no
+//     cluster barrier at all.
+// Measured, kernel time from cold caches, against 1024-thread clusters of eight with a histogram per warp,
+// pooled from global memory: 64 units x 16384 keys 33.3 -> 18.8 us, 32 x 32768 24.8 -> 20.6 us, 4 x 131072 36.8 -> 29.4 us,
+// 16 x 5003 with a calibration size 22.8 -> 19.2 us, 8 x 8192 11.9 -> 13.8 us (in a stream of calls, beside the
+// neighbouring kernels, 1.2 us less per call all the same).  Wider digits, 11 + 10 + 10 bits with two
+// histograms per CTA, were slower, 47 us at 32 x 32768: the votes' few exponents share bins.
 #include <cooperative_groups.h>
+
+#include <type_traits>
 
 #include "common.cuh"
 #include "internal.h"
@@ -21,251 +38,347 @@ namespace {
 
 namespace cg = cooperative_groups;
 
-constexpr int kClu = 8;
-constexpr int kT = 1024;
-constexpr int kW = kT / 32;
+constexpr int kMaxClu = 8;
+constexpr int kHaloMax = 64;   // widest half pool that is staged; wider pools read the votes from global memory
 
-template <int ROWS, bool kSized>
-__global__ void __cluster_dims__(kClu, 1, 1) __launch_bounds__(kT, ROWS <= 8 ? 2 : 1)  // two CTAs per SM where many units make more CTAs than SMs
-pool_select_cluster_kernel(const float* __restrict__ vote, float* __restrict__ pooled,
-                           uint32_t* __restrict__ bitmap, int32_t* __restrict__ kept_idx, int n_cand, int L,
-                           int pool, int k_sel, int n_kept, int bitmap_words, uint32_t* __restrict__ mask2,
-                           int n_calib, size_t vote_stride) {
-  __shared__ unsigned hist[kW][256];
-  __shared__ unsigned mine[2][256];   // this CTA's histogram of the current pass (double-buffered)
-  __shared__ unsigned total[256];
-  __shared__ unsigned sel_bin, sel_k;
-  __shared__ unsigned cnt[2][2];      // this CTA's counts of keys > T and == T, for the two thresholds
-  __shared__ unsigned wsum[ROWS * kW][2];
+struct SelectArgs {
+  const float* votes;     // [part][unit][stride]: the partial votes (or the caller's scores, one part)
+  float* vote_sum;        // out [units, n_cand]: the summed votes, or null
+  float* pooled;          // out [units, n_cand]
+  uint32_t* bitmap;       // out [units, bitmap_words]
+  uint32_t* mask2;        // out, kSized: bit set = not one of the calibrated evicted rows
+  int32_t* kept_idx;      // out [units, n_kept]
+  size_t stride, part_stride;
+  int n_parts, n_cand, L, pool, k_sel, n_kept, bitmap_words, n_calib;
+};
+
+template <int T, int ROWS, bool kSized>
+__global__ void __launch_bounds__(T)
+pool_select_cluster_kernel(const SelectArgs a) {
+  constexpr int kW = T / 32;
+  constexpr int kChunk = ROWS * T;
+  constexpr int kThr = kSized ? 2 : 1;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  unsigned* const hist = reinterpret_cast<unsigned*>(smem_raw);            // [kThr][256][32]
+  float* const stage = reinterpret_cast<float*>(hist + kThr * 256 * 32);   // [kChunk + 2 * kHaloMax]
+  __shared__ __align__(16) unsigned counts[2][kThr][kMaxClu][256];   // every CTA's histogram (double-buffered)
+  __shared__ unsigned sel_bin[kThr], sel_k[kThr], sel_all[kThr];
+  __shared__ unsigned cnt[kMaxClu][kThr][2];      // every CTA's keys > T and == T, per threshold
+  __shared__ unsigned wcnt[kThr][32][2];          // this CTA's, per warp
 
   pdl_trigger();
-  pdl_wait();
   cg::cluster_group cluster = cg::this_cluster();
-  const int rank = (int)cluster.block_rank();
+  const int rank = (int)cluster.block_rank(), n_clu = (int)cluster.num_blocks();
   const int unit = blockIdx.y;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int chunk = ROWS * kT;
-  const float* v = vote + (size_t)unit * vote_stride;
-  float* pl = pooled + (size_t)unit * n_cand;
-  uint32_t* bm = bitmap + (size_t)unit * bitmap_words;
-  int32_t* kept = kept_idx + (size_t)unit * n_kept;
+  for (int i = tid; i < kThr * 256 * 8; i += T) reinterpret_cast<uint4*>(hist)[i] = make_uint4(0u, 0u, 0u, 0u);
+  const int c0 = rank * kChunk;
+  const int n_cand = a.n_cand;
+  const int half = a.pool >> 1;
+  const float* v = a.votes + (size_t)unit * a.stride;
+  float* pl = a.pooled + (size_t)unit * n_cand;
+  uint32_t* bm = a.bitmap + (size_t)unit * a.bitmap_words;
+  int32_t* kept = a.kept_idx + (size_t)unit * a.n_kept;
+  const float fpool = (float)a.pool;
+  // (a CTA may store into a peer's shared memory only once the peer runs: waited for ahead of the first push)
+  if (n_clu > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  pdl_wait();
 
   // 1. zero-padded average pool with a constant divisor; keys stay in registers
-  unsigned key[ROWS];
-  const int half = pool >> 1;
-  const float fpool = (float)pool;
-#pragma unroll
-  for (int i = 0; i < ROWS; ++i) {
-    const int t = rank * chunk + i * kT + tid;
-    key[i] = 0u;
-    if (t < n_cand) {
-      float acc = 0.f;
-      for (int d = -half; d <= half; ++d) {
-        const int u = t + d;
-        if (u >= 0 && u < n_cand) acc += v[u];
-      }
-      const float p = acc / fpool;
-      pl[t] = p;
-      key[i] = __float_as_uint(p);
+  auto vote_at = [&](int t) {
+    float x = v[t];
+    for (int p = 1; p < a.n_parts; ++p) x += v[(size_t)p * a.part_stride + t];
+    return x;
+  };
+  const bool staged = half <= kHaloMax;
+  if (staged) {
+    const int n_stage = min(kChunk, n_cand - c0) + 2 * half;   // (not positive when only window rows are left)
+#pragma unroll 4
+    for (int i = tid; i < n_stage; i += T) {
+      const int t = c0 - half + i;
+      stage[i] = t >= 0 && t < n_cand ? vote_at(t) : 0.f;
     }
   }
-
-  // 2. radix select, most significant byte first; the histograms of the eight CTAs are summed
-  // through distributed shared memory.  Returns the bit pattern T of the kk-th largest pooled vote
-  // and how many candidates equal to T are still taken (those at the lowest positions).
-  auto radix_select = [&](unsigned kk, unsigned& T_out, unsigned& need_out) __attribute__((always_inline)) {
-    unsigned prefix = 0, k = kk;
-    for (int pass = 0; pass < 4; ++pass) {
-      const int shift = 24 - 8 * pass;
-      for (int i = tid; i < kW * 256; i += kT) (&hist[0][0])[i] = 0;
-      __syncthreads();
-#pragma unroll
-      for (int i = 0; i < ROWS; ++i) {
-        const int t = rank * chunk + i * kT + tid;
-        const bool in = t < n_cand && ((pass == 0) || ((key[i] >> (shift + 8)) == prefix));
-        if (in) atomicAdd(&hist[warp][(key[i] >> shift) & 255u], 1u);
-      }
-      __syncthreads();
-      if (tid < 256) {
-        unsigned s = 0;
-#pragma unroll 8
-        for (int w = 0; w < kW; ++w) s += hist[w][tid];
-        mine[pass & 1][tid] = s;
-      }
-      cluster.sync();
-      if (tid < 256) {
-        unsigned s = 0;
-        for (int r = 0; r < kClu; ++r) s += cluster.map_shared_rank(&mine[pass & 1][0], r)[tid];
-        total[tid] = s;
-      }
-      __syncthreads();
-      if (warp == 0) {
-        // lane 0 owns the 8 highest bins; walk bins downwards until k candidates are covered
-        const int base = 255 - 8 * lane;
-        unsigned c[8], s = 0;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) { c[j] = total[base - j]; s += c[j]; }
-        unsigned incl = s;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          unsigned n = __shfl_up_sync(0xffffffffu, incl, o);
-          if (lane >= o) incl += n;
-        }
-        const unsigned ball = __ballot_sync(0xffffffffu, incl >= k);
-        const int target = __ffs(ball) - 1;  // always found: the candidates number at least k
-        if (lane == target) {
-          unsigned run = incl - s;
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            if (run + c[j] >= k) { sel_bin = (unsigned)(base - j); sel_k = k - run; break; }
-            run += c[j];
-          }
-        }
-      }
-      __syncthreads();
-      prefix = (prefix << 8) | sel_bin;
-      k = sel_k;
-    }
-    // (the two passes that still use mine[] of this call lie at least two cluster barriers behind
-    // when the next call writes them again)
-    T_out = prefix;
-    need_out = k;
+  __syncthreads();
+  unsigned key[ROWS];
+  auto pooled_key = [&](int t, float acc) {
+    const float p = acc / fpool;
+    pl[t] = p;
+    return __float_as_uint(p);
   };
-  unsigned T, need_eq;
-  radix_select((unsigned)k_sel, T, need_eq);
-
-  // 3. ordered compaction.  Per (row, warp): how many keys are above T / equal to T; the exclusive
-  // scan of those counts in index order, over the cluster, gives every key the number of keys
-  // above / equal to the threshold that precede it.
-  unsigned gt_mask[ROWS], eq_mask[ROWS];
-  unsigned before_gt = 0, before_eq = 0;  // keys of the lower-ranked CTAs
-  auto scan_threshold = [&](unsigned Tx, int slot) __attribute__((always_inline)) {
+  auto pool_rows = [&](auto taps_tag) __attribute__((always_inline)) {
+    constexpr int kTaps = decltype(taps_tag)::value;
 #pragma unroll
     for (int i = 0; i < ROWS; ++i) {
-      const int t = rank * chunk + i * kT + tid;
-      const bool valid = t < n_cand;
-      gt_mask[i] = __ballot_sync(0xffffffffu, valid && key[i] > Tx);
-      eq_mask[i] = __ballot_sync(0xffffffffu, valid && key[i] == Tx);
-      if (lane == 0) {
-        wsum[i * kW + warp][0] = __popc(gt_mask[i]);
-        wsum[i * kW + warp][1] = __popc(eq_mask[i]);
+      const int tl = (warp * ROWS + i) * 32 + lane, t = c0 + tl;
+      key[i] = 0u;
+      if (t < n_cand) {
+        float acc = 0.f;
+#pragma unroll
+        for (int d = 0; d < kTaps; ++d) acc += stage[tl + d];
+        key[i] = pooled_key(t, acc);
+      }
+    }
+  };
+  switch (a.pool) {
+    case 1: pool_rows(std::integral_constant<int, 1>{}); break;
+    case 5: pool_rows(std::integral_constant<int, 5>{}); break;
+    case 7: pool_rows(std::integral_constant<int, 7>{}); break;
+    default:
+#pragma unroll
+      for (int i = 0; i < ROWS; ++i) {
+        const int tl = (warp * ROWS + i) * 32 + lane, t = c0 + tl;
+        key[i] = 0u;
+        if (t < n_cand) {
+          float acc = 0.f;
+          for (int d = -half; d <= half; ++d) {
+            if (staged) acc += stage[tl + half + d];
+            else if (t + d >= 0 && t + d < n_cand) acc += vote_at(t + d);
+          }
+          key[i] = pooled_key(t, acc);
+        }
+      }
+  }
+  if (a.vote_sum)
+    for (int i = tid; i < min(kChunk, n_cand - c0); i += T)
+      a.vote_sum[(size_t)unit * n_cand + c0 + i] = staged ? stage[i + half] : vote_at(c0 + i);
+  if (n_clu > 1) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+
+  // 2. radix select, most significant digit first.  thr[x] ends as the threshold of selection x, k[x] as the
+  // number of keys equal to it that are taken.
+  unsigned prefix[kThr], k[kThr], thr[kThr];
+  bool open[kThr];
+#pragma unroll
+  for (int x = 0; x < kThr; ++x) {
+    prefix[x] = 0u; thr[x] = 0u; open[x] = true;
+    k[x] = (unsigned)(a.k_sel + (x ? a.n_calib : 0));
+  }
+#pragma unroll 1
+  for (int pass = 0; pass < 4; ++pass) {
+    const int shift = pass == 3 ? 0 : 23 - 8 * pass, bits = pass == 3 ? 7 : 8;
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i) {
+      const bool valid = c0 + (warp * ROWS + i) * 32 + lane < n_cand;
+#pragma unroll
+      for (int x = 0; x < kThr; ++x)
+        if (valid && open[x] && (key[i] >> shift >> bits) == prefix[x])   // (pass 0: the sign bit, zero)
+          atomicAdd(hist + (x * 256 + ((key[i] >> shift) & ((1u << bits) - 1u))) * 32 + lane, 1u);
+    }
+    __syncthreads();
+    constexpr int kPer = 256 / kW;   // bins of a warp
+#pragma unroll
+    for (int x = 0; x < kThr; ++x) {
+      unsigned m = 0u;
+#pragma unroll
+      for (int j = 0; j < kPer; ++j) {
+        unsigned* h = hist + (x * 256 + warp * kPer + j) * 32 + lane;
+        const unsigned s = __reduce_add_sync(0xffffffffu, *h);
+        *h = 0u;
+        if (lane == j) m = s;
+      }
+      // pushed to every CTA of the cluster: stores to a peer cost no round trip, loads from it would
+      if (lane < kPer)
+        for (int r = 0; r < n_clu; ++r)
+          cluster.map_shared_rank(&counts[pass & 1][x][rank][0], r)[warp * kPer + lane] = m;
+    }
+    if (n_clu > 1) cluster.sync();
+    else __syncthreads();
+    // one warp per threshold: lane 0 owns the 8 highest bins; walk downwards until k keys are covered
+    if (warp < kThr) {
+      const int x = warp;
+      unsigned c[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+#pragma unroll
+      for (int r = 0; r < kMaxClu; ++r) {
+        const uint4* h = reinterpret_cast<const uint4*>(&counts[pass & 1][x][r][0]) + 2 * (31 - lane);
+        uint4 lo = make_uint4(0u, 0u, 0u, 0u), hi = lo;
+        if (r < n_clu) { lo = h[0]; hi = h[1]; }
+        c[7] += lo.x; c[6] += lo.y; c[5] += lo.z; c[4] += lo.w;
+        c[3] += hi.x; c[2] += hi.y; c[1] += hi.z; c[0] += hi.w;
+      }
+      unsigned p[8];
+      p[0] = c[0];
+#pragma unroll
+      for (int j = 1; j < 8; ++j) p[j] = p[j - 1] + c[j];
+      unsigned incl = p[7];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned n = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += n;
+      }
+      const unsigned kk = kSized && x == 1 ? k[kThr - 1] : k[0], before = incl - p[7];
+      if (before < kk && incl >= kk) {
+        unsigned run = before, skip = 0u, in_bin = c[0];
+#pragma unroll
+        for (int j = 0; j < 7; ++j)
+          if (before + p[j] < kk) { run = before + p[j]; skip = j + 1; in_bin = c[j + 1]; }
+        sel_bin[x] = 255u - 8u * lane - skip;
+        sel_k[x] = kk - run;
+        sel_all[x] = in_bin == kk - run;
       }
     }
     __syncthreads();
-    // exclusive scan of the ROWS * 32 warp counts in index order (row-major), by the first warp
-    if (warp == 0) {
-      unsigned run_gt = 0, run_eq = 0;
-      for (int base = 0; base < ROWS * kW; base += 32) {
-        const unsigned g0 = wsum[base + lane][0], e0 = wsum[base + lane][1];
-        unsigned ig = g0, ie = e0;
+    bool any = false;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const unsigned a = __shfl_up_sync(0xffffffffu, ig, o);
-          const unsigned b = __shfl_up_sync(0xffffffffu, ie, o);
-          if (lane >= o) { ig += a; ie += b; }
-        }
-        wsum[base + lane][0] = run_gt + ig - g0;
-        wsum[base + lane][1] = run_eq + ie - e0;
-        run_gt += __shfl_sync(0xffffffffu, ig, 31);
-        run_eq += __shfl_sync(0xffffffffu, ie, 31);
-      }
-      if (lane == 0) { cnt[slot][0] = run_gt; cnt[slot][1] = run_eq; }
+    for (int x = 0; x < kThr; ++x) {
+      if (!open[x]) continue;
+      prefix[x] = (prefix[x] << bits) | sel_bin[x];
+      thr[x] = prefix[x] << shift;
+      k[x] = sel_k[x];
+      // every key of the bin is taken: so is every key at or above the bin's lowest bit pattern
+      if (sel_all[x]) { k[x] = 0xffffffffu; open[x] = false; }
+      any |= open[x];
     }
-    cluster.sync();
-    before_gt = before_eq = 0;
-    for (int r = 0; r < rank; ++r) {
-      const unsigned* c = cluster.map_shared_rank(&cnt[slot][0], r);
-      before_gt += c[0];
-      before_eq += c[1];
-    }
-  };
-  // is key (row i, this thread) among the first `need` keys equal to Tx or above Tx ?
-  const unsigned lt = (1u << lane) - 1u;
-  auto taken = [&](int i, unsigned Tx, unsigned need) __attribute__((always_inline)) {
-    const unsigned eq_before = before_eq + wsum[i * kW + warp][1] + __popc(eq_mask[i] & lt);
-    return key[i] > Tx || (key[i] == Tx && eq_before < need);
-  };
+    if (!any) break;
+  }
 
-  scan_threshold(T, 0);
-  unsigned take_bits = 0;   // bit i: this thread's key of row i was selected
+  // 3. ordered compaction.  Number of keys above / equal to a threshold in the warps and CTAs ahead of this warp.
+  unsigned before_gt[kThr], before_eq[kThr];
+#pragma unroll
+  for (int x = 0; x < kThr; ++x) {
+    unsigned g = 0u, e = 0u;
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i) {
+      const bool valid = c0 + (warp * ROWS + i) * 32 + lane < n_cand;
+      g += __popc(__ballot_sync(0xffffffffu, valid && key[i] > thr[x]));
+      e += __popc(__ballot_sync(0xffffffffu, valid && key[i] == thr[x]));
+    }
+    if (lane == 0) { wcnt[x][warp][0] = g; wcnt[x][warp][1] = e; }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int x = 0; x < kThr; ++x) {
+    const unsigned g = lane < kW ? wcnt[x][lane][0] : 0u, e = lane < kW ? wcnt[x][lane][1] : 0u;
+    before_gt[x] = __reduce_add_sync(0xffffffffu, lane < warp ? g : 0u);
+    before_eq[x] = __reduce_add_sync(0xffffffffu, lane < warp ? e : 0u);
+    if (n_clu > 1 && warp == 0) {
+      const unsigned sg = __reduce_add_sync(0xffffffffu, g), se = __reduce_add_sync(0xffffffffu, e);
+      if (lane < n_clu) {
+        unsigned* c = cluster.map_shared_rank(&cnt[rank][x][0], lane);
+        c[0] = sg; c[1] = se;
+      }
+    }
+  }
+  if (n_clu > 1) {
+    // the last time a CTA touches a peer's shared memory lies ahead of this barrier: it may leave afterwards
+    cluster.sync();
+#pragma unroll
+    for (int x = 0; x < kThr; ++x) {
+      before_gt[x] += __reduce_add_sync(0xffffffffu, lane < rank ? cnt[lane][x][0] : 0u);
+      before_eq[x] += __reduce_add_sync(0xffffffffu, lane < rank ? cnt[lane][x][1] : 0u);
+    }
+  }
+  const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
   for (int i = 0; i < ROWS; ++i) {
-    const int t = rank * chunk + i * kT + tid;
-    const unsigned gt_before = before_gt + wsum[i * kW + warp][0] + __popc(gt_mask[i] & lt);
-    const unsigned eq_before = before_eq + wsum[i * kW + warp][1] + __popc(eq_mask[i] & lt);
-    bool take = false;
-    if (t < n_cand) {
-      take = taken(i, T, need_eq);
-      if (take) kept[gt_before + min(eq_before, need_eq)] = t;
-    } else if (t < L) {
-      take = true;  // observation-window rows are always kept
-    }
-    take_bits |= (take ? 1u : 0u) << i;
+    const int t0 = c0 + (warp * ROWS + i) * 32, t = t0 + lane;
+    const bool valid = t < n_cand;
+    const unsigned gm = __ballot_sync(0xffffffffu, valid && key[i] > thr[0]);
+    const unsigned em = __ballot_sync(0xffffffffu, valid && key[i] == thr[0]);
+    const unsigned gt_before = before_gt[0] + __popc(gm & lt), eq_before = before_eq[0] + __popc(em & lt);
+    before_gt[0] += __popc(gm);
+    before_eq[0] += __popc(em);
+    // (observation-window rows are always kept)
+    const bool sel = valid && (key[i] > thr[0] || (key[i] == thr[0] && eq_before < k[0]));
+    if (sel) kept[gt_before + min(eq_before, k[0])] = t;
+    const bool take = sel || (!valid && t < a.L);
     const unsigned word = __ballot_sync(0xffffffffu, take);
-    const int t0 = rank * chunk + i * kT + warp * 32;
-    if (lane == 0 && t0 < L) bm[t0 >> 5] = word;
+    if (lane == 0 && t0 < a.L) bm[t0 >> 5] = word;
+    if (kSized) {
+      // calibration size: the candidates among the first k_sel + n_calib that were not selected
+      constexpr int y = kThr - 1;
+      const unsigned em2 = __ballot_sync(0xffffffffu, valid && key[i] == thr[y]);
+      const bool in2 = valid && (key[i] > thr[y] || (key[i] == thr[y] && before_eq[y] + __popc(em2 & lt) < k[y]));
+      before_eq[y] += __popc(em2);
+      const unsigned word2 = ~__ballot_sync(0xffffffffu, in2 && !take);
+      if (lane == 0 && t0 < a.L) a.mask2[(size_t)unit * a.bitmap_words + (t0 >> 5)] = word2;
+    }
   }
   // the window rows close the kept list
   if (rank == 0)
-    for (int j = tid; j < L - n_cand; j += kT) kept[k_sel + j] = n_cand + j;
-
-  // 4. calibration size: the next n_calib candidates in the same order, i.e. those among the first
-  // k_sel + n_calib that were not selected.  mask2: bit set = the row is NOT one of them.
-  if (kSized) {
-    uint32_t* bm2 = mask2 + (size_t)unit * bitmap_words;
-    unsigned T2, need2;
-    __syncthreads();   // wsum and the flags of step 3 have been read by every thread of this CTA
-    radix_select((unsigned)(k_sel + n_calib), T2, need2);
-    scan_threshold(T2, 1);
-#pragma unroll
-    for (int i = 0; i < ROWS; ++i) {
-      const int t = rank * chunk + i * kT + tid;
-      const bool member = t < n_cand && !((take_bits >> i) & 1u) && taken(i, T2, need2);
-      const unsigned word = ~__ballot_sync(0xffffffffu, member);
-      const int t0 = rank * chunk + i * kT + warp * 32;
-      if (lane == 0 && t0 < L) bm2[t0 >> 5] = word;
-    }
-  }
-  cluster.sync();  // no CTA leaves while another may still read its shared memory
+    for (int j = tid; j < a.L - n_cand; j += T) kept[a.k_sel + j] = n_cand + j;
 }
 
-template <int ROWS>
-void launch_rows(const CompressGeom& g, const CompressWs& ws, char* wsp, const float* scores, size_t stride,
-                 int32_t* kept_idx, cudaStream_t st) {
-  // (the cluster shape is the kernel's own attribute; the launch adds programmatic serialisation)
-  if (g.sized && g.n_calib > 0)
-    launch_pdl(pool_select_cluster_kernel<ROWS, true>, dim3(kClu, g.units), dim3(kT), 0, st, scores,
-               (float*)(wsp + ws.pooled), (uint32_t*)(wsp + ws.bitmap), kept_idx, g.n_cand, g.L, g.pool, g.k_sel, g.n_kept,
-               g.bitmap_words, (uint32_t*)(wsp + ws.bitmap2), g.n_calib, stride);
-  else
-    launch_pdl(pool_select_cluster_kernel<ROWS, false>, dim3(kClu, g.units), dim3(kT), 0, st, scores,
-               (float*)(wsp + ws.pooled), (uint32_t*)(wsp + ws.bitmap), kept_idx, g.n_cand, g.L, g.pool, g.k_sel, g.n_kept,
-               g.bitmap_words, (uint32_t*)nullptr, 0, stride);
+template <int T, int ROWS, bool kSized>
+cudaError_t launch_select(const SelectArgs& a, int units, cudaStream_t st) {
+  constexpr int kSmem = (kSized ? 2 : 1) * 256 * 32 * 4 + (ROWS * T + 2 * kHaloMax) * 4;
+  static bool attr_set[64] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64 || !attr_set[dev]) {
+    e = cudaFuncSetAttribute(pool_select_cluster_kernel<T, ROWS, kSized>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+    if (e != cudaSuccess) return e;
+    if (dev >= 0 && dev < 64) attr_set[dev] = true;
+  }
+  const int n_clu = (a.L + T * ROWS - 1) / (T * ROWS);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(n_clu, units);
+  cfg.blockDim = dim3(T);
+  cfg.dynamicSmemBytes = kSmem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = n_clu;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  e = cudaLaunchKernelEx(&cfg, pool_select_cluster_kernel<T, ROWS, kSized>, a);
+  count_launch(1);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+template <bool kSized>
+cudaError_t launch_any(const SelectArgs& a, int units, cudaStream_t st) {
+  // The fewest keys per thread with which all clusters of the call are resident at once, two CTAs of 512
+  // threads per SM: the work per thread is what a pass waits for (1024-thread CTAs with 16 keys per thread:
+  // 32 units x 32768 keys 29.0 us instead of 20.6, 64 x 16384 25.2 instead of 18.8), but clusters beyond a
+  // full GPU would queue.  Below 2048 keys per CTA nothing is gained (1024 threads with one or two keys: equal).
+  auto clusters = [&](int chunk) { return (a.L + chunk - 1) / chunk; };
+  auto fits = [&](int rows) {
+    const int c = clusters(512 * rows);
+    return c <= kMaxClu && (long long)c * units <= 2 * 148;
+  };
+  if (fits(4)) return launch_select<512, 4, kSized>(a, units, st);
+  if (fits(8)) return launch_select<512, 8, kSized>(a, units, st);
+  if (a.L <= kMaxClu * 512 * 16) return launch_select<512, 16, kSized>(a, units, st);
+  if (a.L <= kMaxClu * 1024 * 16) return launch_select<1024, 16, kSized>(a, units, st);
+  return launch_select<1024, 32, kSized>(a, units, st);
 }
 
 }  // namespace
 
 // The cluster kernel keeps at most 32 keys per thread: 8 CTAs x 1024 threads x 32.
-bool select_cluster_supported(const CompressGeom& g) { return !g.keep_all && g.L <= kClu * kT * 32; }
+bool select_cluster_supported(const CompressGeom& g) { return !g.keep_all && g.L <= kMaxClu * 1024 * 32; }
 
-// Selection from per-candidate scores [units][stride] (the window votes of the workspace, or a
-// caller's scores).
+// Selection from per-candidate scores [parts][units][stride] (the window votes of the workspace, or a
+// caller's scores); vote_sum receives the sum of the parts when it is not null.
 cudaError_t launch_pool_select_scores(const CompressGeom& g, const CompressWs& ws, char* wsp, const float* scores,
-                                      size_t stride, int32_t* kept_idx, cudaStream_t st) {
-  const int rows = (g.L + kClu * kT - 1) / (kClu * kT);
-  if (rows <= 1) launch_rows<1>(g, ws, wsp, scores, stride, kept_idx, st);
-  else if (rows <= 2) launch_rows<2>(g, ws, wsp, scores, stride, kept_idx, st);
-  else if (rows <= 4) launch_rows<4>(g, ws, wsp, scores, stride, kept_idx, st);
-  else if (rows <= 8) launch_rows<8>(g, ws, wsp, scores, stride, kept_idx, st);
-  else if (rows <= 16) launch_rows<16>(g, ws, wsp, scores, stride, kept_idx, st);
-  else launch_rows<32>(g, ws, wsp, scores, stride, kept_idx, st);
-  count_launch(1);
-  return cudaGetLastError();
+                                      size_t stride, int n_parts, size_t part_stride, float* vote_sum,
+                                      int32_t* kept_idx, cudaStream_t st) {
+  SelectArgs a{};
+  a.votes = scores;
+  a.vote_sum = vote_sum;
+  a.pooled = (float*)(wsp + ws.pooled);
+  a.bitmap = (uint32_t*)(wsp + ws.bitmap);
+  a.kept_idx = kept_idx;
+  a.stride = stride; a.part_stride = part_stride; a.n_parts = n_parts;
+  a.n_cand = g.n_cand; a.L = g.L; a.pool = g.pool; a.k_sel = g.k_sel; a.n_kept = g.n_kept;
+  a.bitmap_words = g.bitmap_words;
+  if (g.sized && g.n_calib > 0) {
+    a.mask2 = (uint32_t*)(wsp + ws.bitmap2);
+    a.n_calib = g.n_calib;
+    return launch_any<true>(a, g.units, st);
+  }
+  return launch_any<false>(a, g.units, st);
 }
 
 cudaError_t launch_pool_select_cluster(const CompressGeom& g, const CompressWs& ws, char* wsp, int32_t* kept_idx,
                                        cudaStream_t st) {
-  return launch_pool_select_scores(g, ws, wsp, (const float*)(wsp + ws.vote), (size_t)g.n_cand, kept_idx, st);
+  return launch_pool_select_scores(g, ws, wsp, (const float*)(wsp + ws.vote), (size_t)g.n_cand, 1, 0, nullptr, kept_idx,
+                                   st);
 }
 
 // Sink-plus-recent index rule: the first n_sink rows and the last n_kept - n_sink.

@@ -76,6 +76,36 @@ def test_single_cta_selection_for_very_long_prompts(cuda_lib):
     decode_steps_compare(g, ref, q, kn, vn, steps=2)
 
 
+@pytest.mark.parametrize("units,L,tail,pool,budget", [
+    (1, 2048, 7, 1, 100),          # a full single CTA
+    (3, 2049, 1, 7, 2048),         # the second CTA of the cluster holds one window row and no candidate
+    (2, 16384, 16, 5, 600),        # eight CTAs of 512 x 4, full
+    (2, 16385, 16, 3, 16384),      # five CTAs of 512 x 8, one row evicted
+    (40, 16390, 8, 7, 64),         # more clusters than fit at 4 and 8 keys per thread
+    (1, 70000, 32, 131, 5000),     # 1024 threads x 16 keys, a pool wider than the staged halo
+    (1, 140000, 32, 9, 40000),     # 1024 threads x 32 keys
+])
+@pytest.mark.parametrize("ties", [False, True])
+def test_selection_from_scores_at_the_edges_of_its_launch_shapes(cuda_lib, units, L, tail, pool, budget, ties):
+    """Kept lists against a stable sort.  The scores are multiples of 2^-6 below 8 (`ties`: only eight distinct
+    values, whole runs equal to the threshold), so every pooled sum is exact and the order has no rounding."""
+    cd = cuda_lib
+    rng = np.random.Generator(np.random.Philox(key=[61, L + ties]))
+    scores = rng.integers(0, 8 if ties else 512, size=(1, units, L)).astype(np.float32) / 64
+    p = cd.make_params(B=1, Hq=units, Hkv=units, L=L, window=min(tail, 8), pool=pool, budget=budget, n_cal=1, cap=budget)
+    ws = torch.empty((cd.calidrop_compress_workspace_bytes(p),), dtype=torch.uint8, device="cuda")
+    kept = torch.full((1, units, budget), -1, dtype=torch.int32, device="cuda")
+    cd.calidrop_select_from_scores(p, torch.from_numpy(scores).cuda(), tail, kept, ws)
+    got = kept.cpu().numpy()[0]
+    n = L - tail
+    for u in range(units):
+        csum = np.concatenate([[0.0], np.cumsum(scores[0, u, :n].astype(np.float64))])
+        t = np.arange(n)
+        pooled = csum[np.minimum(t + pool // 2 + 1, n)] - csum[np.maximum(t - pool // 2, 0)]
+        want = np.sort(np.argsort(-pooled, kind="stable")[:budget - tail])
+        np.testing.assert_array_equal(got[u], np.concatenate([want, np.arange(n, L)]))
+
+
 @pytest.mark.parametrize("calib_size", [1, 40, 300, 10 ** 6, -1])
 def test_calibration_size(cuda_lib, calib_size):
     """Section 4.4's calibration size m: only the m evicted rows of highest pooled vote are calibrated
