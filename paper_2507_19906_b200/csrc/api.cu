@@ -78,7 +78,8 @@ CompressWs make_ws(const CompressGeom& g) {
   size_t off = 0;
   const size_t n_cand = (size_t)(g.L > g.W ? g.L - g.W : 0);
   w.vote = off;    off = align_up(off + (size_t)g.units * n_cand * 4, 256);
-  w.vote2 = off;   off = align_up(off + (g.G * g.W > 256 ? (size_t)g.units * n_cand * 4 : 0), 256);
+  w.vote_parts = off;
+  if (score_tc_supported(g)) off = align_up(off + votes_tc_parts(g) * (size_t)g.units * n_cand * 4, 256);
   w.pooled = off;  off = align_up(off + (size_t)g.units * n_cand * 4, 256);
   w.row_lse = off; off = align_up(off + (size_t)g.B * g.Hq * g.W * 4, 256);
   w.bitmap = off;  off = align_up(off + (size_t)g.units * g.bitmap_words * 4, 256);
@@ -263,8 +264,12 @@ int calidrop_compress(const calidrop_params* p, const void* Q_obs, const void* K
     e = tc_path ? launch_votes_tc(g, ws, Q_obs, K, row_lse, wsp, st) : launch_votes(g, ws, Q_obs, K, row_lse, wsp, st);
     if (e != cudaSuccess) return cuda_fail(e);
   }
-  e = select_cluster_supported(g) ? launch_pool_select_cluster(g, ws, wsp, kept_idx, st)
-                                  : launch_pool_select(g, ws, wsp, kept_idx, st);
+  if (select_cluster_supported(g)) {
+    e = launch_pool_select_cluster(g, ws, wsp, tc_path, kept_idx, st);
+  } else {
+    if (tc_path && (e = launch_add_votes(g, ws, wsp, st)) != cudaSuccess) return cuda_fail(e);
+    e = launch_pool_select(g, ws, wsp, kept_idx, st);
+  }
   if (e != cudaSuccess) return cuda_fail(e);
   // the compaction of the retained rows rides on the calibration's second kernel when that runs
   const bool calib_tc = tc_path && calib_tc_supported(g) && !(g.sized && g.n_calib == 0);

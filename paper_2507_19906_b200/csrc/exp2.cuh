@@ -1,0 +1,75 @@
+// exp2 on two pipes.  The special-function unit gives one ex2 per 8 cycles and scheduler for a warp; a softmax
+// over logits that the tensor cores deliver needs nothing else as much, so that unit is what the scoring
+// kernels wait for.  A share of the exponentials is therefore evaluated on the FMA pipe, on PAIRS of values
+// (the packed fp32 instructions do two per issue slot): 2^x = 2^n 2^f with n = round(x), f in [-1/2, 1/2], the
+// second factor a polynomial of degree 5, the first an integer addition to the exponent field.
+// The coefficients are the minimax polynomial of 2^f on [-1/2, 1/2] in relative error (Remez exchange, then
+// rounded to fp32): 7.5e-8, evaluated in fp32 2.1e-7, which is what ex2.approx gives.
+// Measured in a bare loop over accumulators in tensor memory, four warps per scheduler, cycles per warp-wide
+// exponential and scheduler: ex2 on scalars 8.8, on packed arguments 8.6; with 2, 4, 5, 6, 8, 16 pairs of 16 on the
+// polynomial 7.6, 6.9, 6.6, 6.7, 7.7, 12.0.  In the vote kernel, beside its MMAs (32 units x 32768 keys, thousand
+// cycles): 170 without, 131, 133, 135, 138 with 3, 4, 5, 6 of 16.  Hence 3.  (With unpacked arithmetic the polynomial
+// costs ten issue slots per value, and any share of it loses.)
+#pragma once
+
+#include "common.cuh"
+
+namespace calidrop {
+
+using f32x2 = unsigned long long;   // two fp32 in one 64-bit register pair
+
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 pack2(uint32_t a, uint32_t b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(a), "r"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 pack2(float a) { return pack2(a, a); }
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 d;
+  asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
+// 2^x for x <= 127; below -126 (and for -inf) the result is 2^-126 instead of 0.
+__device__ __forceinline__ f32x2 exp2_poly2(f32x2 x) {
+  constexpr float kRound = 12582912.f;   // 1.5 * 2^23: adding it rounds to an integer in the low mantissa bits
+  const float2 v = unpack2(x);
+  x = pack2(fmaxf(v.x, -126.f), fmaxf(v.y, -126.f));
+  const f32x2 t = add2(x, pack2(kRound));
+  const f32x2 f = fma2(add2(t, pack2(-kRound)), pack2(-1.f), x);
+  f32x2 p = fma2(pack2(0.0013276472454890609f), f, pack2(0.009675540961325169f));
+  p = fma2(p, f, pack2(0.05550713092088699f));
+  p = fma2(p, f, pack2(0.24022120237350464f));
+  p = fma2(p, f, pack2(0.6931469440460205f));
+  p = fma2(p, f, pack2(1.0000001192092896f));
+  const float2 pv = unpack2(p), tv = unpack2(t);
+  return pack2(__float_as_uint(pv.x) + (__float_as_uint(tv.x) << 23), __float_as_uint(pv.y) + (__float_as_uint(tv.y) << 23));
+}
+
+__device__ __forceinline__ f32x2 exp2_unit2(f32x2 x) {
+  const float2 v = unpack2(x);
+  return pack2(ex2_approx(v.x), ex2_approx(v.y));
+}
+
+// Pair i of every 16 goes to the polynomial for kPolyPairs of them, evenly spread.
+constexpr int kPolyPairs = 3;
+__host__ __device__ constexpr bool exp2_pair_on_poly(int i) {
+  return ((i % 16 + 1) * kPolyPairs) / 16 > ((i % 16) * kPolyPairs) / 16;
+}
+
+}  // namespace calidrop

@@ -25,7 +25,7 @@ struct CompressGeom {
 
 // Workspace carving of compress (byte offsets, all 256-byte aligned).
 struct CompressWs {
-  size_t vote, vote2, pooled, row_lse, bitmap, stat_part, status, calib_o, calib_l, total;
+  size_t vote, vote_parts, pooled, row_lse, bitmap, stat_part, status, calib_o, calib_l, total;
   size_t bitmap2;     // sized calibration: bit set = the row is NOT one of the calibrated evicted rows
   size_t calib_mask;  // the bitmap the calibration passes mask with: bitmap, or bitmap2 when sized
   int n_tiles;     // 128-key tiles per unit (scalar statistics pass: one partial per tile)
@@ -98,6 +98,8 @@ cudaError_t launch_row_stats_tc(const CompressGeom& g, const CompressWs& ws, con
                                 char* wsp, cudaStream_t st);
 cudaError_t launch_votes_tc(const CompressGeom& g, const CompressWs& ws, const void* Q_obs, const void* K,
                             const float* row_lse, char* wsp, cudaStream_t st);
+int votes_tc_parts(const CompressGeom& g);
+cudaError_t launch_add_votes(const CompressGeom& g, const CompressWs& ws, char* wsp, cudaStream_t st);
 bool calib_tc_supported(const CompressGeom& g);
 void calib_tc_plan(const CompressGeom& g, int* gpb, int* n_cblocks, int* tiles_per_cta, int* max_slots,
                    size_t* parts);
@@ -135,8 +137,8 @@ cudaError_t launch_pool_select(const CompressGeom& g, const CompressWs& ws, char
                                int32_t* kept_idx, cudaStream_t st);
 // select_cluster.cu
 bool select_cluster_supported(const CompressGeom& g);
-cudaError_t launch_pool_select_cluster(const CompressGeom& g, const CompressWs& ws, char* wsp, int32_t* kept_idx,
-                                       cudaStream_t st);
+cudaError_t launch_pool_select_cluster(const CompressGeom& g, const CompressWs& ws, char* wsp, bool in_parts,
+                                       int32_t* kept_idx, cudaStream_t st);
 cudaError_t launch_pool_select_scores(const CompressGeom& g, const CompressWs& ws, char* wsp, const float* scores,
                                       size_t stride, int n_parts, size_t part_stride, float* vote_sum,
                                       int32_t* kept_idx, cudaStream_t st);

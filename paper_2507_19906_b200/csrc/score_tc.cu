@@ -8,8 +8,12 @@
 // the CTA's range crosses into the next virtual unit.
 // Warp roles: four consumer warpgroups in two pairs read the accumulators out of TMEM (one TMEM
 // lane per thread; pair p drains accumulator buffer p, each of its groups half of the columns), one
-// warp is the TMA producer, one warp allocates TMEM and issues the MMAs.  Every MMA has N = 256 where the shape allows it: with both operands in
-// shared memory, narrower tiles are limited by operand fetch, not by the tensor pipe.
+// warp is the TMA producer, one warp allocates TMEM and issues the MMAs.  What bounds both kernels is the
+// exponentials, one per logit; see exp2.cuh.  32 units x 256 rows x 32768 keys: statistics 170 -> 138 thousand
+// cycles (ncu, 92 -> 84 us at the clock the power limit leaves), votes 172 -> 131 (94 -> 80 us), with a share
+// of the exponentials on the FMA pipe and the work between two jobs cut down; either alone gave little (the
+// polynomial without the other change: 173 and 189 thousand cycles).  Every MMA has N = 256 where the shape allows
+// it: with both operands in shared memory, narrower tiles are limited by operand fetch, not by the tensor pipe.
 //
 //   statistics (kVotes = false):  S = Q K^T, 128 query rows on the TMEM lanes, 256 keys per tile.
 //       Thread r keeps the running (max, sum) of exp2(scale2 * s) over the keys row r may see
@@ -18,8 +22,11 @@
 //   votes (kVotes = true):  S^T = K Q^T, 128 KEYS on the TMEM lanes and up to 256 query rows as
 //       columns, so the vote of a key, sum over rows of exp2(scale2 * s - lse2[row]), is a
 //       per-thread sum over the accumulator's columns: no cross-thread reduction and fp32
-//       probabilities throughout.  Candidate keys (t < L - W) are seen by every window row, so this
-//       pass needs no mask.
+//       probabilities throughout.  The groups' halves go out as parts that the selection adds up.
+//       Candidate keys (t < L - W) are seen by every window row, so this pass needs no mask.
+#include <type_traits>
+
+#include "exp2.cuh"
 #include "internal.h"
 #include "tc_common.cuh"
 
@@ -33,9 +40,8 @@ constexpr int kGroups = 4;  // consumer warpgroups (4 warps each), two pairs; pa
 constexpr int kProducerWarp = kGroups * 4;
 constexpr int kMmaWarp = kGroups * 4 + 1;
 constexpr int kThreads = kGroups * 128 + 64;
-constexpr int kTmemCols = 512;  // two accumulators of 256 columns
-constexpr int kBufCols = 256;
-constexpr int kNumBufs = 2;
+constexpr int kTmemCols = 512;  // two accumulators of 256 columns or four of 128
+constexpr int kMaxBufs = 4;
 constexpr int kMaxRows = 512;   // G * W handled by the tiles
 constexpr int kSms = 148;
 
@@ -49,26 +55,26 @@ struct ScoreArgs {
   int total_tiles;    // virtual units * n_tiles
   int tiles_per_cta;
   int stages;         // depth of the key-tile ring
+  int lg_bufs;        // log2 of the accumulator count: two of 256 columns, or four of 128
   int max_slots;      // statistics: partial slots per row (CTAs that can share a virtual unit)
   float scale2;
   const float* row_lse;  // votes: natural-log LSE of every observation row [B, Hq, W]
-  float* vote;           // votes: out [units, n_cand]
-  float* vote2;          // with several row blocks per tile: the partial votes of warpgroup 1 (added to vote afterwards)
-  float2* stat_part;     // statistics: out [row][slot][group] (max, sum) in the log2 domain
+  float* vote_parts;     // votes: out [part][units, n_cand], a part per (row block, column half)
+  float2* stat_part;     // statistics: out [row][slot][2 or 4 groups] (max, sum) in the log2 domain
   unsigned* status;
 };
 
-// exp2 of 32 logits against one reference, four independent partial sums
-__device__ __forceinline__ float sum_exp2_32(const uint32_t (&r)[32], float scale2, float neg_ref) {
-  float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+// sum of exp2 of 32 logits against one reference, four independent partial sums
+__device__ __forceinline__ float sum_exp2_32(const uint32_t (&r)[32], f32x2 sc, f32x2 nr) {
+  f32x2 s0 = 0ull, s1 = 0ull;
 #pragma unroll
   for (int e = 0; e < 32; e += 4) {
-    s0 += ex2_approx(fmaf(__uint_as_float(r[e + 0]), scale2, neg_ref));
-    s1 += ex2_approx(fmaf(__uint_as_float(r[e + 1]), scale2, neg_ref));
-    s2 += ex2_approx(fmaf(__uint_as_float(r[e + 2]), scale2, neg_ref));
-    s3 += ex2_approx(fmaf(__uint_as_float(r[e + 3]), scale2, neg_ref));
+    const f32x2 x0 = fma2(pack2(r[e], r[e + 1]), sc, nr), x1 = fma2(pack2(r[e + 2], r[e + 3]), sc, nr);
+    s0 = add2(s0, exp2_pair_on_poly(e / 2) ? exp2_poly2(x0) : exp2_unit2(x0));
+    s1 = add2(s1, exp2_pair_on_poly(e / 2 + 1) ? exp2_poly2(x1) : exp2_unit2(x1));
   }
-  return (s0 + s1) + (s2 + s3);
+  const float2 v = unpack2(add2(s0, s1));
+  return v.x + v.y;
 }
 
 __device__ __forceinline__ float max_32(const uint32_t (&r)[32]) {
@@ -91,13 +97,11 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
   constexpr int TILE_KEYS = kVotes ? 128 : 256;
   constexpr uint32_t STAGE_BYTES = TILE_KEYS * 256;
   extern __shared__ unsigned char smem_raw[];
-  __shared__ __align__(8) unsigned long long bars[22];
+  __shared__ __align__(8) unsigned long long bars[18];
   __shared__ uint32_t tmem_slot;
   __shared__ Ctl ctl;
-  // votes: -lse2 of the columns this warp reads (128 per row block at most), one copy per warp
-  __shared__ __align__(16) float nlse2_s[kVotes ? kGroups * 4 : 1][kVotes ? 256 : 4];
-  __shared__ float vx[2][128];  // votes: partial vote of the second column half, per pair
-  __shared__ float2 ml_s[kVotes ? 1 : kGroups][kVotes ? 1 : 2][kVotes ? 1 : 128];       // running (max, sum)
+  // votes: -lse2 of the columns this warp reads, one copy per warp
+  __shared__ __align__(16) float nlse2_s[kVotes ? kGroups * 4 : 1][kVotes ? 128 : 4];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int cta = blockIdx.x;
@@ -120,8 +124,6 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
   auto empty_k = [&](int s) { return bar0 + 8u * (6 + s); };
   auto t_full = [&](int b) { return bar0 + 8u * (10 + b); };
   auto t_empty = [&](int b) { return bar0 + 8u * (14 + b); };
-  auto vx_full = [&](int b) { return bar0 + 8u * (18 + b); };
-  auto vx_empty = [&](int b) { return bar0 + 8u * (20 + b); };
 
   if (tid == 0) {
     ctl.abort = 0;
@@ -129,9 +131,9 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
     mbar_init(q_full, 1);
     mbar_init(q_empty, 1);
     for (int s = 0; s < 4; ++s) { mbar_init(full_k(s), 1); mbar_init(empty_k(s), 1); }
-    for (int b = 0; b < kNumBufs; ++b) {
-      mbar_init(t_full(b), 1); mbar_init(t_empty(b), 256);   // a buffer is drained by one pair of warpgroups
-      mbar_init(vx_full(b), 128); mbar_init(vx_empty(b), 128);
+    for (int b = 0; b < kMaxBufs; ++b) {
+      mbar_init(t_full(b), 1);
+      mbar_init(t_empty(b), a.lg_bufs == 2 ? 128 : 256);   // a buffer is drained by one group or by a pair of them
     }
     fence_mbar_init();
   }
@@ -194,13 +196,13 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
         bool ok = true;
         const uint64_t kd = desc_advance(dk0, (uint32_t)s * STAGE_BYTES);
         for (int blk = 0; blk < a.n_blocks; ++blk, ++j) {
-          const int buf = j & (kNumBufs - 1);
-          if (!mbar_wait(&ctl, t_empty(buf), ((j / kNumBufs) & 1) ^ 1, (kVotes ? 34u : 14u) | ((unsigned)j << 8))) {
+          const int buf = j & ((1 << a.lg_bufs) - 1);
+          if (!mbar_wait(&ctl, t_empty(buf), ((j >> a.lg_bufs) & 1) ^ 1, (kVotes ? 34u : 14u) | ((unsigned)j << 8))) {
             ok = false;
             break;
           }
           tc_fence_after_sync();
-          const uint32_t d = tmem_base + (uint32_t)(buf * kBufCols);
+          const uint32_t d = tmem_base + (uint32_t)(buf << (9 - a.lg_bufs));
           const uint64_t qd = desc_advance(dq0, (uint32_t)blk * q_blk_bytes);
           // the second halves (k-steps 4..7) start half a tile further on
           const uint64_t kd2 = desc_advance(kd, STAGE_BYTES / 2), qd2 = desc_advance(qd, q_half_bytes);
@@ -222,164 +224,145 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
   } else {
     // ------------------------------------------------------------ accumulator consumers
     // Thread ct of warpgroup grp owns TMEM lane ct.  The four groups form two pairs; the jobs (key
-    // tile, row block) alternate between the pairs: pair p drains accumulator buffer p, i.e. every
-    // job whose index has parity p, each of its two groups half of the columns.  The pairs run half
-    // a job apart: while one waits for the MMAs of its next job (which cannot start before the
-    // last columns of the current one have been read), the other, two warps per scheduler, keeps the
-    // exponential unit busy; one warp per scheduler alone reaches less than half of that unit's rate.
-    // (Measured at config 3, votes: two groups on the same job 110 us, the groups stalling together
-    // at every job boundary; two groups on alternate jobs 100 us; four accumulators of 128 columns
-    // 110 us, the narrower MMAs costing more than the wait they hide.)
+    // tile, row block) alternate between the pairs: pair p drains accumulator buffer p, each of its two
+    // groups half of the columns.  With two row blocks a pair therefore always has the same one, with one
+    // every second tile.  Votes of at most 128 window rows have four accumulators instead, one per group:
+    // a job is as long as with 256 rows, where half a job per group would double what lies between two
+    // (64 units x 128 rows x 16384 keys: @16k@ us).  While one pair waits for the MMAs of its next job (which cannot start before
+    // the last columns of the current one have been read), the other, two warps per scheduler, keeps
+    // the exponentials going; one warp per scheduler alone reaches less than half of their rate.
+    // (Measured at 32 units x 32768 keys, votes: two groups on the same job 110 us, the groups stalling
+    // together at every job boundary; two groups on alternate jobs 100 us; four accumulators of 128
+    // columns 110 us, the narrower MMAs costing more than the wait they hide.)
+    // What is left between two jobs is kept to a handful of instructions: everything that depends on
+    // the virtual unit is worked out per segment (a run of tiles of one virtual unit), a job's own state
+    // is a tile base and a phase bit, and the halves of a vote go out as they are, to be added by the
+    // selection.  A warp's dependent scalar instructions cost some five cycles each: with a loop over
+    // tiles and blocks, the running statistics in shared memory and the halves of a vote meeting there,
+    // a job carried 190 instructions besides its exponentials, 800 cycles of about 5500.
     const int grp = warp >> 2, ct = tid & 127;
     const int pair = grp >> 1, half = grp & 1;
-    const uint32_t lane_base = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
-    int cur_vu = -1, j = 0;
+    const bool alone = kVotes && a.lg_bufs == 2;   // a buffer per group
+    const int blk = a.n_blocks > 1 ? pair : 0, step = a.n_blocks > 1 ? 1 : (alone ? 4 : 2);
+    const int buf = alone ? grp : pair;
+    // this group's columns of the buffer: [col0, col0 + cw), cw 64, 96 or 128
+    const int cw = kVotes ? (alone ? a.block_rows : a.block_rows >> 1) : TILE_KEYS / 2, col0 = alone ? 0 : half * cw;
+    const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((buf << (9 - a.lg_bufs)) + col0);
+    const uint32_t bar_full = t_full(buf), bar_empty = t_empty(buf);
+    const f32x2 sc = pack2(a.scale2);
+    uint32_t ph = 0;
     bool ok = true;
-    float vsum = 0.f;
 
-    // statistics: store this group's partial (max, sum) of every row of the virtual unit `vu`
-    auto flush_stats = [&](int vu) {
-      const int unit = vu / a.vu_per_unit;
+    int seg0 = 0, seg_tile0 = tile_begin, vu = vu_begin;
+    while (seg0 < nt && ok) {
+      const int seg_n = min(nt - seg0, a.n_tiles - seg_tile0);
+      const int unit = vu / a.vu_per_unit, row0 = (vu - unit * a.vu_per_unit) * a.vu_rows;
       const int hq0 = (unit / Hkv) * a.Hq + (unit % Hkv) * a.G;
-      const int row0 = (vu - unit * a.vu_per_unit) * a.vu_rows;
-      const int slot = cta - (vu * a.n_tiles) / a.tiles_per_cta;
-      for (int blk = 0; blk < a.n_blocks; ++blk) {
-        const int row = row0 + blk * 128 + ct;
-        if (row < a.GW)
-          a.stat_part[(((size_t)hq0 * a.W + row) * a.max_slots + slot) * kGroups + grp] = ml_s[grp][blk][ct];
-      }
-    };
-
-    int vu = vu_begin, tile = tile_begin, unit = vu_begin / a.vu_per_unit;
-    int row0 = (vu - unit * a.vu_per_unit) * a.vu_rows;
-    for (int i = 0; i < nt && ok; ++i, ++tile) {
-      if (tile == a.n_tiles) {
-        tile = 0; ++vu; unit = vu / a.vu_per_unit;
-        row0 = (vu - unit * a.vu_per_unit) * a.vu_rows;
-      }
-      if (vu != cur_vu) {
-        if (kVotes) {
-          // this warp's copy of -lse2 of the unit's window rows (-inf for the padding rows); warps
-          // keep their own copy so that no barrier wider than a warp is needed here
-          const int hq0 = (unit / Hkv) * a.Hq + (unit % Hkv) * a.G;
-          const int cwh = a.block_rows >> 1;   // this group's columns of a row block: [half * cwh, +cwh)
-          __syncwarp();
-          for (int idx = lane; idx < 256; idx += 32) {
-            const int blk = idx >> 7, c = idx & 127;
-            const int r = blk * a.block_rows + half * cwh + c;
-            nlse2_s[warp][idx] = (blk < a.n_blocks && c < cwh && r < a.GW) ? -a.row_lse[(size_t)hq0 * a.W + r] * kLog2e
-                                                                         : -INFINITY;
-          }
-          __syncwarp();
-        } else {
-          if (cur_vu >= 0) flush_stats(cur_vu);
-          for (int blk = 0; blk < 2; ++blk) ml_s[grp][blk][ct] = make_float2(-INFINITY, 0.f);
+      float* vote_out = nullptr;                 // votes: this group's part of the unit's votes
+      float2 ml = make_float2(-1e30f, 0.f);      // statistics: running (max, sum) of this thread's row
+      int lim = 0;                               // statistics: the last key the row may see (causal in the window)
+      if (kVotes) {
+        // this warp's copy of -lse2 of its columns' window rows (-inf for the padding rows); a copy per
+        // warp, so that no barrier wider than a warp is needed here
+        __syncwarp();
+        for (int c = lane; c < cw; c += 32) {
+          const int r = blk * a.block_rows + col0 + c;
+          nlse2_s[warp][c] = r < a.GW ? -a.row_lse[(size_t)hq0 * a.W + r] * kLog2e : -INFINITY;
         }
-        cur_vu = vu;
+        __syncwarp();
+        const int part = alone ? 0 : 2 * blk + half, units = a.total_tiles / a.n_tiles;
+        vote_out = a.vote_parts + ((size_t)part * units + unit) * a.n_cand;
+      } else {
+        lim = min(a.L - 1, a.n_cand + (row0 + blk * 128 + ct) % a.W);
       }
-      const int tbase = tile * TILE_KEYS;
-      for (int blk = 0; blk < a.n_blocks; ++blk, ++j) {
-        if ((j & 1) != pair) continue;
-        const int buf = j & (kNumBufs - 1);
-        const uint32_t lane_addr = lane_base + (uint32_t)(buf * kBufCols);
-        ok = mbar_wait(&ctl, t_full(buf), (j / kNumBufs) & 1, (kVotes ? 35u : 15u) | ((unsigned)j << 8));
+      // the first tile of the segment that is this buffer's: tile i of the CTA goes to buffer i % step
+      const int first = (buf - seg0) & (step - 1);
+      int key0 = (seg_tile0 + first) * TILE_KEYS;
+#pragma unroll 1
+      for (int i = first; i < seg_n; i += step, key0 += step * TILE_KEYS) {
+        ok = mbar_wait(&ctl, bar_full, ph, (kVotes ? 35u : 15u) | ((unsigned)i << 8));
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
+        ph ^= 1u;
         tc_fence_after_sync();
         uint32_t ra[32], rb[32];
         if (kVotes) {
-          const int cw = a.block_rows >> 1;  // columns (query rows) of this group: a multiple of 32
-          const float* nl = nlse2_s[warp] + blk * 128;
-          const uint32_t tcol = lane_addr + (uint32_t)(half * cw);
-          float acc0 = 0.f, acc1 = 0.f, acc2 = 0.f, acc3 = 0.f;  // running vote of this thread's key
+          f32x2 acc0 = 0ull, acc1 = 0ull;  // the vote of this thread's key over this group's columns
           auto add32 = [&](const uint32_t (&r)[32], int c0) {
+            const float* nl = nlse2_s[warp] + c0;
 #pragma unroll
             for (int e = 0; e < 32; e += 4) {
-              const float4 n4 = *reinterpret_cast<const float4*>(nl + c0 + e);
-              acc0 += ex2_approx(fmaf(__uint_as_float(r[e + 0]), a.scale2, n4.x));
-              acc1 += ex2_approx(fmaf(__uint_as_float(r[e + 1]), a.scale2, n4.y));
-              acc2 += ex2_approx(fmaf(__uint_as_float(r[e + 2]), a.scale2, n4.z));
-              acc3 += ex2_approx(fmaf(__uint_as_float(r[e + 3]), a.scale2, n4.w));
+              const ulonglong2 n4 = *reinterpret_cast<const ulonglong2*>(nl + e);
+              const f32x2 x0 = fma2(pack2(r[e], r[e + 1]), sc, n4.x), x1 = fma2(pack2(r[e + 2], r[e + 3]), sc, n4.y);
+              acc0 = add2(acc0, exp2_pair_on_poly(e / 2) ? exp2_poly2(x0) : exp2_unit2(x0));
+              acc1 = add2(acc1, exp2_pair_on_poly(e / 2 + 1) ? exp2_poly2(x1) : exp2_unit2(x1));
             }
           };
-          // chunks of 32 columns alternate between the two register sets (cw is a multiple of 32)
-          tmem_ld32_issue(tcol, ra);
-#pragma unroll 1
-          for (int c0 = 0; c0 < cw; c0 += 64) {
-            tmem_ld_wait(ra);
-            const bool more_b = c0 + 32 < cw;
-            if (more_b) tmem_ld32_issue(tcol + c0 + 32, rb);
-            else { tc_fence_before_sync(); mbar_arrive(t_empty(buf)); }   // all of it is in registers
-            add32(ra, c0);
-            if (more_b) {
-              tmem_ld_wait(rb);
-              if (c0 + 64 < cw) tmem_ld32_issue(tcol + c0 + 64, ra);
-              else { tc_fence_before_sync(); mbar_arrive(t_empty(buf)); }
-              add32(rb, c0 + 32);
+          // chunks of 32 columns alternate between the two register sets; unrolled, since a loop with the
+          // conditions inside took 163 instead of 134 thousand cycles
+          auto drain = [&](auto cw_tag) __attribute__((always_inline)) {
+            constexpr int kCw = decltype(cw_tag)::value;
+            tmem_ld32_issue(taddr, ra);
+#pragma unroll
+            for (int c0 = 0; c0 < kCw; c0 += 64) {
+              tmem_ld_wait(ra);
+              if (c0 + 32 < kCw) tmem_ld32_issue(taddr + c0 + 32, rb);
+              else { tc_fence_before_sync(); mbar_arrive(bar_empty); }   // all of it is in registers
+              add32(ra, c0);
+              if (c0 + 32 < kCw) {
+                tmem_ld_wait(rb);
+                if (c0 + 64 < kCw) tmem_ld32_issue(taddr + c0 + 64, ra);
+                else { tc_fence_before_sync(); mbar_arrive(bar_empty); }
+                add32(rb, c0 + 32);
+              }
             }
-          }
-          // the two halves of the key's vote meet in shared memory; the first group stores the sum
-          const float part = (acc0 + acc1) + (acc2 + acc3);
-          const int jp = j >> 1;   // index of the job among this pair's jobs
-          if (half == 1) {
-            ok = mbar_wait(&ctl, vx_empty(pair), (jp & 1) ^ 1, 37u | ((unsigned)j << 8));
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
-            vx[pair][ct] = part;
-            mbar_arrive(vx_full(pair));
-          } else {
-            ok = mbar_wait(&ctl, vx_full(pair), jp & 1, 38u | ((unsigned)j << 8));
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
-            vsum += part + vx[pair][ct];
-            mbar_arrive(vx_empty(pair));
-            // the vote of the key over this pair's row blocks of the tile; stored after the last of them
-            if (blk + 2 >= a.n_blocks) {
-              const int key = tbase + ct;
-              float* out = (a.n_blocks > 1 && pair == 1) ? a.vote2 : a.vote;
-              if (key < a.n_cand) out[(size_t)unit * a.n_cand + key] = vsum;
-              vsum = 0.f;
-            }
-          }
+          };
+          if (cw == 128) drain(std::integral_constant<int, 128>{});
+          else if (cw == 64) drain(std::integral_constant<int, 64>{});
+          else drain(std::integral_constant<int, 96>{});
+          const float2 acc = unpack2(add2(acc0, acc1));
+          if (key0 + ct < a.n_cand) vote_out[key0 + ct] = acc.x + acc.y;
         } else {
-          float2 ml = ml_s[grp][blk][ct];
-          const int row = row0 + blk * 128 + ct;
-          // local index of the last key this row may see inside the tile (causal inside the window)
-          const int lim = min(a.L - 1, a.n_cand + row % a.W) - tbase;
-          const bool full_tile = __all_sync(0xffffffffu, lim >= TILE_KEYS - 1);
+          const int l0 = lim - (key0 + half * cw);   // index of the row's last key among this group's keys of the tile
+          const bool full = __all_sync(0xffffffffu, l0 >= cw - 1);
           auto fold32 = [&](uint32_t (&r)[32], int c0) {
-            if (!full_tile) {
+            if (!full) {
 #pragma unroll
               for (int e = 0; e < 32; ++e)
-                if (c0 + e > lim) r[e] = 0xff800000u;  // -inf
+                if (c0 + e > l0) r[e] = 0xff800000u;  // -inf
             }
             const float m_new = fmaxf(ml.x, max_32(r) * a.scale2);
-            if (m_new > -INFINITY) {
-              ml.y = ml.y * ex2_approx(ml.x - m_new) + sum_exp2_32(r, a.scale2, -m_new);
-              ml.x = m_new;
-            }
+            ml.y = fmaf(ml.y, ex2_approx(ml.x - m_new), sum_exp2_32(r, sc, pack2(-m_new)));
+            ml.x = m_new;
           };
-          const int cbeg = half * (TILE_KEYS / 2), cend = cbeg + TILE_KEYS / 2;  // this group's keys of the tile
-          tmem_ld32_issue(lane_addr + cbeg, ra);
-#pragma unroll 1
-          for (int c0 = cbeg; c0 < cend; c0 += 64) {
+          tmem_ld32_issue(taddr, ra);
+#pragma unroll
+          for (int c0 = 0; c0 < TILE_KEYS / 2; c0 += 64) {
             tmem_ld_wait(ra);
-            tmem_ld32_issue(lane_addr + c0 + 32, rb);
+            tmem_ld32_issue(taddr + c0 + 32, rb);
             fold32(ra, c0);
             tmem_ld_wait(rb);
-            if (c0 + 64 < cend) {
-              tmem_ld32_issue(lane_addr + c0 + 64, ra);
+            if (c0 + 64 < TILE_KEYS / 2) {
+              tmem_ld32_issue(taddr + c0 + 64, ra);
             } else {
               tc_fence_before_sync();
-              mbar_arrive(t_empty(buf));  // the accumulator is in registers: hand the buffer back early
+              mbar_arrive(bar_empty);  // the accumulator is in registers: hand the buffer back early
             }
             fold32(rb, c0 + 32);
           }
-          ml_s[grp][blk][ct] = ml;
         }
       }
+      if (!kVotes && ok) {
+        // this group's partial (max, sum) of its row; with one row block both pairs have one
+        const int slot = cta - (vu * a.n_tiles) / a.tiles_per_cta;
+        const int row = row0 + blk * 128 + ct, n_part = a.n_blocks > 1 ? 2 : 4;
+        if (row < a.GW)
+          a.stat_part[(((size_t)hq0 * a.W + row) * a.max_slots + slot) * n_part + (a.n_blocks > 1 ? half : grp)] = ml;
+      }
+      seg0 += seg_n;
+      seg_tile0 = 0;
+      ++vu;
     }
-    if (!kVotes && ok && cur_vu >= 0 && !ctl.abort) flush_stats(cur_vu);
   }
 
   // ---------------------------------------------------------------- teardown (every path)
@@ -396,33 +379,41 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
   if (warp == kMmaWarp) tmem_dealloc(tmem_base, kTmemCols);
 }
 
-// Combine the partial statistics of every observation row into its natural-log LSE.  The
-// partials of a row are those of the CTAs whose tile range overlaps the row's virtual unit.
-__global__ void row_lse_from_parts_kernel(const float2* __restrict__ stat_part, float* __restrict__ row_lse,
-                                          int rows, int GW, int vu_per_unit, int n_tiles, int tiles_per_cta,
-                                          int max_slots) {
+// Combine the partial statistics of every observation row into its natural-log LSE, a warp per row (a thread
+// per row walked up to a hundred partials one load after the other: 18.6 us for one prompt of 131072 keys).
+// The partials of a row are those of the CTAs whose tile range overlaps the row's virtual unit.
+__global__ void __launch_bounds__(256)
+row_lse_from_parts_kernel(const float2* __restrict__ stat_part, float* __restrict__ row_lse, int rows, int GW,
+                          int vu_per_unit, int n_tiles, int tiles_per_cta, int max_slots, int n_part) {
   pdl_trigger();
   pdl_wait();
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (r >= rows) return;
   const int unit = r / GW, row = r - unit * GW;
   const int vu = unit * vu_per_unit + row / 256;
   const int first = (vu * n_tiles) / tiles_per_cta, last = ((vu + 1) * n_tiles - 1) / tiles_per_cta;
-  const int n = (last - first + 1) * kGroups;
-  const float2* p = stat_part + (size_t)r * max_slots * kGroups;
-  float m = -INFINITY;
-  for (int i = 0; i < n; ++i) m = fmaxf(m, p[i].x);
-  float l = 0.f;
-  for (int i = 0; i < n; ++i)
-    if (p[i].x > -INFINITY) l += p[i].y * exp2f(p[i].x - m);
-  row_lse[r] = (m + log2f(l)) * kLn2;
+  const int n = (last - first + 1) * n_part;
+  const float2* p = stat_part + (size_t)r * max_slots * n_part;
+  float m = -INFINITY, l = 0.f;
+  for (int i = lane; i < n; i += 32) {
+    const float2 q = p[i];
+    const float mn = fmaxf(m, q.x);
+    l = l * exp2f(m - mn) + q.y * exp2f(q.x - mn);
+    m = mn;
+  }
+  const float M = warp_max(m);
+  l = warp_sum(m > -INFINITY ? l * exp2f(m - M) : 0.f);
+  if (lane == 0) row_lse[r] = (M + log2f(l)) * kLn2;
 }
 
-__global__ void add_votes_kernel(float* __restrict__ vote, const float* __restrict__ vote2, size_t n) {
+__global__ void add_votes_kernel(float* __restrict__ vote, const float* __restrict__ parts, int n_parts, size_t n) {
   pdl_trigger();
   pdl_wait();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) vote[i] += vote2[i];
+  if (i >= n) return;
+  float x = parts[i];
+  for (int p = 1; p < n_parts; ++p) x += parts[(size_t)p * n + i];
+  vote[i] = x;
 }
 
 template <bool kVotes>
@@ -482,6 +473,7 @@ cudaError_t launch_row_stats_tc(const CompressGeom& g, const CompressWs& ws, con
   a.max_slots = (a.n_tiles + a.tiles_per_cta - 1) / a.tiles_per_cta + 1;
   if (a.max_slots * kGroups > ws.stat_slots) return cudaErrorInvalidValue;
   a.stages = 2;  // 64 KB tiles of 256 keys
+  a.lg_bufs = 1;
   a.scale2 = g.scale2;
   a.stat_part = (float2*)(wsp + ws.stat_part);
   a.status = (unsigned*)(wsp + ws.status);
@@ -499,13 +491,18 @@ cudaError_t launch_row_stats_tc(const CompressGeom& g, const CompressWs& ws, con
   e = launch_pdl(score_tc_kernel<false>, dim3(grid), dim3(kThreads), (size_t)smem, st, qm, km, a);
   if (e != cudaSuccess) return e;
   const int rows = g.B * g.Hq * g.W;
-  e = launch_pdl(row_lse_from_parts_kernel, dim3((rows + 127) / 128), dim3(128), 0, st, (const float2*)a.stat_part,
-                 (float*)(wsp + ws.row_lse), rows, GW, a.vu_per_unit, a.n_tiles, a.tiles_per_cta, a.max_slots);
+  e = launch_pdl(row_lse_from_parts_kernel, dim3((rows + 7) / 8), dim3(256), 0, st, (const float2*)a.stat_part,
+                 (float*)(wsp + ws.row_lse), rows, GW, a.vu_per_unit, a.n_tiles, a.tiles_per_cta, a.max_slots,
+                 a.n_blocks > 1 ? 2 : 4);
   count_launch(2);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-// Votes of every candidate key, into ws.vote.
+// Parts of a candidate's vote that launch_votes_tc leaves: one per row block and column half, one in all for
+// at most 128 rows.
+int votes_tc_parts(const CompressGeom& g) { return g.G * g.W <= 128 ? 1 : 2 * ((g.G * g.W + 255) / 256); }
+
+// Partial votes of every candidate key, into ws.vote_parts; the selection adds them up.
 cudaError_t launch_votes_tc(const CompressGeom& g, const CompressWs& ws, const void* Q_obs, const void* K,
                             const float* row_lse, char* wsp, cudaStream_t st) {
   const int GW = g.G * g.W;
@@ -513,18 +510,17 @@ cudaError_t launch_votes_tc(const CompressGeom& g, const CompressWs& ws, const v
   a.Hq = g.Hq; a.G = g.G; a.W = g.W; a.L = g.L; a.n_cand = g.n_cand; a.GW = GW;
   a.vu_per_unit = 1;
   a.vu_rows = 0;
-  // One accumulator of up to 256 row columns per (key tile, row block); with several row blocks
-  // per tile each warpgroup sums the blocks it drains and the two partial votes are added afterwards.
+  // One accumulator of up to 256 row columns per (key tile, row block).
   a.n_blocks = (GW + 255) / 256;
   a.block_rows = ((GW + a.n_blocks - 1) / a.n_blocks + 63) / 64 * 64;
+  a.lg_bufs = a.block_rows <= 128 ? 2 : 1;
   a.n_tiles = (g.n_cand + kTileKeys - 1) / kTileKeys;
   partition_tiles(a, g.units);
   const int q_bytes = a.n_blocks * a.block_rows * 256;
   a.stages = q_bytes <= 65536 ? 4 : (q_bytes <= 98304 ? 3 : 2);
   a.scale2 = g.scale2;
   a.row_lse = row_lse;
-  a.vote = (float*)(wsp + ws.vote);
-  a.vote2 = (float*)(wsp + ws.vote2);
+  a.vote_parts = (float*)(wsp + ws.vote_parts);
   a.status = (unsigned*)(wsp + ws.status);
   CUtensorMap qm, km;
   const uint64_t qd[2] = {(uint64_t)GW, (uint64_t)g.units}, qs[2] = {256, (uint64_t)GW * 256};
@@ -540,12 +536,16 @@ cudaError_t launch_votes_tc(const CompressGeom& g, const CompressWs& ws, const v
   e = launch_pdl(score_tc_kernel<true>, dim3(grid), dim3(kThreads), (size_t)smem, st, qm, km, a);
   if (e != cudaSuccess) return e;
   count_launch(1);
-  if (a.n_blocks > 1) {
-    const size_t n = (size_t)g.units * g.n_cand;
-    e = launch_pdl(add_votes_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, a.vote, (const float*)a.vote2, n);
-    if (e != cudaSuccess) return e;
-    count_launch(1);
-  }
+  return cudaGetLastError();
+}
+
+// The parts added into ws.vote, for the selection that does not add them itself.
+cudaError_t launch_add_votes(const CompressGeom& g, const CompressWs& ws, char* wsp, cudaStream_t st) {
+  const size_t n = (size_t)g.units * g.n_cand;
+  cudaError_t e = launch_pdl(add_votes_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, (float*)(wsp + ws.vote),
+                             (const float*)(wsp + ws.vote_parts), votes_tc_parts(g), n);
+  if (e != cudaSuccess) return e;
+  count_launch(1);
   return cudaGetLastError();
 }
 

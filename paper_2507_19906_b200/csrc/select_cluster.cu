@@ -104,7 +104,7 @@ pool_select_cluster_kernel(const SelectArgs a) {
   auto pooled_key = [&](int t, float acc) {
     const float p = acc / fpool;
     pl[t] = p;
-    return __float_as_uint(p);
+    return (unsigned)max(__float_as_int(p), 0);   // (a score below zero or a negative NaN ranks as zero)
   };
   auto pool_rows = [&](auto taps_tag) __attribute__((always_inline)) {
     constexpr int kTaps = decltype(taps_tag)::value;
@@ -375,10 +375,14 @@ cudaError_t launch_pool_select_scores(const CompressGeom& g, const CompressWs& w
   return launch_any<false>(a, g.units, st);
 }
 
-cudaError_t launch_pool_select_cluster(const CompressGeom& g, const CompressWs& ws, char* wsp, int32_t* kept_idx,
-                                       cudaStream_t st) {
-  return launch_pool_select_scores(g, ws, wsp, (const float*)(wsp + ws.vote), (size_t)g.n_cand, 1, 0, nullptr, kept_idx,
-                                   st);
+// Selection from the window votes of the workspace: ws.vote, or with `in_parts` the partial votes that
+// launch_votes_tc left, whose sum goes to ws.vote on the way.
+cudaError_t launch_pool_select_cluster(const CompressGeom& g, const CompressWs& ws, char* wsp, bool in_parts,
+                                       int32_t* kept_idx, cudaStream_t st) {
+  float* vote = (float*)(wsp + ws.vote);
+  if (!in_parts) return launch_pool_select_scores(g, ws, wsp, vote, (size_t)g.n_cand, 1, 0, nullptr, kept_idx, st);
+  return launch_pool_select_scores(g, ws, wsp, (const float*)(wsp + ws.vote_parts), (size_t)g.n_cand, votes_tc_parts(g),
+                                   (size_t)g.units * g.n_cand, vote, kept_idx, st);
 }
 
 // Sink-plus-recent index rule: the first n_sink rows and the last n_kept - n_sink.
