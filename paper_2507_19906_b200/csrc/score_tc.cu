@@ -175,37 +175,40 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
                       tile * TILE_KEYS, unit);
       }
     }
-  } else if (warp == kMmaWarp) {
+  } else if (__shfl_sync(0xffffffffu, warp, 0) == kMmaWarp) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      const uint32_t idesc = umma_idesc(128, kVotes ? a.block_rows : TILE_KEYS, false, false);
-      // Descriptors are built once per buffer; a k-step adds a constant to the address field (the
-      // issuing thread's own instructions between two MMAs are what limits the issue rate).
-      const uint64_t dq0 = smem_desc_sw128(q_base, 16u, 1024u);
-      const uint64_t dk0 = smem_desc_sw128(k_base, 16u, 1024u);
-      int cur_vu = -1, seg = 0, j = 0, vu = vu_begin, tile = tile_begin;
-      for (int i = 0; i < nt; ++i, ++tile) {
-        if (tile == a.n_tiles) { tile = 0; ++vu; }
-        if (vu != cur_vu) {
-          if (!mbar_wait(&ctl, q_full, seg & 1, (kVotes ? 32u : 12u) | ((unsigned)i << 8))) break;
-          cur_vu = vu;
-          ++seg;
-        }
-        const int s = i % a.stages;
-        if (!mbar_wait(&ctl, full_k(s), (i / a.stages) & 1, (kVotes ? 33u : 13u) | ((unsigned)i << 8))) break;
-        bool ok = true;
-        const uint64_t kd = desc_advance(dk0, (uint32_t)s * STAGE_BYTES);
-        for (int blk = 0; blk < a.n_blocks; ++blk, ++j) {
-          const int buf = j & ((1 << a.lg_bufs) - 1);
-          if (!mbar_wait(&ctl, t_empty(buf), ((j >> a.lg_bufs) & 1) ^ 1, (kVotes ? 34u : 14u) | ((unsigned)j << 8))) {
-            ok = false;
-            break;
-          }
-          tc_fence_after_sync();
-          const uint32_t d = tmem_base + (uint32_t)(buf << (9 - a.lg_bufs));
-          const uint64_t qd = desc_advance(dq0, (uint32_t)blk * q_blk_bytes);
-          // the second halves (k-steps 4..7) start half a tile further on
-          const uint64_t kd2 = desc_advance(kd, STAGE_BYTES / 2), qd2 = desc_advance(qd, q_half_bytes);
+    // The whole warp walks the loop and one lane issues: the values are then warp-uniform, and the operands
+    // of an MMA come from uniform registers as they are.  With one lane in a loop of its own the eight MMAs of a job
+    // took 560 cycles to issue and a job 1700 in all, which was the pace of the votes of 128 rows (64 units x 16384
+    // keys: 64.8 -> 50 us, 5.3 TB/s of keys).  The shuffle makes the role of this warp uniform to the compiler; the
+    // consumers keep the plain index, with which they need fewer registers.
+    const uint32_t idesc = umma_idesc(128, kVotes ? a.block_rows : TILE_KEYS, false, false);
+    // Descriptors are built once per buffer; a k-step adds a constant to the address field.
+    const uint64_t dq0 = smem_desc_sw128(q_base, 16u, 1024u);
+    const uint64_t dk0 = smem_desc_sw128(k_base, 16u, 1024u);
+    const bool leader = elect_one();
+    int seg = 0, j = 0, s = 0, tile = tile_begin;
+    uint32_t s_ph = 0;
+    bool first = true, ok = true;
+    for (int i = 0; i < nt && ok; ++i) {
+      if (first) {
+        ok = __all_sync(0xffffffffu, mbar_wait(&ctl, q_full, seg & 1, (kVotes ? 32u : 12u) | ((unsigned)i << 8)));
+        if (!ok) break;
+        ++seg;
+      }
+      ok = __all_sync(0xffffffffu, mbar_wait(&ctl, full_k(s), s_ph, (kVotes ? 33u : 13u) | ((unsigned)i << 8)));
+      if (!ok) break;
+      const uint64_t kd = desc_advance(dk0, (uint32_t)s * STAGE_BYTES);
+      for (int blk = 0; blk < a.n_blocks; ++blk, ++j) {
+        const int buf = j & ((1 << a.lg_bufs) - 1);
+        ok = __all_sync(0xffffffffu, mbar_wait(&ctl, t_empty(buf), ((j >> a.lg_bufs) & 1) ^ 1, (kVotes ? 34u : 14u) | ((unsigned)j << 8)));
+        if (!ok) break;
+        tc_fence_after_sync();
+        const uint32_t d = tmem_base + (uint32_t)(buf << (9 - a.lg_bufs));
+        const uint64_t qd = desc_advance(dq0, (uint32_t)blk * q_blk_bytes);
+        // the second halves (k-steps 4..7) start half a tile further on
+        const uint64_t kd2 = desc_advance(kd, STAGE_BYTES / 2), qd2 = desc_advance(qd, q_half_bytes);
+        if (leader) {
           umma_ss_imm<0>(d, kVotes ? kd : qd, kVotes ? qd : kd, idesc);
 #pragma unroll
           for (int kk = 1; kk < 4; ++kk)
@@ -215,11 +218,18 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
             umma_ss_imm<1>(d, desc_advance(kVotes ? kd2 : qd2, kk * 32u), desc_advance(kVotes ? qd2 : kd2, kk * 32u), idesc);
           umma_commit(t_full(buf));
         }
-        if (!ok) break;
-        umma_commit(empty_k(s));
-        const bool last_of_vu = (i == nt - 1) || (tile == a.n_tiles - 1);
-        if (last_of_vu) umma_commit(q_empty);
+        __syncwarp();
       }
+      if (!ok) break;
+      ++tile;
+      first = tile == a.n_tiles;
+      if (first) tile = 0;
+      if (leader) {
+        umma_commit(empty_k(s));
+        if (first || i == nt - 1) umma_commit(q_empty);
+      }
+      __syncwarp();
+      if (++s == a.stages) { s = 0; s_ph ^= 1u; }
     }
   } else {
     // ------------------------------------------------------------ accumulator consumers
@@ -228,7 +238,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
     // groups half of the columns.  With two row blocks a pair therefore always has the same one, with one
     // every second tile.  Votes of at most 128 window rows have four accumulators instead, one per group:
     // a job is as long as with 256 rows, where half a job per group would double what lies between two
-    // (64 units x 128 rows x 16384 keys: @16k@ us).  While one pair waits for the MMAs of its next job (which cannot start before
+    // (64 units x 16384 keys: whole call 199 -> 193 us).  While one pair waits for the MMAs of its next job (which cannot start before
     // the last columns of the current one have been read), the other, two warps per scheduler, keeps
     // the exponentials going; one warp per scheduler alone reaches less than half of their rate.
     // (Measured at 32 units x 32768 keys, votes: two groups on the same job 110 us, the groups stalling

@@ -100,6 +100,19 @@ __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
 }
 
+// One lane of a converged warp, the same one every time.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n"
+      ".reg .pred p;\n"
+      "elect.sync _|p, 0xffffffff;\n"
+      "selp.u32 %0, 1, 0, p;\n"
+      "}\n"
+      : "=r"(p));
+  return p != 0;
+}
+
 // ---------------------------------------------------------------- tensor memory
 // Whole-warp calls.  The allocated base address (lane 0, first column) is written to smem_dst.
 __device__ __forceinline__ void tmem_alloc(uint32_t smem_dst, uint32_t ncols) {
@@ -236,12 +249,10 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
                : "memory");
 }
 
-// ---- lean issue: the MMA-issuing thread is ONE thread, whose dependent scalar instructions cost
-// several cycles each, so every instruction between two MMAs counts (measured: an issue loop that
-// rebuilds its descriptors from addresses runs at 100-150 cycles per 128x128x16 MMA whatever the
-// operands; with the descriptors prepared and the accumulate flag an immediate the same MMAs run
-// at 64 cycles, the tensor pipe's own rate, even as one dependent chain).  So descriptors are built
-// once per buffer and advanced by adding a compile-time byte offset to their address field.
+// ---- lean issue: whatever lies between two MMAs of the issuing warp counts.  Descriptors are built once per
+// buffer and advanced by adding a compile-time byte offset to their address field, and the issuing warp
+// walks its loop as a whole with one elected lane issuing (see elect_one), so that the operands sit in uniform
+// registers.
 __device__ __forceinline__ uint64_t desc_advance(uint64_t desc, uint32_t bytes) {
   uint2 v = *reinterpret_cast<uint2*>(&desc);
   v.x += bytes >> 4;   // the address field holds bytes / 16 in the low bits; tiles never wrap it
