@@ -14,12 +14,9 @@
 // every p <= 1 and no running maximum or rescaling is needed: the partial (O, l) of the key ranges
 // simply add up.  calib_reduce_kernel sums them in a fixed order and writes O_c = O / l,
 // LSE_c = lse + log l, C_q.
-// Warp roles: two softmax warpgroups (group g takes the tiles with local index i % 2 == g), two TMA
-// producer warps (Q_c and K; V), and two MMA-issuing warps, one for S and one for P.V: a single
-// thread's dependent scalar instructions cost several cycles each, and with the waits and commits of
-// both chains on one thread the issue, not the tensor pipe, set the pace (a lone chain of eight
-// 128x128x16 MMAs runs at the pipe's 64 cycles each once its descriptors are prepared; no
-// interleaving of chains is needed).
+// Warp roles: four softmax warpgroups in two pairs (pair p takes the tiles whose local index has parity p), two
+// TMA producer warps (Q_c and K; V), and two MMA-issuing warps, one for S and one for P.V: what a warp has to
+// go through between two MMAs adds up, and one warp for both chains set the pace, not the tensor pipe.
 // Tensor memory: three S/P buffers of 128 columns at 0, 128, 256 and O at 384.  Tile i lives in buffer
 // i % 3: S(i) arrives there, and its probabilities, rounded to bf16, overwrite the first 64 columns in
 // place (a thread stores the P of 32 keys only after the S of those columns is in its registers).  A
@@ -28,6 +25,7 @@
 // (with two S buffers and a P buffer per group it did, for about a third of its time).
 #include <type_traits>
 
+#include "exp2.cuh"
 #include "internal.h"
 #include "tc_common.cuh"
 
@@ -146,7 +144,7 @@ calib_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
         if (tile == a.n_tiles) { tile = 0; ++unit; vu += a.n_cblocks; }
         if (i == 0 || tile == 0) {
           // the Q_c block of the next virtual unit replaces the current one once its MMAs are done
-          if (seg > 0 && !mbar_wait(&ctl, q_empty, (seg - 1) & 1, 20u | ((unsigned)i << 8))) break;
+          if (seg > 0 && !mbar_wait_far(&ctl, q_empty, (seg - 1) & 1, 20u | ((unsigned)i << 8))) break;
           const int g0 = (vu - unit * a.n_cblocks) * a.gpb;
           mbar_arrive_expect_tx(q_full, 2u * (uint32_t)(a.gpb * a.n_cal) * kLineBytes);
           for (int half = 0; half < 2; ++half)
@@ -155,7 +153,7 @@ calib_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
         }
         const int s = i % kStages;
         // slot s is free when S(i-3), which read it, is done: the barrier that hands S to the softmax group
-        if (!mbar_wait(&ctl, s_full(s), ((i / kStages) & 1) ^ 1, 21u | ((unsigned)i << 8))) break;
+        if (!mbar_wait_far(&ctl, s_full(s), ((i / kStages) & 1) ^ 1, 21u | ((unsigned)i << 8))) break;
         mbar_arrive_expect_tx(full_k(s), kTileBytes);
         for (int half = 0; half < 2; ++half)
           tma_load_3d(k_base + s * kTileBytes + half * (kTileBytes / 2), &k_map, full_k(s), half * kHalfCols,
@@ -171,102 +169,104 @@ calib_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
         if (tile == a.n_tiles) { tile = 0; ++unit; }
         const int s = i % kStages;
         // slot s is free when the P.V of tile i-3 is done: the barrier that frees its S/P buffer
-        if (!mbar_wait(&ctl, buf_free(s), ((i / kStages) & 1) ^ 1, 22u | ((unsigned)i << 8))) break;
+        if (!mbar_wait_far(&ctl, buf_free(s), ((i / kStages) & 1) ^ 1, 22u | ((unsigned)i << 8))) break;
         mbar_arrive_expect_tx(full_v(s), kTileBytes);
         for (int half = 0; half < 2; ++half)
           tma_load_3d(v_base + s * kTileBytes + half * (kTileBytes / 2), &v_map, full_v(s), half * kHalfCols,
                       tile * kTileKeys, unit);
       }
     }
-  } else if (warp == kMmaWarp) {
+  } else if (__shfl_sync(0xffffffffu, warp, 0) == kMmaWarp) {
     // ------------------------------------------------------------ issuer of the S MMAs
-    // The MMAs have two issuing threads, one for S = Q_c K^T and one for O += P V.  One thread for
-    // both was the bottleneck of this kernel: besides its sixteen MMAs a tile it has three waits and
-    // five commits to go through, each of them some hundred cycles of dependent scalar instructions
-    // for a single thread (measured: 2900 cycles a tile against 1024 of tensor-pipe time, the softmax
-    // groups waiting for S half of the time).  The two chains touch different accumulators; what
-    // orders them is the barriers, not the issue order.
+    // The MMAs have two issuing warps, one for S = Q_c K^T and one for O += P V: what a warp has to go
+    // through between two MMAs (waits of about 100 cycles each, commits, 60 cycles per MMA) adds up to more than the
+    // tensor pipe needs for a tile when one warp issues both chains (1830 cycles a tile against 1024).  The
+    // two chains touch different accumulators; what orders them is the barriers, not the issue order.
     // S(t) goes into buffer t % 3 as soon as the P.V of tile t-3 has completed (buf_free).  S never
     // runs ahead across a change of virtual unit: its Q_c block is only loaded once the current unit's
     // S MMAs are done.
-    if (lane == 0) {
-      const uint32_t idesc = umma_idesc(128, 128, false, false);     // S: A = Q_c, B = K tile, K-major
-      // Descriptors are built once per buffer and a k-step adds a constant to the address field: the
-      // issuing thread's own instructions between two MMAs are what limits the issue rate.
-      const uint64_t dq = smem_desc_sw128(q_base, 16u, 1024u);
-      const uint64_t dk0 = smem_desc_sw128(k_base, 16u, 1024u);
-      // The loop is kept short on purpose: between two tiles this one thread runs dependent scalar
-      // instructions at several cycles each, and whatever it spends there the tensor pipe idles.
-      // b = t % 3 is the tile's buffer and its K slot, ph = (t / 3) & 1 their phase.
-      int seg = 0, tile = tile_begin, b = 0;
-      uint32_t ph = 0;
-      bool first = true;
-      for (int t = 0; t < nt; ++t) {
-        if (first) {
-          // new virtual unit: its Q_c block must have landed
-          if (!mbar_wait(&ctl, q_full, seg & 1, 23u | ((unsigned)t << 8))) break;
-          ++seg;
-        }
-        if (t >= kBufs && !mbar_wait(&ctl, buf_free(b), ph ^ 1u, 29u | ((unsigned)t << 8))) break;
-        if (!mbar_wait(&ctl, full_k(b), ph, 24u | ((unsigned)t << 8))) break;
-        tc_fence_after_sync();
-        const uint32_t d = tmem_base + (uint32_t)(b * 128);
-        const uint64_t kd = desc_advance(dk0, (uint32_t)b * kTileBytes);
+    // Each of the two warps walks its loop as a whole with one elected lane issuing: the operands of the
+    // MMAs are then in uniform registers (a lane in a loop of its own took 100 cycles per MMA).  Together with
+    // the packed exponentials of the softmax groups, 32 units x 256 rows x 32768 keys: 212 -> 196 thousand cycles;
+    // calls of 8 units x 8192 keys 50.2 -> 49.0 us.  The operands then bound it: S reads 64 KB and P.V 32 KB of shared
+    // memory per tile while TMA writes 64 KB, 1280 cycles at 128 bytes a cycle against 1024 of the tensor pipe.
+    const uint32_t idesc = umma_idesc(128, 128, false, false);     // S: A = Q_c, B = K tile, K-major
+    const uint64_t dq = smem_desc_sw128(q_base, 16u, 1024u);
+    const uint64_t dk0 = smem_desc_sw128(k_base, 16u, 1024u);
+    const bool leader = elect_one();
+    // b = t % 3 is the tile's buffer and its K slot, ph = (t / 3) & 1 their phase.
+    int seg = 0, tile = tile_begin, b = 0;
+    uint32_t ph = 0;
+    bool first = true, ok = true;
+#pragma unroll 1
+    for (int t = 0; t < nt; ++t) {
+      if (first) {
+        // new virtual unit: its Q_c block must have landed
+        ok = mbar_wait_far(&ctl, q_full, seg & 1, 23u | ((unsigned)t << 8));
+        ++seg;
+      }
+      ok = ok && mbar_wait_far(&ctl, full_k(b), ph, 24u | ((unsigned)t << 8));
+      if (t >= kBufs) ok = ok && mbar_wait_far(&ctl, buf_free(b), ph ^ 1u, 29u | ((unsigned)t << 8));
+      if (!__all_sync(0xffffffffu, ok)) break;
+      tc_fence_after_sync();
+      const uint32_t d = tmem_base + (uint32_t)(b * 128);
+      const uint64_t kd = desc_advance(dk0, (uint32_t)b * kTileBytes);
+      ++tile;
+      first = tile == a.n_tiles;
+      if (first) tile = 0;
+      if (leader) {
         umma_ss_imm<0>(d, dq, kd, idesc);
 #pragma unroll
         for (int kk = 1; kk < kD / 16; ++kk)
           umma_ss_imm<1>(d, desc_advance(dq, kmajor_step_bytes(kTileBytes / 2, kk)),
                          desc_advance(kd, kmajor_step_bytes(kTileBytes / 2, kk)), idesc);
-        umma_commit(s_full(b));   // to the softmax group, and to the K producer: the slot is free
-        ++tile;
-        first = tile == a.n_tiles;
-        if (first) tile = 0;
+        umma_commit(s_full(b));   // to the softmax groups, and to the K producer: the slot is free
         // every S of the unit has been issued by its last tile: Q_c may be replaced once they are done
         if (first || t == nt - 1) umma_commit(q_empty);
-        if (++b == kBufs) { b = 0; ph ^= 1u; }
       }
+      __syncwarp();
+      if (++b == kBufs) { b = 0; ph ^= 1u; }
     }
-  } else if (warp == kPvWarp) {
+  } else if (__shfl_sync(0xffffffffu, warp, 0) == kPvWarp) {
     // ------------------------------------------------------------ issuer of the P.V MMAs
-    if (lane == 0) {
-      const uint32_t idesc_o = umma_idesc(128, 128, false, true);    // O: A = P (TMEM), B = V tile, MN-major
-      const uint32_t tmem_o = tmem_base + kColO;
-      // V tile with the keys as K, i.e. MN-major: blocks of 64 head-dim elements are half a tile
-      // apart, groups of 8 keys 1024 bytes apart
-      const uint64_t dv0 = smem_desc_sw128(v_base, kTileBytes / 2, 1024u);
-      // P.V(i): A = P in tensor memory, 16 keys = 8 columns per step
-      auto pv_steps = [&](int b, auto first_tag) {
-        constexpr bool kFirst = decltype(first_tag)::value;
+    const uint32_t idesc_o = umma_idesc(128, 128, false, true);    // O: A = P (TMEM), B = V tile, MN-major
+    const uint32_t tmem_o = tmem_base + kColO;
+    // V tile with the keys as K, i.e. MN-major: blocks of 64 head-dim elements are half a tile
+    // apart, groups of 8 keys 1024 bytes apart
+    const uint64_t dv0 = smem_desc_sw128(v_base, kTileBytes / 2, 1024u);
+    const bool leader = elect_one();
+    int seg = 0, tile = tile_begin, b = 0;
+    uint32_t ph = 0;
+    bool first = true, ok = true;
+#pragma unroll 1
+    for (int i = 0; i < nt; ++i) {
+      if (first) {
+        // O of the previous unit must have been read out before the first P.V overwrites it
+        if (seg > 0) ok = mbar_wait_far(&ctl, o_empty, (seg - 1) & 1, 25u | ((unsigned)i << 8));
+        ++seg;
+      }
+      ok = ok && mbar_wait_far(&ctl, full_v(b), ph, 27u | ((unsigned)i << 8));
+      ok = ok && mbar_wait_far(&ctl, p_full(b), ph, 26u | ((unsigned)i << 8));
+      if (!__all_sync(0xffffffffu, ok)) break;
+      tc_fence_after_sync();
+      const uint32_t acc0 = first ? 0u : 1u;
+      ++tile;
+      first = tile == a.n_tiles;
+      if (first) tile = 0;
+      if (leader) {
+        // P.V(i): A = P in tensor memory, 16 keys = 8 columns per step; the P of keys 64..127 sits at columns 64..95
         const uint64_t vd = desc_advance(dv0, (uint32_t)b * kTileBytes);
         const uint32_t pa = tmem_base + (uint32_t)(b * 128);
-        if (kFirst) umma_ts_imm<0>(tmem_o, pa, vd, idesc_o);
-        else umma_ts_imm<1>(tmem_o, pa, vd, idesc_o);
+        umma_ts(tmem_o, pa, vd, idesc_o, acc0);
 #pragma unroll
-        for (int kk = 1; kk < kTileKeys / 16; ++kk)   // the P of keys 64..127 sits at columns 64..95
+        for (int kk = 1; kk < kTileKeys / 16; ++kk)
           umma_ts_imm<1>(tmem_o, pa + (uint32_t)((kk >> 2) * 64 + (kk & 3) * 8),
                          desc_advance(vd, (uint32_t)kk * 16u * kLineBytes), idesc_o);
-      };
-      int seg = 0, tile = tile_begin, b = 0;
-      uint32_t ph = 0;
-      bool first = true;
-      for (int i = 0; i < nt; ++i) {
-        if (first) {
-          // O of the previous unit must have been read out before the first P.V overwrites it
-          if (seg > 0 && !mbar_wait(&ctl, o_empty, (seg - 1) & 1, 25u | ((unsigned)i << 8))) break;
-          ++seg;
-        }
-        if (!mbar_wait(&ctl, p_full(b), ph, 26u | ((unsigned)i << 8))) break;
-        if (!mbar_wait(&ctl, full_v(b), ph, 27u | ((unsigned)i << 8))) break;
-        tc_fence_after_sync();
-        if (first) pv_steps(b, std::true_type{});
-        else pv_steps(b, std::false_type{});
         umma_commit(buf_free(b));   // to the S issuer, and to the V producer: the slot is free
-        ++tile;
-        first = tile == a.n_tiles;
-        if (first) tile = 0;
         if (first || i == nt - 1) umma_commit(o_full);
-        if (++b == kBufs) { b = 0; ph ^= 1u; }
       }
+      __syncwarp();
+      if (++b == kBufs) { b = 0; ph ^= 1u; }
     }
   } else {
     // ------------------------------------------------------------ softmax threads (one row each)
@@ -274,7 +274,8 @@ calib_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
     const int pair = grp >> 1, half = grp & 1;
     const uint32_t lane_bits = (uint32_t)((warp & 3) * 32) << 16;
     const uint32_t lane_addr = tmem_base + lane_bits;
-    float l0 = 0.f, l1 = 0.f, nlse2 = -INFINITY;
+    f32x2 lsum = 0ull, nl2 = pack2(-INFINITY);   // row sum in two parts; -lse2 of the row
+    const f32x2 sc = pack2(a.scale2);
     int seg = 0;
     bool ok = true, valid = false;
 
@@ -298,7 +299,8 @@ calib_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
             *reinterpret_cast<uint4*>(orow + c0 + e) = make_uint4(ov[e], ov[e + 1], ov[e + 2], ov[e + 3]);
         }
       }
-      if (valid) a.l_part[(part * kGroups + grp) * 128 + r] = l0 + l1;
+      const float2 l = unpack2(lsum);
+      if (valid) a.l_part[(part * kGroups + grp) * 128 + r] = l.x + l.y;
       tc_fence_before_sync();
       mbar_arrive(o_empty);
       return true;
@@ -310,10 +312,10 @@ calib_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
       const int g0 = cb * a.gpb;
       const int rows = min(a.gpb, a.G - g0) * a.n_cal;
       valid = r < rows;
-      nlse2 = -INFINITY;
+      nl2 = pack2(-INFINITY);
       if (valid) {
         const int g = g0 + r / a.n_cal, c = r - (r / a.n_cal) * a.n_cal;
-        nlse2 = -a.row_lse[(size_t)(hq0 + g) * a.W + (a.W - a.n_cal + c)] * kLog2e;
+        nl2 = pack2(-a.row_lse[(size_t)(hq0 + g) * a.W + (a.W - a.n_cal + c)] * kLog2e);
       }
     };
 
@@ -340,21 +342,29 @@ calib_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
     };
     // probabilities of 32 keys -> bf16 pairs -> 16 columns at paddr.  The
     // kept-key word is the same for every row of the tile, so the test on it is uniform; most
-    // words have no kept key (the kept keys are a few per cent and come in runs).
+    // words have no kept key (the kept keys are a few per cent and come in runs, so that a word with one
+    // still has bytes without).
     auto soft32 = [&](uint32_t (&sv)[32], uint32_t paddr, uint32_t w) {
 #pragma unroll
-      for (int e = 0; e < 32; ++e)
-        sv[e] = __float_as_uint(ex2_approx(fmaf(__uint_as_float(sv[e]), a.scale2, nlse2)));
+      for (int e = 0; e < 32; e += 2) {
+        const f32x2 x = fma2(pack2(sv[e], sv[e + 1]), sc, nl2);
+        const float2 p = unpack2(exp2_pair_on_poly(e / 2) ? exp2_poly2(x) : exp2_unit2(x));
+        sv[e] = __float_as_uint(p.x);
+        sv[e + 1] = __float_as_uint(p.y);
+      }
       if (w != 0u) {
 #pragma unroll
-        for (int e = 0; e < 32; ++e)
-          if ((w >> e) & 1u) sv[e] = 0u;
+        for (int e8 = 0; e8 < 32; e8 += 8)
+          if ((w >> e8) & 0xffu) {
+#pragma unroll
+            for (int e = e8; e < e8 + 8; ++e)
+              if ((w >> e) & 1u) sv[e] = 0u;
+          }
       }
       uint32_t packed[16];
 #pragma unroll
       for (int e = 0; e < 32; e += 2) {
-        l0 += __uint_as_float(sv[e]);
-        l1 += __uint_as_float(sv[e + 1]);
+        lsum = add2(lsum, pack2(sv[e], sv[e + 1]));
         packed[e >> 1] = pack_bf16(__uint_as_float(sv[e]), __uint_as_float(sv[e + 1]));
       }
       tmem_st16(paddr, packed);
@@ -372,10 +382,12 @@ calib_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
       while (t0 >= a.n_tiles) { t0 -= a.n_tiles; ++u0; }
       load_words(u0, t0, next_raw);
     }
+    int b = pair;            // S/P buffer of the pair's next tile, and the phase of its barriers
+    uint32_t ph = 0;
     int seg_first = 0, seg_tile0 = tile_begin, seg_unit = unit_begin, seg_vu = vu_begin;
     while (seg_first < nt) {
       const int seg_end = seg_first + min(nt - seg_first, a.n_tiles - seg_tile0);
-      l0 = l1 = 0.f;
+      lsum = 0ull;
       load_q(seg_vu);
       ++seg;
 #pragma unroll 1
@@ -388,11 +400,10 @@ calib_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
           load_words(u2, t2, next_raw);
         }
         if (tile == a.n_tiles - 1) tail_mask(tile, word);
-        const int b = i % kBufs;
         // S(i) of this group's keys; their P goes to the first 32 of the same 64 columns, which this
         // group alone reads, each 16 columns only after the S they held is in registers
         const uint32_t taddr = lane_addr + (uint32_t)(b * 128 + half * 64);
-        ok = mbar_wait(&ctl, s_full(b), (i / kBufs) & 1, 28u | ((unsigned)i << 8));
+        ok = mbar_wait(&ctl, s_full(b), ph, 28u | ((unsigned)i << 8));
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         tc_fence_after_sync();
@@ -406,6 +417,8 @@ calib_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
         tmem_st_wait();
         tc_fence_before_sync();
         mbar_arrive(p_full(b));
+        b += 2;   // the pair's next tile
+        if (b >= kBufs) { b -= kBufs; ph ^= 1u; }
       }
       if (!ok) break;
       ok = store_partial(seg_vu);

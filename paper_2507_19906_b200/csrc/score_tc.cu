@@ -192,16 +192,16 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
     bool first = true, ok = true;
     for (int i = 0; i < nt && ok; ++i) {
       if (first) {
-        ok = __all_sync(0xffffffffu, mbar_wait(&ctl, q_full, seg & 1, (kVotes ? 32u : 12u) | ((unsigned)i << 8)));
+        ok = __all_sync(0xffffffffu, mbar_wait_far(&ctl, q_full, seg & 1, (kVotes ? 32u : 12u) | ((unsigned)i << 8)));
         if (!ok) break;
         ++seg;
       }
-      ok = __all_sync(0xffffffffu, mbar_wait(&ctl, full_k(s), s_ph, (kVotes ? 33u : 13u) | ((unsigned)i << 8)));
+      ok = __all_sync(0xffffffffu, mbar_wait_far(&ctl, full_k(s), s_ph, (kVotes ? 33u : 13u) | ((unsigned)i << 8)));
       if (!ok) break;
       const uint64_t kd = desc_advance(dk0, (uint32_t)s * STAGE_BYTES);
       for (int blk = 0; blk < a.n_blocks; ++blk, ++j) {
         const int buf = j & ((1 << a.lg_bufs) - 1);
-        ok = __all_sync(0xffffffffu, mbar_wait(&ctl, t_empty(buf), ((j >> a.lg_bufs) & 1) ^ 1, (kVotes ? 34u : 14u) | ((unsigned)j << 8)));
+        ok = __all_sync(0xffffffffu, mbar_wait_far(&ctl, t_empty(buf), ((j >> a.lg_bufs) & 1) ^ 1, (kVotes ? 34u : 14u) | ((unsigned)j << 8)));
         if (!ok) break;
         tc_fence_after_sync();
         const uint32_t d = tmem_base + (uint32_t)(buf << (9 - a.lg_bufs));

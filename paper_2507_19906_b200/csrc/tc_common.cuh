@@ -62,8 +62,7 @@ struct Ctl {
 
 // Wait for the phase with the given parity to complete.  Returns false when the CTA is aborting
 // (this wait expired, or another thread's did).
-__device__ __forceinline__ bool mbar_wait(Ctl* ctl, uint32_t bar, uint32_t parity, unsigned code) {
-  if (mbar_try_wait(bar, parity)) return true;
+__device__ __forceinline__ bool mbar_wait_poll(Ctl* ctl, uint32_t bar, uint32_t parity, unsigned code) {
   long long t0 = 0;
   unsigned polls = 0;
   while (!mbar_try_wait(bar, parity)) {
@@ -79,6 +78,17 @@ __device__ __forceinline__ bool mbar_wait(Ctl* ctl, uint32_t bar, uint32_t parit
     }
   }
   return true;
+}
+__device__ __forceinline__ bool mbar_wait(Ctl* ctl, uint32_t bar, uint32_t parity, unsigned code) {
+  return mbar_try_wait(bar, parity) || mbar_wait_poll(ctl, bar, parity, code);
+}
+// The same with the polling out of line, for the warps that issue MMAs or copies: they share the instruction
+// caches with consumers whose unrolled loops stream through them, and pay for every line of code they touch.
+static __device__ __noinline__ bool mbar_wait_poll_far(Ctl* ctl, uint32_t bar, uint32_t parity, unsigned code) {
+  return mbar_wait_poll(ctl, bar, parity, code);
+}
+__device__ __forceinline__ bool mbar_wait_far(Ctl* ctl, uint32_t bar, uint32_t parity, unsigned code) {
+  return mbar_try_wait(bar, parity) || mbar_wait_poll_far(ctl, bar, parity, code);
 }
 
 // ---------------------------------------------------------------- TMA tile loads (no cluster forms)
