@@ -186,8 +186,8 @@ int calidrop_calibrate(const calidrop_params* p,
  *     Q_full in  [B, Hq, L, D] bf16, every prompt query (its last `window` rows are Q_obs)
  *     K      in  [B, Hkv, L, D] bf16
  *     scores out [B, Hkv, L] f32
- *     workspace: calidrop_accumulated_scores_workspace_bytes(p) bytes (the row statistics,
- *            4 B Hq L), 256-byte aligned; WORKSPACE_TOO_SMALL otherwise
+ *     workspace: calidrop_accumulated_scores_workspace_bytes(p) bytes (the row statistics and the
+ *            heads' column sums, 4 B Hq L each), 256-byte aligned; WORKSPACE_TOO_SMALL otherwise
  */
 int calidrop_select_streaming(const calidrop_params* p, int32_t n_sink, int32_t* kept_idx, void* stream);
 int calidrop_select_from_scores(const calidrop_params* p, const float* scores, int32_t tail, int32_t* kept_idx,

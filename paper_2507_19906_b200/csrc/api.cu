@@ -334,7 +334,7 @@ int calidrop_calibrate(const calidrop_params* p, const void* Q_obs, const void* 
 
 size_t calidrop_accumulated_scores_workspace_bytes(const calidrop_params* p) {
   if (check_compress(p) != CALIDROP_OK) return 0;
-  return align_up((size_t)p->B * p->Hq * p->L * 4, 256);
+  return accum_scores_workspace_bytes(p->B, p->Hq, p->L);
 }
 
 int calidrop_accumulated_scores(const calidrop_params* p, const void* Q_full, const void* K, float* scores,
@@ -348,7 +348,7 @@ int calidrop_accumulated_scores(const calidrop_params* p, const void* Q_full, co
   if (workspace_bytes < calidrop_accumulated_scores_workspace_bytes(p)) return CALIDROP_WORKSPACE_TOO_SMALL;
   if (!device_supported()) return CALIDROP_UNSUPPORTED;
   const CompressGeom g = make_geom(p);
-  cudaError_t e = launch_accum_scores(p->B, p->Hq, p->Hkv, p->L, g.scale2, Q_full, K, (float*)workspace, scores,
+  cudaError_t e = launch_accum_scores(p->B, p->Hq, p->Hkv, p->L, g.scale2, Q_full, K, (char*)workspace, scores,
                                       (cudaStream_t)stream);
   return e == cudaSuccess ? CALIDROP_OK : cuda_fail(e);
 }

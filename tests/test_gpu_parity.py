@@ -843,6 +843,35 @@ def test_h2o_accumulated_scores_from_the_library(cuda_lib, B, Hq, Hkv, L):
     assert cd.calidrop_accumulated_scores(p, None, to_dev(Kb), scores, ws, check=False) == cd.INVALID_ARG
 
 
+@pytest.mark.parametrize("B,Hq,Hkv,L", [
+    (1, 1, 1, 1),        # a single key
+    (1, 2, 1, 127),      # one partial row tile
+    (1, 3, 3, 128),      # full row tile, half a column tile
+    (2, 2, 1, 129),      # the second row tile holds one row, its job's second half is not seen
+    (1, 2, 2, 257),      # the second column tile holds one column
+    (2, 40, 8, 1025),    # 720 items: several per CTA, forwards and backwards, with odd and even job counts
+])
+def test_accumulated_scores_at_the_edges_of_their_tiles(cuda_lib, B, Hq, Hkv, L):
+    """Against attention in fp64.  A score sums up to G L probabilities, each with a relative error of about 2^-22
+    from exp2, 2^-24 |logit| from the fp32 logits and statistics; 2e-5 covers them tenfold."""
+    cd = cuda_lib
+    gen = torch.Generator(device="cuda").manual_seed(L)
+    Q = (2.0 * torch.randn((B, Hq, L, 128), generator=gen, device="cuda")).to(torch.bfloat16)
+    K = torch.randn((B, Hkv, L, 128), generator=gen, device="cuda").to(torch.bfloat16)
+    p = cd.make_params(B=B, Hq=Hq, Hkv=Hkv, L=L, window=1, pool=1, budget=L, n_cal=1, cap=L)
+    ws = torch.empty((cd.calidrop_accumulated_scores_workspace_bytes(p),), dtype=torch.uint8, device="cuda")
+    scores = torch.full((B, Hkv, L), -1.0, dtype=torch.float32, device="cuda")
+    cd.calidrop_accumulated_scores(p, Q, K, scores, ws)
+    G = Hq // Hkv
+    ref = torch.zeros((B, Hkv, L), dtype=torch.float64, device="cuda")
+    mask = torch.ones((L, L), dtype=torch.bool, device="cuda").triu(1)
+    for b in range(B):
+        for hq in range(Hq):
+            s = (Q[b, hq].double() @ K[b, hq // G].double().T) / 128 ** 0.5
+            ref[b, hq // G] += torch.softmax(s.masked_fill_(mask, -float("inf")), -1).sum(0)
+    torch.testing.assert_close(scores.double(), ref, rtol=2e-5, atol=1e-6)
+
+
 def test_calls_enqueued_back_to_back_give_the_results_of_calls_run_one_at_a_time(cuda_lib):
     """The kernels of a compress call start beside the end of their predecessors (programmatic dependent
     launch) and a decode launch prefetches ahead of its dependency wait: a stream of calls with no
