@@ -1,13 +1,17 @@
-"""ctypes binding of the C-ABI library (argument marshalling only).
+"""Binding of the C-ABI library (argument marshalling only).
 
 Every function here has the name of the `extern "C"` entry point it forwards to.  Tensors
 are torch CUDA tensors used purely as device memory; the current torch stream is passed as
-the library's stream.  Nothing in this module computes: if the shared library is missing the
-import of any entry point fails loudly, there is no fallback.
+the library's stream.  The entry points that a serving loop calls for every layer and token go
+through a small native module (csrc/marshal.cpp), the others through ctypes.  Nothing in this
+module computes: if the shared library is missing the import of any entry point fails loudly,
+there is no fallback.
 """
 from __future__ import annotations
 
 import ctypes as C
+import importlib.machinery
+import importlib.util
 import os
 from dataclasses import dataclass
 
@@ -16,7 +20,9 @@ import torch
 _HERE = os.path.dirname(os.path.abspath(__file__))
 # CALIDROP_LIB selects another build of the same library (e.g. an instrumented one).
 LIB_PATH = os.environ.get("CALIDROP_LIB") or os.path.join(_HERE, "libcalidrop.so")
+MARSHAL_PATH = os.path.join(_HERE, "_marshal.so")
 _lib = None
+_native = None
 
 OK, INVALID_ARG, UNSUPPORTED, WORKSPACE_TOO_SMALL, CUDA_ERROR, SCRATCH_LIMIT = 0, -1, -2, -3, -4, -5
 STATIC_SCRATCH_BYTES = 4 << 20
@@ -58,14 +64,24 @@ class CalidropError(RuntimeError):
         super().__init__(f"{where}: status {status} ({status_string(status)})")
 
 
+def _load_native():
+    """The marshalling module, forwarding to the library at LIB_PATH."""
+    loader = importlib.machinery.ExtensionFileLoader("_marshal", MARSHAL_PATH)
+    module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_marshal", loader))
+    loader.exec_module(module)
+    module.open(LIB_PATH)
+    return module
+
+
 def load():
     """Load libcalidrop.so (built in-tree by paper_2507_19906_b200/build.py)."""
-    global _lib
+    global _lib, _native
     if _lib is not None:
         return _lib
-    if not os.path.exists(LIB_PATH):
-        raise ImportError(f"{LIB_PATH} is not built; run `python -m paper_2507_19906_b200.build` "
-                          "(there is no CPU fallback)")
+    for path in (LIB_PATH, MARSHAL_PATH):
+        if not os.path.exists(path):
+            raise ImportError(f"{path} is not built; run `python -m paper_2507_19906_b200.build` "
+                              "(there is no CPU fallback)")
     lib = C.CDLL(LIB_PATH)
     lib.calidrop_compress_workspace_bytes.restype = C.c_size_t
     lib.calidrop_compress_workspace_bytes.argtypes = [C.POINTER(Params)]
@@ -113,8 +129,15 @@ def load():
     lib.calidrop_status_string.argtypes = [C.c_int]
     lib.calidrop_version.restype = C.c_int
     lib.calidrop_launch_count.restype = C.c_uint64
+    _native = _load_native()
     _lib = lib
     return lib
+
+
+def native():
+    if _native is None:
+        load()
+    return _native
 
 
 def make_params(*, B, Hq, Hkv, L=1, window=1, pool=1, budget=1, n_cal=1, cap, D=128,
@@ -174,9 +197,7 @@ def calidrop_compress_workspace_layout(p: Params) -> CompressLayout:
 
 def calidrop_compress(p, Q_obs, K, V, lse_obs, kept_idx, K_kept, V_kept, O_c, LSE_c, C_q, workspace,
                       check=True) -> int:
-    rc = load().calidrop_compress(C.byref(p), _ptr(Q_obs), _ptr(K), _ptr(V), _ptr(lse_obs), _ptr(kept_idx),
-                                  _ptr(K_kept), _ptr(V_kept), _ptr(O_c), _ptr(LSE_c), _ptr(C_q),
-                                  _ptr(workspace), workspace.numel() * workspace.element_size(), _stream())
+    rc = (_native or native()).compress(p, Q_obs, K, V, lse_obs, kept_idx, K_kept, V_kept, O_c, LSE_c, C_q, workspace)
     if check:
         _check(rc, "calidrop_compress")
     return rc
@@ -184,34 +205,28 @@ def calidrop_compress(p, Q_obs, K, V, lse_obs, kept_idx, K_kept, V_kept, O_c, LS
 
 def calidrop_calibrate(p, Q_obs, K, V, lse_obs, kept_idx, K_kept, V_kept, O_c, LSE_c, C_q, workspace,
                        check=True) -> int:
-    rc = load().calidrop_calibrate(C.byref(p), _ptr(Q_obs), _ptr(K), _ptr(V), _ptr(lse_obs), _ptr(kept_idx),
-                                   _ptr(K_kept), _ptr(V_kept), _ptr(O_c), _ptr(LSE_c), _ptr(C_q),
-                                   _ptr(workspace), workspace.numel() * workspace.element_size(), _stream())
+    rc = (_native or native()).calibrate(p, Q_obs, K, V, lse_obs, kept_idx, K_kept, V_kept, O_c, LSE_c, C_q, workspace)
     if check:
         _check(rc, "calidrop_calibrate")
     return rc
 
 
 def calidrop_gather_evicted(p, K, V, kept_idx, evict_idx, K_evict, V_evict, workspace, check=True) -> int:
-    rc = load().calidrop_gather_evicted(C.byref(p), _ptr(K), _ptr(V), _ptr(kept_idx), _ptr(evict_idx),
-                                        _ptr(K_evict), _ptr(V_evict), _ptr(workspace),
-                                        workspace.numel() * workspace.element_size(), _stream())
+    rc = (_native or native()).gather_evicted(p, K, V, kept_idx, evict_idx, K_evict, V_evict, workspace)
     if check:
         _check(rc, "calidrop_gather_evicted")
     return rc
 
 
 def calidrop_recalibrate(p, q, K_evict, V_evict, n_evict, slot, O_c, LSE_c, C_q, workspace, check=True) -> int:
-    rc = load().calidrop_recalibrate(C.byref(p), _ptr(q), _ptr(K_evict), _ptr(V_evict), int(n_evict), int(slot),
-                                     _ptr(O_c), _ptr(LSE_c), _ptr(C_q), _ptr(workspace),
-                                     workspace.numel() * workspace.element_size(), _stream())
+    rc = (_native or native()).recalibrate(p, q, K_evict, V_evict, n_evict, slot, O_c, LSE_c, C_q, workspace)
     if check:
         _check(rc, "calidrop_recalibrate")
     return rc
 
 
 def calidrop_select_streaming(p, n_sink, kept_idx, check=True) -> int:
-    rc = load().calidrop_select_streaming(C.byref(p), int(n_sink), _ptr(kept_idx), _stream())
+    rc = (_native or native()).select_streaming(p, n_sink, kept_idx)
     if check:
         _check(rc, "calidrop_select_streaming")
     return rc
@@ -222,16 +237,14 @@ def calidrop_accumulated_scores_workspace_bytes(p: Params) -> int:
 
 
 def calidrop_accumulated_scores(p, Q_full, K, scores, workspace, check=True) -> int:
-    rc = load().calidrop_accumulated_scores(C.byref(p), _ptr(Q_full), _ptr(K), _ptr(scores), _ptr(workspace),
-                                            workspace.numel() * workspace.element_size(), _stream())
+    rc = (_native or native()).accumulated_scores(p, Q_full, K, scores, workspace)
     if check:
         _check(rc, "calidrop_accumulated_scores")
     return rc
 
 
 def calidrop_select_from_scores(p, scores, tail, kept_idx, workspace, check=True) -> int:
-    rc = load().calidrop_select_from_scores(C.byref(p), _ptr(scores), int(tail), _ptr(kept_idx), _ptr(workspace),
-                                            workspace.numel() * workspace.element_size(), _stream())
+    rc = (_native or native()).select_from_scores(p, scores, tail, kept_idx, workspace)
     if check:
         _check(rc, "calidrop_select_from_scores")
     return rc
@@ -276,11 +289,8 @@ def calidrop_decode_workspace_init(workspace) -> int:
 
 def calidrop_decode(p, q, k_new, v_new, K_kept, V_kept, kv_len, O_c, LSE_c, C_q, out, lse_out, flags,
                     workspace, check=True) -> int:
-    rc = load().calidrop_decode(C.byref(p), _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(K_kept), _ptr(V_kept),
-                                int(kv_len), _ptr(O_c), _ptr(LSE_c), _ptr(C_q), _ptr(out), _ptr(lse_out),
-                                _ptr(flags), _ptr(workspace), workspace.numel() * workspace.element_size(),
-                                _stream())
-    if check:
+    rc = (_native or native()).decode(p, q, k_new, v_new, K_kept, V_kept, kv_len, O_c, LSE_c, C_q, out, lse_out, flags, workspace)
+    if check and rc:
         _check(rc, "calidrop_decode")
     return rc
 
@@ -288,9 +298,7 @@ def calidrop_decode(p, q, k_new, v_new, K_kept, V_kept, kv_len, O_c, LSE_c, C_q,
 def calidrop_decode_static(p, q, k_new, v_new, K_kept, V_kept, kv_len, O_c, LSE_c, C_q, out, lse_out, flags,
                            check=True) -> int:
     """calidrop_decode with the library's built-in scratch: no workspace argument, nothing allocated."""
-    rc = load().calidrop_decode_static(C.byref(p), _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(K_kept),
-                                       _ptr(V_kept), int(kv_len), _ptr(O_c), _ptr(LSE_c), _ptr(C_q), _ptr(out),
-                                       _ptr(lse_out), _ptr(flags), _stream())
+    rc = (_native or native()).decode_static(p, q, k_new, v_new, K_kept, V_kept, kv_len, O_c, LSE_c, C_q, out, lse_out, flags)
     if check:
         _check(rc, "calidrop_decode_static")
     return rc
@@ -306,8 +314,7 @@ def make_decode_layers(layers):
 
 
 def calidrop_decode_batched(p, layer_array, kv_len, workspace, check=True) -> int:
-    rc = load().calidrop_decode_batched(C.byref(p), len(layer_array), layer_array, int(kv_len), _ptr(workspace),
-                                        workspace.numel() * workspace.element_size(), _stream())
+    rc = (_native or native()).decode_batched(p, layer_array, kv_len, workspace)
     if check:
         _check(rc, "calidrop_decode_batched")
     return rc

@@ -281,6 +281,42 @@ def test_invalid_arguments_have_no_effect(cuda_lib):
     assert "invalid" in cd.status_string(cd.INVALID_ARG)
 
 
+def test_binding_refuses_what_it_cannot_pass_on(cuda_lib):
+    """The native marshalling: tensors, addresses, None and integers of any integer type go through; strided
+    tensors, wrong counts and other objects raise before anything is enqueued."""
+    cd = cuda_lib
+    cfg = wl.small_config()
+    Q, K, V = _inputs(cfg)
+    g = gpu_compress(Q, K, V, window=8, pool=5, budget=40, n_cal=1, cap=42)
+    p, st = g.p, g.st
+    q = to_dev(wl.gen_decode_inputs(cfg, Q, steps=1)[0][0])
+    out = torch.full((1, 4, 128), 7.0, dtype=torch.bfloat16, device="cuda")
+
+    def call(qq=q, kv_len=40, oo=out, ws=st.ws_decode):
+        return cd.calidrop_decode(p, qq, None, None, st.K_kept, st.V_kept, kv_len, st.O_c, st.LSE_c, st.C_q, oo, None, None,
+                                  ws)
+
+    launches = cd.calidrop_launch_count()
+    with pytest.raises(AssertionError):
+        call(qq=torch.empty((1, 4, 256), dtype=torch.bfloat16, device="cuda")[:, :, ::2])
+    with pytest.raises(TypeError):
+        call(qq="q")
+    with pytest.raises(TypeError):
+        call(ws=None)
+    with pytest.raises(OverflowError):
+        call(kv_len=1 << 40)
+    with pytest.raises(cd.CalidropError):
+        call(qq=None)
+    with pytest.raises(TypeError):
+        cd.native().decode(p, q)
+    assert cd.calidrop_launch_count() == launches and torch.all(out == 7.0)
+    call(kv_len=np.int32(40))
+    want = out.clone()
+    out.zero_()
+    call(qq=q.data_ptr(), oo=out.data_ptr())
+    assert torch.equal(out, want)
+
+
 def test_batched_layers_match_single_layer_calls(cuda_lib):
     cd = cuda_lib
     cfg = wl.small_config(B=2, Hq=4, Hkv=2, L=260, window=8, pool=5, budget=40, layers=3)
