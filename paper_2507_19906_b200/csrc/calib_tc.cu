@@ -441,7 +441,7 @@ calib_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
 }
 
 // One warp per (batch, query head, calibration row): sum the partials of the CTAs that shared the
-// row's virtual unit, in order, then O_c = O / l, LSE_c = lse + log l (zeros and -inf when nothing
+// row's virtual unit, in a fixed order, then O_c = O / l, LSE_c = lse + log l (zeros and -inf when nothing
 // was evicted), C_q = the query.  The blocks beyond the reduction's compact the retained rows.
 __global__ void __launch_bounds__(256)
 calib_reduce_kernel(const __nv_bfloat16* __restrict__ Q_obs, const float* __restrict__ row_lse,
@@ -466,13 +466,23 @@ calib_reduce_kernel(const __nv_bfloat16* __restrict__ Q_obs, const float* __rest
   const int vu = unit * n_cblocks + cb;
   const int first = (unit * n_tiles) / tiles_per_cta, last = ((unit + 1) * n_tiles - 1) / tiles_per_cta;
   const size_t part0 = (size_t)vu * max_slots;
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  const int n = last - first + 1;
+  // the row sums: the lanes take the slots' and groups' partials side by side
   float l = 0.f;
-  for (int s = 0; s <= last - first; ++s) {
-    const float4 v = *reinterpret_cast<const float4*>(o_part + ((part0 + s) * 128 + r) * kD + 4 * lane);
-    acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
-    for (int grp = 0; grp < kGroups; ++grp) l += l_part[((part0 + s) * kGroups + grp) * 128 + r];
+  for (int i = lane; i < n * kGroups; i += 32) l += l_part[(part0 * kGroups + i) * 128 + r];
+  // O: the slots in order, eight loads in flight (one after the other, a unit spread over 16 CTAs cost 10 us)
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  const float4* op = reinterpret_cast<const float4*>(o_part + (part0 * 128 + r) * kD) + lane;
+  constexpr int kSlotStride = 128 * kD / 4;
+  for (int s0 = 0; s0 < n; s0 += 8) {
+    float4 v[8];
+#pragma unroll
+    for (int s = 0; s < 8; ++s)
+      v[s] = s0 + s < n ? op[(size_t)(s0 + s) * kSlotStride] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int s = 0; s < 8; ++s) { acc.x += v[s].x; acc.y += v[s].y; acc.z += v[s].z; acc.w += v[s].w; }
   }
+  l = warp_sum(l);
   const int qrow = W - n_cal + c;
   float4 out = make_float4(0.f, 0.f, 0.f, 0.f);
   float lse = -INFINITY;
