@@ -249,19 +249,21 @@ int calidrop_compress(const calidrop_params* p, const void* Q_obs, const void* K
 
   cudaStream_t st = (cudaStream_t)stream;
   char* wsp = (char*)workspace;
-  cudaError_t e = cudaMemsetAsync(wsp + ws.status, 0, 4, st);
-  if (e != cudaSuccess) return cuda_fail(e);
   // The contractions run on the tensor cores whenever the tiles cover the shape; the scalar
   // kernels remain for the rest (more than 512 window rows per kv head, budget >= L).
   const bool tc_path = score_tc_supported(g);
+  // the error word is cleared by the call's first tensor-core kernel, where it has one
+  cudaError_t e = tc_path ? cudaSuccess : cudaMemsetAsync(wsp + ws.status, 0, 4, st);
+  if (e != cudaSuccess) return cuda_fail(e);
   const float* row_lse = lse_obs;
   if (!g.keep_all) {
     if (!row_lse) {
-      e = tc_path ? launch_row_stats_tc(g, ws, Q_obs, K, wsp, st) : launch_row_stats(g, ws, Q_obs, K, wsp, st);
+      e = tc_path ? launch_row_stats_tc(g, ws, Q_obs, K, wsp, true, st) : launch_row_stats(g, ws, Q_obs, K, wsp, st);
       if (e != cudaSuccess) return cuda_fail(e);
       row_lse = (const float*)(wsp + ws.row_lse);
     }
-    e = tc_path ? launch_votes_tc(g, ws, Q_obs, K, row_lse, wsp, st) : launch_votes(g, ws, Q_obs, K, row_lse, wsp, st);
+    e = tc_path ? launch_votes_tc(g, ws, Q_obs, K, row_lse, wsp, lse_obs != nullptr, st)
+                : launch_votes(g, ws, Q_obs, K, row_lse, wsp, st);
     if (e != cudaSuccess) return cuda_fail(e);
   }
   if (select_cluster_supported(g)) {
@@ -282,7 +284,7 @@ int calidrop_compress(const calidrop_params* p, const void* Q_obs, const void* K
   if (g.sized && g.n_calib == 0)
     e = launch_calib_none(g, Q_obs, O_c, LSE_c, C_q, st);
   else
-    e = calib_tc ? launch_calib_tc(g, ws, Q_obs, K, V, row_lse, wsp, O_c, LSE_c, C_q, ga, st)
+    e = calib_tc ? launch_calib_tc(g, ws, Q_obs, K, V, row_lse, wsp, O_c, LSE_c, C_q, ga, false, st)
                  : launch_calib_direct(g, ws, Q_obs, K, V, wsp, O_c, LSE_c, C_q, st);
   if (e != cudaSuccess) return cuda_fail(e);
   return CALIDROP_OK;
@@ -306,27 +308,28 @@ int calidrop_calibrate(const calidrop_params* p, const void* Q_obs, const void* 
 
   cudaStream_t st = (cudaStream_t)stream;
   char* wsp = (char*)workspace;
-  cudaError_t e = cudaMemsetAsync(wsp + ws.status, 0, 4, st);
+  const bool tc_path = score_tc_supported(g), calib_tc = tc_path && calib_tc_supported(g);
+  // the error word is cleared by the call's first tensor-core kernel, where it has one
+  const bool stats_tc = tc_path && !lse_obs;
+  cudaError_t e = stats_tc || calib_tc ? cudaSuccess : cudaMemsetAsync(wsp + ws.status, 0, 4, st);
   if (e != cudaSuccess) return cuda_fail(e);
-  const bool tc_path = score_tc_supported(g);
   // the calibration probabilities refer to the full-row softmax: its row LSE comes from the caller
   // or from the statistics pass of the scoring
   const float* row_lse = lse_obs;
   if (!g.keep_all && !row_lse) {
-    e = tc_path ? launch_row_stats_tc(g, ws, Q_obs, K, wsp, st) : launch_row_stats(g, ws, Q_obs, K, wsp, st);
+    e = tc_path ? launch_row_stats_tc(g, ws, Q_obs, K, wsp, true, st) : launch_row_stats(g, ws, Q_obs, K, wsp, st);
     if (e != cudaSuccess) return cuda_fail(e);
     row_lse = (const float*)(wsp + ws.row_lse);
   }
   e = launch_bitmap_from_indices(g, ws, wsp, kept_idx, st);
   if (e != cudaSuccess) return cuda_fail(e);
-  const bool calib_tc = tc_path && calib_tc_supported(g);
   if (!calib_tc) {
     e = launch_gather(g, K, V, kept_idx, K_kept, V_kept, st);
     if (e != cudaSuccess) return cuda_fail(e);
   }
   const GatherArgs ga{(const uint4*)K, (const uint4*)V, kept_idx, (uint4*)K_kept, (uint4*)V_kept,
                       g.L, g.n_kept, g.cap, g.units};
-  e = calib_tc ? launch_calib_tc(g, ws, Q_obs, K, V, row_lse, wsp, O_c, LSE_c, C_q, ga, st)
+  e = calib_tc ? launch_calib_tc(g, ws, Q_obs, K, V, row_lse, wsp, O_c, LSE_c, C_q, ga, !stats_tc, st)
                : launch_calib_direct(g, ws, Q_obs, K, V, wsp, O_c, LSE_c, C_q, st);
   if (e != cudaSuccess) return cuda_fail(e);
   return CALIDROP_OK;

@@ -63,6 +63,7 @@ struct CalibArgs {
   float* o_part;           // [virtual unit][slot][128][128]
   float* l_part;           // [virtual unit][slot][group][128]
   unsigned* status;
+  int clear_status;        // the first kernel of a call clears the error word
 };
 
 __global__ void __launch_bounds__(kThreads, 1)
@@ -126,6 +127,7 @@ calib_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
   tc_fence_after_sync();
   const uint32_t tmem_base = tmem_slot;
   pdl_wait();   // everything above ran beside the previous kernel's end; global memory from here on
+  if (a.clear_status && blockIdx.x == 0 && tid == 0) *a.status = 0u;   // (see score_tc.cu)
 
   // first tile of a run of tiles of one virtual unit inside this CTA's range
   // (the position inside the tile space is tracked incrementally: no division per tile)
@@ -522,8 +524,9 @@ void calib_tc_plan(const CompressGeom& g, int* gpb, int* n_cblocks, int* tiles_p
 
 cudaError_t launch_calib_tc(const CompressGeom& g, const CompressWs& ws, const void* Q_obs, const void* K,
                             const void* V, const float* row_lse, char* wsp, float* O_c, float* LSE_c, void* C_q,
-                            const GatherArgs& gather, cudaStream_t st) {
+                            const GatherArgs& gather, bool first, cudaStream_t st) {
   CalibArgs a{};
+  a.clear_status = first;
   a.Hq = g.Hq; a.G = g.G; a.W = g.W; a.L = g.L; a.n_cand = g.n_cand; a.n_cal = g.n_cal;
   size_t parts;
   calib_tc_plan(g, &a.gpb, &a.n_cblocks, &a.tiles_per_cta, &a.max_slots, &parts);

@@ -95,9 +95,9 @@ cudaError_t launch_calib_direct(const CompressGeom& g, const CompressWs& ws, con
 int pick_tile_splits(int groups, int n_tiles, int min_tiles);
 bool score_tc_supported(const CompressGeom& g);
 cudaError_t launch_row_stats_tc(const CompressGeom& g, const CompressWs& ws, const void* Q_obs, const void* K,
-                                char* wsp, cudaStream_t st);
+                                char* wsp, bool first, cudaStream_t st);
 cudaError_t launch_votes_tc(const CompressGeom& g, const CompressWs& ws, const void* Q_obs, const void* K,
-                            const float* row_lse, char* wsp, cudaStream_t st);
+                            const float* row_lse, char* wsp, bool first, cudaStream_t st);
 int votes_tc_parts(const CompressGeom& g);
 cudaError_t launch_add_votes(const CompressGeom& g, const CompressWs& ws, char* wsp, cudaStream_t st);
 bool calib_tc_supported(const CompressGeom& g);
@@ -117,7 +117,7 @@ struct GatherArgs {
 };
 cudaError_t launch_calib_tc(const CompressGeom& g, const CompressWs& ws, const void* Q_obs, const void* K,
                             const void* V, const float* row_lse, char* wsp, float* O_c, float* LSE_c, void* C_q,
-                            const GatherArgs& gather, cudaStream_t st);
+                            const GatherArgs& gather, bool first, cudaStream_t st);
 #ifdef __CUDACC__
 // Rows [16 bx, 16 bx + 16) of unit `unit`: 16 lanes x 16 bytes per row, 256 threads.
 __device__ __forceinline__ void gather_rows16(const GatherArgs& a, int bx, int unit, int tid) {

@@ -62,6 +62,7 @@ struct ScoreArgs {
   float* vote_parts;     // votes: out [part][units, n_cand], a part per (row block, column half)
   float2* stat_part;     // statistics: out [row][slot][2 or 4 groups] (max, sum) in the log2 domain
   unsigned* status;
+  int clear_status;      // the first kernel of a call clears the error word
 };
 
 // sum of exp2 of 32 logits against one reference, four independent partial sums
@@ -146,6 +147,9 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
   tc_fence_after_sync();
   const uint32_t tmem_base = tmem_slot;
   pdl_wait();   // everything above ran beside the previous kernel's end; global memory from here on
+  // (an error code is stored seconds into a wait, long after this; a memset ahead of the kernel would cost the chain
+  // of programmatic launches 2 us)
+  if (a.clear_status && blockIdx.x == 0 && tid == 0) *a.status = 0u;
 
   if (warp == kProducerWarp) {
     // ------------------------------------------------------------ TMA producer
@@ -468,11 +472,13 @@ bool score_tc_supported(const CompressGeom& g) {
   return !g.keep_all && g.G * g.W <= kMaxRows && g.W <= 128 && g.n_cand >= 1;
 }
 
-// Statistics (row LSE) of the G*W observation rows of every unit, into ws.row_lse.
+// Statistics (row LSE) of the G*W observation rows of every unit, into ws.row_lse.  `first`: of a call, the kernel
+// then clears the workspace's error word.
 cudaError_t launch_row_stats_tc(const CompressGeom& g, const CompressWs& ws, const void* Q_obs, const void* K,
-                                char* wsp, cudaStream_t st) {
+                                char* wsp, bool first, cudaStream_t st) {
   const int GW = g.G * g.W;
   ScoreArgs a{};
+  a.clear_status = first;
   a.Hq = g.Hq; a.G = g.G; a.W = g.W; a.L = g.L; a.n_cand = g.n_cand; a.GW = GW;
   a.vu_per_unit = (GW + 255) / 256;
   a.vu_rows = 256;
@@ -514,9 +520,10 @@ int votes_tc_parts(const CompressGeom& g) { return g.G * g.W <= 128 ? 1 : 2 * ((
 
 // Partial votes of every candidate key, into ws.vote_parts; the selection adds them up.
 cudaError_t launch_votes_tc(const CompressGeom& g, const CompressWs& ws, const void* Q_obs, const void* K,
-                            const float* row_lse, char* wsp, cudaStream_t st) {
+                            const float* row_lse, char* wsp, bool first, cudaStream_t st) {
   const int GW = g.G * g.W;
   ScoreArgs a{};
+  a.clear_status = first;
   a.Hq = g.Hq; a.G = g.G; a.W = g.W; a.L = g.L; a.n_cand = g.n_cand; a.GW = GW;
   a.vu_per_unit = 1;
   a.vu_rows = 0;
