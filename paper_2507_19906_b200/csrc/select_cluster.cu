@@ -1,6 +1,6 @@
 // Pooling + per-(batch, kv-head) top-k on thread-block clusters.
 //
-// A cluster of 1..8 CTAs shares a unit: CTA r owns the contiguous key range [r * chunk, (r + 1) * chunk),
+// A cluster of 1..16 CTAs shares a unit: CTA r owns the contiguous key range [r * chunk, (r + 1) * chunk),
 // every thread keeps its ROWS keys (pooled votes as fp32 bit patterns; non-negative, so unsigned order is
 // numeric order) in registers, and the CTAs exchange only histograms and counts through distributed
 // shared memory.  Exact radix select, digits of 8 + 8 + 8 + 7 bits (the sign bit is zero), finds a threshold
@@ -25,8 +25,11 @@
 // 16 x 5003 with a calibration size 22.8 -> 19.2 us, 8 x 8192 11.9 -> 13.8 us (in a stream of calls, beside the
 // neighbouring kernels, 1.2 us less per call all the same).  Wider digits, 11 + 10 + 10 bits with two
 // histograms per CTA, were slower, 47 us at 32 x 32768: the votes' few exponents share bins.
+// Then, the partial votes loaded in batches (they were a chain of round trips) and sixteen CTAs for a unit where few
+// units share the GPU: compress calls of 4 x 131072 keys 339 -> 325 us, 32 x 32768 379 -> 371 us, 64 x 16384 184 -> 180 us.
 #include <cooperative_groups.h>
 
+#include <atomic>
 #include <type_traits>
 
 #include "common.cuh"
@@ -38,7 +41,7 @@ namespace {
 
 namespace cg = cooperative_groups;
 
-constexpr int kMaxClu = 8;
+constexpr int kPortableClu = 8, kMaxClu = 16;   // clusters of more than eight CTAs where few units leave the GPU idle
 constexpr int kHaloMax = 64;   // widest half pool that is staged; wider pools read the votes from global memory
 
 struct SelectArgs {
@@ -52,7 +55,8 @@ struct SelectArgs {
   int n_parts, n_cand, L, pool, k_sel, n_kept, bitmap_words, n_calib;
 };
 
-template <int T, int ROWS, bool kSized>
+// kClu: the most CTAs a cluster of this instantiation has.
+template <int T, int ROWS, bool kSized, int kClu>
 __global__ void __launch_bounds__(T)
 pool_select_cluster_kernel(const SelectArgs a) {
   constexpr int kW = T / 32;
@@ -60,10 +64,11 @@ pool_select_cluster_kernel(const SelectArgs a) {
   constexpr int kThr = kSized ? 2 : 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned* const hist = reinterpret_cast<unsigned*>(smem_raw);            // [kThr][256][32]
-  float* const stage = reinterpret_cast<float*>(hist + kThr * 256 * 32);   // [kChunk + 2 * kHaloMax]
-  __shared__ __align__(16) unsigned counts[2][kThr][kMaxClu][256];   // every CTA's histogram (double-buffered)
+  unsigned* const counts = hist + kThr * 256 * 32;   // [2][kThr][kClu][256]: every CTA's histogram (double-buffered)
+  float* const stage = reinterpret_cast<float*>(counts + 2 * kThr * kClu * 256);   // [kChunk + 2 * kHaloMax]
+  auto counts_of = [&](int buf, int x, int r) { return counts + ((buf * kThr + x) * kClu + r) * 256; };
   __shared__ unsigned sel_bin[kThr], sel_k[kThr], sel_all[kThr];
-  __shared__ unsigned cnt[kMaxClu][kThr][2];      // every CTA's keys > T and == T, per threshold
+  __shared__ unsigned cnt[kClu][kThr][2];         // every CTA's keys > T and == T, per threshold
   __shared__ unsigned wcnt[kThr][32][2];          // this CTA's, per warp
 
   pdl_trigger();
@@ -93,11 +98,38 @@ pool_select_cluster_kernel(const SelectArgs a) {
   const bool staged = half <= kHaloMax;
   if (staged) {
     const int n_stage = min(kChunk, n_cand - c0) + 2 * half;   // (not positive when only window rows are left)
-#pragma unroll 4
-    for (int i = tid; i < n_stage; i += T) {
-      const int t = c0 - half + i;
-      stage[i] = t >= 0 && t < n_cand ? vote_at(t) : 0.f;
-    }
+    float* const vs = a.vote_sum ? a.vote_sum + (size_t)unit * n_cand : nullptr;
+    // up to 16 loads of a thread in flight: one position after the other, a thread of a 131072-key prompt walked 64
+    // dependent round trips here (4 parts of 16 keys; 30.5 thousand cycles, now 4)
+    auto stage_parts = [&](auto parts_tag) __attribute__((always_inline)) {
+      constexpr int kParts = decltype(parts_tag)::value;
+      constexpr int kBatch = ROWS < 16 / kParts ? ROWS : 16 / kParts;
+#pragma unroll 1
+      for (int i0 = tid; i0 < n_stage; i0 += kBatch * T) {
+        float x[kBatch][kParts];
+#pragma unroll
+        for (int j = 0; j < kBatch; ++j) {
+          const int i = i0 + j * T, t = c0 - half + i;
+          const bool in = i < n_stage && t >= 0 && t < n_cand;
+#pragma unroll
+          for (int q = 0; q < kParts; ++q) x[j][q] = in ? __ldcg(v + (size_t)q * a.part_stride + t) : 0.f;
+        }
+#pragma unroll
+        for (int j = 0; j < kBatch; ++j) {
+          const int i = i0 + j * T, own = i - half;
+          float sum = x[j][0];
+#pragma unroll
+          for (int q = 1; q < kParts; ++q) sum += x[j][q];
+          if (i < n_stage) {
+            stage[i] = sum;
+            if (vs && own >= 0 && own < min(kChunk, n_cand - c0)) vs[c0 + own] = sum;
+          }
+        }
+      }
+    };
+    if (a.n_parts == 1) stage_parts(std::integral_constant<int, 1>{});
+    else if (a.n_parts == 2) stage_parts(std::integral_constant<int, 2>{});
+    else stage_parts(std::integral_constant<int, 4>{});
   }
   __syncthreads();
   unsigned key[ROWS];
@@ -139,9 +171,9 @@ pool_select_cluster_kernel(const SelectArgs a) {
         }
       }
   }
-  if (a.vote_sum)
+  if (a.vote_sum && !staged)
     for (int i = tid; i < min(kChunk, n_cand - c0); i += T)
-      a.vote_sum[(size_t)unit * n_cand + c0 + i] = staged ? stage[i + half] : vote_at(c0 + i);
+      a.vote_sum[(size_t)unit * n_cand + c0 + i] = vote_at(c0 + i);
   if (n_clu > 1) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
 
   // 2. radix select, most significant digit first.  thr[x] ends as the threshold of selection x, k[x] as the
@@ -179,7 +211,7 @@ pool_select_cluster_kernel(const SelectArgs a) {
       // pushed to every CTA of the cluster: stores to a peer cost no round trip, loads from it would
       if (lane < kPer)
         for (int r = 0; r < n_clu; ++r)
-          cluster.map_shared_rank(&counts[pass & 1][x][rank][0], r)[warp * kPer + lane] = m;
+          cluster.map_shared_rank(counts_of(pass & 1, x, rank), r)[warp * kPer + lane] = m;
     }
     if (n_clu > 1) cluster.sync();
     else __syncthreads();
@@ -188,8 +220,8 @@ pool_select_cluster_kernel(const SelectArgs a) {
       const int x = warp;
       unsigned c[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
 #pragma unroll
-      for (int r = 0; r < kMaxClu; ++r) {
-        const uint4* h = reinterpret_cast<const uint4*>(&counts[pass & 1][x][r][0]) + 2 * (31 - lane);
+      for (int r = 0; r < kClu; ++r) {
+        const uint4* h = reinterpret_cast<const uint4*>(counts_of(pass & 1, x, r)) + 2 * (31 - lane);
         uint4 lo = make_uint4(0u, 0u, 0u, 0u), hi = lo;
         if (r < n_clu) { lo = h[0]; hi = h[1]; }
         c[7] += lo.x; c[6] += lo.y; c[5] += lo.z; c[4] += lo.w;
@@ -298,37 +330,75 @@ pool_select_cluster_kernel(const SelectArgs a) {
     for (int j = tid; j < a.L - n_cand; j += T) kept[a.k_sel + j] = n_cand + j;
 }
 
-template <int T, int ROWS, bool kSized>
-cudaError_t launch_select(const SelectArgs& a, int units, cudaStream_t st) {
-  constexpr int kSmem = (kSized ? 2 : 1) * 256 * 32 * 4 + (ROWS * T + 2 * kHaloMax) * 4;
-  static bool attr_set[64] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-    e = cudaFuncSetAttribute(pool_select_cluster_kernel<T, ROWS, kSized>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) attr_set[dev] = true;
+template <int T, int ROWS, bool kSized, int kClu>
+struct Launch {
+  static constexpr int kSmem = ((kSized ? 2 : 1) * (256 * 32 + 2 * kClu * 256) + ROWS * T + 2 * kHaloMax) * 4;
+
+  static void config(int n_clu, int units, cudaStream_t st, cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&attr)[2]) {
+    cfg = cudaLaunchConfig_t{};
+    cfg.gridDim = dim3(n_clu, units);
+    cfg.blockDim = dim3(T);
+    cfg.dynamicSmemBytes = kSmem;
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = n_clu;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
   }
-  const int n_clu = (a.L + T * ROWS - 1) / (T * ROWS);
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(n_clu, units);
-  cfg.blockDim = dim3(T);
-  cfg.dynamicSmemBytes = kSmem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = n_clu;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 2;
-  e = cudaLaunchKernelEx(&cfg, pool_select_cluster_kernel<T, ROWS, kSized>, a);
-  count_launch(1);
-  return e != cudaSuccess ? e : cudaGetLastError();
-}
+
+  // What the current device needs set up once.  `resident`: clusters of kClu CTAs it runs at the same time (only asked
+  // for beyond the portable size, where the shape of the device's processor clusters decides).
+  static cudaError_t setup(int* resident) {
+    static std::atomic<int> known[64];   // 0: not set up yet, else 1 + resident
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const bool slot = dev >= 0 && dev < 64;
+    int n = slot ? known[dev].load(std::memory_order_acquire) : 0;
+    if (n == 0) {
+      auto* kernel = pool_select_cluster_kernel<T, ROWS, kSized, kClu>;
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+      if (e != cudaSuccess) return e;
+      int active = 0;
+      if (kClu > kPortableClu) {
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return e;
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute attr[2];
+        config(kClu, 1, nullptr, cfg, attr);
+        cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&active, kernel, &cfg) != cudaSuccess) {
+          cudaGetLastError();   // no such cluster on this device
+          active = 0;
+        }
+      }
+      n = 1 + active;
+      if (slot) known[dev].store(n, std::memory_order_release);
+    }
+    if (resident) *resident = n - 1;
+    return cudaSuccess;
+  }
+
+  static bool all_resident(const SelectArgs& a, int units) {
+    int resident = 0;
+    return a.L <= kClu * T * ROWS && setup(&resident) == cudaSuccess && units <= resident;
+  }
+
+  static cudaError_t run(const SelectArgs& a, int units, cudaStream_t st) {
+    cudaError_t e = setup(nullptr);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[2];
+    config((a.L + T * ROWS - 1) / (T * ROWS), units, st, cfg, attr);
+    e = cudaLaunchKernelEx(&cfg, pool_select_cluster_kernel<T, ROWS, kSized, kClu>, a);
+    count_launch(1);
+    return e != cudaSuccess ? e : cudaGetLastError();
+  }
+};
 
 template <bool kSized>
 cudaError_t launch_any(const SelectArgs& a, int units, cudaStream_t st) {
@@ -339,19 +409,26 @@ cudaError_t launch_any(const SelectArgs& a, int units, cudaStream_t st) {
   auto clusters = [&](int chunk) { return (a.L + chunk - 1) / chunk; };
   auto fits = [&](int rows) {
     const int c = clusters(512 * rows);
-    return c <= kMaxClu && (long long)c * units <= 2 * 148;
+    return c <= kPortableClu && (long long)c * units <= 2 * 148;
   };
-  if (fits(4)) return launch_select<512, 4, kSized>(a, units, st);
-  if (fits(8)) return launch_select<512, 8, kSized>(a, units, st);
-  if (a.L <= kMaxClu * 512 * 16) return launch_select<512, 16, kSized>(a, units, st);
-  if (a.L <= kMaxClu * 1024 * 16) return launch_select<1024, 16, kSized>(a, units, st);
-  return launch_select<1024, 32, kSized>(a, units, st);
+  if (fits(4)) return Launch<512, 4, kSized, kPortableClu>::run(a, units, st);
+  if (fits(8)) return Launch<512, 8, kSized, kPortableClu>::run(a, units, st);
+  // Longer prompts of few units: up to sixteen CTAs per unit, half the keys per thread.
+  if (a.L > kPortableClu * 512 * 8) {
+    using C8 = Launch<1024, 8, kSized, kMaxClu>;
+    using C16 = Launch<1024, 16, kSized, kMaxClu>;
+    if (C8::all_resident(a, units)) return C8::run(a, units, st);
+    if (a.L > kPortableClu * 1024 * 16 && C16::all_resident(a, units)) return C16::run(a, units, st);
+  }
+  if (a.L <= kPortableClu * 512 * 16) return Launch<512, 16, kSized, kPortableClu>::run(a, units, st);
+  if (a.L <= kPortableClu * 1024 * 16) return Launch<1024, 16, kSized, kPortableClu>::run(a, units, st);
+  return Launch<1024, 32, kSized, kPortableClu>::run(a, units, st);
 }
 
 }  // namespace
 
 // The cluster kernel keeps at most 32 keys per thread: 8 CTAs x 1024 threads x 32.
-bool select_cluster_supported(const CompressGeom& g) { return !g.keep_all && g.L <= kMaxClu * 1024 * 32; }
+bool select_cluster_supported(const CompressGeom& g) { return !g.keep_all && g.L <= kPortableClu * 1024 * 32; }
 
 // Selection from per-candidate scores [parts][units][stride] (the window votes of the workspace, or a
 // caller's scores); vote_sum receives the sum of the parts when it is not null.

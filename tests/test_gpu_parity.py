@@ -106,6 +106,18 @@ def test_selection_from_scores_at_the_edges_of_its_launch_shapes(cuda_lib, units
         np.testing.assert_array_equal(got[u], np.concatenate([want, np.arange(n, L)]))
 
 
+@pytest.mark.parametrize("units,L,tail,pool,budget", [
+    (1, 32769, 1, 7, 300),         # five CTAs of 1024 x 8, the last with one window row only
+    (2, 131072, 64, 5, 4096),      # sixteen CTAs, full
+    (1, 131073, 9, 1, 131000),     # nine CTAs of 1024 x 16
+    (40, 33000, 8, 7, 64),         # more clusters of sixteen than run at once: eight CTAs of 512 x 16
+    (30, 66000, 8, 3, 500),        # ... of 1024 x 16
+])
+def test_selection_on_clusters_of_more_than_eight(cuda_lib, units, L, tail, pool, budget):
+    """As above, with the clusters of up to sixteen CTAs that long prompts of few units get, and past their edge."""
+    test_selection_from_scores_at_the_edges_of_its_launch_shapes(cuda_lib, units, L, tail, pool, budget, False)
+
+
 @pytest.mark.parametrize("calib_size", [1, 40, 300, 10 ** 6, -1])
 def test_calibration_size(cuda_lib, calib_size):
     """Section 4.4's calibration size m: only the m evicted rows of highest pooled vote are calibrated
