@@ -404,11 +404,8 @@ int calidrop_gather_evicted(const calidrop_params* p, const void* K, const void*
   if (!device_supported()) return CALIDROP_UNSUPPORTED;
   cudaStream_t st = (cudaStream_t)stream;
   char* wsp = (char*)workspace;
-  cudaError_t e = cudaSuccess;
   // sized calibration: the mask of the calibrated rows is the one calidrop_compress left in this workspace
-  if (!g.sized) e = launch_bitmap_from_indices(g, ws, wsp, kept_idx, st);
-  if (e != cudaSuccess) return cuda_fail(e);
-  e = launch_evicted_indices(g, ws, wsp, evict_idx, st);
+  cudaError_t e = launch_evicted_indices(g, ws, wsp, kept_idx, evict_idx, st);
   if (e != cudaSuccess) return cuda_fail(e);
   const int n_evict = g.n_calib;
   e = launch_gather_rows(g, K, V, evict_idx, n_evict, n_evict, K_evict, V_evict, st);

@@ -161,8 +161,8 @@ cudaError_t launch_decode(const DecodeArgsT<kDecodeMaxLayers>& a, cudaStream_t s
 // The same stream over the evicted KV (K, V of the layer = the compacted evicted rows), rewriting
 // row recal_slot of O_c, LSE_c, C_q (Algorithm 2, lines 4-6).
 cudaError_t launch_recalibrate(const DecodeArgsT<1>& a, cudaStream_t st);
-cudaError_t launch_evicted_indices(const CompressGeom& g, const CompressWs& ws, char* wsp, int32_t* evict_idx,
-                                   cudaStream_t st);
+cudaError_t launch_evicted_indices(const CompressGeom& g, const CompressWs& ws, char* wsp, const int32_t* kept_idx,
+                                   int32_t* evict_idx, cudaStream_t st);
 // Calibration size -1: no row is calibrated (O_c = 0, LSE_c = -inf, C_q = the calibration queries).
 cudaError_t launch_calib_none(const CompressGeom& g, const void* Q_obs, float* O_c, float* LSE_c, void* C_q,
                               cudaStream_t st);

@@ -176,6 +176,8 @@ __global__ void bitmap_from_indices_kernel(const int32_t* __restrict__ kept_idx,
 
 // K_kept[u, i, :] = K[u, kept_idx[u, i], :], same for V; 16 lanes x 16 bytes per row.
 __global__ void __launch_bounds__(256) gather_kernel(const GatherArgs a) {
+  pdl_trigger();
+  pdl_wait();
   gather_rows16(a, blockIdx.x, blockIdx.y, threadIdx.x);
 }
 
@@ -196,66 +198,92 @@ cudaError_t launch_pool_select(const CompressGeom& g, const CompressWs& ws, char
   return cudaGetLastError();
 }
 
-// Ascending list of the evicted candidates of a unit: the zero bits of its kept bitmap below n_cand.
-// One CTA per unit; thread i owns a contiguous run of bitmap words, so a block-wide exclusive scan of
-// the per-thread counts gives every thread the position of its first index.
-__global__ void __launch_bounds__(kSelThreads)
-evicted_indices_kernel(const uint32_t* __restrict__ bitmap, int32_t* __restrict__ evict_idx, int n_cand, int n_evict,
-                       int bitmap_words) {
-  __shared__ unsigned warp_sum[kSelThreads / 32];
-  const int unit = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint32_t* bm = bitmap + (size_t)unit * bitmap_words;
-  int32_t* out = evict_idx + (size_t)unit * n_evict;
+// Ascending list of the evicted candidates: the zero bits below n_cand of a bitmap, which is either given
+// (kFromList = false) or built here from the kept list, in shared memory.  A CTA emits the rows of kEvictSlice words of a
+// unit (8192 rows); for the position of its first one it counts the zero bits ahead of it itself, which is cheaper than
+// a second kernel or a chain through the CTAs.  32 units x 32768 rows: 31 us as memset, bitmap kernel and one CTA per unit;
+// the recompute pass around it 280 -> 257 us.  A warp emits a word at a time, so its stores are consecutive.
+constexpr int kEvictSlice = 256;                    // words per CTA, one per thread
+constexpr int kEvictListWords = 40 * 1024 / 4;      // longest bitmap that is built in shared memory (327680 rows)
+
+template <bool kFromList>
+__global__ void __launch_bounds__(kEvictSlice)
+evicted_indices_kernel(const int32_t* __restrict__ kept_idx, const uint32_t* __restrict__ bitmap,
+                       int32_t* __restrict__ evict_idx, int n_kept, int n_cand, int n_evict, int bitmap_words) {
+  extern __shared__ uint32_t list_bits[];           // kFromList: the unit's words up to the end of this slice
+  __shared__ unsigned warp_tot[2][kEvictSlice / 32];
+  pdl_trigger();
+  pdl_wait();
+  const int unit = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n_words = (n_cand + 31) >> 5;
-  const int wpt = (n_words + kSelThreads - 1) / kSelThreads;
-  const int w0 = tid * wpt, w1 = min(n_words, w0 + wpt);
+  const int w0 = blockIdx.x * kEvictSlice, w_end = min(n_words, w0 + kEvictSlice);
+  const uint32_t* bm = bitmap + (size_t)unit * bitmap_words;
+  if (kFromList) {
+    for (int w = tid; w < w_end; w += kEvictSlice) list_bits[w] = 0u;
+    __syncthreads();
+    const int32_t* kept = kept_idx + (size_t)unit * n_kept;
+#pragma unroll 4
+    for (int i = tid; i < n_kept; i += kEvictSlice) {
+      const int t = kept[i];
+      if (t >= 0 && (t >> 5) < w_end) atomicOr(&list_bits[t >> 5], 1u << (t & 31));
+    }
+    __syncthreads();
+  }
   auto zeros_of = [&](int w) {
-    uint32_t z = ~bm[w];
+    uint32_t z = kFromList ? ~list_bits[w] : ~__ldcg(bm + w);
     const int rem = n_cand - (w << 5);
     if (rem < 32) z &= (1u << rem) - 1u;
     return z;
   };
-  // entries that no zero bit fills (a kept list with fewer candidates than expected leaves fewer
-  // evicted rows than n_evict) hold -1, which the gather skips
-  for (int i = tid; i < n_evict; i += kSelThreads) out[i] = -1;
-  __syncthreads();
-  unsigned cnt = 0;
-  for (int w = w0; w < w1; ++w) cnt += __popc(zeros_of(w));
-  unsigned incl = cnt;
+  unsigned ahead = 0u;                              // zero bits ahead of the slice
+#pragma unroll 4
+  for (int w = tid; w < w0; w += kEvictSlice) ahead += __popc(zeros_of(w));
+  const uint32_t mine = w0 + tid < w_end ? zeros_of(w0 + tid) : 0u;
+  unsigned incl = __popc(mine);
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const unsigned n = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl += n;
   }
-  if (lane == 31) warp_sum[warp] = incl;
+  ahead = __reduce_add_sync(0xffffffffu, ahead);
+  if (lane == 31) { warp_tot[0][warp] = ahead; warp_tot[1][warp] = incl; }
   __syncthreads();
-  if (warp == 0) {
-    unsigned v = lane < kSelThreads / 32 ? warp_sum[lane] : 0u, iv = v;
+  unsigned base = 0u, total = 0u;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned n = __shfl_up_sync(0xffffffffu, iv, o);
-      if (lane >= o) iv += n;
-    }
-    if (lane < kSelThreads / 32) warp_sum[lane] = iv - v;
+  for (int w = 0; w < kEvictSlice / 32; ++w) {
+    base += warp_tot[0][w] + (w < warp ? warp_tot[1][w] : 0u);
+    total += warp_tot[0][w] + warp_tot[1][w];
   }
-  __syncthreads();
-  unsigned pos = warp_sum[warp] + incl - cnt;
-  for (int w = w0; w < w1; ++w) {
-    uint32_t z = zeros_of(w);
-    while (z) {
-      const int b = __ffs(z) - 1;
-      z &= z - 1;
-      if (pos < (unsigned)n_evict) out[pos] = (w << 5) + b;
-      ++pos;
-    }
+  int32_t* out = evict_idx + (size_t)unit * n_evict;
+  const unsigned first = base + incl - __popc(mine);   // position of the first zero bit of this thread's word
+#pragma unroll 4
+  for (int k = 0; k < 32; ++k) {
+    const uint32_t z = __shfl_sync(0xffffffffu, mine, k);
+    const unsigned pos = __shfl_sync(0xffffffffu, first, k) + __popc(z & ((1u << lane) - 1u));
+    if (((z >> lane) & 1u) && pos < (unsigned)n_evict) out[pos] = (w0 + warp * 32 + k) * 32 + lane;
   }
+  // entries that no zero bit fills (a kept list with fewer candidates than expected leaves fewer
+  // evicted rows than n_evict) hold -1, which the gather skips
+  if (blockIdx.x == gridDim.x - 1)
+    for (unsigned i = total + tid; i < (unsigned)n_evict; i += kEvictSlice) out[i] = -1;
 }
 
-cudaError_t launch_evicted_indices(const CompressGeom& g, const CompressWs& ws, char* wsp, int32_t* evict_idx,
-                                   cudaStream_t st) {
-  // the zero bits below n_cand of the kept bitmap, or of the calibration mask when the calibration is sized
-  evicted_indices_kernel<<<g.units, kSelThreads, 0, st>>>((const uint32_t*)(wsp + ws.calib_mask), evict_idx, g.n_cand,
-                                                          g.n_calib, g.bitmap_words);
+// The rows of a kept list that are not in it, or (sized calibration) the zero bits of the calibration mask.
+cudaError_t launch_evicted_indices(const CompressGeom& g, const CompressWs& ws, char* wsp, const int32_t* kept_idx,
+                                   int32_t* evict_idx, cudaStream_t st) {
+  const int n_words = (g.n_cand + 31) / 32;
+  const dim3 grid((n_words + kEvictSlice - 1) / kEvictSlice, g.units), block(kEvictSlice);
+  const uint32_t* mask = (const uint32_t*)(wsp + ws.calib_mask);
+  cudaError_t e;
+  if (!g.sized && n_words <= kEvictListWords) {
+    e = launch_pdl(evicted_indices_kernel<true>, grid, block, (size_t)n_words * 4, st, kept_idx, mask, evict_idx, g.n_kept,
+                   g.n_cand, g.n_calib, g.bitmap_words);
+  } else {
+    if (!g.sized && (e = launch_bitmap_from_indices(g, ws, wsp, kept_idx, st)) != cudaSuccess) return e;
+    e = launch_pdl(evicted_indices_kernel<false>, grid, block, 0, st, kept_idx, mask, evict_idx, g.n_kept, g.n_cand,
+                   g.n_calib, g.bitmap_words);
+  }
+  if (e != cudaSuccess) return e;
   count_launch(1);
   return cudaGetLastError();
 }
@@ -299,7 +327,8 @@ cudaError_t launch_gather_rows(const CompressGeom& g, const void* K, const void*
                                int out_rows, void* K_out, void* V_out, cudaStream_t st) {
   dim3 grid((n_rows + 15) / 16, g.units);
   const GatherArgs a{(const uint4*)K, (const uint4*)V, idx, (uint4*)K_out, (uint4*)V_out, g.L, n_rows, out_rows, g.units};
-  gather_kernel<<<grid, 256, 0, st>>>(a);
+  cudaError_t e = launch_pdl(gather_kernel, grid, dim3(256), 0, st, a);
+  if (e != cudaSuccess) return e;
   count_launch(1);
   return cudaGetLastError();
 }

@@ -667,6 +667,39 @@ def test_calibrate_with_a_supplied_kept_list(cuda_lib, B, Hq, Hkv, L, W, budget,
 
 
 # ---------------------------------------------------------------- the recompute branch (Algorithm 2, lines 3-8)
+@pytest.mark.parametrize("units,L,W,budget", [
+    (3, 8192 + 8, 8, 40),         # one slice of the index kernel, full
+    (3, 8192 + 9, 8, 8000),       # one candidate in the second slice, most rows kept
+    (1, 40000, 32, 64),           # five slices
+    (1, 330000, 8, 16),           # a bitmap longer than the one built in shared memory
+])
+def test_evicted_list_at_the_edges_of_its_slices(cuda_lib, units, L, W, budget):
+    """The complement of a caller's list, in any order and with entries twice or outside the prompt: those leave fewer
+    kept rows, and the rows past the budgeted number of evicted ones are dropped."""
+    cd = cuda_lib
+    rng = np.random.Generator(np.random.Philox(key=[67, L]))
+    kept = np.stack([rng.permutation(L - W)[:budget] for _ in range(units)]).astype(np.int32)
+    kept[0, 0], kept[0, 1] = -5, L + 3
+    kept[-1, 2] = kept[-1, 3]
+    p = cd.make_params(B=1, Hq=units, Hkv=units, L=L, window=W, pool=1, budget=budget, n_cal=1, cap=budget)
+    n_e = L - budget
+    K = torch.arange(L, device="cuda").view(1, 1, L, 1).expand(1, units, L, 128).to(torch.bfloat16).contiguous()
+    V = -K
+    ws = torch.empty((cd.calidrop_compress_workspace_bytes(p),), dtype=torch.uint8, device="cuda")
+    ev = torch.empty((1, units, n_e), dtype=torch.int32, device="cuda")
+    K_e = torch.zeros((1, units, n_e, 128), dtype=torch.bfloat16, device="cuda")
+    V_e = torch.zeros_like(K_e)
+    cd.calidrop_gather_evicted(p, K, V, torch.from_numpy(kept[None]).cuda(), ev, K_e, V_e, ws)
+    got = ev.cpu().numpy()[0]
+    for u in range(units):
+        want = np.setdiff1d(np.arange(L - W), kept[u])[:n_e]
+        np.testing.assert_array_equal(got[u, :len(want)], want)
+        assert (got[u, len(want):] == -1).all()
+        rows = torch.from_numpy(want).cuda()
+        assert torch.equal(K_e[0, u, :len(want)], K[0, u, rows]) and torch.equal(V_e[0, u, :len(want)], V[0, u, rows])
+        assert not K_e[0, u, len(want):].any()
+
+
 @pytest.mark.parametrize("B,Hq,Hkv,L,W,budget,n_cal,slot", [
     (1, 4, 2, 600, 16, 80, 1, 0),          # the paper's single calibration query
     (2, 8, 2, 1500, 32, 256, 4, 2),        # G = 4, one of four rows rewritten
