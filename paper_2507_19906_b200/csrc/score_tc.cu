@@ -110,8 +110,13 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
   const int g_end = min(a.total_tiles, g_begin + a.tiles_per_cta);
   const int nt = g_end - g_begin;
   const int Hkv = a.Hq / a.G;
+  // The statistics walk their range upwards and the votes downwards: the keys that the pass ahead read last are still in
+  // L2, and so are those that the votes read last when the calibration, upwards again, starts.
   // (the position inside the tile space is tracked incrementally: no division per tile)
-  const int vu_begin = g_begin / a.n_tiles, tile_begin = g_begin - vu_begin * a.n_tiles;
+  const int g_first = kVotes ? max(g_end - 1, g_begin) : g_begin;
+  const int vu_begin = g_first / a.n_tiles, tile_begin = g_first - vu_begin * a.n_tiles;
+  constexpr int kDir = kVotes ? -1 : 1;
+  const int unit_tile0 = kVotes ? a.n_tiles - 1 : 0, past_tile = kVotes ? -1 : a.n_tiles;  // a virtual unit's first tile, past its last
 
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t q_half_bytes = (uint32_t)a.block_rows * kLineBytes;
@@ -157,8 +162,8 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
       tma_prefetch_desc(&q_map);
       tma_prefetch_desc(&k_map);
       int cur_vu = -1, seg = 0, vu = vu_begin, tile = tile_begin, unit = vu_begin / a.vu_per_unit;
-      for (int i = 0; i < nt; ++i, ++tile) {
-        if (tile == a.n_tiles) { tile = 0; ++vu; unit = vu / a.vu_per_unit; }
+      for (int i = 0; i < nt; ++i, tile += kDir) {
+        if (tile == past_tile) { tile = unit_tile0; vu += kDir; unit = vu / a.vu_per_unit; }
         if (vu != cur_vu) {
           // the query rows of the next virtual unit replace the current ones once its MMAs are done
           if (seg > 0 && !mbar_wait(&ctl, q_empty, (seg - 1) & 1, (kVotes ? 36u : 16u) | ((unsigned)i << 8))) break;
@@ -225,9 +230,9 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
         __syncwarp();
       }
       if (!ok) break;
-      ++tile;
-      first = tile == a.n_tiles;
-      if (first) tile = 0;
+      tile += kDir;
+      first = tile == past_tile;
+      if (first) tile = unit_tile0;
       if (leader) {
         umma_commit(empty_k(s));
         if (first || i == nt - 1) umma_commit(q_empty);
@@ -269,7 +274,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
 
     int seg0 = 0, seg_tile0 = tile_begin, vu = vu_begin;
     while (seg0 < nt && ok) {
-      const int seg_n = min(nt - seg0, a.n_tiles - seg_tile0);
+      const int seg_n = min(nt - seg0, kVotes ? seg_tile0 + 1 : a.n_tiles - seg_tile0);
       const int unit = vu / a.vu_per_unit, row0 = (vu - unit * a.vu_per_unit) * a.vu_rows;
       const int hq0 = (unit / Hkv) * a.Hq + (unit % Hkv) * a.G;
       float* vote_out = nullptr;                 // votes: this group's part of the unit's votes
@@ -291,9 +296,9 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
       }
       // the first tile of the segment that is this buffer's: tile i of the CTA goes to buffer i % step
       const int first = (buf - seg0) & (step - 1);
-      int key0 = (seg_tile0 + first) * TILE_KEYS;
+      int key0 = (seg_tile0 + kDir * first) * TILE_KEYS;
 #pragma unroll 1
-      for (int i = first; i < seg_n; i += step, key0 += step * TILE_KEYS) {
+      for (int i = first; i < seg_n; i += step, key0 += kDir * step * TILE_KEYS) {
         ok = mbar_wait(&ctl, bar_full, ph, (kVotes ? 35u : 15u) | ((unsigned)i << 8));
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
@@ -374,8 +379,8 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
           a.stat_part[(((size_t)hq0 * a.W + row) * a.max_slots + slot) * n_part + (a.n_blocks > 1 ? half : grp)] = ml;
       }
       seg0 += seg_n;
-      seg_tile0 = 0;
-      ++vu;
+      seg_tile0 = unit_tile0;
+      vu += kDir;
     }
   }
 
