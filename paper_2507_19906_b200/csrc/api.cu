@@ -146,23 +146,34 @@ DecodeWs make_decode_ws(const calidrop_params* p) {
 
 // Split plan and workspace carving of one decode-kernel launch over `cap_rows`-row caches.
 DecodeCommon plan_decode(const calidrop_params* p, const DecodeWs& w, int n_layers, int kv_len, int n_kv,
-                         bool has_new, int cap_rows, void* workspace) {
+                         bool has_new, int cap_rows, bool recal, void* workspace) {
   DecodeCommon a{};
   a.B = p->B; a.Hq = p->Hq; a.Hkv = p->Hkv; a.G = p->Hq / p->Hkv; a.n_cal = p->n_cal; a.cap = cap_rows;
   a.kv_len = kv_len; a.n_kv = n_kv; a.has_new = has_new ? 1 : 0;
   a.units = p->B * p->Hkv; a.n_layers = n_layers;
-  // the splits of a unit form one thread-block cluster: 1, 2, 4 or 8 CTAs
-  int want = decode_nsplit(a.units * n_layers, n_kv);
+  // The splits of a unit form one thread-block cluster of 1, 2, 4, 8 or 16 CTAs, or several clusters that meet through the
+  // workspace.  What a choice costs, in microseconds: the clusters that the device does not hold at once queue for a
+  // second round (eight CTAs: 15 clusters on a B200, whose processor clusters differ in size; 16 units on clusters of
+  // eight took two rounds); a round is a fixed chain (4.4) and the longest slice, at 5.8 ns per row of one CTA or at the
+  // rate of the memory if that is less; the meeting of several clusters costs 4, that of sixteen CTAs 1.4 more than of
+  // eight.  Measured per launch: 4 units x 4333 rows 7.4 (8 CTAs) and 7.0 (16), x 2100 rows 6.2 and 6.8, x 15000 rows
+  // 15.1 and 11.0; 8 units x 20000 rows on 16 clusters of eight 29.5.
+  const int units_total = a.units * n_layers;
+  int want = decode_nsplit(units_total, n_kv);
   if (want > w.max_split) want = w.max_split;
-  a.nsplit = 1;
-  while (a.nsplit * 2 <= want && a.nsplit < 8) a.nsplit *= 2;
-  // Few units with a long cache: several clusters per unit, combined through the workspace.  That
-  // combine costs about 4 us (fences, a ticket, a round trip through L2), as much as a CTA needs
-  // to stream a thousand rows, so a unit is split only while every CTA keeps at least 1024 rows.
-  a.nclu = want / a.nsplit;
-  const int rows_single = (n_kv + a.nsplit - 1) / a.nsplit;
-  if (a.nclu > rows_single / 1024) a.nclu = rows_single / 1024;
-  if (a.nclu < 1) a.nclu = 1;
+  const double memory = (double)units_total * n_kv * kRowBytes * 2 / 6.3e6;
+  double best = 0.0;
+  a.nsplit = a.nclu = 1;
+  for (int ns = 1; ns <= (recal ? 8 : 16) && ns <= want; ns *= 2) {
+    const int resident = want > 1 ? decode_resident_clusters(ns) : 1;
+    for (int nc = 1; resident > 0 && nc <= 8 && ns * nc <= want; ++nc) {
+      const int rounds = (units_total * nc + resident - 1) / resident;
+      const double rows = (double)((n_kv + ns * nc - 1) / (ns * nc));
+      const double slice = rows * 5.8e-3, share = memory / rounds;
+      const double t = rounds * (4.4 + (slice > share ? slice : share)) + (nc > 1 ? 4.0 : 0.0) + (ns > 8 ? 1.4 : 0.0);
+      if ((ns == 1 && nc == 1) || t < best) { best = t; a.nsplit = ns; a.nclu = nc; }
+    }
+  }
   a.rows_per_split = (n_kv + a.nsplit * a.nclu - 1) / (a.nsplit * a.nclu);
   a.scale2 = scale2_of(p);
   a.theta1 = p->theta1; a.theta2 = p->theta2; a.always_apply = p->theta2 <= -1.0f;
@@ -456,7 +467,7 @@ int calidrop_recalibrate(const calidrop_params* p, const void* q, const void* K_
   if (workspace_bytes < w.per_layer) return CALIDROP_WORKSPACE_TOO_SMALL;
   if (!device_supported()) return CALIDROP_UNSUPPORTED;
   DecodeArgsT<1> args{};
-  args.c = plan_decode(p, w, 1, n_evict, n_evict, false, n_evict, workspace);
+  args.c = plan_decode(p, w, 1, n_evict, n_evict, false, n_evict, true, workspace);
   args.c.recal_slot = slot;
   args.layer[0] = DecodeLayerPtrs{q, nullptr, nullptr, const_cast<void*>(K_evict), const_cast<void*>(V_evict), O_c,
                                   LSE_c, C_q, nullptr, nullptr, nullptr};
@@ -503,7 +514,7 @@ int calidrop_decode_batched(const calidrop_params* p, int32_t n_layers, const ca
   if (workspace_bytes < w.per_layer * (size_t)n_layers) return CALIDROP_WORKSPACE_TOO_SMALL;
   if (!device_supported()) return CALIDROP_UNSUPPORTED;
 
-  DecodeCommon a = plan_decode(p, w, n_layers, kv_len, n_kv, has_new, p->cap, workspace);
+  DecodeCommon a = plan_decode(p, w, n_layers, kv_len, n_kv, has_new, p->cap, false, workspace);
   cudaError_t e;
   if (n_layers == 1) {
     DecodeArgsT<1> args{};

@@ -8,11 +8,12 @@
 // what matters is how the bytes get to the SM and how short the chain after the last byte is.
 //
 // Grid: (split, batch*kv-head, layer); the splits of one (unit, layer) form thread-block
-// clusters of 1, 2, 4 or 8 CTAs.  A CTA has one producer warp and eight stream warps.  The
+// clusters of 1, 2, 4, 8 or 16 CTAs.  A CTA has one producer warp and eight stream warps.  The
 // producer moves the CTA's slice of K and V through a ring of six 64-row slots with TMA
 // (128-byte swizzle, so ldmatrix is conflict-free and no load instruction per 16 bytes is
 // spent on the stream); each slot is consumed by four stream warps, 16 rows each, with their
-// own online softmax.  The products are taken transposed, keys on the 16-row side of the MMA and
+// own online softmax.  Launches of more (unit, layer) pairs than SMs take smaller CTAs, several to an
+// SM, one per pair (ShapePair, ShapeNarrow).  The products are taken transposed, keys on the 16-row side of the MMA and
 // the (at most eight) heads on its 8-column side, so that no half of a tile is padding:
 //   S^T[16 keys x 8 heads]   = K_blk[16 x 128] . Q^T[128 x 8]          (8 MMAs)
 //   O^T[128 dims x 8 heads] += V_blk^T[128 x 16 keys] . P^T[16 x 8]     (8 MMAs)
@@ -20,8 +21,8 @@
 // finishes a slice of the 128 output dimensions for all heads of the group, and each CTA pushes
 // its partial of a slice into the shared memory of the slice's owner with asynchronous stores that
 // report their bytes to an mbarrier there, so that every CTA waits for its own data only and then
-// reduces local data.  Only when very few units share a very long cache
-// (more than 1024 rows per CTA even with a cluster of eight) does a unit get up to eight clusters;
+// reduces local data.  Where few units share a very long cache (see
+// plan_decode) a unit gets up to eight clusters;
 // each writes its combined partial, its (max, sum) pair and its best similarity to the workspace, and
 // the CTA that takes the last ticket of the unit's arrival counter merges them and resets the counter.
 //
@@ -38,6 +39,8 @@
 //   * the cache stream carries an evict-first L2 hint, the calibration state an evict-last hint.
 #include <cooperative_groups.h>
 
+#include <atomic>
+
 #include "common.cuh"
 #include "internal.h"
 #include "tc_common.cuh"
@@ -48,22 +51,33 @@ namespace {
 
 namespace cg = cooperative_groups;
 
-constexpr int kStreamWarps = 8;
-constexpr int kThreads = (kStreamWarps + 1) * 32;  // the last warp is the producer
 constexpr int kBlkRows = 16;                        // rows of one warp's MMA block
-constexpr int kSlotRows = 64;                       // rows per ring slot: four blocks
-constexpr int kSlotsWide = 6;    // ring of a launch with one CTA per SM at most: 192 KB
-constexpr int kSlotsNarrow = 3;  // ring of a launch with more CTAs than SMs: 96 KB, two CTAs per SM
-constexpr int kPlaneBytes = kSlotRows * 128;        // 64 rows x 64 columns of bf16 (one TMA box)
-constexpr int kSlotBytes = 4 * kPlaneBytes;         // K low / K high / V low / V high column halves
-constexpr int smem_bytes(int slots) { return slots * kSlotBytes + 1024; }  // + slack for the 1024-byte alignment
+constexpr int kWideRows = 64;                       // rows of the boxes of whole slots in the wide shape
+// The shape of a CTA: ring slots of kRows rows, each consumed by kRows / 16 warps, kWarps stream warps in two groups on
+// alternate slots, kCtas CTAs per SM.
+template <int kSlots_, int kRows_, int kCtas_, int kClu_>
+struct Shape {
+  static constexpr int kSlots = kSlots_, kRows = kRows_, kCtas = kCtas_;
+  static constexpr int kClu = kClu_;                // the most CTAs of a cluster
+  static constexpr int kSubs = kRows / kBlkRows;    // warps per slot
+  static constexpr int kStreamWarps = 2 * kSubs;
+  static constexpr int kThreads = (kStreamWarps + 1) * 32;   // the last warp is the producer
+  static constexpr int kPlaneBytes = kRows * 128;   // rows x 64 columns of bf16
+  static constexpr int kSlotBytes = 4 * kPlaneBytes;         // K low / K high / V low / V high column halves
+  static constexpr int kSmemBytes = kSlots * kSlotBytes + 1024;   // + slack for the 1024-byte alignment
+};
+using ShapeWide = Shape<6, kWideRows, 1, 8>;     // a launch with one CTA per SM at most: 192 KB
+using ShapeCluster16 = Shape<6, kWideRows, 1, 16>;  // few units with a longer cache (see plan_decode)
+using ShapePair = Shape<3, kWideRows, 2, 1>;     // a launch with up to two CTAs per SM: 96 KB
+using ShapeNarrow = Shape<3, 32, 4, 1>;          // more than that: 48 KB, four CTAs per SM
 constexpr int kWoStride = kD + 4;  // row stride of the per-warp partial outputs: heads land in distinct banks
 constexpr long long kWaitLimitCycles = 2000000000ll;  // about a second: a wait this long has failed
 
-// Byte offset of 16-byte chunk `chunk` (0..15) of row `row` (0..63) inside the K or V part of a
-// slot: two column halves, each a [64 rows][128 bytes] plane in the 128-byte swizzle TMA writes.
+// Byte offset of 16-byte chunk `chunk` (0..15) of row `row` inside the K or V part of a
+// slot: two column halves, each a [rows][128 bytes] plane in the 128-byte swizzle TMA writes.
+template <class S>
 __device__ __forceinline__ uint32_t plane_off(int row, int chunk) {
-  return (uint32_t)((chunk >> 3) * kPlaneBytes + row * 128 + (((chunk & 7) ^ (row & 7)) << 4));
+  return (uint32_t)((chunk >> 3) * S::kPlaneBytes + row * 128 + (((chunk & 7) ^ (row & 7)) << 4));
 }
 
 __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t x) {
@@ -146,6 +160,13 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, unsigned bytes, uint32_t bar, uint64_t pol) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(dst),
+      "l"(src), "r"(bytes), "r"(bar), "l"(pol)
+      : "memory");
+}
+
 // L2 eviction policies.  The retained cache is read once per call and is far larger than what the
 // next call on the same state finds in L2 again, so its lines are marked to go first; the
 // calibration state (C_q, the chosen O_c rows, LSE_c) is small and read by every call, so its
@@ -191,17 +212,20 @@ struct RhoLoad {
   uint4 q0, q1, c0, c1;
 };
 
-__device__ __forceinline__ void rho_accumulate(const RhoLoad& r, float& dot, float& qq, float& cc) {
-  const uint32_t qw[8] = {r.q0.x, r.q0.y, r.q0.z, r.q0.w, r.q1.x, r.q1.y, r.q1.z, r.q1.w};
-  const uint32_t cw[8] = {r.c0.x, r.c0.y, r.c0.z, r.c0.w, r.c1.x, r.c1.y, r.c1.z, r.c1.w};
+__device__ __forceinline__ void rho_accumulate(const uint4& q, const uint4& c, float& dot, float& qq, float& cc) {
+  const uint32_t qw[4] = {q.x, q.y, q.z, q.w}, cw[4] = {c.x, c.y, c.z, c.w};
 #pragma unroll
-  for (int j = 0; j < 8; ++j) {
+  for (int j = 0; j < 4; ++j) {
     const float a0 = bf16_lo(qw[j]), a1 = bf16_hi(qw[j]);
     const float b0 = bf16_lo(cw[j]), b1 = bf16_hi(cw[j]);
     dot = fmaf(a0, b0, fmaf(a1, b1, dot));
     qq = fmaf(a0, a0, fmaf(a1, a1, qq));
     cc = fmaf(b0, b0, fmaf(b1, b1, cc));
   }
+}
+__device__ __forceinline__ void rho_accumulate(const RhoLoad& r, float& dot, float& qq, float& cc) {
+  rho_accumulate(r.q0, r.c0, dot, qq, cc);
+  rho_accumulate(r.q1, r.c1, dot, qq, cc);
 }
 
 // Order-preserving map of a float onto unsigned integers; with the row index in the low word,
@@ -224,13 +248,17 @@ __device__ __forceinline__ void cluster_wait() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Gate and merge of one output element (Eq. 1-2): (acc, M, Lsum) is the unnormalised partial of
+// Gate and merge (Eq. 1-2) of `kN` neighbouring output elements of a head: (acc, M, Lsum) is the unnormalised partial of
 // the retained cache in the log2 domain, best the chosen (similarity, calibration row) key.
-__device__ __forceinline__ void merge_store(const DecodeCommon& a, const DecodeLayerPtrs& P, int hq, int d, float acc,
-                                            float M, float Lsum, unsigned long long best, float lse_c, float oc) {
+template <int kN>
+__device__ __forceinline__ void merge_store(const DecodeCommon& a, const DecodeLayerPtrs& P, int hq, int d,
+                                            const float (&acc)[kN], float M, float Lsum, unsigned long long best,
+                                            float lse_c, const float (&oc)[kN]) {
   const int cs = (int)(unsigned)(best & 0xffffffffull);
   const float rho = rank_key_value(best);
-  float outv = __fdividef(acc, Lsum);  // O_a
+  float outv[kN];
+#pragma unroll
+  for (int e = 0; e < kN; ++e) outv[e] = __fdividef(acc[e], Lsum);  // O_a
   float lse2 = M + __log2f(Lsum);      // LSE_a (log2 domain)
   const bool apply = (a.always_apply || rho > a.theta2) && (lse_c > -INFINITY);
   if (apply) {
@@ -239,15 +267,23 @@ __device__ __forceinline__ void merge_store(const DecodeCommon& a, const DecodeL
     const float mx = fmaxf(lse2, lc2);
     const float ea = ex2_approx(lse2 - mx), ec = ex2_approx(lc2 - mx);
     const float inv = __fdividef(1.f, ea + ec);  // the sum is in [1, 2]
-    outv = (ea * inv) * outv + (ec * inv) * oc;
+#pragma unroll
+    for (int e = 0; e < kN; ++e) outv[e] = (ea * inv) * outv[e] + (ec * inv) * oc[e];
     lse2 = mx + __log2f(ea + ec);
   }
-  reinterpret_cast<__nv_bfloat16*>(P.out)[(size_t)hq * kD + d] = __float2bfloat16_rn(outv);
+  __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(P.out) + (size_t)hq * kD + d;
+  if constexpr (kN == 4) *reinterpret_cast<uint2*>(out) = make_uint2(pack_bf16(outv[0], outv[1]), pack_bf16(outv[2], outv[3]));
+  else *out = __float2bfloat16_rn(outv[0]);
   if (d == 0) {
     if (P.lse_out) P.lse_out[hq] = lse2 * kLn2;
     if (P.flags)
       P.flags[hq] = (uint8_t)((apply ? 1 : 0) | (rho < a.theta1 ? 2 : 0) | (a.n_cal <= 64 ? (cs << 2) : 0));
   }
+}
+__device__ __forceinline__ void merge_store(const DecodeCommon& a, const DecodeLayerPtrs& P, int hq, int d, float acc,
+                                            float M, float Lsum, unsigned long long best, float lse_c, float oc) {
+  const float acc1[1] = {acc}, oc1[1] = {oc};
+  merge_store<1>(a, P, hq, d, acc1, M, Lsum, best, lse_c, oc1);
 }
 
 // Algorithm 2, lines 4-6, for the launches that recompute a calibration entry: the attention of the
@@ -263,19 +299,21 @@ __device__ __forceinline__ void recal_store(const DecodeCommon& a, const DecodeL
 }
 
 // RECAL = false: the decode step.  RECAL = true: the same stream over the evicted KV, without the
-// similarity and the gate, ending in recal_store.  kSlots: ring depth (six slots and one CTA per
-// SM, or three slots and two CTAs per SM for launches of many short, independent slices, where the
-// fixed chain of one CTA is what a second resident CTA can overlap).
-template <int NL, bool RECAL, int kSlots>
-__global__ void __launch_bounds__(kThreads, kSlots > 3 ? 1 : 2)
+// similarity and the gate, ending in recal_store.  S: the shape of a CTA.
+template <int NL, bool RECAL, class S>
+__global__ void __launch_bounds__(S::kThreads, S::kCtas)
 decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
+  constexpr int kSlots = S::kSlots, kSlotRows = S::kRows, kSubs = S::kSubs, kStreamWarps = S::kStreamWarps;
+  constexpr int kThreads = S::kThreads, kPlaneBytes = S::kPlaneBytes, kSlotBytes = S::kSlotBytes;
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long s_full[kSlots][2], s_empty[kSlots][2];
   __shared__ unsigned long long s_best[kMaxG];     // best (similarity, row) of this CTA's calibration rows
   __shared__ unsigned long long s_bestall[kMaxG];  // ... of the whole cluster
   __shared__ __align__(16) float s_xpart[kMaxG * kD];  // [source split][head][dim of this CTA's slice]
-  __shared__ __align__(16) float s_xml[8][kMaxG][2];   // [source split][head] (max, sum)
+  __shared__ __align__(16) float s_xml[S::kClu][kMaxG][2];   // [source split][head] (max, sum)
   __shared__ __align__(8) unsigned long long s_push;  // counts the bytes pushed to this CTA by the cluster
+  __shared__ __align__(16) uint4 s_q[S::kClu == 1 && !RECAL ? kMaxG * kD / 8 : 1];  // the unit's queries
+  __shared__ __align__(8) unsigned long long s_qfull;
   __shared__ int s_abort;
   __shared__ unsigned s_ticket;
 
@@ -307,10 +345,12 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
     }
   }
   cg::cluster_group cluster = cg::this_cluster();
-  const int gs = blockIdx.x;             // split index over the whole unit
-  const int split = gs % a.nsplit;       // rank inside the cluster
-  const int clu = gs / a.nsplit;         // cluster of this unit
-  const int n_gs = a.nsplit * a.nclu;
+  constexpr bool kOne = S::kClu == 1;    // a unit is one CTA's: nothing to combine across CTAs
+  const int nsplit = kOne ? 1 : a.nsplit, nclu = kOne ? 1 : a.nclu;
+  const int gs = kOne ? 0 : blockIdx.x;  // split index over the whole unit
+  const int split = gs % nsplit;         // rank inside the cluster
+  const int clu = gs / nsplit;           // cluster of this unit
+  const int n_gs = nsplit * nclu;
   const int unit = blockIdx.y, layer = blockIdx.z;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int gq = lane >> 2, tq = lane & 3;  // MMA fragment coordinates
@@ -324,7 +364,11 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
 
   const int r0 = min(a.n_kv, gs * a.rows_per_split);
   const int r1 = min(a.n_kv, r0 + a.rows_per_split);
-  const int n_sb = (r1 - r0 + kSlotRows - 1) / kSlotRows;  // ring fills of this CTA
+  // Ring fills of this CTA: the K/V rows, and with one CTA per unit the unit's calibration queries ahead of them, 32 rows
+  // per warp of the slot.
+  constexpr int kCalRows = kSubs * 32;
+  const int n_cf = kOne && !RECAL ? (a.G * a.n_cal + kCalRows - 1) / kCalRows : 0;
+  const int n_sb = n_cf + (r1 - r0 + kSlotRows - 1) / kSlotRows;
 
   const uint64_t pol_stream = policy_evict_first(), pol_keep = policy_evict_last();
   const uint32_t ring = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -338,8 +382,9 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
   if (tid == 0) {
     for (int s = 0; s < kSlots; ++s)
       for (int p = 0; p < 2; ++p) {
+        if (s == 0 && p == 0) mbar_init(smem_u32(&s_qfull), 1);
         mbar_init(smem_u32(&s_full[s][p]), 1);    // the producer's arrive with the byte count
-        mbar_init(smem_u32(&s_empty[s][p]), 4);   // one lane of each of the slot's four warps
+        mbar_init(smem_u32(&s_empty[s][p]), kSubs);   // one lane of each of the slot's warps
       }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     s_abort = 0;
@@ -349,7 +394,7 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
     // (max, sum) pairs here: G * dpc * 4 + G * 8 bytes each
     mbar_init(smem_u32(&s_push), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    mbar_expect_tx(smem_u32(&s_push), (uint32_t)(a.nsplit * a.G * (kD / a.nsplit * 4 + 8)));
+    if (!kOne) mbar_expect_tx(smem_u32(&s_push), (uint32_t)(nsplit * a.G * (kD / nsplit * 4 + 8)));
     asm volatile("prefetch.tensormap [%0];" ::"l"(&TM.k64) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&TM.v64) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&TM.k16) : "memory");
@@ -379,10 +424,10 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
   const uint4* qp0 = reinterpret_cast<const uint4*>(q + (size_t)(hq0 + pg0) * kD + sub4 * 32);
   const uint4* cp0 = reinterpret_cast<const uint4*>(Cq + ((size_t)(hq0 + pg0) * a.n_cal + pc0) * kD + sub4 * 32);
   const uint32_t* qr0 = reinterpret_cast<const uint32_t*>(q + (size_t)(hq0 + min(gq, a.G - 1)) * kD) + tq;
-  const int dpc = kD / a.nsplit, lg_dpc = 31 - __clz(dpc);  // nsplit is a power of two
+  const int dpc = kD / nsplit, lg_dpc = 31 - __clz(dpc);  // nsplit is a power of two
   const int n_items = a.G * dpc;
-  const bool single = a.nclu == 1;
-  const bool early = !RECAL && single && n_items <= kThreads;  // one output element per thread at most
+  const bool single = nclu == 1;
+  const bool early = !kOne && !RECAL && single && n_items <= kThreads;  // one output element per thread at most
   const int eg = min(tid >> lg_dpc, a.G - 1), ed = split * dpc + (tid & (dpc - 1));
   const float* oc_base = P.O_c + (size_t)(hq0 + eg) * a.n_cal * kD + ed;
   const float* lsec_base = P.LSE_c + (size_t)(hq0 + eg) * a.n_cal;
@@ -400,9 +445,20 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
     const int s = sb % kSlots, k = sb / kSlots;
     const uint32_t bar = smem_u32(&s_full[s][k & 1]);
     const uint32_t dst = ring + s * kSlotBytes;
-    const int row0 = r0 + sb * kSlotRows;
+    if (kOne && sb < n_cf) {
+      const int rows = min(kCalRows, a.G * a.n_cal - sb * kCalRows);
+      const unsigned bytes = (unsigned)rows * kRowBytes, q_bytes = (unsigned)a.G * kRowBytes;
+      if (sb == 0) {
+        mbar_expect_tx(smem_u32(&s_qfull), q_bytes);
+        bulk_load(smem_u32(s_q), q + (size_t)hq0 * kD, q_bytes, smem_u32(&s_qfull), pol_keep);
+      }
+      mbar_expect_tx(bar, bytes);
+      bulk_load(dst, Cq + ((size_t)hq0 * a.n_cal + sb * kCalRows) * kD, bytes, bar, pol_keep);
+      return;
+    }
+    const int row0 = r0 + (sb - n_cf) * kSlotRows;
     const int nrows = min(kSlotRows, r1 - row0);
-    if (nrows == kSlotRows) {
+    if (kSlotRows == kWideRows && nrows == kSlotRows) {
       mbar_expect_tx(bar, kSlotBytes);
       tma_load_3d(dst, &TM.k64, bar, 0, row0, unit, pol_stream);
       tma_load_3d(dst + kPlaneBytes, &TM.k64, bar, 64, row0, unit, pol_stream);
@@ -462,7 +518,7 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
   }
   RhoLoad rl[2];
   rl[0] = RhoLoad{}; rl[1] = RhoLoad{};
-  if (pi0 < pairs) {
+  if (!kOne && pi0 < pairs) {
     rl[0].q0 = __ldg(qp0); rl[0].q1 = __ldg(qp0 + 1);
     rl[0].c0 = ldg_keep(cp0, pol_keep); rl[0].c1 = ldg_keep(cp0 + 1, pol_keep);
     rl[1].q0 = __ldg(qp0 + 2); rl[1].q1 = __ldg(qp0 + 3);
@@ -481,6 +537,7 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
   // CTA barrier and arrive relaxed, and the producer warp, which has time, makes the one release
   // for the CTA.
   auto rho_rest = [&]() {
+    if (kOne) return;
     rho_finish(pi0, pg0, pc0, rl);
     for (int base = kPairsPerPass; base < pairs; base += kPairsPerPass) {
       const int pi = base + pi0;
@@ -490,6 +547,41 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
     if (warp != kStreamWarps) {
       asm volatile("barrier.cta.arrive 1, %0;" ::"n"(kThreads) : "memory");
       asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    }
+  };
+  // One CTA per unit: the similarities of a slot of calibration queries, a row per lane.  (Loaded through registers, four
+  // lanes to a row, the passes were a chain of round trips that held the stream up: 73 instead of 60 us for 2048 caches
+  // of 231 rows.)
+  // The sums are those of the other shapes, to the bit, so that no near-tie between two rows depends on the shape: quarters
+  // of a row, each in ascending order, added in pairs.  (Every second group of four lanes takes a pair's quarters the other way
+  // round, which halves the bank conflicts; lanes that start up to three chunks apart and meet in no bank were slower,
+  // 63.5 us.)
+  auto rho_slot = [&](int s, int sb, int sub) {
+    const int rows = a.G * a.n_cal, r = sb * kCalRows + sub * 32 + lane;
+    const int g_lo = (sb * kCalRows + sub * 32) / a.n_cal, g = r < rows ? r / a.n_cal : -1, c = r - g * a.n_cal;
+    if (g_lo >= a.G) return;                          // (the same for the whole warp)
+    const uint4* crow = reinterpret_cast<const uint4*>(ring_ptr + s * kSlotBytes) + (sub * 32 + lane) * (kD / 8);
+    const uint4* qrow = s_q + (g < 0 ? 0 : g) * (kD / 8);
+    float dot = 0.f, qq = 0.f, cc = 0.f;
+    const int parity = (lane >> 2) & 1;
+#pragma unroll 1
+    for (int pair = 0; pair < 2; ++pair) {
+      float d[2] = {0.f, 0.f}, dq[2] = {0.f, 0.f}, dc[2] = {0.f, 0.f};
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int chunk = (2 * pair + (e ^ parity)) * 4;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) rho_accumulate(qrow[chunk + j], crow[chunk + j], d[e], dq[e], dc[e]);
+      }
+      dot += d[0] + d[1]; qq += dq[0] + dq[1]; cc += dc[0] + dc[1];
+    }
+    const float rho = (qq > 0.f && cc > 0.f) ? dot / (sqrtf(qq) * sqrtf(cc)) : 0.f;
+    const unsigned hi = (unsigned)(rank_key(rho, 0) >> 32);
+    const int g_hi = min(a.G - 1, (sb * kCalRows + sub * 32 + 31) / a.n_cal);
+    for (int gg = g_lo; gg <= g_hi; ++gg) {
+      const unsigned m = __reduce_max_sync(0xffffffffu, g == gg ? hi : 0u);
+      const unsigned cm = __reduce_max_sync(0xffffffffu, g == gg && hi == m ? (unsigned)c : 0u);
+      if (lane == 0) atomicMax(&s_best[gg], ((unsigned long long)m << 32) | cm);
     }
   };
 
@@ -512,12 +604,14 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
     // with the last fill under way the producer has nothing left to move: it settles the
     // calibration row (best similarity over the cluster, ties to the largest row index) while the
     // stream warps are still busy
-    asm volatile("barrier.cta.sync 1, %0;" ::"n"(kThreads) : "memory");  // the stream warps' updates of s_best
-    cluster_arrive();  // (A) with the release for the whole CTA
-    cluster_wait();    //     every CTA's s_best can be read
-    if (lane < a.G) {
+    if (!kOne) asm volatile("barrier.cta.sync 1, %0;" ::"n"(kThreads) : "memory");  // the stream warps' updates of s_best
+    if (!kOne) {
+      cluster_arrive();  // (A) with the release for the whole CTA
+      cluster_wait();    //     every CTA's s_best can be read
+    }
+    if (!kOne && lane < a.G) {
       unsigned long long best = 0ull;
-      for (int s = 0; s < a.nsplit; ++s) {
+      for (int s = 0; s < nsplit; ++s) {
         const unsigned long long k = *cluster.map_shared_rank(&s_best[lane], s);
         best = k > best ? k : best;
       }
@@ -525,21 +619,23 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
     }
   } else {
     // ---- (3) stream warps
-    const int group = warp >> 2, sub = warp & 3;
+    const int group = warp / kSubs, sub = warp % kSubs;
     const int mid = lane >> 3;
     bool rho_done = false;
     for (int sb = group; sb < n_sb; sb += 2) {
       const int s = sb % kSlots, k = sb / kSlots;
       const bool ok = mbar_wait(smem_u32(&s_full[s][k & 1]), (k >> 1) & 1, abort_flag, a.status, 0x200u + sb);
-      const int row_base = r0 + sb * kSlotRows + sub * kBlkRows;
-      if (ok && row_base < r1) {
+      const int row_base = r0 + (sb - n_cf) * kSlotRows + sub * kBlkRows;
+      if (kOne && sb < n_cf) {
+        if (!RECAL && ok && mbar_wait(smem_u32(&s_qfull), 0, abort_flag, a.status, 0x400u)) rho_slot(s, sb, sub);
+      } else if (ok && row_base < r1) {
         const uint32_t sK = ring + s * kSlotBytes;
         const uint32_t sV = sK + 2 * kPlaneBytes;
         // D1: the warp that meets row kv_len takes it from k_new / v_new (the cache row has not
         // been written yet: what arrived for it is stale) and appends it to the cache
         if (a.has_new && a.kv_len >= row_base && a.kv_len < row_base + kBlkRows) {
           const int chunk = lane & 15;
-          const int rs = a.kv_len - (r0 + sb * kSlotRows);  // row inside the slot
+          const int rs = a.kv_len - (r0 + (sb - n_cf) * kSlotRows);  // row inside the slot
           const unsigned char* src = (const unsigned char*)(lane < 16 ? P.k_new : P.v_new) +
                                      (size_t)unit * kRowBytes + chunk * 16;
           const uint4 v = *reinterpret_cast<const uint4*>(src);
@@ -547,7 +643,7 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
                                 ((size_t)unit * a.cap + a.kv_len) * kRowBytes + chunk * 16;
           *reinterpret_cast<uint4*>(dstg) = v;
           *reinterpret_cast<uint4*>(ring_ptr + s * kSlotBytes + (lane < 16 ? 0 : 2 * kPlaneBytes) +
-                                    plane_off(rs, chunk)) = v;
+                                    plane_off<S>(rs, chunk)) = v;
           __syncwarp();
         }
         // S^T: two accumulators (even and odd k-steps) halve the dependent chain
@@ -555,7 +651,7 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
 #pragma unroll
         for (int kk = 0; kk < kD / 16; ++kk) {
           uint32_t a0, a1, a2, a3;
-          ldmatrix_x4(sK + plane_off(sub * kBlkRows + (lane & 7) + (mid & 1) * 8, kk * 2 + (mid >> 1)), a0, a1, a2, a3);
+          ldmatrix_x4(sK + plane_off<S>(sub * kBlkRows + (lane & 7) + (mid & 1) * 8, kk * 2 + (mid >> 1)), a0, a1, a2, a3);
           if (kk & 1) mma_bf16_16816(sb2, a0, a1, a2, a3, qa[kk][0], qa[kk][1]);
           else mma_bf16_16816(sa, a0, a1, a2, a3, qa[kk][0], qa[kk][1]);
         }
@@ -585,7 +681,7 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
 #pragma unroll
         for (int n = 0; n < kD / 16; ++n) {
           uint32_t a0, a1, a2, a3;
-          ldmatrix_x4_trans(sV + plane_off(sub * kBlkRows + (lane & 7) + (mid >> 1) * 8, n * 2 + (mid & 1)), a0, a1, a2, a3);
+          ldmatrix_x4_trans(sV + plane_off<S>(sub * kBlkRows + (lane & 7) + (mid >> 1) * 8, n * 2 + (mid & 1)), a0, a1, a2, a3);
           mma_bf16_16816(o[n], a0, a1, a2, a3, pb0, pb1);
         }
       }
@@ -602,11 +698,11 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
   }
 
   // ---- (4) the chosen O_c elements and LSE_c start their way while the partials are combined
-  if (warp < kStreamWarps) cluster_wait();  // (A): the stream warps only pass it
+  if (!kOne && warp < kStreamWarps) cluster_wait();  // (A): the stream warps only pass it
   __syncthreads();  // all warps are done with the ring: reuse it for the combine
   // the common case has one output element per thread at most: its O_c element and LSE_c are
   // loaded now and arrive while the partials are combined
-  if (!RECAL && (!single || n_items > kThreads)) {
+  if (!kOne && !RECAL && (!single || n_items > kThreads)) {
     if (tid < a.G && single) {
       const size_t crow = (size_t)(hq0 + tid) * a.n_cal + (unsigned)(s_bestall[tid] & 0xffffffffull);
       const float* orow = P.O_c + crow * kD;
@@ -622,7 +718,16 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
     oc_early = ldg_keep(oc_base + (size_t)cs * kD, pol_keep);
   }
 
-  // ---- (5) CTA combine of the eight stream warps, pushed to the owners of the output slices:
+  // one CTA per unit: a warp per head, four elements per thread, the first head's O_c on its way now
+  uint4 oc_one = make_uint4(0u, 0u, 0u, 0u);
+  auto load_oc = [&](int g) {
+    const size_t crow = (size_t)(hq0 + g) * a.n_cal + (unsigned)(s_best[g] & 0xffffffffull);
+    oc_one = ldg_keep(reinterpret_cast<const uint4*>(P.O_c + crow * kD) + lane, pol_keep);
+    lse_c_early = ldg_keep(P.LSE_c + crow, pol_keep);
+  };
+  if (kOne && !RECAL && warp < min(kStreamWarps, a.G)) load_oc(warp);
+
+  // ---- (5) CTA combine of the stream warps, pushed to the owners of the output slices:
   // CTA r of the cluster owns dimensions [r * dpc, (r + 1) * dpc) of every head of the group
   float* wo = reinterpret_cast<float*>(ring_ptr);          // [warp][8][kWoStride]
   float* wml = wo + kStreamWarps * kMaxG * kWoStride;       // [warp][8][2]
@@ -639,13 +744,39 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
     }
   }
   __syncthreads();
-  // 256 threads: thread t owns dimensions 2 (t & 63) and 2 (t & 63) + 1 of head (t >> 6) + 4k, so the
+  if constexpr (kOne) {
+    if (warp < kStreamWarps) {
+      for (int g = warp; g < a.G; g += kStreamWarps) {
+        if (!RECAL && g != warp) load_oc(g);
+        float mw[kStreamWarps], M = -INFINITY, Lsum = 0.f, acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int w = 0; w < kStreamWarps; ++w) { mw[w] = wml[(w * kMaxG + g) * 2]; M = fmaxf(M, mw[w]); }
+#pragma unroll
+        for (int w = 0; w < kStreamWarps; ++w) {
+          const float sc = mw[w] > -INFINITY ? ex2_approx(mw[w] - M) : 0.f;
+          const float4 v = *reinterpret_cast<const float4*>(wo + (w * kMaxG + g) * kWoStride + 4 * lane);
+          Lsum = fmaf(wml[(w * kMaxG + g) * 2 + 1], sc, Lsum);
+          acc[0] = fmaf(v.x, sc, acc[0]); acc[1] = fmaf(v.y, sc, acc[1]);
+          acc[2] = fmaf(v.z, sc, acc[2]); acc[3] = fmaf(v.w, sc, acc[3]);
+        }
+        if constexpr (RECAL) {
+          for (int e = 0; e < 4; ++e) recal_store(a, P, hq0 + g, 4 * lane + e, acc[e], M, Lsum);
+        } else {
+          const float oc[4] = {__uint_as_float(oc_one.x), __uint_as_float(oc_one.y), __uint_as_float(oc_one.z),
+                               __uint_as_float(oc_one.w)};
+          merge_store<4>(a, P, hq0 + g, 4 * lane, acc, M, Lsum, s_best[g], lse_c_early, oc);
+        }
+      }
+    }
+    return;
+  }
+  // the stream warps' threads: thread t owns dimensions 2 (t & 63) and 2 (t & 63) + 1 of every kStreamWarps / 2-th head, so the
   // scale factors of the eight warps are worked out once for two elements, which go to their owner
   // in one 8-byte store; all loads are done before the pushes (stores through generic pointers,
   // which the compiler will not move loads across)
-  if (tid < 256) {
+  if (tid < kStreamWarps * 32) {
     const int d0 = 2 * (tid & 63);
-    for (int g = tid >> 6; g < a.G; g += 4) {
+    for (int g = tid >> 6; g < a.G; g += kStreamWarps / 2) {
       float mw[kStreamWarps], M = -INFINITY;
 #pragma unroll
       for (int w = 0; w < kStreamWarps; ++w) { mw[w] = wml[(w * kMaxG + g) * 2]; M = fmaxf(M, mw[w]); }
@@ -661,7 +792,7 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
       const int own = d0 >> lg_dpc;  // dpc is even: both dimensions have the same owner
       push_f32x2(cluster_addr(smem_u32(s_xpart + (split * kMaxG + g) * dpc + (d0 - own * dpc)), own), acc0, acc1,
                  cluster_addr(smem_u32(&s_push), own));
-      if ((tid & 63) < a.nsplit) {  // the (max, sum) pair of this split goes to every CTA of the cluster
+      if ((tid & 63) < nsplit) {  // the (max, sum) pair of this split goes to every CTA of the cluster
         push_f32x2(cluster_addr(smem_u32(&s_xml[split][g][0]), tid & 63), M, Lsum,
                    cluster_addr(smem_u32(&s_push), tid & 63));
       }
@@ -682,10 +813,10 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
     const int g = item >> lg_dpc, dl = item & (dpc - 1), d = split * dpc + dl;
     const int hq = hq0 + g;
     const unsigned long long best = s_bestall[g];
-    float ms[8], ls[8], xs[8], M = -INFINITY;
+    float ms[S::kClu], ls[S::kClu], xs[S::kClu], M = -INFINITY;
 #pragma unroll
-    for (int s = 0; s < 8; ++s) {  // all loads first (nsplit <= 8)
-      const bool on = s < a.nsplit;
+    for (int s = 0; s < S::kClu; ++s) {  // all loads first
+      const bool on = s < nsplit;
       ms[s] = on ? s_xml[s][g][0] : -INFINITY;
       ls[s] = on ? s_xml[s][g][1] : 0.f;
       xs[s] = on ? s_xpart[(s * kMaxG + g) * dpc + dl] : 0.f;
@@ -693,7 +824,7 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
     }
     float Lsum = 0.f, acc = 0.f;
 #pragma unroll
-    for (int s = 0; s < 8; ++s) {
+    for (int s = 0; s < S::kClu; ++s) {
       const float sc = ms[s] > -INFINITY ? ex2_approx(ms[s] - M) : 0.f;
       Lsum = fmaf(ls[s], sc, Lsum);
       acc = fmaf(xs[s], sc, acc);
@@ -712,7 +843,7 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
       }
     } else {
       // this cluster's partial goes to the workspace; (M, Lsum, best) are the same in all its CTAs
-      const size_t pc = ((size_t)lu * a.nclu + clu) * kMaxG + g;
+      const size_t pc = ((size_t)lu * nclu + clu) * kMaxG + g;
       a.part_o[pc * kD + d] = acc;
       if (d == 0) {
         a.part_ml[pc * 2] = M;
@@ -731,13 +862,13 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
       __threadfence();
       for (int gd = tid; gd < a.G * kD; gd += kThreads) {
         const int g = gd / kD, d = gd % kD;
-        const size_t pu = (size_t)lu * a.nclu * kMaxG + g;
+        const size_t pu = (size_t)lu * nclu * kMaxG + g;
         unsigned long long best = 0ull;
         float ms[8], ls[8], os[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
           ms[c] = -INFINITY; ls[c] = 0.f; os[c] = 0.f;
-          if (c < a.nclu) {
+          if (c < nclu) {
             const size_t pc = pu + (size_t)c * kMaxG;
             const unsigned long long k = __ldcg(a.part_best + pc);
             best = k > best ? k : best;
@@ -783,7 +914,7 @@ bool make_decode_maps(const DecodeCommon& c, const DecodeLayerPtrs& L, DecodeLay
   static thread_local Entry table[kEntries];
   static thread_local int next = 0;
   const uint64_t strides[2] = {(uint64_t)kRowBytes, (uint64_t)c.cap * kRowBytes};
-  const uint32_t box64[2] = {(uint32_t)kSlotRows, 1}, box16[2] = {(uint32_t)kBlkRows, 1};
+  const uint32_t box64[2] = {(uint32_t)kWideRows, 1}, box16[2] = {(uint32_t)kBlkRows, 1};
   const uint64_t dims_v16[2] = {(uint64_t)(c.kv_len > 0 ? c.kv_len : 1), (uint64_t)c.units};
   for (int i = 0; i < kEntries; ++i) {
     const Entry& e = table[i];
@@ -806,22 +937,27 @@ bool make_decode_maps(const DecodeCommon& c, const DecodeLayerPtrs& L, DecodeLay
 
 namespace {
 
-template <int NL, bool RECAL, int kSlots>
+template <int NL, bool RECAL, class S>
+cudaError_t setup_decode(int dev) {
+  static std::atomic<bool> done[64];
+  if (dev >= 0 && dev < 64 && done[dev].load(std::memory_order_acquire)) return cudaSuccess;
+  cudaError_t e = cudaFuncSetAttribute(decode_kernel<NL, RECAL, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kSmemBytes);
+  if (e == cudaSuccess && S::kClu > 8)
+    e = cudaFuncSetAttribute(decode_kernel<NL, RECAL, S>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev].store(true, std::memory_order_release);
+  return e;
+}
+
+template <int NL, bool RECAL, class S>
 cudaError_t launch_decode_s(const DecodeArgsT<NL>& a, cudaStream_t st) {
-  constexpr int kSmemBytes = smem_bytes(kSlots);
-  static bool attr_set[64] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = setup_decode<NL, RECAL, S>(dev);
   if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-    e = cudaFuncSetAttribute(decode_kernel<NL, RECAL, kSlots>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) attr_set[dev] = true;
-  }
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(a.c.nsplit * a.c.nclu, a.c.units, a.c.n_layers);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = kSmemBytes;
+  cfg.blockDim = dim3(S::kThreads);
+  cfg.dynamicSmemBytes = S::kSmemBytes;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;  // the splits of a unit are one cluster
@@ -832,21 +968,27 @@ cudaError_t launch_decode_s(const DecodeArgsT<NL>& a, cudaStream_t st) {
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  e = cudaLaunchKernelEx(&cfg, decode_kernel<NL, RECAL, kSlots>, a);
+  e = cudaLaunchKernelEx(&cfg, decode_kernel<NL, RECAL, S>, a);
   if (e != cudaSuccess) return e;
   count_launch(1);
   return cudaGetLastError();
 }
 
-// More CTAs than SMs and short slices (a stack of small caches in one launch): the narrow ring, so
-// that two CTAs share an SM and one's fixed chain overlaps the other's stream.  Long slices keep the
-// wide ring, which they need to stream at full rate (measured: 32 layers of 129-384 rows 115 -> 95 us
-// with the narrow ring, 8 caches of 2049 rows 53 -> 57 us).
+// More units than SMs (a stack of caches in one launch), a CTA each: smaller rings, fewer warps and the calibration queries
+// through the ring, so that several CTAs share an SM and one's fixed chain overlaps the others' streams.  Two CTAs per SM
+// as long as that is all of them, else four.  Against the wide ring, one CTA per SM (us): 256 caches of 2049 rows 56.8 ->
+// 48.9, 192 of 800 28.6 -> 20.1, 1024 of 1000 122 -> 107, 512 of 800 62 -> 46.5; 704 of 1300 equal and 384 of 2000 75 -> 80: long
+// slices of more CTAs than fit two to an SM keep it.  2048 of 231 rows: two CTAs of eight stream warps with the similarities
+// through registers 88.9, four of four warps 73, with the calibration queries through the ring 60 (48 for the bytes).
+constexpr int kNarrowRows = 1024;
 template <int NL, bool RECAL>
 cudaError_t launch_decode_t(const DecodeArgsT<NL>& a, cudaStream_t st) {
   const long long ctas = (long long)a.c.nsplit * a.c.nclu * a.c.units * a.c.n_layers;
-  const bool narrow = ctas > kDecodeTargetCtas && a.c.rows_per_split <= 8 * kSlotRows;
-  return narrow ? launch_decode_s<NL, RECAL, kSlotsNarrow>(a, st) : launch_decode_s<NL, RECAL, kSlotsWide>(a, st);
+  if (ctas > 2 * kDecodeTargetCtas && a.c.rows_per_split <= kNarrowRows) return launch_decode_s<NL, RECAL, ShapeNarrow>(a, st);
+  if (ctas > kDecodeTargetCtas && ctas <= 2 * kDecodeTargetCtas) return launch_decode_s<NL, RECAL, ShapePair>(a, st);
+  if constexpr (!RECAL)
+    if (a.c.nsplit > 8) return launch_decode_s<NL, RECAL, ShapeCluster16>(a, st);
+  return launch_decode_s<NL, RECAL, ShapeWide>(a, st);
 }
 
 }  // namespace
@@ -854,6 +996,36 @@ cudaError_t launch_decode_t(const DecodeArgsT<NL>& a, cudaStream_t st) {
 cudaError_t launch_decode(const DecodeArgsT<1>& a, cudaStream_t st) { return launch_decode_t<1, false>(a, st); }
 cudaError_t launch_decode(const DecodeArgsT<kDecodeMaxLayers>& a, cudaStream_t st) {
   return launch_decode_t<kDecodeMaxLayers, false>(a, st);
+}
+int decode_resident_clusters(int ctas) {
+  static std::atomic<int> known[64][5];   // per device and log2 of the size; 0: not asked yet, else 1 + clusters
+  int dev = 0, lg = 0;
+  while ((1 << lg) < ctas) ++lg;
+  if (lg > 4 || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  int n = known[dev][lg].load(std::memory_order_acquire);
+  if (n == 0) {
+    // (the kernels of one shape differ in their arguments only)
+    int active = 0;
+    if (setup_decode<1, false, ShapeCluster16>(dev) != cudaSuccess) return 0;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(ShapeCluster16::kThreads);
+    cfg.dynamicSmemBytes = ShapeCluster16::kSmemBytes;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = ctas;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&active, decode_kernel<1, false, ShapeCluster16>, &cfg) != cudaSuccess) {
+      cudaGetLastError();   // no such cluster on this device
+      active = 0;
+    }
+    n = 1 + active;
+    known[dev][lg].store(n, std::memory_order_release);
+  }
+  return n - 1;
 }
 cudaError_t launch_recalibrate(const DecodeArgsT<1>& a, cudaStream_t st) { return launch_decode_t<1, true>(a, st); }
 

@@ -61,7 +61,7 @@ constexpr int kDecodeTargetCtas = 148;  // one CTA of a launch on each of the 14
 struct DecodeCommon {
   int B, Hq, Hkv, G, n_cal, cap, kv_len, n_kv, has_new;
   int units, n_layers, rows_per_split;
-  int nsplit;  // CTAs per cluster (1, 2, 4 or 8): the splits combined through distributed shared memory
+  int nsplit;  // CTAs per cluster (1, 2, 4, 8 or 16): the splits combined through distributed shared memory
   int nclu;    // clusters per (layer, unit); more than one only when few units share a long cache
   float scale2, theta1, theta2;
   int always_apply;
@@ -160,6 +160,8 @@ cudaError_t launch_decode(const DecodeArgsT<1>& a, cudaStream_t st);
 cudaError_t launch_decode(const DecodeArgsT<kDecodeMaxLayers>& a, cudaStream_t st);
 // The same stream over the evicted KV (K, V of the layer = the compacted evicted rows), rewriting
 // row recal_slot of O_c, LSE_c, C_q (Algorithm 2, lines 4-6).
+// Clusters of `ctas` CTAs of the decode kernel, one CTA per SM, that the current device runs at the same time (0: none).
+int decode_resident_clusters(int ctas);
 cudaError_t launch_recalibrate(const DecodeArgsT<1>& a, cudaStream_t st);
 cudaError_t launch_evicted_indices(const CompressGeom& g, const CompressWs& ws, char* wsp, const int32_t* kept_idx,
                                    int32_t* evict_idx, cudaStream_t st);

@@ -570,6 +570,62 @@ def test_decode_ignores_cache_rows_beyond_kv_len(cuda_lib, B, Hq, Hkv, kv0, step
         np.testing.assert_array_equal(to_bits(st.K_kept)[:, :, kv0 + t + 1:], Kk[:, :, kv0 + t + 1:])
 
 
+@pytest.mark.parametrize("units,layers,G,kv,n_cal", [
+    (80, 2, 1, 64, 1),        # two CTAs per SM: one calibration row, one whole slot and the appended row
+    (80, 3, 4, 700, 33),      # ... 132 calibration rows, four of them in a second slot
+    (20, 8, 3, 2100, 64),     # ... a long slice
+    (80, 4, 8, 0, 64),        # four CTAs per SM: the appended row alone
+    (75, 5, 7, 32, 100),      # ... eleven slots of calibration rows, the last with 60; 300 rows of n_cal above 64
+    (80, 4, 2, 1023, 16),     # ... the longest slice of this shape
+    (80, 4, 2, 1024, 16),     # one more row: the wide ring, more CTAs than SMs
+    (3, 1, 7, 4400, 5),       # clusters of sixteen, five calibration rows over sixteen CTAs
+    (1, 2, 8, 9001, 64),      # ... or several clusters of eight
+    (16, 1, 4, 2100, 8),      # more clusters of eight than the GPU holds at once: clusters of four
+])
+def test_decode_launch_shapes_against_fp32(cuda_lib, units, layers, G, kv, n_cal):
+    """Every shape that the launch rules choose between, at its edges, against the same step in fp32: outputs are bf16
+    of values below about 2 (tolerances of the other parity tests); the calibration row is the one the query was
+    drawn around, far from any tie."""
+    cd = cuda_lib
+    gen = torch.Generator(device="cuda").manual_seed(units * 7 + kv)
+    rn = lambda *sh: torch.randn(sh, generator=gen, device="cuda")
+    Hq, cap = units * G, kv + 3
+    p = cd.make_params(B=1, Hq=Hq, Hkv=units, n_cal=n_cal, cap=cap)
+    p.theta1, p.theta2 = 0.7, -1.0
+    bf = torch.bfloat16
+    ins = []
+    for i in range(layers):
+        pick = torch.randint(n_cal, (1, Hq), generator=gen, device="cuda")
+        C_q = rn(1, Hq, n_cal, 128).to(bf)
+        q = (C_q.float().gather(2, pick[..., None, None].expand(-1, -1, 1, 128))[:, :, 0] + 0.3 * rn(1, Hq, 128)).to(bf)
+        ins.append(dict(q=q, k_new=rn(1, units, 128).to(bf), v_new=rn(1, units, 128).to(bf),
+                        K_kept=rn(1, units, cap, 128).to(bf), V_kept=rn(1, units, cap, 128).to(bf),
+                        O_c=rn(1, Hq, n_cal, 128), LSE_c=rn(1, Hq, n_cal) + 6, C_q=C_q,
+                        out=torch.empty((1, Hq, 128), dtype=bf, device="cuda"),
+                        lse_out=torch.empty((1, Hq), device="cuda"),
+                        flags=torch.empty((1, Hq), dtype=torch.uint8, device="cuda"), pick=pick))
+    ws = torch.zeros((cd.calidrop_decode_workspace_bytes(p, cap) * layers,), dtype=torch.uint8, device="cuda")
+    cd.calidrop_decode_batched(p, cd.make_decode_layers([{k: v for k, v in d.items() if k != "pick"} for d in ins]), kv, ws)
+    torch.cuda.synchronize()
+    off = cd.calidrop_decode_workspace_status_offset(p)
+    assert int(ws[off:off + 4].view(torch.int32).item()) == 0
+    for d in ins:
+        assert torch.equal(d["K_kept"][:, :, kv], d["k_new"]) and torch.equal(d["V_kept"][:, :, kv], d["v_new"])
+        if n_cal <= 64:
+            assert torch.equal((d["flags"] >> 2).long(), d["pick"])
+        K, V = (d[k][0, :, :kv + 1].float() for k in ("K_kept", "V_kept"))
+        s = torch.einsum("ugd,utd->ugt", d["q"].float().view(units, G, 128).double(), K.double()) / 128 ** 0.5
+        la = torch.logsumexp(s, -1)
+        oa = torch.einsum("ugt,utd->ugd", torch.softmax(s, -1), V.double())
+        lc = d["LSE_c"].gather(2, d["pick"][..., None])[..., 0].view(units, G).double()
+        oc = d["O_c"].gather(2, d["pick"][..., None, None].expand(-1, -1, 1, 128)).view(units, G, 128).double()
+        lse = torch.logaddexp(la, lc)
+        want = torch.exp(la - lse)[..., None] * oa + torch.exp(lc - lse)[..., None] * oc
+        assert (d["out"].double().view(units, G, 128) - want).abs().max() < 2e-2 * max(1.0, want.abs().max().item() / 2)
+        assert (d["out"].double().view(units, G, 128) - want).abs().mean() < 2e-3
+        assert (d["lse_out"].double().view(units, G) - lse).abs().max() < 1e-3
+
+
 def test_batched_layers_with_several_clusters_per_unit(cuda_lib):
     """Two layers of one unit with 17000 cached rows in one launch: every (layer, unit) is split over
     two clusters that meet through the workspace, each layer with its own counters and partials.
