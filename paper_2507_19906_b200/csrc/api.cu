@@ -268,12 +268,13 @@ int calidrop_compress(const calidrop_params* p, const void* Q_obs, const void* K
   if (e != cudaSuccess) return cuda_fail(e);
   const float* row_lse = lse_obs;
   if (!g.keep_all) {
+    const bool in_votes = tc_path && !lse_obs && votes_combine_stats(g);   // the row LSE comes out of the votes' kernel
     if (!row_lse) {
-      e = tc_path ? launch_row_stats_tc(g, ws, Q_obs, K, wsp, true, st) : launch_row_stats(g, ws, Q_obs, K, wsp, st);
+      e = tc_path ? launch_row_stats_tc(g, ws, Q_obs, K, wsp, true, !in_votes, st) : launch_row_stats(g, ws, Q_obs, K, wsp, st);
       if (e != cudaSuccess) return cuda_fail(e);
       row_lse = (const float*)(wsp + ws.row_lse);
     }
-    e = tc_path ? launch_votes_tc(g, ws, Q_obs, K, row_lse, wsp, lse_obs != nullptr, st)
+    e = tc_path ? launch_votes_tc(g, ws, Q_obs, K, in_votes ? nullptr : row_lse, wsp, lse_obs != nullptr, st)
                 : launch_votes(g, ws, Q_obs, K, row_lse, wsp, st);
     if (e != cudaSuccess) return cuda_fail(e);
   }
@@ -328,7 +329,7 @@ int calidrop_calibrate(const calidrop_params* p, const void* Q_obs, const void* 
   // or from the statistics pass of the scoring
   const float* row_lse = lse_obs;
   if (!g.keep_all && !row_lse) {
-    e = tc_path ? launch_row_stats_tc(g, ws, Q_obs, K, wsp, true, st) : launch_row_stats(g, ws, Q_obs, K, wsp, st);
+    e = tc_path ? launch_row_stats_tc(g, ws, Q_obs, K, wsp, true, true, st) : launch_row_stats(g, ws, Q_obs, K, wsp, st);
     if (e != cudaSuccess) return cuda_fail(e);
     row_lse = (const float*)(wsp + ws.row_lse);
   }

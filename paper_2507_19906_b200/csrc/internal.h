@@ -95,7 +95,8 @@ cudaError_t launch_calib_direct(const CompressGeom& g, const CompressWs& ws, con
 int pick_tile_splits(int groups, int n_tiles, int min_tiles);
 bool score_tc_supported(const CompressGeom& g);
 cudaError_t launch_row_stats_tc(const CompressGeom& g, const CompressWs& ws, const void* Q_obs, const void* K,
-                                char* wsp, bool first, cudaStream_t st);
+                                char* wsp, bool first, bool combine, cudaStream_t st);
+bool votes_combine_stats(const CompressGeom& g);
 cudaError_t launch_votes_tc(const CompressGeom& g, const CompressWs& ws, const void* Q_obs, const void* K,
                             const float* row_lse, char* wsp, bool first, cudaStream_t st);
 int votes_tc_parts(const CompressGeom& g);

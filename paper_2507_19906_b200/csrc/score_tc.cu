@@ -45,6 +45,18 @@ constexpr int kMaxBufs = 4;
 constexpr int kMaxRows = 512;   // G * W handled by the tiles
 constexpr int kSms = 148;
 
+// Where the partial statistics of a row lie: those of the CTAs whose tile range overlaps the row's virtual unit.
+struct StatParts {
+  const float2* part;   // [row][slot][n_part] (max, sum)
+  int vu_per_unit, n_tiles, tiles_per_cta, max_slots, n_part;
+  __device__ __forceinline__ const float2* of(int unit, int GW, int row, int* n) const {
+    const int vu = unit * vu_per_unit + row / 256;
+    const int first = (vu * n_tiles) / tiles_per_cta, last = ((vu + 1) * n_tiles - 1) / tiles_per_cta;
+    *n = (last - first + 1) * n_part;
+    return part + (size_t)(unit * GW + row) * max_slots * n_part;
+  }
+};
+
 struct ScoreArgs {
   int Hq, G, W, L, n_cand, GW;
   int vu_per_unit;    // virtual units per (batch, kv-head) unit
@@ -61,6 +73,10 @@ struct ScoreArgs {
   const float* row_lse;  // votes: natural-log LSE of every observation row [B, Hq, W]
   float* vote_parts;     // votes: out [part][units, n_cand], a part per (row block, column half)
   float2* stat_part;     // statistics: out [row][slot][2 or 4 groups] (max, sum) in the log2 domain
+  // votes: the statistics' partials, combined here (StatParts::part null: row_lse is given)
+  StatParts stats;
+  float* lse_out;        // ... and the natural-log LSE for the calibration
+  int lg_tpr;            // ... log2 of the threads that share a row
   unsigned* status;
   int clear_status;      // the first kernel of a call clears the error word
 };
@@ -103,6 +119,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
   __shared__ Ctl ctl;
   // votes: -lse2 of the columns this warp reads, one copy per warp
   __shared__ __align__(16) float nlse2_s[kVotes ? kGroups * 4 : 1][kVotes ? 128 : 4];
+  __shared__ float lse_s[kVotes ? 2 : 1][kVotes ? kMaxRows : 1];   // combined here: the LSE of the CTA's (at most two) units
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int cta = blockIdx.x;
@@ -272,6 +289,47 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
     uint32_t ph = 0;
     bool ok = true;
 
+    const int unit_lo = g_begin / a.n_tiles;
+    const bool combine = kVotes && a.stats.part != nullptr;
+    if (combine) {
+      // Row LSE of this CTA's units from the partial statistics, by the consumers while the first keys are on their way:
+      // cheaper than a kernel of its own as long as the partials are few (see votes_combine_stats).
+      const int tpr = 1 << a.lg_tpr, row = tid >> a.lg_tpr, sub = tid & (tpr - 1);
+      const int unit_hi = (g_end - 1) / a.n_tiles;
+      for (int unit = unit_lo; unit <= unit_hi; ++unit) {
+        float m = -1e30f, l = 0.f;
+        if (row < a.GW) {
+          int n;
+          const float2* p = a.stats.of(unit, a.GW, row, &n);
+          for (int i0 = sub; i0 < n; i0 += 4 * tpr) {
+            float2 v[4];
+            float mn = m;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              v[k] = i0 + k * tpr < n ? __ldcg(p + i0 + k * tpr) : make_float2(-1e30f, 0.f);
+              mn = fmaxf(mn, v[k].x);
+            }
+            l *= exp2f(m - mn);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) l += v[k].y * exp2f(v[k].x - mn);
+            m = mn;
+          }
+        }
+        for (int o = 1; o < tpr; o <<= 1) {
+          const float m2 = __shfl_xor_sync(0xffffffffu, m, o), l2 = __shfl_xor_sync(0xffffffffu, l, o);
+          const float mn = fmaxf(m, m2);
+          l = l * exp2f(m - mn) + l2 * exp2f(m2 - mn);
+          m = mn;
+        }
+        if (row < a.GW && sub == 0) {
+          const float lse = (m + log2f(l)) * kLn2;
+          lse_s[unit - unit_lo][row] = lse;
+          const int tile0 = unit * a.n_tiles;   // the CTA that has the unit's first tile hands it on
+          if (g_begin <= tile0 && tile0 < g_end) a.lse_out[(size_t)unit * a.GW + row] = lse;
+        }
+      }
+      asm volatile("barrier.cta.sync 1, %0;" ::"n"(kGroups * 128) : "memory");
+    }
     int seg0 = 0, seg_tile0 = tile_begin, vu = vu_begin;
     while (seg0 < nt && ok) {
       const int seg_n = min(nt - seg0, kVotes ? seg_tile0 + 1 : a.n_tiles - seg_tile0);
@@ -286,7 +344,8 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
         __syncwarp();
         for (int c = lane; c < cw; c += 32) {
           const int r = blk * a.block_rows + col0 + c;
-          nlse2_s[warp][c] = r < a.GW ? -a.row_lse[(size_t)hq0 * a.W + r] * kLog2e : -INFINITY;
+          const float lse = r >= a.GW ? INFINITY : combine ? lse_s[unit - unit_lo][r] : a.row_lse[(size_t)hq0 * a.W + r];
+          nlse2_s[warp][c] = -lse * kLog2e;
         }
         __syncwarp();
         const int part = alone ? 0 : 2 * blk + half, units = a.total_tiles / a.n_tiles;
@@ -400,19 +459,15 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
 
 // Combine the partial statistics of every observation row into its natural-log LSE, a warp per row (a thread
 // per row walked up to a hundred partials one load after the other: 18.6 us for one prompt of 131072 keys).
-// The partials of a row are those of the CTAs whose tile range overlaps the row's virtual unit.
 __global__ void __launch_bounds__(256)
-row_lse_from_parts_kernel(const float2* __restrict__ stat_part, float* __restrict__ row_lse, int rows, int GW,
-                          int vu_per_unit, int n_tiles, int tiles_per_cta, int max_slots, int n_part) {
+row_lse_from_parts_kernel(const StatParts stats, float* __restrict__ row_lse, int rows, int GW) {
   pdl_trigger();
   pdl_wait();
   const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (r >= rows) return;
-  const int unit = r / GW, row = r - unit * GW;
-  const int vu = unit * vu_per_unit + row / 256;
-  const int first = (vu * n_tiles) / tiles_per_cta, last = ((vu + 1) * n_tiles - 1) / tiles_per_cta;
-  const int n = (last - first + 1) * n_part;
-  const float2* p = stat_part + (size_t)r * max_slots * n_part;
+  const int unit = r / GW;
+  int n;
+  const float2* p = stats.of(unit, GW, r - unit * GW, &n);
   float m = -INFINITY, l = 0.f;
   for (int i = lane; i < n; i += 32) {
     const float2 q = p[i];
@@ -477,13 +532,11 @@ bool score_tc_supported(const CompressGeom& g) {
   return !g.keep_all && g.G * g.W <= kMaxRows && g.W <= 128 && g.n_cand >= 1;
 }
 
-// Statistics (row LSE) of the G*W observation rows of every unit, into ws.row_lse.  `first`: of a call, the kernel
-// then clears the workspace's error word.
-cudaError_t launch_row_stats_tc(const CompressGeom& g, const CompressWs& ws, const void* Q_obs, const void* K,
-                                char* wsp, bool first, cudaStream_t st) {
+namespace {
+
+// The statistics' tile partition, which the kernels that combine its partials need too.
+void plan_stats(const CompressGeom& g, ScoreArgs& a) {
   const int GW = g.G * g.W;
-  ScoreArgs a{};
-  a.clear_status = first;
   a.Hq = g.Hq; a.G = g.G; a.W = g.W; a.L = g.L; a.n_cand = g.n_cand; a.GW = GW;
   a.vu_per_unit = (GW + 255) / 256;
   a.vu_rows = 256;
@@ -492,6 +545,46 @@ cudaError_t launch_row_stats_tc(const CompressGeom& g, const CompressWs& ws, con
   a.n_tiles = (g.L + 255) / 256;
   partition_tiles(a, g.units * a.vu_per_unit);
   a.max_slots = (a.n_tiles + a.tiles_per_cta - 1) / a.tiles_per_cta + 1;
+}
+
+StatParts stat_parts(const ScoreArgs& a, const float2* part) {
+  return StatParts{part, a.vu_per_unit, a.n_tiles, a.tiles_per_cta, a.max_slots, a.n_blocks > 1 ? 2 : 4};
+}
+
+void plan_votes(const CompressGeom& g, ScoreArgs& a) {
+  const int GW = g.G * g.W;
+  a.Hq = g.Hq; a.G = g.G; a.W = g.W; a.L = g.L; a.n_cand = g.n_cand; a.GW = GW;
+  a.vu_per_unit = 1;
+  a.vu_rows = 0;
+  // One accumulator of up to 256 row columns per (key tile, row block).
+  a.n_blocks = (GW + 255) / 256;
+  a.block_rows = ((GW + a.n_blocks - 1) / a.n_blocks + 63) / 64 * 64;
+  a.lg_bufs = a.block_rows <= 128 ? 2 : 1;
+  a.n_tiles = (g.n_cand + kTileKeys - 1) / kTileKeys;
+  partition_tiles(a, g.units);
+}
+
+}  // namespace
+
+// Whether the votes combine the partial statistics themselves: every CTA then reads the partials of its one or two
+// units, so they must be few.  Whole compress calls with the kernel of its own and without: 8 units of 9 KB 28.2 -> 27.6 us,
+// 32 of 24 KB (32768 keys) about 1 % less, 8 of 69 KB (8192 keys) 44.6 -> 45.2.
+bool votes_combine_stats(const CompressGeom& g) {
+  ScoreArgs st{}, vt{};
+  plan_stats(g, st);
+  plan_votes(g, vt);
+  const StatParts p = stat_parts(st, nullptr);
+  return vt.tiles_per_cta <= vt.n_tiles && (size_t)st.GW * p.max_slots * p.n_part * sizeof(float2) <= 32768;
+}
+
+// Statistics of the G*W observation rows of every unit: the partials and, unless the votes combine them, the row LSE
+// into ws.row_lse.  `first`: of a call, the kernel then clears the workspace's error word.
+cudaError_t launch_row_stats_tc(const CompressGeom& g, const CompressWs& ws, const void* Q_obs, const void* K,
+                                char* wsp, bool first, bool combine, cudaStream_t st) {
+  const int GW = g.G * g.W;
+  ScoreArgs a{};
+  a.clear_status = first;
+  plan_stats(g, a);
   if (a.max_slots * kGroups > ws.stat_slots) return cudaErrorInvalidValue;
   a.stages = 2;  // 64 KB tiles of 256 keys
   a.lg_bufs = 1;
@@ -511,11 +604,13 @@ cudaError_t launch_row_stats_tc(const CompressGeom& g, const CompressWs& ws, con
   const int grid = (a.total_tiles + a.tiles_per_cta - 1) / a.tiles_per_cta;
   e = launch_pdl(score_tc_kernel<false>, dim3(grid), dim3(kThreads), (size_t)smem, st, qm, km, a);
   if (e != cudaSuccess) return e;
-  const int rows = g.B * g.Hq * g.W;
-  e = launch_pdl(row_lse_from_parts_kernel, dim3((rows + 7) / 8), dim3(256), 0, st, (const float2*)a.stat_part,
-                 (float*)(wsp + ws.row_lse), rows, GW, a.vu_per_unit, a.n_tiles, a.tiles_per_cta, a.max_slots,
-                 a.n_blocks > 1 ? 2 : 4);
-  count_launch(2);
+  count_launch(1);
+  if (combine) {
+    const int rows = g.B * g.Hq * g.W;
+    e = launch_pdl(row_lse_from_parts_kernel, dim3((rows + 7) / 8), dim3(256), 0, st, stat_parts(a, a.stat_part),
+                   (float*)(wsp + ws.row_lse), rows, GW);
+    count_launch(1);
+  }
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -523,21 +618,21 @@ cudaError_t launch_row_stats_tc(const CompressGeom& g, const CompressWs& ws, con
 // at most 128 rows.
 int votes_tc_parts(const CompressGeom& g) { return g.G * g.W <= 128 ? 1 : 2 * ((g.G * g.W + 255) / 256); }
 
-// Partial votes of every candidate key, into ws.vote_parts; the selection adds them up.
+// Partial votes of every candidate key, into ws.vote_parts; the selection adds them up.  row_lse null: combined from the
+// partials that the statistics left in the workspace, and written to ws.row_lse.
 cudaError_t launch_votes_tc(const CompressGeom& g, const CompressWs& ws, const void* Q_obs, const void* K,
                             const float* row_lse, char* wsp, bool first, cudaStream_t st) {
   const int GW = g.G * g.W;
   ScoreArgs a{};
   a.clear_status = first;
-  a.Hq = g.Hq; a.G = g.G; a.W = g.W; a.L = g.L; a.n_cand = g.n_cand; a.GW = GW;
-  a.vu_per_unit = 1;
-  a.vu_rows = 0;
-  // One accumulator of up to 256 row columns per (key tile, row block).
-  a.n_blocks = (GW + 255) / 256;
-  a.block_rows = ((GW + a.n_blocks - 1) / a.n_blocks + 63) / 64 * 64;
-  a.lg_bufs = a.block_rows <= 128 ? 2 : 1;
-  a.n_tiles = (g.n_cand + kTileKeys - 1) / kTileKeys;
-  partition_tiles(a, g.units);
+  plan_votes(g, a);
+  if (!row_lse) {
+    ScoreArgs sa{};
+    plan_stats(g, sa);
+    a.stats = stat_parts(sa, (const float2*)(wsp + ws.stat_part));
+    a.lse_out = (float*)(wsp + ws.row_lse);
+    while (a.lg_tpr < 5 && (GW << (a.lg_tpr + 1)) <= kGroups * 128) ++a.lg_tpr;
+  }
   const int q_bytes = a.n_blocks * a.block_rows * 256;
   a.stages = q_bytes <= 65536 ? 4 : (q_bytes <= 98304 ? 3 : 2);
   a.scale2 = g.scale2;

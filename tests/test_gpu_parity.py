@@ -76,6 +76,32 @@ def test_single_cta_selection_for_very_long_prompts(cuda_lib):
     decode_steps_compare(g, ref, q, kn, vn, steps=2)
 
 
+@pytest.mark.parametrize("units,G,W,L", [
+    (3, 1, 8, 300),        # combined by the votes: 32 threads share a row, two statistics tiles
+    (2, 8, 64, 700),       # ... 512 rows in two virtual units, a thread each
+    (40, 4, 16, 1500),     # ... CTAs whose range spans two units
+    (1, 4, 32, 20000),     # too many partials for it: a kernel of its own
+    (300, 1, 8, 140),      # ... CTAs of more than two units
+])
+def test_row_lse_of_the_statistics(cuda_lib, units, G, W, L):
+    """Row LSE that a compress call leaves in its workspace, against fp64.  A logit is a sum of 128 exact products in
+    fp32: an error of 128 * 2^-24 of a sum of magnitudes below 13 at the most, 1e-4."""
+    cd = cuda_lib
+    gen = torch.Generator(device="cuda").manual_seed(L)
+    rn = lambda *sh: torch.randn(sh, generator=gen, device="cuda").to(torch.bfloat16)
+    Q, K, V = rn(1, units * G, W, 128), rn(1, units, L, 128), rn(1, units, L, 128)
+    p = cd.make_params(B=1, Hq=units * G, Hkv=units, L=L, window=W, pool=5, budget=W + 20, n_cal=1, cap=W + 20)
+    st = cd.alloc_layer_state(p)
+    cd.calidrop_compress(p, Q, K, V, None, st.kept_idx, st.K_kept, st.V_kept, st.O_c, st.LSE_c, st.C_q, st.ws_compress)
+    torch.cuda.synchronize()
+    off = cd.calidrop_compress_workspace_layout(p).row_lse_offset
+    got = st.ws_compress[off:off + units * G * W * 4].view(torch.float32).view(units, G * W)
+    s = torch.einsum("urd,utd->urt", Q.view(units, G * W, 128).double(), K[0].double()) / 128 ** 0.5
+    last = L - W + torch.arange(G * W, device="cuda") % W
+    s.masked_fill_(torch.arange(L, device="cuda")[None, None] > last[None, :, None], -float("inf"))
+    assert (got.double() - torch.logsumexp(s, -1)).abs().max() < 1e-4
+
+
 @pytest.mark.parametrize("units,L,tail,pool,budget", [
     (1, 2048, 7, 1, 100),          # a full single CTA
     (3, 2049, 1, 7, 2048),         # the second CTA of the cluster holds one window row and no candidate
