@@ -350,7 +350,7 @@ calib_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
 #pragma unroll
       for (int e = 0; e < 32; e += 2) {
         const f32x2 x = fma2(pack2(sv[e], sv[e + 1]), sc, nl2);
-        const float2 p = unpack2(exp2_pair_on_poly(e / 2) ? exp2_poly2(x) : exp2_unit2(x));
+        const float2 p = unpack2(exp2_pair<true>(x, e / 2));
         sv[e] = __float_as_uint(p.x);
         sv[e + 1] = __float_as_uint(p.y);
       }

@@ -2,7 +2,7 @@
 // over logits that the tensor cores deliver needs nothing else as much, so that unit is what the scoring
 // kernels wait for.  A share of the exponentials is therefore evaluated on the FMA pipe, on PAIRS of values
 // (the packed fp32 instructions do two per issue slot): 2^x = 2^n 2^f with n = round(x), f in [-1/2, 1/2], the
-// second factor a polynomial of degree 5, the first an integer addition to the exponent field.
+// second factor a polynomial of degree 5, the first put together in the exponent field.
 // The coefficients are the minimax polynomial of 2^f on [-1/2, 1/2] in relative error (Remez exchange, then
 // rounded to fp32): 7.5e-8, evaluated in fp32 2.1e-7, which is what ex2.approx gives.
 // Measured in a bare loop over accumulators in tensor memory, four warps per scheduler, cycles per warp-wide
@@ -45,11 +45,26 @@ __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
   return d;
 }
 
-// 2^x for x <= 127; below -126 (and for -inf) the result is 2^-126 instead of 0.
-__device__ __forceinline__ f32x2 exp2_poly2(f32x2 x) {
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
+// 2^x as a product of two factors, the second a power of two.  The argument is held at -127 from below, where the power
+// of two is 0: like ex2.approx.ftz, the result underflows to 0 below -126, so that a sum over masked or far smaller
+// logits is 0 and not a count of them.  kAbove: the argument may exceed 127 (it is then held at 128, and the result is
+// infinite from 127.5 on); for logits relative to their own row's maximum or sum it cannot.
+struct Exp2Factors {
+  f32x2 p, pow2;
+};
+template <bool kAbove>
+__device__ __forceinline__ Exp2Factors exp2_factors(f32x2 x) {
   constexpr float kRound = 12582912.f;   // 1.5 * 2^23: adding it rounds to an integer in the low mantissa bits
-  const float2 v = unpack2(x);
-  x = pack2(fmaxf(v.x, -126.f), fmaxf(v.y, -126.f));
+  float2 v = unpack2(x);
+  v.x = fmaxf(v.x, -127.f); v.y = fmaxf(v.y, -127.f);
+  if (kAbove) { v.x = fminf(v.x, 128.f); v.y = fminf(v.y, 128.f); }
+  x = pack2(v.x, v.y);
   const f32x2 t = add2(x, pack2(kRound));
   const f32x2 f = fma2(add2(t, pack2(-kRound)), pack2(-1.f), x);
   f32x2 p = fma2(pack2(0.0013276472454890609f), f, pack2(0.009675540961325169f));
@@ -57,8 +72,8 @@ __device__ __forceinline__ f32x2 exp2_poly2(f32x2 x) {
   p = fma2(p, f, pack2(0.24022120237350464f));
   p = fma2(p, f, pack2(0.6931469440460205f));
   p = fma2(p, f, pack2(1.0000001192092896f));
-  const float2 pv = unpack2(p), tv = unpack2(t);
-  return pack2(__float_as_uint(pv.x) + (__float_as_uint(tv.x) << 23), __float_as_uint(pv.y) + (__float_as_uint(tv.y) << 23));
+  const float2 tv = unpack2(t);
+  return {p, pack2((__float_as_uint(tv.x) << 23) + 0x3f800000u, (__float_as_uint(tv.y) << 23) + 0x3f800000u)};
 }
 
 __device__ __forceinline__ f32x2 exp2_unit2(f32x2 x) {
@@ -70,6 +85,20 @@ __device__ __forceinline__ f32x2 exp2_unit2(f32x2 x) {
 constexpr int kPolyPairs = 3;
 __host__ __device__ constexpr bool exp2_pair_on_poly(int i) {
   return ((i % 16 + 1) * kPolyPairs) / 16 > ((i % 16) * kPolyPairs) / 16;
+}
+
+// 2^x and acc + 2^x of pair i (the addition costs the polynomial's pairs nothing: it takes the place of the product).
+template <bool kAbove>
+__device__ __forceinline__ f32x2 exp2_pair(f32x2 x, int i) {
+  if (!exp2_pair_on_poly(i)) return exp2_unit2(x);
+  const Exp2Factors e = exp2_factors<kAbove>(x);
+  return mul2(e.p, e.pow2);
+}
+template <bool kAbove>
+__device__ __forceinline__ f32x2 add_exp2_pair(f32x2 acc, f32x2 x, int i) {
+  if (!exp2_pair_on_poly(i)) return add2(acc, exp2_unit2(x));
+  const Exp2Factors e = exp2_factors<kAbove>(x);
+  return fma2(e.p, e.pow2, acc);
 }
 
 }  // namespace calidrop

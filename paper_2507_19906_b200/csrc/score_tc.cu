@@ -87,8 +87,8 @@ __device__ __forceinline__ float sum_exp2_32(const uint32_t (&r)[32], f32x2 sc, 
 #pragma unroll
   for (int e = 0; e < 32; e += 4) {
     const f32x2 x0 = fma2(pack2(r[e], r[e + 1]), sc, nr), x1 = fma2(pack2(r[e + 2], r[e + 3]), sc, nr);
-    s0 = add2(s0, exp2_pair_on_poly(e / 2) ? exp2_poly2(x0) : exp2_unit2(x0));
-    s1 = add2(s1, exp2_pair_on_poly(e / 2 + 1) ? exp2_poly2(x1) : exp2_unit2(x1));
+    s0 = add_exp2_pair<false>(s0, x0, e / 2);
+    s1 = add_exp2_pair<false>(s1, x1, e / 2 + 1);
   }
   const float2 v = unpack2(add2(s0, s1));
   return v.x + v.y;
@@ -372,8 +372,8 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
             for (int e = 0; e < 32; e += 4) {
               const ulonglong2 n4 = *reinterpret_cast<const ulonglong2*>(nl + e);
               const f32x2 x0 = fma2(pack2(r[e], r[e + 1]), sc, n4.x), x1 = fma2(pack2(r[e + 2], r[e + 3]), sc, n4.y);
-              acc0 = add2(acc0, exp2_pair_on_poly(e / 2) ? exp2_poly2(x0) : exp2_unit2(x0));
-              acc1 = add2(acc1, exp2_pair_on_poly(e / 2 + 1) ? exp2_poly2(x1) : exp2_unit2(x1));
+              acc0 = add_exp2_pair<true>(acc0, x0, e / 2);
+              acc1 = add_exp2_pair<true>(acc1, x1, e / 2 + 1);
             }
           };
           // chunks of 32 columns alternate between the two register sets; unrolled, since a loop with the

@@ -102,6 +102,68 @@ def test_row_lse_of_the_statistics(cuda_lib, units, G, W, L):
     assert (got.double() - torch.logsumexp(s, -1)).abs().max() < 1e-4
 
 
+@pytest.mark.parametrize("gap_one,gap_rest", [(78, 78), (78, 140), (140, 140)])
+def test_calibration_of_evicted_rows_with_almost_no_attention(cuda_lib, gap_one, gap_rest):
+    """The kept rows lead the evicted ones by `gap` nats, one row per kv head by another gap.  A probability below 2^-126
+    is 0 and adds nothing; where all of them are, the row has no calibration: O_c = 0, LSE_c = -inf, not applied.  The
+    one row at 78 nats is e^-82 of the softmax, far from the rest at e^-144."""
+    cd = cuda_lib
+    units, G, W, L, n_heavy = 2, 2, 16, 3000, 64
+    gen = torch.Generator(device="cuda").manual_seed(gap_one + gap_rest)
+    rn = lambda *sh: torch.randn(sh, generator=gen, device="cuda")
+    e = rn(units, 128).sign()
+    Q = (2.0 * e[None, :, None, None, :]).expand(1, units, G, W, 128).reshape(1, units * G, W, 128).to(torch.bfloat16)
+    level = torch.full((units, L), -gap_rest / 2.0, device="cuda")
+    level[:, L - W:] = 0.0
+    at = torch.randperm(L - W, generator=gen, device="cuda")
+    level[:, at[:n_heavy]] = gap_rest / 2.0
+    level[:, at[n_heavy]] = gap_rest / 2.0 - gap_one
+    # a key of `a` times the signs has the logit 2 a 128 / sqrt(128)
+    K = ((level / (2 * 128 ** 0.5))[..., None] * e[:, None]).to(torch.bfloat16)[None].contiguous()
+    V = rn(1, units, L, 128).to(torch.bfloat16)
+    budget = W + n_heavy
+    p = cd.make_params(B=1, Hq=units * G, Hkv=units, L=L, window=W, pool=1, budget=budget, n_cal=W, cap=budget, theta2=-1.0)
+    st = cd.alloc_layer_state(p)
+    cd.calidrop_compress(p, Q, K, V, None, st.kept_idx, st.K_kept, st.V_kept, st.O_c, st.LSE_c, st.C_q, st.ws_compress)
+    assert torch.equal(st.kept_idx[0, :, :n_heavy].long(), at[:n_heavy].sort().values.expand(units, -1))
+    out = torch.empty((1, units * G, 128), dtype=torch.bfloat16, device="cuda")
+    flags = torch.empty((1, units * G), dtype=torch.uint8, device="cuda")
+    cd.calidrop_decode(p, Q[:, :, -1].contiguous(), None, None, st.K_kept, st.V_kept, budget, st.O_c, st.LSE_c, st.C_q, out,
+                       None, flags, st.ws_decode)
+    if gap_one > 100:
+        assert torch.all(st.LSE_c == -float("inf")) and not st.O_c.any() and not (flags & 1).any()
+        return
+    evicted = torch.ones(L, dtype=torch.bool, device="cuda")
+    evicted[L - W:] = False
+    evicted[at[:n_heavy]] = False
+    s = torch.einsum("urd,utd->urt", Q.view(units, G * W, 128).double(), K[0].double())[..., evicted] / 128 ** 0.5
+    assert (st.LSE_c.view(units, G * W).double() - torch.logsumexp(s, -1)).abs().max() < 1e-3
+    want = torch.softmax(s, -1) @ V[0][:, evicted].double()
+    assert (st.O_c.view(units, G * W, 128).double() - want).abs().max() < 2e-2
+    assert (flags & 1).all()
+
+
+def test_votes_with_a_row_lse_far_below_the_logits(cuda_lib):
+    """A caller's row LSE is not validated: one row's that is 200 nats too low makes every vote overflow to infinity,
+    whichever of the 32 columns the row is, and the lowest candidates win."""
+    cd = cuda_lib
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    rn = lambda *sh: torch.randn(sh, generator=gen, device="cuda").to(torch.bfloat16)
+    L, W, G, budget = 900, 8, 4, 60
+    Q, K, V = rn(1, G, W, 128), rn(1, 1, L, 128), rn(1, 1, L, 128)
+    p = cd.make_params(B=1, Hq=G, Hkv=1, L=L, window=W, pool=1, budget=budget, n_cal=1, cap=budget)
+    st = cd.alloc_layer_state(p)
+    off = cd.calidrop_compress_workspace_layout(p).vote_offset
+    for row in range(G * W):
+        lse = torch.full((G * W,), 7.0, device="cuda")
+        lse[row] = -200.0
+        cd.calidrop_compress(p, Q, K, V, lse.view(1, G, W), st.kept_idx, st.K_kept, st.V_kept, st.O_c, st.LSE_c, st.C_q,
+                             st.ws_compress)
+        votes = st.ws_compress[off:off + 4 * (L - W)].view(torch.float32)
+        assert torch.all(votes == float("inf")), row
+        assert torch.equal(st.kept_idx[0, 0, :budget - W].long(), torch.arange(budget - W, device="cuda"))
+
+
 @pytest.mark.parametrize("units,L,tail,pool,budget", [
     (1, 2048, 7, 1, 100),          # a full single CTA
     (3, 2049, 1, 7, 2048),         # the second CTA of the cluster holds one window row and no candidate
