@@ -51,6 +51,18 @@ __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
   return d;
 }
 
+// fmaxf and fminf return the other operand for a NaN, and a NaN logit would leave no trace
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float min_nan(float a, float b) {
+  float r;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
 // 2^x as a product of two factors, the second a power of two.  The argument is held at -127 from below, where the power
 // of two is 0: like ex2.approx.ftz, the result underflows to 0 below -126, so that a sum over masked or far smaller
 // logits is 0 and not a count of them.  kAbove: the argument may exceed 127 (it is then held at 128, and the result is
@@ -62,8 +74,8 @@ template <bool kAbove>
 __device__ __forceinline__ Exp2Factors exp2_factors(f32x2 x) {
   constexpr float kRound = 12582912.f;   // 1.5 * 2^23: adding it rounds to an integer in the low mantissa bits
   float2 v = unpack2(x);
-  v.x = fmaxf(v.x, -127.f); v.y = fmaxf(v.y, -127.f);
-  if (kAbove) { v.x = fminf(v.x, 128.f); v.y = fminf(v.y, 128.f); }
+  v.x = max_nan(v.x, -127.f); v.y = max_nan(v.y, -127.f);
+  if (kAbove) { v.x = min_nan(v.x, 128.f); v.y = min_nan(v.y, 128.f); }
   x = pack2(v.x, v.y);
   const f32x2 t = add2(x, pack2(kRound));
   const f32x2 f = fma2(add2(t, pack2(-kRound)), pack2(-1.f), x);

@@ -164,6 +164,37 @@ def test_votes_with_a_row_lse_far_below_the_logits(cuda_lib):
         assert torch.equal(st.kept_idx[0, 0, :budget - W].long(), torch.arange(budget - W, device="cuda"))
 
 
+def test_nan_inputs_leave_a_nan_wherever_they_lie(cuda_lib):
+    """One NaN in a key or query row reaches every result that depends on it, at every position inside the 32 logits that
+    a thread works on at a time: row LSE, votes, accumulated scores; a calibration over such a key is none."""
+    cd = cuda_lib
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    rn = lambda *sh: torch.randn(sh, generator=gen, device="cuda").to(torch.bfloat16)
+    L, W, G, budget = 300, 8, 4, 60
+    Q, K, V, Q_full = rn(1, G, W, 128), rn(1, 1, L, 128), rn(1, 1, L, 128), rn(1, G, L, 128)
+    p = cd.make_params(B=1, Hq=G, Hkv=1, L=L, window=W, pool=1, budget=budget, n_cal=W, cap=budget)
+    st = cd.alloc_layer_state(p)
+    lay = cd.calidrop_compress_workspace_layout(p)
+    get = lambda off, n: st.ws_compress[off:off + 4 * n].view(torch.float32)
+    lse = torch.full((1, G, W), 7.0, device="cuda")
+    outs = (st.K_kept, st.V_kept, st.O_c, st.LSE_c, st.C_q, st.ws_compress)
+    scores = torch.empty((1, 1, L), device="cuda")
+    ws = torch.empty((cd.calidrop_accumulated_scores_workspace_bytes(p),), dtype=torch.uint8, device="cuda")
+    kept = torch.arange(L - budget, L, dtype=torch.int32, device="cuda").view(1, 1, budget)
+    for t in range(32):
+        Kt, Qt = K.clone(), Q.clone()
+        Kt[0, 0, 32 + t, 5] = float("nan")
+        Qt.view(G * W, 128)[t, 5] = float("nan")
+        cd.calidrop_compress(p, Q, Kt, V, None, st.kept_idx, *outs)
+        assert torch.all(torch.isnan(get(lay.row_lse_offset, G * W))), t
+        cd.calidrop_compress(p, Qt, K, V, lse, st.kept_idx, *outs)
+        assert torch.all(torch.isnan(get(lay.vote_offset, L - W))), t
+        cd.calidrop_calibrate(p, Q, Kt, V, lse, kept, *outs)
+        assert torch.all(st.LSE_c == -float("inf")) and not st.O_c.any(), t
+        cd.calidrop_accumulated_scores(p, Q_full, Kt, scores, ws)
+        assert torch.all(torch.isnan(scores)), t
+
+
 @pytest.mark.parametrize("units,L,tail,pool,budget", [
     (1, 2048, 7, 1, 100),          # a full single CTA
     (3, 2049, 1, 7, 2048),         # the second CTA of the cluster holds one window row and no candidate
