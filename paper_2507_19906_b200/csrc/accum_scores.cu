@@ -203,13 +203,19 @@ accum_tc_kernel(const __grid_constant__ CUtensorMap a_map, const __grid_constant
       float2 ml = make_float2(-1e30f, 0.f);    // row statistics: running (max, sum)
       f32x2 acc0 = 0ull, acc1 = 0ull;          // column sums
       const int first = (pair ^ j0) & 1;
+      int nan_at = -1;                         // column sums: the last query of this lane's whose statistics are NaN
 #pragma unroll 1
       for (int j = first; j < n_jobs; j += 2) {
         if (kSums) {
           if (!have_nl) load_nl(head, ct0 + j);
+          // A query whose statistics are NaN must reach the keys it sees and no others, but a masked logit of -inf does not
+          // outweigh it: it is left out of the sums (fmaxf drops a NaN), and its position is kept until the item's end.
           __syncwarp();
 #pragma unroll
-          for (int q = 0; q < 4; ++q) nlse2_s[warp][q * 32 + lane] = nl_next[q];
+          for (int q = 0; q < 4; ++q) {
+            if (nl_next[q] != nl_next[q]) nan_at = (ct0 + j) * kCols + half * 128 + q * 32 + lane;
+            nlse2_s[warp][q * 32 + lane] = fmaxf(nl_next[q], -INFINITY);
+          }
           __syncwarp();
           have_nl = j + 2 < n_jobs;
           if (have_nl) load_nl(head, ct0 + j + 2);
@@ -289,7 +295,8 @@ accum_tc_kernel(const __grid_constant__ CUtensorMap a_map, const __grid_constant
       const int xslot = n & 1;
       if (kSums) {
         const float2 v = unpack2(add2(acc0, acc1));
-        ml = make_float2(0.f, v.x + v.y);
+        nan_at = __reduce_max_sync(0xffffffffu, nan_at);
+        ml = make_float2(0.f, nan_at >= rt * kRows + row ? __uint_as_float(0x7fc00000u) : v.x + v.y);
       }
       if (grp != 0) {
         ok = __all_sync(0xffffffffu, mbar_wait(&ctl, x_empty(xslot), ((n >> 1) & 1) ^ 1, 56u));

@@ -195,6 +195,28 @@ def test_nan_inputs_leave_a_nan_wherever_they_lie(cuda_lib):
         assert torch.all(torch.isnan(scores)), t
 
 
+@pytest.mark.parametrize("L", [100, 300, 650])
+def test_nan_query_reaches_the_keys_it_sees_only(cuda_lib, L):
+    """Accumulated scores with a NaN in one query row: NaN up to its own position, as without it from there on."""
+    cd = cuda_lib
+    gen = torch.Generator(device="cuda").manual_seed(L)
+    rn = lambda *sh: torch.randn(sh, generator=gen, device="cuda").to(torch.bfloat16)
+    G = 2
+    Q, K = rn(1, G, L, 128), rn(1, 1, L, 128)
+    p = cd.make_params(B=1, Hq=G, Hkv=1, L=L, window=1, pool=1, budget=L, n_cal=1, cap=L)
+    want, got = (torch.empty((1, 1, L), device="cuda") for _ in range(2))
+    ws = torch.empty((cd.calidrop_accumulated_scores_workspace_bytes(p),), dtype=torch.uint8, device="cuda")
+    cd.calidrop_accumulated_scores(p, Q, K, want, ws)
+    for i in [0, 1, 10, 31, 32, 63, 64, 127, 128, 129, 255, 256, 300, 511, L - 1]:
+        if i >= L:
+            continue
+        Qn = Q.clone()
+        Qn[0, 1, i, 77] = float("nan")
+        cd.calidrop_accumulated_scores(p, Qn, K, got, ws)
+        assert torch.all(torch.isnan(got[0, 0, :i + 1])), i
+        assert torch.equal(got[0, 0, i + 1:], want[0, 0, i + 1:]), i
+
+
 @pytest.mark.parametrize("units,L,tail,pool,budget", [
     (1, 2048, 7, 1, 100),          # a full single CTA
     (3, 2049, 1, 7, 2048),         # the second CTA of the cluster holds one window row and no candidate
