@@ -2,12 +2,14 @@
 // over logits that the tensor cores deliver needs nothing else as much, so that unit is what the scoring
 // kernels wait for.  A share of the exponentials is therefore evaluated on the FMA pipe, on PAIRS of values
 // (the packed fp32 instructions do two per issue slot): 2^x = 2^n 2^f with n = round(x), f in [-1/2, 1/2], the
-// second factor a polynomial of degree 5, the first put together in the exponent field.
-// The coefficients are the minimax polynomial of 2^f on [-1/2, 1/2] in relative error (Remez exchange, then
-// rounded to fp32): 7.5e-8, evaluated in fp32 2.1e-7, which is what ex2.approx gives.
+// second factor a polynomial of degree 6, the first put together in the exponent field.
+// The coefficients are the minimax polynomial of 2^f on [-1/2, 1/2] in relative error (Remez exchange), rounded to fp32
+// one after the other from 1 upwards with the rest fitted again: 3e-9; evaluated in fp32 6.5e-8 at most, 2.6e-8 rms and
+// no bias, where ex2.approx has 1.4e-7, 6e-8 rms and a bias of -5e-8 (measured on [-30, 0]).  Degree 5 has 7.5e-8
+// before any rounding and 6.5e-8 rms after it, and sums of exponentials were less exact with it than with ex2.
 // Measured in a bare loop over accumulators in tensor memory, four warps per scheduler, cycles per warp-wide
-// exponential and scheduler: ex2 on scalars 8.8, on packed arguments 8.6; with 2, 4, 5, 6, 8, 16 pairs of 16 on the
-// polynomial 7.6, 6.9, 6.6, 6.7, 7.7, 12.0.  In the vote kernel, beside its MMAs (32 units x 32768 keys, thousand
+// exponential and scheduler (degree 5): ex2 on scalars 8.8, on packed arguments 8.6; with 2, 4, 5, 6, 8, 16 pairs of 16 on
+// the polynomial 7.6, 6.9, 6.6, 6.7, 7.7, 12.0.  In the vote kernel, beside its MMAs (32 units x 32768 keys, thousand
 // cycles): 170 without, 131, 133, 135, 138 with 3, 4, 5, 6 of 16.  Hence 3.  (With unpacked arithmetic the polynomial
 // costs ten issue slots per value, and any share of it loses.)
 #pragma once
@@ -73,17 +75,20 @@ struct Exp2Factors {
 template <bool kAbove>
 __device__ __forceinline__ Exp2Factors exp2_factors(f32x2 x) {
   constexpr float kRound = 12582912.f;   // 1.5 * 2^23: adding it rounds to an integer in the low mantissa bits
+  constexpr float kExp2Poly[7] = {1.f, 0.6931471824645996f, 0.24022647738456726f, 0.05550359934568405f,
+                                  0.009618505835533142f, 0.0013390806270763278f, 0.00015326471475418657f};
   float2 v = unpack2(x);
   v.x = max_nan(v.x, -127.f); v.y = max_nan(v.y, -127.f);
   if (kAbove) { v.x = min_nan(v.x, 128.f); v.y = min_nan(v.y, 128.f); }
   x = pack2(v.x, v.y);
   const f32x2 t = add2(x, pack2(kRound));
   const f32x2 f = fma2(add2(t, pack2(-kRound)), pack2(-1.f), x);
-  f32x2 p = fma2(pack2(0.0013276472454890609f), f, pack2(0.009675540961325169f));
-  p = fma2(p, f, pack2(0.05550713092088699f));
-  p = fma2(p, f, pack2(0.24022120237350464f));
-  p = fma2(p, f, pack2(0.6931469440460205f));
-  p = fma2(p, f, pack2(1.0000001192092896f));
+  f32x2 p = fma2(pack2(kExp2Poly[6]), f, pack2(kExp2Poly[5]));
+  p = fma2(p, f, pack2(kExp2Poly[4]));
+  p = fma2(p, f, pack2(kExp2Poly[3]));
+  p = fma2(p, f, pack2(kExp2Poly[2]));
+  p = fma2(p, f, pack2(kExp2Poly[1]));
+  p = fma2(p, f, pack2(kExp2Poly[0]));
   const float2 tv = unpack2(t);
   return {p, pack2((__float_as_uint(tv.x) << 23) + 0x3f800000u, (__float_as_uint(tv.y) << 23) + 0x3f800000u)};
 }
