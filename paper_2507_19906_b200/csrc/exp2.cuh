@@ -98,6 +98,13 @@ __device__ __forceinline__ f32x2 exp2_unit2(f32x2 x) {
   return pack2(ex2_approx(v.x), ex2_approx(v.y));
 }
 
+// 2^x of one value on the FMA pipe, for the few factors by which partial sums are brought to a common maximum: they
+// multiply whole sums, and the unit's bias of -5e-8 would add up from step to step.
+__device__ __forceinline__ float exp2_unbiased(float x) {
+  const Exp2Factors e = exp2_factors<false>(pack2(x));
+  return unpack2(mul2(e.p, e.pow2)).x;
+}
+
 // Pair i of every 16 goes to the polynomial for kPolyPairs of them, evenly spread.
 constexpr int kPolyPairs = 3;
 __host__ __device__ constexpr bool exp2_pair_on_poly(int i) {

@@ -309,20 +309,19 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
               v[k] = i0 + k * tpr < n ? __ldcg(p + i0 + k * tpr) : make_float2(-1e30f, 0.f);
               mn = fmaxf(mn, v[k].x);
             }
-            l *= exp2f(m - mn);
+            l *= exp2_unbiased(m - mn);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) l += v[k].y * exp2f(v[k].x - mn);
+            for (int k = 0; k < 4; ++k) l += v[k].y * exp2_unbiased(v[k].x - mn);
             m = mn;
           }
         }
-        for (int o = 1; o < tpr; o <<= 1) {
-          const float m2 = __shfl_xor_sync(0xffffffffu, m, o), l2 = __shfl_xor_sync(0xffffffffu, l, o);
-          const float mn = fmaxf(m, m2);
-          l = l * exp2f(m - mn) + l2 * exp2f(m2 - mn);
-          m = mn;
-        }
+        // (the maximum first, then one factor per thread: factors on every level of the exchange would add up their errors)
+        float M = m;
+        for (int o = 1; o < tpr; o <<= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+        l *= exp2_unbiased(m - M);
+        for (int o = 1; o < tpr; o <<= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
         if (row < a.GW && sub == 0) {
-          const float lse = (m + log2f(l)) * kLn2;
+          const float lse = (M + log2f(l)) * kLn2;
           lse_s[unit - unit_lo][row] = lse;
           const int tile0 = unit * a.n_tiles;   // the CTA that has the unit's first tile hands it on
           if (g_begin <= tile0 && tile0 < g_end) a.lse_out[(size_t)unit * a.GW + row] = lse;
@@ -472,11 +471,11 @@ row_lse_from_parts_kernel(const StatParts stats, float* __restrict__ row_lse, in
   for (int i = lane; i < n; i += 32) {
     const float2 q = p[i];
     const float mn = fmaxf(m, q.x);
-    l = l * exp2f(m - mn) + q.y * exp2f(q.x - mn);
+    l = l * exp2_unbiased(m - mn) + q.y * exp2_unbiased(q.x - mn);
     m = mn;
   }
   const float M = warp_max(m);
-  l = warp_sum(m > -INFINITY ? l * exp2f(m - M) : 0.f);
+  l = warp_sum(m > -INFINITY ? l * exp2_unbiased(m - M) : 0.f);
   if (lane == 0) row_lse[r] = (M + log2f(l)) * kLn2;
 }
 
