@@ -69,7 +69,7 @@ def _load_native():
     loader = importlib.machinery.ExtensionFileLoader("_marshal", MARSHAL_PATH)
     module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_marshal", loader))
     loader.exec_module(module)
-    module.open(LIB_PATH)
+    module.open(LIB_PATH, Params, DecodeLayer)
     return module
 
 

@@ -22,6 +22,9 @@ namespace {
 CALIDROP_ENTRIES(DECLARE)
 #undef DECLARE
 
+PyTypeObject* params_type = nullptr;   // the binding's ctypes structures (see open)
+PyTypeObject* layer_type = nullptr;
+
 // The positional arguments of one call.  A conversion that fails sets a Python error, after which `ok` is
 // false and the entry point is not called.
 struct Args {
@@ -69,7 +72,6 @@ struct Args {
   }
   // address of a ctypes structure or array
   void* buf(int i) {
-    if (!ok || a[i] == Py_None) return nullptr;
     Py_buffer v;
     if (PyObject_GetBuffer(a[i], &v, PyBUF_SIMPLE) != 0) { ok = false; return nullptr; }
     void* p = v.buf;
@@ -82,7 +84,25 @@ struct Args {
     if (n < 0) ok = false;
     return n;
   }
-  const calidrop_params* params(int i) { return (const calidrop_params*)buf(i); }
+  // Structures are taken by their type, as ctypes would: a buffer of other bytes would be read as pointers and sizes.
+  const calidrop_params* params(int i) {
+    if (!ok) return nullptr;
+    if (PyObject_TypeCheck(a[i], params_type)) return (const calidrop_params*)buf(i);
+    PyErr_SetString(PyExc_TypeError, "a Params structure expected");
+    ok = false;
+    return nullptr;
+  }
+  const calidrop_decode_layer* layers(int i) {
+    if (!ok) return nullptr;
+    PyObject* element = PyObject_GetAttrString((PyObject*)Py_TYPE(a[i]), "_type_");   // of an array type
+    if (!element) PyErr_Clear();
+    const bool match = element && element == (PyObject*)layer_type && PyObject_CheckBuffer(a[i]);
+    Py_XDECREF(element);
+    if (match) return (const calidrop_decode_layer*)buf(i);
+    PyErr_SetString(PyExc_TypeError, "an array of DecodeLayer structures expected");
+    ok = false;
+    return nullptr;
+  }
   void* stream() {
     if (!ok) return nullptr;
     try {
@@ -99,9 +119,11 @@ struct Args {
 template <typename F, typename... A>
 PyObject* forward(Args& x, F f, A... v) {
   if (!x.ok) return nullptr;
+  void* const stream = x.stream();
+  if (!x.ok) return nullptr;
   int rc;
   Py_BEGIN_ALLOW_THREADS   // a launch may have to wait for room in the stream's queue
-  rc = f(v...);
+  rc = f(v..., stream);
   Py_END_ALLOW_THREADS
   return PyLong_FromLong(rc);
 }
@@ -114,29 +136,41 @@ PyObject* forward(Args& x, F f, A... v) {
   }
 
 ENTRY(compress, 12, x.params(0), x.ptr(1), x.ptr(2), x.ptr(3), (const float*)x.ptr(4), (int32_t*)x.ptr(5), x.ptr(6),
-      x.ptr(7), (float*)x.ptr(8), (float*)x.ptr(9), x.ptr(10), x.ptr(11), x.nbytes(11), x.stream())
+      x.ptr(7), (float*)x.ptr(8), (float*)x.ptr(9), x.ptr(10), x.ptr(11), x.nbytes(11))
 ENTRY(calibrate, 12, x.params(0), x.ptr(1), x.ptr(2), x.ptr(3), (const float*)x.ptr(4), (const int32_t*)x.ptr(5),
-      x.ptr(6), x.ptr(7), (float*)x.ptr(8), (float*)x.ptr(9), x.ptr(10), x.ptr(11), x.nbytes(11), x.stream())
+      x.ptr(6), x.ptr(7), (float*)x.ptr(8), (float*)x.ptr(9), x.ptr(10), x.ptr(11), x.nbytes(11))
 ENTRY(gather_evicted, 8, x.params(0), x.ptr(1), x.ptr(2), (const int32_t*)x.ptr(3), (int32_t*)x.ptr(4), x.ptr(5),
-      x.ptr(6), x.ptr(7), x.nbytes(7), x.stream())
+      x.ptr(6), x.ptr(7), x.nbytes(7))
 ENTRY(recalibrate, 10, x.params(0), x.ptr(1), x.ptr(2), x.ptr(3), x.i32(4), x.i32(5), (float*)x.ptr(6),
-      (float*)x.ptr(7), x.ptr(8), x.ptr(9), x.nbytes(9), x.stream())
-ENTRY(accumulated_scores, 5, x.params(0), x.ptr(1), x.ptr(2), (float*)x.ptr(3), x.ptr(4), x.nbytes(4), x.stream())
-ENTRY(select_from_scores, 5, x.params(0), (const float*)x.ptr(1), x.i32(2), (int32_t*)x.ptr(3), x.ptr(4), x.nbytes(4),
-      x.stream())
-ENTRY(select_streaming, 3, x.params(0), x.i32(1), (int32_t*)x.ptr(2), x.stream())
+      (float*)x.ptr(7), x.ptr(8), x.ptr(9), x.nbytes(9))
+ENTRY(accumulated_scores, 5, x.params(0), x.ptr(1), x.ptr(2), (float*)x.ptr(3), x.ptr(4), x.nbytes(4))
+ENTRY(select_from_scores, 5, x.params(0), (const float*)x.ptr(1), x.i32(2), (int32_t*)x.ptr(3), x.ptr(4), x.nbytes(4))
+ENTRY(select_streaming, 3, x.params(0), x.i32(1), (int32_t*)x.ptr(2))
 ENTRY(decode, 14, x.params(0), x.ptr(1), x.ptr(2), x.ptr(3), x.ptr(4), x.ptr(5), x.i32(6), (const float*)x.ptr(7),
-      (const float*)x.ptr(8), x.ptr(9), x.ptr(10), (float*)x.ptr(11), (uint8_t*)x.ptr(12), x.ptr(13), x.nbytes(13),
-      x.stream())
-ENTRY(decode_batched, 4, x.params(0), (int32_t)x.len(1), (const calidrop_decode_layer*)x.buf(1), x.i32(2), x.ptr(3),
-      x.nbytes(3), x.stream())
+      (const float*)x.ptr(8), x.ptr(9), x.ptr(10), (float*)x.ptr(11), (uint8_t*)x.ptr(12), x.ptr(13), x.nbytes(13))
+ENTRY(decode_batched, 4, x.params(0), (int32_t)x.len(1), x.layers(1), x.i32(2), x.ptr(3),
+      x.nbytes(3))
 ENTRY(decode_static, 13, x.params(0), x.ptr(1), x.ptr(2), x.ptr(3), x.ptr(4), x.ptr(5), x.i32(6), (const float*)x.ptr(7),
-      (const float*)x.ptr(8), x.ptr(9), x.ptr(10), (float*)x.ptr(11), (uint8_t*)x.ptr(12), x.stream())
+      (const float*)x.ptr(8), x.ptr(9), x.ptr(10), (float*)x.ptr(11), (uint8_t*)x.ptr(12))
 
-// open(path): the shared library whose entry points the functions forward to
-PyObject* py_open(PyObject*, PyObject* path) {
-  const char* s = PyUnicode_AsUTF8(path);
+// open(path, Params, DecodeLayer): the shared library whose entry points the functions forward to, and the ctypes
+// structures of its arguments
+PyObject* py_open(PyObject*, PyObject* const* args, Py_ssize_t n) {
+  if (n != 3 || !PyType_Check(args[1]) || !PyType_Check(args[2]))
+    return PyErr_Format(PyExc_TypeError, "a path and two structure types expected");
+  const char* s = PyUnicode_AsUTF8(args[0]);
   if (!s) return nullptr;
+  for (int i = 1; i < 3; ++i) {
+    PyObject* o = PyObject_CallNoArgs(args[i]);
+    Py_buffer v;
+    if (!o) return nullptr;
+    const bool buffer = PyObject_GetBuffer(o, &v, PyBUF_SIMPLE) == 0;
+    Py_DECREF(o);
+    if (!buffer) return nullptr;
+    const bool same = v.len == (Py_ssize_t)(i == 1 ? sizeof(calidrop_params) : sizeof(calidrop_decode_layer));
+    PyBuffer_Release(&v);
+    if (!same) return PyErr_Format(PyExc_TypeError, "the structure's size is not the library's");
+  }
   void* h = dlopen(s, RTLD_NOW | RTLD_LOCAL);
   if (!h) return PyErr_Format(PyExc_ImportError, "%s", dlerror());
 #define RESOLVE(name)                                                                               \
@@ -144,11 +178,13 @@ PyObject* py_open(PyObject*, PyObject* path) {
   if (!f_##name) return PyErr_Format(PyExc_ImportError, "%s does not export calidrop_" #name, s);
   CALIDROP_ENTRIES(RESOLVE)
 #undef RESOLVE
+  params_type = (PyTypeObject*)Py_NewRef(args[1]);
+  layer_type = (PyTypeObject*)Py_NewRef(args[2]);
   Py_RETURN_NONE;
 }
 
 PyMethodDef methods[] = {
-    {"open", py_open, METH_O, nullptr},
+    {"open", (PyCFunction)(void (*)(void))py_open, METH_FASTCALL, nullptr},
 #define METHOD(name) {#name, (PyCFunction)(void (*)(void))py_##name, METH_FASTCALL, nullptr},
     CALIDROP_ENTRIES(METHOD)
 #undef METHOD

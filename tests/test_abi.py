@@ -5,6 +5,7 @@ import os
 import re
 
 import pytest
+import torch
 
 from paper_2507_19906_b200 import binding as cd
 from paper_2507_19906_b200 import build as cdbuild
@@ -105,3 +106,30 @@ def test_entry_points_of_the_other_eviction_rules_and_the_offload_validate_on_th
     # calibration size below -1 is no setting
     bad = cd.make_params(B=1, Hq=4, Hkv=2, L=300, window=8, pool=1, budget=40, n_cal=1, cap=40, calib_size=-2)
     assert cd.calidrop_compress_workspace_bytes(bad) == 0
+
+
+def test_native_marshalling_takes_structures_by_their_type(lib):
+    """Bytes of the right or the wrong length, another structure or an array of one are refused, not read as pointers."""
+    p = cd.make_params(B=1, Hq=4, Hkv=2, L=300, window=8, pool=1, budget=40, n_cal=1, cap=40)
+    none = [None] * 10
+    for bad in (b"", bytes(p), bytes(8), cd.DecodeLayer(), (cd.Params * 1)(), None, 0, ctypes.byref(p)):
+        with pytest.raises(TypeError):
+            cd.native().select_streaming(bad, 4, None)
+        with pytest.raises(TypeError):
+            cd.calidrop_compress(bad, *none, torch.empty(0, dtype=torch.uint8))
+    ws = torch.empty(0, dtype=torch.uint8)
+    for bad in (b"", bytes(ctypes.sizeof(cd.DecodeLayer)), (cd.Params * 2)(), (ctypes.c_void_p * 11)(), [cd.DecodeLayer()],
+                None, ctypes.pointer(cd.DecodeLayer())):
+        with pytest.raises(TypeError):
+            cd.calidrop_decode_batched(p, bad, 1, ws)
+
+    class Derived(cd.Params):
+        pass
+
+    # what is of the type goes through to the library: no device here, or its refusal of a null pointer
+    for good in (p, Derived.from_buffer_copy(p)):
+        try:
+            assert cd.calidrop_select_streaming(good, 4, None, check=False) == cd.INVALID_ARG
+            assert cd.calidrop_decode_batched(good, (cd.DecodeLayer * 2)(), 1, ws, check=False) == cd.INVALID_ARG
+        except RuntimeError:
+            assert not torch.cuda.is_available()
