@@ -37,28 +37,73 @@ struct Args {
   void* ptr(int i) {
     PyObject* o = a[i];
     if (!ok || o == Py_None) return nullptr;
-    if (THPVariable_Check(o)) {
-      const at::Tensor& t = THPVariable_Unpack(o);
-      if (t.is_contiguous()) return t.data_ptr();
-      PyErr_SetString(PyExc_AssertionError, "tensors passed to the library must be contiguous");
-      ok = false;
-      return nullptr;
+    if (PyLong_Check(o)) return address(o);
+    if (THPVariable_CheckExact(o)) {
+      // (torch throws for a tensor without memory of its own, sparse or wrapped: no exception may leave through
+      // the interpreter's frames, and the tensor's own methods raise it properly)
+      try {
+        const at::Tensor& t = THPVariable_Unpack(o);
+        if (t.is_contiguous()) return t.data_ptr();
+        not_contiguous();
+        return nullptr;
+      } catch (...) {
+      }
     }
-    if (PyLong_Check(o)) {
-      void* p = PyLong_AsVoidPtr(o);
-      ok = !PyErr_Occurred();
-      return p;
-    }
-    PyErr_SetString(PyExc_TypeError, "a tensor, an address or None expected");
-    ok = false;
-    return nullptr;
+    // subclasses of torch.Tensor and anything else with its methods
+    if (!method(o, "data_ptr")) return nullptr;
+    PyObject* contiguous = call(o, "is_contiguous");
+    if (!contiguous) return nullptr;
+    const int c = PyObject_IsTrue(contiguous);
+    Py_DECREF(contiguous);
+    if (c < 0) ok = false;
+    else if (c == 0) not_contiguous();
+    if (!ok) return nullptr;
+    PyObject* p = call(o, "data_ptr");
+    if (!p) return nullptr;
+    void* const r = address(p);
+    Py_DECREF(p);
+    return r;
   }
   size_t nbytes(int i) {
+    PyObject* o = a[i];
     if (!ok) return 0;
-    if (THPVariable_Check(a[i])) return THPVariable_Unpack(a[i]).nbytes();
-    PyErr_SetString(PyExc_TypeError, "the workspace must be a tensor");
+    if (THPVariable_CheckExact(o)) {
+      try {
+        return THPVariable_Unpack(o).nbytes();
+      } catch (...) {
+      }
+    }
+    if (!method(o, "element_size")) return 0;
+    size_t bytes = 1;
+    for (const char* m : {"numel", "element_size"}) {
+      PyObject* v = call(o, m);
+      if (!v) return 0;
+      bytes *= PyLong_AsSize_t(v);
+      Py_DECREF(v);
+      if (PyErr_Occurred()) { ok = false; return 0; }
+    }
+    return bytes;
+  }
+  void not_contiguous() {
+    PyErr_SetString(PyExc_AssertionError, "tensors passed to the library must be contiguous");
     ok = false;
-    return 0;
+  }
+  void* address(PyObject* o) {
+    void* p = PyLong_AsVoidPtr(o);
+    if (!p && PyErr_Occurred()) ok = false;
+    return p;
+  }
+  bool method(PyObject* o, const char* name) {
+    if (!PyObject_HasAttrString(o, name)) {
+      PyErr_SetString(PyExc_TypeError, "a tensor, an address or None expected");
+      ok = false;
+    }
+    return ok;
+  }
+  PyObject* call(PyObject* o, const char* name) {
+    PyObject* r = PyObject_CallMethod(o, name, nullptr);
+    if (!r) ok = false;
+    return r;
   }
   int32_t i32(int i) {
     if (!ok) return 0;

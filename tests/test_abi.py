@@ -133,3 +133,53 @@ def test_native_marshalling_takes_structures_by_their_type(lib):
             assert cd.calidrop_decode_batched(good, (cd.DecodeLayer * 2)(), 1, ws, check=False) == cd.INVALID_ARG
         except RuntimeError:
             assert not torch.cuda.is_available()
+
+
+def test_native_marshalling_leaves_errors_of_tensors_to_python(lib):
+    """A tensor for which torch throws raises in Python (a C++ exception would end the process), and subclasses or
+    wrappers are asked through their own methods."""
+    p = cd.make_params(B=1, Hq=4, Hkv=2, L=300, window=8, pool=1, budget=40, n_cal=1, cap=40)
+    ws = torch.empty(256, dtype=torch.uint8)
+    none = [None] * 10
+
+    def call(q, ws=ws):
+        return cd.calidrop_decode(p, q, *none[:4], 1, *none[:6], ws, check=False)
+
+    with pytest.raises((AssertionError, RuntimeError)):
+        call(torch.eye(4).to_sparse())
+    with pytest.raises(RuntimeError, match="storage"):
+        torch.vmap(lambda x: call(x) + x)(torch.ones(2, 4))
+    with pytest.raises(AssertionError):
+        call(torch.ones(4, 4).t())
+
+    asked = []
+
+    class Wrapper:
+        def is_contiguous(self):
+            asked.append("is_contiguous")
+            return len(asked) < 3
+
+        def data_ptr(self):
+            asked.append("data_ptr")
+            return 0
+
+        def numel(self):
+            return 256
+
+        def element_size(self):
+            raise KeyError("no size")
+
+    try:                                           # no device here, or the library's refusal of a null pointer
+        assert call(Wrapper()) == cd.INVALID_ARG
+    except RuntimeError:
+        assert not torch.cuda.is_available()
+    assert asked == ["is_contiguous", "data_ptr"]
+    with pytest.raises(AssertionError):
+        call(Wrapper())
+    with pytest.raises(KeyError):
+        call(None, Wrapper())
+    for bad in ("q", 1.5, [1]):
+        with pytest.raises(TypeError):
+            call(bad)
+        with pytest.raises(TypeError):
+            call(None, bad)
