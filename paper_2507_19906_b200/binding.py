@@ -17,10 +17,12 @@ from dataclasses import dataclass
 
 import torch
 
+from .build import marshal_path
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 # CALIDROP_LIB selects another build of the same library (e.g. an instrumented one).
 LIB_PATH = os.environ.get("CALIDROP_LIB") or os.path.join(_HERE, "libcalidrop.so")
-MARSHAL_PATH = os.path.join(_HERE, "_marshal.so")
+MARSHAL_PATH = marshal_path()
 _lib = None
 _native = None
 

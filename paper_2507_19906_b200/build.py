@@ -11,13 +11,20 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libcalidrop.so")
 MARSHAL_SRC = os.path.join(CSRC, "marshal.cpp")
-MARSHAL = os.path.join(HERE, "_marshal.so")
 HEADER = os.path.join(os.path.dirname(HERE), "include", "calidrop.h")
 
 NVCC_FLAGS = [
     "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
     "-Xcompiler", "-fPIC", "-shared", "--expt-relaxed-constexpr",
 ]
+
+
+def marshal_path() -> str:
+    """The marshalling module, named after the Python and the torch whose binary interfaces it is compiled against, so
+    that a module built for others is never loaded."""
+    import torch
+
+    return os.path.join(HERE, f"_marshal.{sys.implementation.cache_tag}-torch{torch.__version__}.so")
 
 
 def sources():
@@ -37,14 +44,15 @@ def _older(target, deps) -> bool:
 
 
 def is_stale() -> bool:
-    return _older(LIB, _deps()) or _older(MARSHAL, [MARSHAL_SRC, HEADER])
+    return _older(LIB, _deps()) or _older(marshal_path(), [MARSHAL_SRC, HEADER])
 
 
 def _build_marshal() -> None:
     import torch
     from torch.utils import cpp_extension
 
-    tmp = MARSHAL + f".{os.getpid()}.tmp"
+    target = marshal_path()
+    tmp = target + f".{os.getpid()}.tmp"
     libs = cpp_extension.library_paths("cuda")
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared",
            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
@@ -53,11 +61,11 @@ def _build_marshal() -> None:
     cmd += ["-o", tmp, MARSHAL_SRC] + [f"-L{p}" for p in libs] + \
         ["-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-ldl"]
     subprocess.check_call(cmd)
-    os.replace(tmp, MARSHAL)
+    os.replace(tmp, target)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    if force or _older(MARSHAL, [MARSHAL_SRC, HEADER]):
+    if force or _older(marshal_path(), [MARSHAL_SRC, HEADER]):
         _build_marshal()
     if not force and not _older(LIB, _deps()):
         return LIB

@@ -183,3 +183,11 @@ def test_native_marshalling_leaves_errors_of_tensors_to_python(lib):
             call(bad)
         with pytest.raises(TypeError):
             call(None, bad)
+
+
+def test_marshalling_module_of_another_torch_counts_as_stale(lib, monkeypatch):
+    """The module is compiled against the binary interface of a Python and a torch: another version of either needs a
+    build of its own and never loads this one."""
+    assert not cdbuild.is_stale() and os.path.exists(cdbuild.marshal_path())
+    monkeypatch.setattr(torch, "__version__", "0.0.0")
+    assert cdbuild.is_stale() and not os.path.exists(cdbuild.marshal_path())
