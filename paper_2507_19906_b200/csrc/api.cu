@@ -86,8 +86,8 @@ CompressWs make_ws(const CompressGeom& g) {
   w.bitmap2 = off; off = align_up(off + (g.sized ? (size_t)g.units * g.bitmap_words * 4 : 0), 256);
   w.calib_mask = g.sized ? w.bitmap2 : w.bitmap;
   w.n_tiles = (g.L + 127) / 128;
-  w.stat_slots = w.n_tiles > 320 ? w.n_tiles : 320;
-  w.stat_part = off; off = align_up(off + (size_t)g.B * g.Hq * g.W * w.stat_slots * 8, 256);
+  const size_t stat_slots = score_tc_supported(g) ? row_stats_tc_slots(g) : w.n_tiles;   // partials of an observation row
+  w.stat_part = off; off = align_up(off + (size_t)g.B * g.Hq * g.W * stat_slots * 8, 256);
   w.status = off;    off = align_up(off + 4, 256);
   w.calib_o = w.calib_l = off;
   if (score_tc_supported(g) && calib_tc_supported(g)) {

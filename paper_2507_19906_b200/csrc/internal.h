@@ -29,7 +29,6 @@ struct CompressWs {
   size_t bitmap2;     // sized calibration: bit set = the row is NOT one of the calibrated evicted rows
   size_t calib_mask;  // the bitmap the calibration passes mask with: bitmap, or bitmap2 when sized
   int n_tiles;     // 128-key tiles per unit (scalar statistics pass: one partial per tile)
-  int stat_slots;  // (max, sum) partial slots per observation row in stat_part
 };
 
 struct DecodeLayerPtrs {
@@ -94,6 +93,7 @@ cudaError_t launch_calib_direct(const CompressGeom& g, const CompressWs& ws, con
 // score_tc.cu / calib_tc.cu: the tcgen05 + TMA path
 int pick_tile_splits(int groups, int n_tiles, int min_tiles);
 bool score_tc_supported(const CompressGeom& g);
+size_t row_stats_tc_slots(const CompressGeom& g);   // (max, sum) partials of an observation row
 cudaError_t launch_row_stats_tc(const CompressGeom& g, const CompressWs& ws, const void* Q_obs, const void* K,
                                 char* wsp, bool first, bool combine, cudaStream_t st);
 bool votes_combine_stats(const CompressGeom& g);

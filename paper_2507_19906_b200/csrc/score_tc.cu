@@ -565,6 +565,12 @@ void plan_votes(const CompressGeom& g, ScoreArgs& a) {
 
 }  // namespace
 
+size_t row_stats_tc_slots(const CompressGeom& g) {
+  ScoreArgs a{};
+  plan_stats(g, a);
+  return (size_t)a.max_slots * stat_parts(a, nullptr).n_part;
+}
+
 // Whether the votes combine the partial statistics themselves: every CTA then reads the partials of its one or two
 // units, so they must be few.  Whole compress calls with the kernel of its own and without: 8 units of 9 KB 28.2 -> 27.6 us,
 // 32 of 24 KB (32768 keys) about 1 % less, 8 of 69 KB (8192 keys) 44.6 -> 45.2.
@@ -584,7 +590,6 @@ cudaError_t launch_row_stats_tc(const CompressGeom& g, const CompressWs& ws, con
   ScoreArgs a{};
   a.clear_status = first;
   plan_stats(g, a);
-  if (a.max_slots * kGroups > ws.stat_slots) return cudaErrorInvalidValue;
   a.stages = 2;  // 64 KB tiles of 256 keys
   a.lg_bufs = 1;
   a.scale2 = g.scale2;

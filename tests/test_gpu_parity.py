@@ -82,6 +82,10 @@ def test_single_cta_selection_for_very_long_prompts(cuda_lib):
     (40, 4, 16, 1500),     # ... CTAs whose range spans two units
     (1, 4, 32, 20000),     # too many partials for it: a kernel of its own
     (300, 1, 8, 140),      # ... CTAs of more than two units
+    (1, 4, 32, 20225),     # one unit: 80 tiles on a CTA each, 81 slots of four partials
+    (1, 4, 64, 32768),     # ... 129 slots of two
+    (1, 1, 8, 32768),      # ... of four
+    (1, 2, 16, 65536),     # ... two tiles a CTA
 ])
 def test_row_lse_of_the_statistics(cuda_lib, units, G, W, L):
     """Row LSE that a compress call leaves in its workspace, against fp64.  A logit is a sum of 128 exact products in
