@@ -356,15 +356,9 @@ accum_group_sum_kernel(const float* __restrict__ part, float* __restrict__ score
 
 template <bool kSums>
 cudaError_t launch_pass(const AccumArgs& a, const CUtensorMap& am, const CUtensorMap& bm, cudaStream_t st) {
-  static bool attr_set[64] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  static OncePerDevice granted;
+  cudaError_t e = grant_smem(accum_tc_kernel<kSums>, kSmem, granted);
   if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-    e = cudaFuncSetAttribute(accum_tc_kernel<kSums>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) attr_set[dev] = true;
-  }
   return launch_pdl(accum_tc_kernel<kSums>, dim3(a.items < kSms ? a.items : kSms), dim3(kThreads), (size_t)kSmem, st, am, bm, a);
 }
 

@@ -550,15 +550,9 @@ cudaError_t launch_calib_tc(const CompressGeom& g, const CompressWs& ws, const v
   const uint32_t kb[2] = {(uint32_t)kTileKeys, 1};
   if (!make_tensor_map_bf16(&km, K, 3, kd, ks, kb) || !make_tensor_map_bf16(&vm, V, 3, kd, ks, kb))
     return cudaErrorInvalidValue;
-  static bool attr_set[64] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  static OncePerDevice granted;
+  cudaError_t e = grant_smem(calib_tc_kernel, kSmemBytes, granted);
   if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-    e = cudaFuncSetAttribute(calib_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) attr_set[dev] = true;
-  }
   const int grid = (a.total_tiles + a.tiles_per_cta - 1) / a.tiles_per_cta * a.n_cblocks;
   e = launch_pdl(calib_tc_kernel, dim3(grid), dim3(kThreads), (size_t)kSmemBytes, st, qm, km, vm, a);
   if (e != cudaSuccess) return e;

@@ -1,6 +1,8 @@
 // Internal launcher interface between the C-ABI layer (api.cu) and the kernels.
 #pragma once
 
+#include <atomic>
+
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <stddef.h>
@@ -173,6 +175,21 @@ cudaError_t launch_calib_none(const CompressGeom& g, const void* Q_obs, float* O
 void count_launch(int n = 1);
 
 #ifdef __CUDACC__
+// Lets `kernel` use `bytes` of dynamic shared memory, once per device; `done` is the kernel's own.  Threads may race
+// here: all of them set the same value, so `bytes` must be the most that any launch of the kernel asks for.
+using OncePerDevice = std::atomic<bool>[64];
+template <typename... Params>
+cudaError_t grant_smem(void (*kernel)(Params...), int bytes, OncePerDevice& done) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const bool slot = dev >= 0 && dev < 64;
+  if (slot && done[dev].load(std::memory_order_acquire)) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess && slot) done[dev].store(true, std::memory_order_release);
+  return e;
+}
+
 // Launch with the programmatic-serialisation attribute (see pdl_wait in common.cuh).
 template <typename... Params, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {

@@ -489,16 +489,17 @@ __global__ void add_votes_kernel(float* __restrict__ vote, const float* __restri
   vote[i] = x;
 }
 
+// The query rows of a virtual unit and the ring of key tiles share this much, however they divide it.
+constexpr int kSmemMax = 192 * 1024 + 1024;
+
 template <bool kVotes>
-cudaError_t set_smem_limit(int bytes) {
-  static int granted[64] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+cudaError_t launch_score(const CUtensorMap& qm, const CUtensorMap& km, const ScoreArgs& a, int smem, cudaStream_t st) {
+  static OncePerDevice granted;
+  if (smem > kSmemMax) return cudaErrorInvalidValue;
+  cudaError_t e = grant_smem(score_tc_kernel<kVotes>, kSmemMax, granted);
   if (e != cudaSuccess) return e;
-  if (dev >= 0 && dev < 64 && granted[dev] >= bytes) return cudaSuccess;
-  e = cudaFuncSetAttribute(score_tc_kernel<kVotes>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess && dev >= 0 && dev < 64) granted[dev] = bytes;
-  return e;
+  const int grid = (a.total_tiles + a.tiles_per_cta - 1) / a.tiles_per_cta;
+  return launch_pdl(score_tc_kernel<kVotes>, dim3(grid), dim3(kThreads), (size_t)smem, st, qm, km, a);
 }
 
 // Equal contiguous tile ranges over at most one CTA per SM.
@@ -603,10 +604,7 @@ cudaError_t launch_row_stats_tc(const CompressGeom& g, const CompressWs& ws, con
   if (!make_tensor_map_bf16(&qm, Q_obs, 3, qd, qs, qb) || !make_tensor_map_bf16(&km, K, 3, kd, ks, kb))
     return cudaErrorInvalidValue;
   const int smem = a.n_blocks * 128 * 256 + a.stages * 256 * 256 + 1024;
-  cudaError_t e = set_smem_limit<false>(smem);
-  if (e != cudaSuccess) return e;
-  const int grid = (a.total_tiles + a.tiles_per_cta - 1) / a.tiles_per_cta;
-  e = launch_pdl(score_tc_kernel<false>, dim3(grid), dim3(kThreads), (size_t)smem, st, qm, km, a);
+  cudaError_t e = launch_score<false>(qm, km, a, smem, st);
   if (e != cudaSuccess) return e;
   count_launch(1);
   if (combine) {
@@ -651,10 +649,7 @@ cudaError_t launch_votes_tc(const CompressGeom& g, const CompressWs& ws, const v
   if (!make_tensor_map_bf16(&qm, Q_obs, 3, qd, qs, qb) || !make_tensor_map_bf16(&km, K, 3, kd, ks, kb))
     return cudaErrorInvalidValue;
   const int smem = q_bytes + a.stages * kKvTileBytes + 1024;
-  cudaError_t e = set_smem_limit<true>(smem);
-  if (e != cudaSuccess) return e;
-  const int grid = (a.total_tiles + a.tiles_per_cta - 1) / a.tiles_per_cta;
-  e = launch_pdl(score_tc_kernel<true>, dim3(grid), dim3(kThreads), (size_t)smem, st, qm, km, a);
+  cudaError_t e = launch_score<true>(qm, km, a, smem, st);
   if (e != cudaSuccess) return e;
   count_launch(1);
   return cudaGetLastError();

@@ -4,6 +4,10 @@ Tolerances: kept-index sets bit-exact except near-tie swaps
 (oracle pooled votes within 1e-5 relative); K_kept/V_kept/C_q bit-exact; O_c and decode
 outputs within max-abs 2e-2 and mean-abs 2e-3; LSE_c and the output LSE within 1e-3.
 """
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -1152,6 +1156,46 @@ def test_accumulated_scores_at_the_edges_of_their_tiles(cuda_lib, B, Hq, Hkv, L)
             s = (Q[b, hq].double() @ K[b, hq // G].double().T) / 128 ** 0.5
             ref[b, hq // G] += torch.softmax(s.masked_fill_(mask, -float("inf")), -1).sum(0)
     torch.testing.assert_close(scores.double(), ref, rtol=2e-5, atol=1e-6)
+
+
+def test_first_calls_of_several_threads_with_different_window_sizes(cuda_lib):
+    """Threads whose first calls need different amounts of shared memory of the same kernel start at the same moment, in a
+    process of its own (what a launch sets up once per device is not set up yet there).  (The two can interleave in
+    an order that leaves the lower limit; whether they do is up to the scheduler.)"""
+    code = """
+import threading, torch
+from paper_2507_19906_b200 import binding as cd
+cd.load()
+L, W, budget, out, errors = 700, 32, 80, {}, []
+def state(G):
+    gen = torch.Generator(device="cuda").manual_seed(G)
+    rn = lambda *sh: torch.randn(sh, generator=gen, device="cuda").to(torch.bfloat16)
+    p = cd.make_params(B=1, Hq=G, Hkv=1, L=L, window=W, pool=1, budget=budget, n_cal=W, cap=budget)
+    return p, rn(1, G, W, 128), rn(1, 1, L, 128), rn(1, 1, L, 128), cd.alloc_layer_state(p)
+def run(p, Q, K, V, st):
+    cd.calidrop_compress(p, Q, K, V, None, st.kept_idx, st.K_kept, st.V_kept, st.O_c, st.LSE_c, st.C_q, st.ws_compress)
+states = {G: state(G) for G in range(1, 9)}
+torch.cuda.synchronize()
+start = threading.Barrier(len(states))
+def work(G):
+    with torch.cuda.stream(torch.cuda.Stream()):
+        start.wait()
+        try:
+            for _ in range(20): run(*states[G])
+        except Exception as e:
+            errors.append((G, e))
+threads = [threading.Thread(target=work, args=(G,)) for G in states]
+[t.start() for t in threads]; [t.join() for t in threads]
+torch.cuda.synchronize()
+assert not errors, errors
+for G, s in states.items():
+    got = [t.clone() for t in (s[4].kept_idx, s[4].O_c, s[4].LSE_c)]
+    run(*s)
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(got, (s[4].kept_idx, s[4].O_c, s[4].LSE_c))), G
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    subprocess.run([sys.executable, "-c", code], cwd=root, check=True, timeout=300)
 
 
 def test_calls_enqueued_back_to_back_give_the_results_of_calls_run_one_at_a_time(cuda_lib):
