@@ -302,6 +302,20 @@ int calidrop_decode_workspace_init(void* workspace, size_t workspace_bytes, void
 size_t calidrop_decode_workspace_status_offset(const calidrop_params* p);
 
 /*
+ * How a decode launch over n_rows cached rows (kv_len, and one more when the step appends) of n_layers layers would be
+ * laid out on the current device, for diagnostics and tests; with `recalibrate` the launch of
+ * calidrop_recalibrate over n_rows evicted rows (n_layers is then 1).  Nothing is enqueued.  The results of a step do
+ * not depend on the layout beyond rounding.  Returns CALIDROP_OK, INVALID_ARG or UNSUPPORTED.
+ */
+typedef struct calidrop_decode_layout {
+  int32_t cluster_ctas;        /* CTAs of a thread-block cluster, which share a (layer, unit)'s rows      */
+  int32_t clusters_per_unit;   /* more than one: they meet through the workspace                        */
+  int32_t ctas_per_sm;         /* 1, 2 or 4                                                               */
+} calidrop_decode_layout;
+int calidrop_decode_plan(const calidrop_params* p, int32_t n_layers, int32_t n_rows, int32_t recalibrate,
+                         calidrop_decode_layout* out);
+
+/*
  * One decode step for one layer (Algorithm 2, lines 1-2 and 9-14).
  *
  * Per (b, query head hq of kv head h):

@@ -37,7 +37,7 @@ EXPORTS = [
     "calidrop_accumulated_scores_workspace_bytes", "calidrop_accumulated_scores",
     "calidrop_compress_workspace_layout",
     "calidrop_decode_workspace_bytes", "calidrop_decode_workspace_init",
-    "calidrop_decode_workspace_status_offset", "calidrop_decode",
+    "calidrop_decode_workspace_status_offset", "calidrop_decode_plan", "calidrop_decode",
     "calidrop_decode_batched", "calidrop_decode_static", "calidrop_compress_host", "calidrop_decode_host",
     "calidrop_status_string", "calidrop_version", "calidrop_launch_count",
 ]
@@ -58,6 +58,10 @@ class CompressLayout(C.Structure):
 class DecodeLayer(C.Structure):
     _fields_ = [(n, C.c_void_p) for n in
                 ("q", "k_new", "v_new", "K_kept", "V_kept", "O_c", "LSE_c", "C_q", "out", "lse_out", "flags")]
+
+
+class DecodeLayout(C.Structure):
+    _fields_ = [(n, C.c_int32) for n in ("cluster_ctas", "clusters_per_unit", "ctas_per_sm")]
 
 
 class CalidropError(RuntimeError):
@@ -114,6 +118,8 @@ def load():
     lib.calidrop_calibrate.argtypes = [C.POINTER(Params)] + [vp] * 11 + [C.c_size_t, vp]
     lib.calidrop_decode_workspace_status_offset.restype = C.c_size_t
     lib.calidrop_decode_workspace_status_offset.argtypes = [C.POINTER(Params)]
+    lib.calidrop_decode_plan.restype = C.c_int
+    lib.calidrop_decode_plan.argtypes = [C.POINTER(Params), C.c_int32, C.c_int32, C.c_int32, C.POINTER(DecodeLayout)]
     lib.calidrop_decode_workspace_init.restype = C.c_int
     lib.calidrop_decode_workspace_init.argtypes = [vp, C.c_size_t, vp]
     lib.calidrop_decode.restype = C.c_int
@@ -189,6 +195,12 @@ def calidrop_decode_workspace_bytes(p: Params, kv_len_max: int) -> int:
 
 def calidrop_decode_workspace_status_offset(p: Params) -> int:
     return int(load().calidrop_decode_workspace_status_offset(C.byref(p)))
+
+
+def calidrop_decode_plan(p: Params, n_layers: int, n_rows: int, recalibrate: bool = False) -> DecodeLayout:
+    out = DecodeLayout()
+    _check(load().calidrop_decode_plan(C.byref(p), n_layers, n_rows, int(recalibrate), C.byref(out)), "calidrop_decode_plan")
+    return out
 
 
 def calidrop_compress_workspace_layout(p: Params) -> CompressLayout:

@@ -539,6 +539,18 @@ int calidrop_decode_batched(const calidrop_params* p, int32_t n_layers, const ca
   return e == cudaSuccess ? CALIDROP_OK : cuda_fail(e);
 }
 
+int calidrop_decode_plan(const calidrop_params* p, int32_t n_layers, int32_t n_rows, int32_t recalibrate,
+                         calidrop_decode_layout* out) {
+  int rc = check_common(p);
+  if (rc != CALIDROP_OK) return rc;
+  if (!out || n_rows < 1 || n_layers < 1 || n_layers > kDecodeMaxLayers || (recalibrate && n_layers != 1))
+    return CALIDROP_INVALID_ARG;
+  if (!device_supported()) return CALIDROP_UNSUPPORTED;
+  const DecodeCommon a = plan_decode(p, make_decode_ws(p), n_layers, n_rows, n_rows, false, n_rows, recalibrate != 0, nullptr);
+  *out = calidrop_decode_layout{a.nsplit, a.nclu, decode_ctas_per_sm(a)};
+  return CALIDROP_OK;
+}
+
 int calidrop_decode(const calidrop_params* p, const void* q, const void* k_new, const void* v_new,
                     void* K_kept, void* V_kept, int32_t kv_len, const float* O_c, const float* LSE_c,
                     const void* C_q, void* out, float* lse_out, uint8_t* flags, void* workspace,

@@ -981,17 +981,25 @@ cudaError_t launch_decode_s(const DecodeArgsT<NL>& a, cudaStream_t st) {
 // slices of more CTAs than fit two to an SM keep it.  2048 of 231 rows: two CTAs of eight stream warps with the similarities
 // through registers 88.9, four of four warps 73, with the calibration queries through the ring 60 (48 for the bytes).
 constexpr int kNarrowRows = 1024;
+
 template <int NL, bool RECAL>
 cudaError_t launch_decode_t(const DecodeArgsT<NL>& a, cudaStream_t st) {
-  const long long ctas = (long long)a.c.nsplit * a.c.nclu * a.c.units * a.c.n_layers;
-  if (ctas > 2 * kDecodeTargetCtas && a.c.rows_per_split <= kNarrowRows) return launch_decode_s<NL, RECAL, ShapeNarrow>(a, st);
-  if (ctas > kDecodeTargetCtas && ctas <= 2 * kDecodeTargetCtas) return launch_decode_s<NL, RECAL, ShapePair>(a, st);
+  switch (decode_ctas_per_sm(a.c)) {
+    case 4: return launch_decode_s<NL, RECAL, ShapeNarrow>(a, st);
+    case 2: return launch_decode_s<NL, RECAL, ShapePair>(a, st);
+  }
   if constexpr (!RECAL)
     if (a.c.nsplit > 8) return launch_decode_s<NL, RECAL, ShapeCluster16>(a, st);
   return launch_decode_s<NL, RECAL, ShapeWide>(a, st);
 }
 
 }  // namespace
+
+int decode_ctas_per_sm(const DecodeCommon& c) {
+  const long long ctas = (long long)c.nsplit * c.nclu * c.units * c.n_layers;
+  if (ctas > 2 * kDecodeTargetCtas && c.rows_per_split <= kNarrowRows) return 4;
+  return ctas > kDecodeTargetCtas && ctas <= 2 * kDecodeTargetCtas ? 2 : 1;
+}
 
 cudaError_t launch_decode(const DecodeArgsT<1>& a, cudaStream_t st) { return launch_decode_t<1, false>(a, st); }
 cudaError_t launch_decode(const DecodeArgsT<kDecodeMaxLayers>& a, cudaStream_t st) {

@@ -163,9 +163,11 @@ cudaError_t launch_decode(const DecodeArgsT<1>& a, cudaStream_t st);
 cudaError_t launch_decode(const DecodeArgsT<kDecodeMaxLayers>& a, cudaStream_t st);
 // The same stream over the evicted KV (K, V of the layer = the compacted evicted rows), rewriting
 // row recal_slot of O_c, LSE_c, C_q (Algorithm 2, lines 4-6).
+cudaError_t launch_recalibrate(const DecodeArgsT<1>& a, cudaStream_t st);
 // Clusters of `ctas` CTAs of the decode kernel, one CTA per SM, that the current device runs at the same time (0: none).
 int decode_resident_clusters(int ctas);
-cudaError_t launch_recalibrate(const DecodeArgsT<1>& a, cudaStream_t st);
+// CTAs that share an SM in the shape that a launch takes (see launch_decode_t).
+int decode_ctas_per_sm(const DecodeCommon& c);
 cudaError_t launch_evicted_indices(const CompressGeom& g, const CompressWs& ws, char* wsp, const int32_t* kept_idx,
                                    int32_t* evict_idx, cudaStream_t st);
 // Calibration size -1: no row is calibrated (O_c = 0, LSE_c = -inf, C_q = the calibration queries).

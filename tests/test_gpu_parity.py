@@ -665,8 +665,8 @@ def test_config5_last_query_only(cuda_lib):
     (2, 8, 2, 60, 8, 2),      # the appended row crosses the first 64-row slot boundary
     (1, 7, 1, 1020, 10, 5),   # ... and a 16-row block boundary deep in a slice
     (3, 8, 8, 250, 4, 1),     # 24 units: clusters of 4, slices of about 64 rows
-    (1, 4, 1, 16500, 3, 2),   # one unit, 16500 rows: two clusters per unit meet through the workspace
-    (1, 8, 2, 40000, 2, 1),   # two units, 40000 rows each: four clusters per unit
+    (1, 4, 1, 16500, 3, 2),   # one unit, 16500 rows: several clusters meet through the workspace
+    (1, 8, 2, 40000, 2, 1),   # two units, 40000 rows each: several clusters per unit
 ])
 def test_decode_ignores_cache_rows_beyond_kv_len(cuda_lib, B, Hq, Hkv, kv0, steps, n_cal):
     """The cache rows at and beyond kv_len belong to the caller and may hold anything; here they
@@ -719,19 +719,21 @@ def test_decode_ignores_cache_rows_beyond_kv_len(cuda_lib, B, Hq, Hkv, kv0, step
         np.testing.assert_array_equal(to_bits(st.K_kept)[:, :, kv0 + t + 1:], Kk[:, :, kv0 + t + 1:])
 
 
-@pytest.mark.parametrize("units,layers,G,kv,n_cal", [
-    (80, 2, 1, 64, 1),        # two CTAs per SM: one calibration row, one whole slot and the appended row
-    (80, 3, 4, 700, 33),      # ... 132 calibration rows, four of them in a second slot
-    (20, 8, 3, 2100, 64),     # ... a long slice
-    (80, 4, 8, 0, 64),        # four CTAs per SM: the appended row alone
-    (75, 5, 7, 32, 100),      # ... eleven slots of calibration rows, the last with 60; 300 rows of n_cal above 64
-    (80, 4, 2, 1023, 16),     # ... the longest slice of this shape
-    (80, 4, 2, 1024, 16),     # one more row: the wide ring, more CTAs than SMs
-    (3, 1, 7, 4400, 5),       # clusters of sixteen, five calibration rows over sixteen CTAs
-    (1, 2, 8, 9001, 64),      # ... or several clusters of eight
-    (16, 1, 4, 2100, 8),      # more clusters of eight than the GPU holds at once: clusters of four
+@pytest.mark.parametrize("units,layers,G,kv,n_cal,layout", [
+    # layout: CTAs of a cluster, clusters per unit, CTAs per SM
+    (80, 2, 1, 64, 1, (1, 1, 2)),         # one calibration row, one whole slot and the appended row
+    (80, 3, 4, 700, 33, (1, 1, 2)),       # 132 calibration rows, four of them in a second slot
+    (20, 8, 3, 2100, 64, (1, 1, 2)),      # a long slice
+    (80, 4, 8, 0, 64, (1, 1, 4)),         # the appended row alone
+    (75, 5, 7, 32, 100, (1, 1, 4)),       # eleven slots of calibration rows, the last with 60; n_cal above 64
+    (80, 4, 2, 1023, 16, (1, 1, 4)),      # the longest slice of this shape
+    (80, 4, 2, 1024, 16, (1, 1, 1)),      # one more row: the wide ring, more CTAs than SMs
+    (3, 1, 7, 4400, 5, (16, 1, 1)),       # five calibration rows over sixteen CTAs
+    (1, 2, 8, 9001, 64, (16, 1, 1)),      # ... 64, in two layers
+    (1, 2, 8, 17000, 64, (8, 5, 1)),      # several clusters of eight
+    (16, 1, 4, 2100, 8, (4, 1, 1)),       # more clusters of eight than the GPU holds at once
 ])
-def test_decode_launch_shapes_against_fp32(cuda_lib, units, layers, G, kv, n_cal):
+def test_decode_launch_shapes_against_fp32(cuda_lib, units, layers, G, kv, n_cal, layout):
     """Every shape that the launch rules choose between, at its edges, against the same step in fp32: outputs are bf16
     of values below about 2 (tolerances of the other parity tests); the calibration row is the one the query was
     drawn around, far from any tie."""
@@ -741,6 +743,8 @@ def test_decode_launch_shapes_against_fp32(cuda_lib, units, layers, G, kv, n_cal
     Hq, cap = units * G, kv + 3
     p = cd.make_params(B=1, Hq=Hq, Hkv=units, n_cal=n_cal, cap=cap)
     p.theta1, p.theta2 = 0.7, -1.0
+    plan = cd.calidrop_decode_plan(p, layers, kv + 1)
+    assert (plan.cluster_ctas, plan.clusters_per_unit, plan.ctas_per_sm) == layout
     bf = torch.bfloat16
     ins = []
     for i in range(layers):
@@ -777,7 +781,7 @@ def test_decode_launch_shapes_against_fp32(cuda_lib, units, layers, G, kv, n_cal
 
 def test_batched_layers_with_several_clusters_per_unit(cuda_lib):
     """Two layers of one unit with 17000 cached rows in one launch: every (layer, unit) is split over
-    two clusters that meet through the workspace, each layer with its own counters and partials.
+    several clusters that meet through the workspace, each layer with its own counters and partials.
     Checked against the oracle, twice on the same workspace (the counters must come back to zero)."""
     cd = cuda_lib
     rng = np.random.Generator(np.random.Philox(key=[91, 5]))
@@ -786,6 +790,7 @@ def test_batched_layers_with_several_clusters_per_unit(cuda_lib):
     bits = lambda x: wl.f32_to_bf16_bits(np.ascontiguousarray(x, dtype=np.float32))
     p = cd.make_params(B=B, Hq=Hq, Hkv=Hkv, L=kv0 + 64, window=8, pool=7, budget=kv0, n_cal=n_cal, cap=cap)
     p.theta1, p.theta2 = 0.7, -1.0
+    assert cd.calidrop_decode_plan(p, NL, kv0 + 1).clusters_per_unit > 1
     ws = torch.zeros((cd.calidrop_decode_workspace_bytes(p, cap) * NL,), dtype=torch.uint8, device="cuda")
     host, layers = [], []
     for _ in range(NL):
@@ -905,10 +910,42 @@ def test_evicted_list_at_the_edges_of_its_slices(cuda_lib, units, L, W, budget):
         assert not K_e[0, u, len(want):].any()
 
 
+@pytest.mark.parametrize("units,G,n_evict,layout", [
+    (160, 3, 300, (1, 1, 2)),     # two CTAs per SM
+    (300, 1, 1, (1, 1, 4)),       # four: a single row
+    (300, 2, 1024, (1, 1, 4)),    # ... the longest slice of this shape
+    (300, 1, 1025, (1, 1, 1)),    # one more row: the wide ring, more CTAs than SMs
+    (2, 8, 2000, (8, 1, 1)),      # clusters of eight at the most
+])
+def test_recalibrate_launch_shapes_against_fp64(cuda_lib, units, G, n_evict, layout):
+    """Every shape that a recomputation takes: O_c within the tolerance of bf16 probabilities, the other rows untouched."""
+    cd = cuda_lib
+    gen = torch.Generator(device="cuda").manual_seed(units + n_evict)
+    rn = lambda *sh: torch.randn(sh, generator=gen, device="cuda")
+    Hq, n_cal, slot = units * G, 3, 1
+    p = cd.make_params(B=1, Hq=Hq, Hkv=units, n_cal=n_cal, cap=1)
+    plan = cd.calidrop_decode_plan(p, 1, n_evict, True)
+    assert (plan.cluster_ctas, plan.clusters_per_unit, plan.ctas_per_sm) == layout
+    q, K, V = (rn(*sh).to(torch.bfloat16) for sh in ((1, Hq, 128), (1, units, n_evict, 128), (1, units, n_evict, 128)))
+    O_c, LSE_c, C_q = rn(1, Hq, n_cal, 128), rn(1, Hq, n_cal), rn(1, Hq, n_cal, 128).to(torch.bfloat16)
+    before = [t.clone() for t in (O_c, LSE_c, C_q)]
+    ws = torch.zeros((cd.calidrop_decode_workspace_bytes(p, n_evict),), dtype=torch.uint8, device="cuda")
+    cd.calidrop_recalibrate(p, q, K, V, n_evict, slot, O_c, LSE_c, C_q, ws)
+    off = cd.calidrop_decode_workspace_status_offset(p)
+    assert int(ws[off:off + 4].view(torch.int32).item()) == 0
+    s = torch.einsum("ugd,utd->ugt", q.view(units, G, 128).double(), K[0].double()) / 128 ** 0.5
+    want = torch.einsum("ugt,utd->ugd", torch.softmax(s, -1), V[0].double()).view(1, Hq, 128)
+    assert (O_c[:, :, slot].double() - want).abs().max() < 2e-2 and (O_c[:, :, slot].double() - want).abs().mean() < 2e-3
+    assert (LSE_c[:, :, slot].double() - torch.logsumexp(s, -1).view(1, Hq)).abs().max() < 1e-3
+    assert torch.equal(C_q[:, :, slot], q)
+    for got, was in zip((O_c, LSE_c, C_q), before):
+        assert torch.equal(got[:, :, ::2], was[:, :, ::2])
+
+
 @pytest.mark.parametrize("B,Hq,Hkv,L,W,budget,n_cal,slot", [
     (1, 4, 2, 600, 16, 80, 1, 0),          # the paper's single calibration query
     (2, 8, 2, 1500, 32, 256, 4, 2),        # G = 4, one of four rows rewritten
-    (1, 7, 1, 20000, 64, 2048, 64, 63),    # one unit, 17952 evicted rows: two clusters per unit
+    (1, 7, 1, 20000, 64, 2048, 64, 63),    # one unit, 17952 evicted rows: several clusters of eight
 ])
 def test_gather_evicted_and_recalibrate(cuda_lib, B, Hq, Hkv, L, W, budget, n_cal, slot):
     cd = cuda_lib

@@ -56,7 +56,7 @@ def test_static_scratch_decode_matches_workspace_decode_twice(cuda_lib):
 
 
 def test_static_scratch_carries_the_partials_of_a_unit_split_over_clusters(cuda_lib):
-    """One unit with 17000 cached rows: the unit is split over two clusters, whose partial results,
+    """One unit with 17000 cached rows: the unit is split over several clusters, whose partial results,
     arrival counter and error word all live in the built-in array.  Two calls in a row on the shared
     array, each checked against the workspace entry point and against the oracle; the device's free
     memory must not move (nothing is allocated or freed by the calls)."""
@@ -70,6 +70,7 @@ def test_static_scratch_carries_the_partials_of_a_unit_split_over_clusters(cuda_
     p = cd.make_params(B=B, Hq=Hq, Hkv=Hkv, L=kv0 + 64, window=8, pool=7, budget=kv0, n_cal=n_cal, cap=cap)
     p.theta1, p.theta2 = 0.7, -1.0
     assert cd.calidrop_decode_workspace_bytes(p, cap) <= cd.STATIC_SCRATCH_BYTES
+    assert cd.calidrop_decode_plan(p, 1, kv0 + 1).clusters_per_unit > 1
     Kk = np.zeros((B, Hkv, cap, D), dtype=np.uint16); Vk = np.zeros_like(Kk)
     Kk[:, :, :kv0] = bits(rng.standard_normal((B, Hkv, kv0, D)))
     Vk[:, :, :kv0] = bits(rng.standard_normal((B, Hkv, kv0, D)))
