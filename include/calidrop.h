@@ -28,8 +28,8 @@
  *   - The library allocates nothing and owns no buffer: all of them, including the workspaces,
  *     belong to the caller.  Two things outlast a call.  (1) calidrop_decode_static's built-in
  *     scratch array (see there).  (2) Small per-thread and per-device tables of derived values:
- *     whether a kernel's shared-memory attribute has been set on a device, the argument block of
- *     the batched decode, and the TMA descriptors of the caches the decode entry points have
+ *     whether a kernel's shared-memory attribute has been set on a device and how many clusters of
+ *     a size the device holds at once, the argument block of the batched decode, and the TMA descriptors of the caches the decode entry points have
  *     seen, keyed by the cache's addresses, capacity and unit count.  A descriptor is a pure
  *     function of its key, so a table entry is never stale and is never dereferenced by the
  *     library itself; freeing a cache needs no call into the library.
@@ -205,7 +205,7 @@ int calidrop_accumulated_scores(const calidrop_params* p, const void* Q_full, co
  *   evict_idx out [B, Hkv, n_evict] i32, n_evict = L - budget: the rows of [0, L - window) that
  *             kept_idx does not list, ascending
  *   K_evict, V_evict out [B, Hkv, n_evict, D] bf16: bit copies of those rows
- *   workspace as for calidrop_compress (its kept bitmap is rebuilt from kept_idx)
+ *   workspace as for calidrop_compress (a long prompt's kept bitmap is rebuilt there from kept_idx)
  * With calib_size = m > 0 the rows are the m calibrated ones (n_evict = min(m, L - budget)): which
  * they are depends on the votes, so `workspace` must then be the workspace of the calidrop_compress
  * call that wrote kept_idx (same parameters), not used for anything else in between; that call

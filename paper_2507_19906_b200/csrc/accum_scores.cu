@@ -366,7 +366,8 @@ size_t rows_bytes(int B, int Hq, int L) { return ((size_t)B * Hq * L * 4 + 255) 
 
 }  // namespace
 
-// Row statistics, the heads' parts, and a word for the error code of the bounded waits.
+// Row statistics, the heads' parts, and a word where the bounded waits leave their code.  No entry point reads it and
+// nothing clears it: a wait that ran out shows as NaN rows.
 size_t accum_scores_workspace_bytes(int B, int Hq, int L) { return 2 * rows_bytes(B, Hq, L) + 256; }
 
 cudaError_t launch_accum_scores(int B, int Hq, int Hkv, int L, float scale2, const void* Q_full, const void* K,

@@ -114,8 +114,8 @@ int device_supported() {
   return major_of[dev] == 10;
 }
 
-// Split-K factor of the decode launch: one CTA per SM at most (a CTA's ring takes most of an SM's
-// shared memory), never fewer than 32 rows per split.
+// The most CTAs that may share a unit: a launch whose units are split has one CTA per SM at most (a CTA's ring then
+// takes most of an SM's shared memory), never fewer than 32 rows per split.
 int decode_nsplit(int units_total, int n_kv) {
   int ns = kDecodeTargetCtas / units_total;
   if (ns < 1) ns = 1;

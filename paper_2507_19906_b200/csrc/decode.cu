@@ -28,8 +28,7 @@
 //
 // A launch moves only tens of MB, so its latency chain matters as much as its bandwidth:
 //   * the launch carries the programmatic-serialisation attribute and the kernel, first thing,
-//     prefetches the head of its K/V slice into L2, ahead of the dependency wait; the ring takes
-//     most of an SM's shared memory, so a launch has one CTA per SM at most;
+//     prefetches the head of its K/V slice into L2, ahead of the dependency wait;
 //   * everything that does not need the predecessor's results (barrier setup, the address
 //     arithmetic of all later loads) is done ahead of the wait as well;
 //   * the similarity work (which needs only q and C_q) runs while the first slots are in flight,
@@ -435,10 +434,10 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
   __syncthreads();  // barriers initialised, s_best cleared: nothing of this needs the predecessor
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
-  // One ring fill: rows [r0 + sb * 64, ...) of K and V into slot sb % 3.  Whole slots take four
-  // 64-row boxes; the ragged last slot takes 16-row boxes for the row groups that hold valid rows,
-  // so a split never pulls more than 15 rows of its neighbour.  Only a 16-row box can reach past
-  // row kv_len: the V map of those boxes ends at kv_len, so such V rows arrive as zeros (a zero
+  // One ring fill into slot sb % kSlots: calibration queries first where they go through the ring, then kSlotRows rows of
+  // K and V.  Whole slots of 64 rows take four 64-row boxes; slots of 32 rows and the ragged last one take 16-row boxes
+  // for the row groups that hold valid rows, so a split never pulls more than 15 rows of its neighbour.  Only a 16-row
+  // box can reach past row kv_len: the V map of those boxes ends at kv_len, so such V rows arrive as zeros (a zero
   // probability times whatever lies in the caller's memory could still be a NaN); the K rows
   // arrive as they lie in memory and their scores are masked.
   auto fill = [&](int sb) {
@@ -478,7 +477,7 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
   };
 
   // ---- (1) cosine similarities of this CTA's calibration rows: four lanes per (head, row) pair,
-  // 72 pairs per pass; the best pair per head goes to s_best while the first slots are in flight
+  // kPairsPerPass pairs per pass; the best pair per head goes to s_best while the first slots are in flight
   auto rho_load = [&](int pi, RhoLoad (&r)[2]) {
     r[0] = RhoLoad{}; r[1] = RhoLoad{};
     if (pi < pairs) {
