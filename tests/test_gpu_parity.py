@@ -7,6 +7,7 @@ outputs within max-abs 2e-2 and mean-abs 2e-3; LSE_c and the output LSE within 1
 import os
 import subprocess
 import sys
+import threading
 
 import numpy as np
 import pytest
@@ -1195,6 +1196,42 @@ def test_accumulated_scores_at_the_edges_of_their_tiles(cuda_lib, B, Hq, Hkv, L)
     torch.testing.assert_close(scores.double(), ref, rtol=2e-5, atol=1e-6)
 
 
+def test_a_thread_may_start_with_a_call_of_the_library(cuda_lib):
+    """A thread that has made no other CUDA call has no current context yet; prompts and decode steps alike."""
+    cd = cuda_lib
+    cfg = wl.small_config()
+    Q, K, V = _inputs(cfg)
+    args = dict(window=8, pool=5, budget=40, n_cal=1, cap=42)
+    want = gpu_compress(Q, K, V, **args)
+    st, p = want.st, want.p
+    dQ, dK, dV = to_dev(Q), to_dev(K), to_dev(V)
+    q = dQ[:, :, -1].contiguous()
+    out = torch.empty((2,) + tuple(q.shape), dtype=torch.bfloat16, device="cuda")
+    K_kept, V_kept = st.K_kept.clone(), st.V_kept.clone()      # caches whose descriptors no call has made yet
+    st2 = cd.alloc_layer_state(p)
+    torch.cuda.synchronize()
+    errors = []
+
+    def work(f):
+        try:
+            f()
+        except Exception as e:
+            errors.append(e)
+
+    def decode(kc, vc, o):
+        cd.calidrop_decode(p, q, None, None, kc, vc, 40, st.O_c, st.LSE_c, st.C_q, o, None, None, st.ws_decode)
+
+    for f in (lambda: cd.calidrop_compress(p, dQ, dK, dV, None, st2.kept_idx, st2.K_kept, st2.V_kept, st2.O_c, st2.LSE_c, st2.C_q,
+                                           st2.ws_compress),
+              lambda: decode(K_kept, V_kept, out[0])):
+        t = threading.Thread(target=work, args=(f,))
+        t.start()
+        t.join()
+    assert not errors, errors
+    decode(st.K_kept, st.V_kept, out[1])
+    assert torch.equal(st2.kept_idx, st.kept_idx) and torch.equal(st2.O_c, st.O_c) and torch.equal(out[0], out[1])
+
+
 def test_first_calls_of_several_threads_with_different_window_sizes(cuda_lib):
     """Threads whose first calls need different amounts of shared memory of the same kernel start at the same moment, in a
     process of its own (what a launch sets up once per device is not set up yet there).  (The two can interleave in
@@ -1216,6 +1253,7 @@ torch.cuda.synchronize()
 start = threading.Barrier(len(states))
 def work(G):
     with torch.cuda.stream(torch.cuda.Stream()):
+        torch.zeros(1, device="cuda")
         start.wait()
         try:
             for _ in range(20): run(*states[G])
