@@ -39,7 +39,7 @@ FALLBACK_HBM_GBS, FALLBACK_BF16_TFLOPS = 6650.0, 1590.0
 # ncu capture late in an eager sequence of launches with the caches left as the launches before it
 # left them (the median launch: a sixth of the cache is still in L2; from flushed caches a launch
 # reads 35.9 MB, its algorithmic bytes); reported only for that workload.
-DECODE_DRAM_TRAFFIC_PER_LAUNCH = 29636608
+DECODE_DRAM_TRAFFIC_PER_LAUNCH = 29683200
 
 
 def load_peaks():

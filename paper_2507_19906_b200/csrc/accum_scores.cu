@@ -17,8 +17,8 @@
 // in the order of their cost, forwards and backwards in turn, so that all CTAs end together.  Roles as in
 // the window scoring: four consumer warpgroups in two pairs on alternate jobs, each group half of the columns, a TMA
 // producer, an MMA-issuing warp.  What bounds it is the exponentials, one per visible logit and pass (see exp2.cuh).
-// Measured at 32 query heads on 8 kv heads, 8192 tokens: 308 + 321 us (501 and 529 thousand cycles, the
-// special-function unit 78 % and 71 % busy), against 1302 + 1313 us with 64 x 64 tiles on mma.sync.
+// Measured at 32 query heads on 8 kv heads, 8192 tokens: 312 + 331 us (506 and 539 thousand cycles, the
+// special-function unit 77 % and 70 % busy), against 1302 + 1313 us with 64 x 64 tiles on mma.sync.
 #include <type_traits>
 
 #include "exp2.cuh"

@@ -190,7 +190,7 @@ calib_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
     // Each of the two warps walks its loop as a whole with one elected lane issuing: the operands of the
     // MMAs are then in uniform registers (a lane in a loop of its own took 100 cycles per MMA).  Together with
     // the packed exponentials of the softmax groups, 32 units x 256 rows x 32768 keys: 212 -> 196 thousand cycles;
-    // calls of 8 units x 8192 keys 50.2 -> 49.0 us.  The operands then bound it: S reads 64 KB and P.V 32 KB of shared
+    // calls of 8 units x 8192 keys 50.2 -> 49.0 us (198 with the exponential that underflows).  The operands then bound it: S reads 64 KB and P.V 32 KB of shared
     // memory per tile while TMA writes 64 KB, 1280 cycles at 128 bytes a cycle against 1024 of the tensor pipe.
     const uint32_t idesc = umma_idesc(128, 128, false, false);     // S: A = Q_c, B = K tile, K-major
     const uint64_t dq = smem_desc_sw128(q_base, 16u, 1024u);

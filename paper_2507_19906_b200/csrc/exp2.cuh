@@ -9,9 +9,10 @@
 // before any rounding and 6.5e-8 rms after it, and sums of exponentials were less exact with it than with ex2.
 // Measured in a bare loop over accumulators in tensor memory, four warps per scheduler, cycles per warp-wide
 // exponential and scheduler (degree 5): ex2 on scalars 8.8, on packed arguments 8.6; with 2, 4, 5, 6, 8, 16 pairs of 16 on
-// the polynomial 7.6, 6.9, 6.6, 6.7, 7.7, 12.0.  In the vote kernel, beside its MMAs (32 units x 32768 keys, thousand
-// cycles): 170 without, 131, 133, 135, 138 with 3, 4, 5, 6 of 16.  Hence 3.  (With unpacked arithmetic the polynomial
-// costs ten issue slots per value, and any share of it loses.)
+// the polynomial 7.6, 6.9, 6.6, 6.7, 7.7, 12.0.  Whole calls, us, with 0, 2, 3, 4 pairs of 16 (degree 6): 32 units x
+// 256 rows x 32768 keys 379, 376, 371, 373; 4 x 448 x 131072 337, 332, 327, 328; accumulated scores of 32 heads x 8192
+// tokens 728, 716, 708, 719; 8 x 128 x 8192 46.7, 46.2, 44.7, 44.5.  Hence 3.  (With unpacked arithmetic the
+// polynomial costs ten issue slots per value, and any share of it loses.)
 #pragma once
 
 #include "common.cuh"

@@ -9,8 +9,8 @@
 // Warp roles: four consumer warpgroups in two pairs read the accumulators out of TMEM (one TMEM
 // lane per thread; pair p drains accumulator buffer p, each of its groups half of the columns), one
 // warp is the TMA producer, one warp allocates TMEM and issues the MMAs.  What bounds both kernels is the
-// exponentials, one per logit; see exp2.cuh.  32 units x 256 rows x 32768 keys: statistics 170 -> 138 thousand
-// cycles (ncu, 92 -> 84 us at the clock the power limit leaves), votes 172 -> 131 (94 -> 80 us), with a share
+// exponentials, one per logit; see exp2.cuh.  32 units x 256 rows x 32768 keys: statistics 170 -> 140 thousand
+// cycles (ncu, 92 -> 85 us at the clock the power limit leaves), votes 172 -> 142 (94 -> 86 us), with a share
 // of the exponentials on the FMA pipe and the work between two jobs cut down; either alone gave little (the
 // polynomial without the other change: 173 and 189 thousand cycles).  Every MMA has N = 256 where the shape allows
 // it: with both operands in shared memory, narrower tiles are limited by operand fetch, not by the tensor pipe.

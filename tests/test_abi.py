@@ -98,9 +98,9 @@ def test_entry_points_of_the_other_eviction_rules_and_the_offload_validate_on_th
     assert lib.calidrop_select_from_scores(pp, ptr, 40, ptr, ptr, 1 << 30, None) == cd.INVALID_ARG
     assert lib.calidrop_select_from_scores(pp, None, 20, ptr, ptr, 1 << 30, None) == cd.INVALID_ARG
     assert lib.calidrop_select_from_scores(pp, ptr, 20, ptr, ptr, 16, None) == cd.WORKSPACE_TOO_SMALL
-    # accumulated scores: workspace = 4 B Hq L bytes, rounded up to 256
+    # accumulated scores: the workspace holds row statistics and parts, 4 B Hq L bytes each at the least
     need = cd.calidrop_accumulated_scores_workspace_bytes(p)
-    assert need >= 4 * 1 * 4 * 300 and need % 256 == 0
+    assert need >= 2 * 4 * 1 * 4 * 300 and need % 256 == 0
     assert lib.calidrop_accumulated_scores(pp, None, ptr, ptr, ptr, need, None) == cd.INVALID_ARG
     assert lib.calidrop_accumulated_scores(pp, ptr, ptr, ptr, ptr, need - 256, None) == cd.WORKSPACE_TOO_SMALL
     # calibration size below -1 is no setting
