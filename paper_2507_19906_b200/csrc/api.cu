@@ -263,6 +263,14 @@ int calidrop_compress(const calidrop_params* p, const void* Q_obs, const void* K
   // The contractions run on the tensor cores whenever the tiles cover the shape; the scalar
   // kernels remain for the rest (more than 512 window rows per kv head, budget >= L).
   const bool tc_path = score_tc_supported(g);
+  const GatherArgs ga{(const uint4*)K, (const uint4*)V, kept_idx, (uint4*)K_kept, (uint4*)V_kept,
+                      g.L, g.n_kept, g.cap, g.units};
+  if (tc_path) {   // short prompts: the whole step in one kernel
+    bool taken = false;
+    cudaError_t ec = launch_compress_cluster(g, ws, Q_obs, K, V, lse_obs, wsp, kept_idx, O_c, LSE_c, C_q, ga, &taken, st);
+    if (ec != cudaSuccess) return cuda_fail(ec);
+    if (taken) return CALIDROP_OK;
+  }
   // the error word is cleared by the call's first tensor-core kernel, where it has one
   cudaError_t e = tc_path ? cudaSuccess : cudaMemsetAsync(wsp + ws.status, 0, 4, st);
   if (e != cudaSuccess) return cuda_fail(e);
@@ -291,8 +299,6 @@ int calidrop_compress(const calidrop_params* p, const void* Q_obs, const void* K
     e = launch_gather(g, K, V, kept_idx, K_kept, V_kept, st);
     if (e != cudaSuccess) return cuda_fail(e);
   }
-  const GatherArgs ga{(const uint4*)K, (const uint4*)V, kept_idx, (uint4*)K_kept, (uint4*)V_kept,
-                      g.L, g.n_kept, g.cap, g.units};
   if (g.sized && g.n_calib == 0)
     e = launch_calib_none(g, Q_obs, O_c, LSE_c, C_q, st);
   else

@@ -16,7 +16,7 @@ import torch
 import oracle
 from paper_2507_19906_b200 import workload as wl
 
-from gpu_util import (assert_close_lse, assert_close_out, compare_compress, decode_steps_compare,
+from gpu_util import (assert_close_lse, assert_close_out, check_kept_sets, compare_compress, decode_steps_compare,
                       gpu_compress, to_bits, to_dev)
 
 pytestmark = pytest.mark.gpu
@@ -313,6 +313,64 @@ def test_calibration_size(cuda_lib, calib_size):
     q, kn, vn = wl.gen_decode_inputs(cfg, Q, steps=3)
     decode_steps_compare(g, ref, q, kn, vn, steps=3)
 
+
+ONE_KERNEL = [
+    # B, Hq, Hkv, L, W, pool, budget, n_cal, calib_size, kernels (1: the cluster kernel; else the separate ones)
+    (1, 1, 1, 136, 8, 7, 40, 1, 0, 1),           # two CTAs, the second has window rows only
+    (1, 2, 1, 128 * 3 + 33, 32, 1, 70, 32, 0, 1),   # 64 window rows (two copies of them on the lanes), one candidate in the last tile
+    (1, 5, 1, 2048, 8, 9, 200, 8, 0, 1),         # sixteen CTAs of a tile, 40 rows, a pool without a kernel of its own
+    (2, 5, 1, 2300, 24, 129, 300, 24, 500, 1),   # 120 rows, the widest pool that the kernel takes, a calibration size
+    (1, 4, 1, 900, 32, 5, 899, 32, 0, 1),        # a single evicted candidate, 128 calibration rows
+    (3, 8, 8, 1300, 16, 7, 17, 1, 3, 1),         # 24 units, 16 rows; one candidate kept, three calibrated
+    (1, 100, 100, 300, 8, 7, 50, 8, 0, 1),       # one CTA to a unit
+    (1, 100, 100, 128 * 17 + 5, 8, 5, 60, 2, 40, 1),   # ... of 18 tiles: the groups take tiles of their own in the votes
+    (1, 3, 1, 900, 64, 7, 200, 3, 0, 5),         # 192 rows: the separate kernels, the row LSE combined by the votes
+    (1, 100, 100, 900, 128, 131, 300, 2, 0, 5),  # a pool wider than the halo
+]
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,L,W,pool,budget,n_cal,calib_size,kernels", ONE_KERNEL)
+@pytest.mark.parametrize("octaves", [None, 0, 24, -40])
+def test_compress_in_one_kernel(cuda_lib, B, Hq, Hkv, L, W, pool, budget, n_cal, calib_size, kernels, octaves):
+    """Units that a cluster holds take one kernel.  With `octaves` the caller supplies the row LSE, less that many factors of
+    two: the votes then lie inside, above and below the range that the first selection pass resolves.  Rounding the
+    shifted row LSE moves a vote by 2^-18 of itself at most (|lse| below 64), the same for all keys of a row."""
+    from paper_2507_19906_b200 import binding as cd
+    cfg = wl.small_config(B=B, Hq=Hq, Hkv=Hkv, L=L, window=W, pool=pool, budget=budget, steps=1, n_sink=2,
+                          n_heavy=max(1, L // 50))
+    Q, K, V = _inputs(cfg)
+    m = None if calib_size == 0 else calib_size
+    orc = oracle.compress(Q, K, V, window=W, pool=pool, budget=budget, n_cal=n_cal, cap=budget, calib_size=m)
+    p = cd.make_params(B=B, Hq=Hq, Hkv=Hkv, L=L, window=W, pool=pool, budget=budget, n_cal=n_cal, cap=budget,
+                       calib_size=calib_size)
+    st = cd.alloc_layer_state(p)
+    dQ, dK, dV = to_dev(Q), to_dev(K), to_dev(V)
+    lse = None
+    if octaves is not None:
+        lse = torch.from_numpy((orc.row_lse - octaves * np.log(2.0)).astype(np.float32)).cuda()
+    before = cd.calidrop_launch_count()
+    cd.calidrop_compress(p, dQ, dK, dV, lse, st.kept_idx, st.K_kept, st.V_kept, st.O_c, st.LSE_c, st.C_q, st.ws_compress)
+    torch.cuda.synchronize()
+    launched = cd.calidrop_launch_count() - before
+    assert launched == kernels - (octaves is not None and kernels > 1)
+    lay = cd.calidrop_compress_workspace_layout(p)
+    assert int(st.ws_compress[lay.status_offset:lay.status_offset + 4].view(torch.int32).item()) == 0
+    ws = lambda off, ref: st.ws_compress[off:off + 4 * ref.size].view(torch.float32).cpu().numpy().reshape(ref.shape)
+    scale, rtol = 2.0 ** (octaves or 0), 2e-5 if not octaves else 4e-5
+    np.testing.assert_allclose(ws(lay.vote_offset, orc.vote), orc.vote * scale, rtol=rtol, atol=1e-9 * scale)
+    np.testing.assert_allclose(ws(lay.pooled_offset, orc.pooled), orc.pooled * scale, rtol=rtol, atol=1e-9 * scale)
+    if octaves is None:
+        np.testing.assert_allclose(ws(lay.row_lse_offset, orc.row_lse), orc.row_lse, atol=2e-5)
+    kept = st.kept_idx.cpu().numpy()
+    swaps = check_kept_sets(kept, orc)
+    np.testing.assert_array_equal(to_bits(st.C_q), orc.C_q)
+    for b in range(B):
+        for h in range(Hkv):
+            np.testing.assert_array_equal(to_bits(st.K_kept)[b, h], K[b, h][kept[b, h]])
+            np.testing.assert_array_equal(to_bits(st.V_kept)[b, h], V[b, h][kept[b, h]])
+    if swaps == 0:   # (neither depends on the shift)
+        assert_close_lse(st.LSE_c.cpu().numpy(), orc.LSE_c, "LSE_c")
+        assert_close_out(st.O_c.cpu().numpy(), orc.O_c, "O_c")
 
 def test_supplied_row_lse_matches_self_computed(cuda_lib):
     cfg = wl.small_config(B=1, Hq=4, Hkv=2, L=400, window=16, pool=7, budget=64)
