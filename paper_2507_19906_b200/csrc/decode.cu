@@ -32,7 +32,7 @@
 //   * everything that does not need the predecessor's results (barrier setup, the address
 //     arithmetic of all later loads) is done ahead of the wait as well;
 //   * the similarity work (which needs only q and C_q) runs while the first slots are in flight,
-//     and the cluster exchanges each CTA's best (similarity, row) pair early; the producer warp,
+//     and each CTA's best (similarity, row) pairs are pushed to the others early; the producer warp,
 //     idle once the last slot is on its way, settles the calibration row meanwhile, and the chosen
 //     O_c elements are fetched while the partial outputs are combined;
 //   * the cache stream carries an evict-first L2 hint, the calibration state an evict-last hint.
@@ -207,6 +207,12 @@ __device__ __forceinline__ void push_f32x2(uint32_t remote, float x, float y, ui
                : "memory");
 }
 
+__device__ __forceinline__ void push_u64(uint32_t remote, unsigned long long x, uint32_t remote_bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.u64 [%0], %1, [%2];" ::"r"(remote), "l"(x),
+               "r"(remote_bar)
+               : "memory");
+}
+
 struct RhoLoad {
   uint4 q0, q1, c0, c1;
 };
@@ -240,9 +246,6 @@ __device__ __forceinline__ float rank_key_value(unsigned long long k) {
   return __uint_as_float(u);
 }
 
-__device__ __forceinline__ void cluster_arrive() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-}
 __device__ __forceinline__ void cluster_wait() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
@@ -308,6 +311,8 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
   __shared__ __align__(8) unsigned long long s_full[kSlots][2], s_empty[kSlots][2];
   __shared__ unsigned long long s_best[kMaxG];     // best (similarity, row) of this CTA's calibration rows
   __shared__ unsigned long long s_bestall[kMaxG];  // ... of the whole cluster
+  __shared__ __align__(8) unsigned long long s_bestx[S::kClu][kMaxG];   // ... of every CTA, pushed by them
+  __shared__ __align__(8) unsigned long long s_bestbar;
   __shared__ __align__(16) float s_xpart[kMaxG * kD];  // [source split][head][dim of this CTA's slice]
   __shared__ __align__(16) float s_xml[S::kClu][kMaxG][2];   // [source split][head] (max, sum)
   __shared__ __align__(8) unsigned long long s_push;  // counts the bytes pushed to this CTA by the cluster
@@ -392,8 +397,10 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
     // every CTA of the cluster (this one included) pushes its partial of this CTA's slice and its
     // (max, sum) pairs here: G * dpc * 4 + G * 8 bytes each
     mbar_init(smem_u32(&s_push), 1);
+    mbar_init(smem_u32(&s_bestbar), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     if (!kOne) mbar_expect_tx(smem_u32(&s_push), (uint32_t)(nsplit * a.G * (kD / nsplit * 4 + 8)));
+    if (!kOne && !RECAL) mbar_expect_tx(smem_u32(&s_bestbar), (uint32_t)(nsplit * a.G * 8));
     asm volatile("prefetch.tensormap [%0];" ::"l"(&TM.k64) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&TM.v64) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&TM.k16) : "memory");
@@ -432,6 +439,8 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
   const float* lsec_base = P.LSE_c + (size_t)(hq0 + eg) * a.n_cal;
   asm volatile("" ::"l"(qp0), "l"(cp0), "l"(qr0), "l"(oc_base), "l"(lsec_base), "r"(pg0), "r"(pc0));
   __syncthreads();  // barriers initialised, s_best cleared: nothing of this needs the predecessor
+  // (A) arrived at once, waited for ahead of a warp's first push: every CTA of the cluster runs, its barriers are set up
+  if (!kOne) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
   // One ring fill into slot sb % kSlots: calibration queries first where they go through the ring, then kSlotRows rows of
@@ -530,11 +539,8 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
     __syncwarp();
   }
   // The similarities are finished by the producer warp at once and by a stream warp after its first
-  // slot, whose data is already there when the query arrives.  (A) then says this CTA's s_best is
-  // final.  Publishing it to the cluster takes a release fence, which is slow while the stream is
-  // in flight; the stream warps therefore only hand their updates to the producer warp through a
-  // CTA barrier and arrive relaxed, and the producer warp, which has time, makes the one release
-  // for the CTA.
+  // slot, whose data is already there when the query arrives.  The stream warps then hand their updates of s_best to the
+  // producer warp through a CTA barrier, and that one, which has time, pushes them to the CTAs of the cluster.
   auto rho_rest = [&]() {
     if (kOne) return;
     rho_finish(pi0, pg0, pc0, rl);
@@ -543,10 +549,7 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
       rho_load(pi, rl);
       rho_finish(pi, pi < pairs ? pi % a.G : 0, c_begin + (pi < pairs ? pi / a.G : 0), rl);
     }
-    if (warp != kStreamWarps) {
-      asm volatile("barrier.cta.arrive 1, %0;" ::"n"(kThreads) : "memory");
-      asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-    }
+    if (warp != kStreamWarps) asm volatile("barrier.cta.arrive 1, %0;" ::"n"(kThreads) : "memory");
   };
   // One CTA per unit: the similarities of a slot of calibration queries, a row per lane.  (Loaded through registers, four
   // lanes to a row, the passes were a chain of round trips that held the stream up: 73 instead of 60 us for 2048 caches
@@ -604,17 +607,25 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
     // calibration row (best similarity over the cluster, ties to the largest row index) while the
     // stream warps are still busy
     if (!kOne) asm volatile("barrier.cta.sync 1, %0;" ::"n"(kThreads) : "memory");  // the stream warps' updates of s_best
-    if (!kOne) {
-      cluster_arrive();  // (A) with the release for the whole CTA
-      cluster_wait();    //     every CTA's s_best can be read
-    }
-    if (!kOne && lane < a.G) {
-      unsigned long long best = 0ull;
-      for (int s = 0; s < nsplit; ++s) {
-        const unsigned long long k = *cluster.map_shared_rank(&s_best[lane], s);
-        best = k > best ? k : best;
+    if (!kOne) cluster_wait();   // (A)
+    if (!kOne && !RECAL) {
+      // Pushed like the partial outputs below.  (Published by a release of the whole CTA at a cluster barrier and read from
+      // the peers, this took a microsecond of fence while copies are in flight and a chain of remote loads: 8 units of 129
+      // rows 4.96 -> 4.5 us a launch, longer streams cover it.)
+      for (int i = lane; i < a.G * nsplit; i += 32) {
+        const int g = i % a.G, r = i / a.G;
+        push_u64(cluster_addr(smem_u32(&s_bestx[split][g]), r), s_best[g], cluster_addr(smem_u32(&s_bestbar), r));
       }
-      s_bestall[lane] = best;
+      mbar_wait_sit_out(smem_u32(&s_bestbar), 0, abort_flag, a.status, 0x500u);
+      if (lane < a.G) {
+        unsigned long long best = 0ull;
+#pragma unroll
+        for (int s = 0; s < S::kClu; ++s) {
+          const unsigned long long k = s < nsplit ? s_bestx[s][lane] : 0ull;
+          best = k > best ? k : best;
+        }
+        s_bestall[lane] = best;
+      }
     }
   } else {
     // ---- (3) stream warps
@@ -697,7 +708,7 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
   }
 
   // ---- (4) the chosen O_c elements and LSE_c start their way while the partials are combined
-  if (!kOne && warp < kStreamWarps) cluster_wait();  // (A): the stream warps only pass it
+  if (!kOne && warp < kStreamWarps) cluster_wait();  // (A)
   __syncthreads();  // all warps are done with the ring: reuse it for the combine
   // the common case has one output element per thread at most: its O_c element and LSE_c are
   // loaded now and arrive while the partials are combined
@@ -798,10 +809,9 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
     }
   }
   // (B) everything pushed to this CTA has arrived when its byte count is complete.  No cluster
-  // barrier: a CTA waits for its own data only, and it cannot leave before the others have read its
-  // s_best, because their pushes, which it waits for, come after those reads.  That argument needs
-  // the wait to be sat out: a CTA whose earlier wait ran out (abort flag raised) must not skip it,
-  // or its peers, which always reach their pushes, would read and write the shared memory of a
+  // barrier: a CTA waits for its own data only, and nothing else of a peer touches its shared memory.
+  // The wait has to be sat out: a CTA whose earlier wait ran out (abort flag raised) must not skip it,
+  // or its peers, which always reach their pushes, would write to the shared memory of a
   // CTA that has left.  Only the wait's own time limit remains as the way out.
   mbar_wait_sit_out(smem_u32(&s_push), 0, abort_flag, a.status, 0x300u);
 
