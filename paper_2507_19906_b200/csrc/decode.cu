@@ -207,6 +207,12 @@ __device__ __forceinline__ void push_f32x2(uint32_t remote, float x, float y, ui
                : "memory");
 }
 
+__device__ __forceinline__ void push_f32x4(uint32_t remote, float4 v, uint32_t remote_bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(
+                   remote),
+               "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(remote_bar)
+               : "memory");
+}
 __device__ __forceinline__ void push_u64(uint32_t remote, unsigned long long x, uint32_t remote_bar) {
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.u64 [%0], %1, [%2];" ::"r"(remote), "l"(x),
                "r"(remote_bar)
@@ -433,8 +439,10 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
   const int dpc = kD / nsplit, lg_dpc = 31 - __clz(dpc);  // nsplit is a power of two
   const int n_items = a.G * dpc;
   const bool single = nclu == 1;
-  const bool early = !kOne && !RECAL && single && n_items <= kThreads;  // one output element per thread at most
-  const int eg = min(tid >> lg_dpc, a.G - 1), ed = split * dpc + (tid & (dpc - 1));
+  // threads that share an output element in the finish, each with up to four splits: as many as there are threads for
+  const int lg_sub = nsplit >= 4 && n_items * 4 <= kThreads ? 2 : nsplit >= 2 && n_items * 2 <= kThreads ? 1 : 0;
+  const bool early = !kOne && !RECAL && single && n_items << lg_sub <= kThreads;  // one output element per thread at most
+  const int eg = min(tid >> lg_sub >> lg_dpc, a.G - 1), ed = split * dpc + ((tid >> lg_sub) & (dpc - 1));
   const float* oc_base = P.O_c + (size_t)(hq0 + eg) * a.n_cal * kD + ed;
   const float* lsec_base = P.LSE_c + (size_t)(hq0 + eg) * a.n_cal;
   asm volatile("" ::"l"(qp0), "l"(cp0), "l"(qr0), "l"(oc_base), "l"(lsec_base), "r"(pg0), "r"(pc0));
@@ -612,9 +620,14 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
       // Pushed like the partial outputs below.  (Published by a release of the whole CTA at a cluster barrier and read from
       // the peers, this took a microsecond of fence while copies are in flight and a chain of remote loads: 8 units of 129
       // rows 4.96 -> 4.5 us a launch, longer streams cover it.)
-      for (int i = lane; i < a.G * nsplit; i += 32) {
-        const int g = i % a.G, r = i / a.G;
-        push_u64(cluster_addr(smem_u32(&s_bestx[split][g]), r), s_best[g], cluster_addr(smem_u32(&s_bestbar), r));
+      if ((lane & 7) < a.G) {
+        const unsigned long long mine = s_best[lane & 7];
+#pragma unroll
+        for (int r0 = 0; r0 < S::kClu; r0 += 4) {
+          const int r = r0 + (lane >> 3);
+          if (r < nsplit)
+            push_u64(cluster_addr(smem_u32(&s_bestx[split][lane & 7]), r), mine, cluster_addr(smem_u32(&s_bestbar), r));
+        }
       }
       mbar_wait_sit_out(smem_u32(&s_bestbar), 0, abort_flag, a.status, 0x500u);
       if (lane < a.G) {
@@ -722,7 +735,7 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
     }
   }
   float lse_c_early = 0.f, oc_early = 0.f;
-  if (early && tid < n_items) {
+  if (early && tid < n_items << lg_sub) {
     const unsigned cs = (unsigned)(s_bestall[eg] & 0xffffffffull);
     lse_c_early = ldg_keep(lsec_base + cs, pol_keep);
     oc_early = ldg_keep(oc_base + (size_t)cs * kD, pol_keep);
@@ -780,33 +793,28 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
     }
     return;
   }
-  // the stream warps' threads: thread t owns dimensions 2 (t & 63) and 2 (t & 63) + 1 of every kStreamWarps / 2-th head, so the
-  // scale factors of the eight warps are worked out once for two elements, which go to their owner
-  // in one 8-byte store; all loads are done before the pushes (stores through generic pointers,
-  // which the compiler will not move loads across)
-  if (tid < kStreamWarps * 32) {
-    const int d0 = 2 * (tid & 63);
-    for (int g = tid >> 6; g < a.G; g += kStreamWarps / 2) {
-      float mw[kStreamWarps], M = -INFINITY;
+  // A warp per head, four elements a lane: the scale factors of the stream warps are worked out once for four elements,
+  // which go to their owner in one 16-byte store; all loads are done before the pushes (stores through generic pointers,
+  // which the compiler will not move loads across).
+  if (warp < min(kStreamWarps, a.G)) {
+    const int g = warp, d0 = 4 * lane;
+    float mw[kStreamWarps], M = -INFINITY, Lsum = 0.f;
 #pragma unroll
-      for (int w = 0; w < kStreamWarps; ++w) { mw[w] = wml[(w * kMaxG + g) * 2]; M = fmaxf(M, mw[w]); }
-      float Lsum = 0.f, acc0 = 0.f, acc1 = 0.f;
+    for (int w = 0; w < kStreamWarps; ++w) { mw[w] = wml[(w * kMaxG + g) * 2]; M = fmaxf(M, mw[w]); }
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-      for (int w = 0; w < kStreamWarps; ++w) {
-        const float sc = mw[w] > -INFINITY ? ex2_approx(mw[w] - M) : 0.f;
-        const float2 wv = *reinterpret_cast<const float2*>(wo + (w * kMaxG + g) * kWoStride + d0);
-        Lsum = fmaf(wml[(w * kMaxG + g) * 2 + 1], sc, Lsum);
-        acc0 = fmaf(wv.x, sc, acc0);
-        acc1 = fmaf(wv.y, sc, acc1);
-      }
-      const int own = d0 >> lg_dpc;  // dpc is even: both dimensions have the same owner
-      push_f32x2(cluster_addr(smem_u32(s_xpart + (split * kMaxG + g) * dpc + (d0 - own * dpc)), own), acc0, acc1,
-                 cluster_addr(smem_u32(&s_push), own));
-      if ((tid & 63) < nsplit) {  // the (max, sum) pair of this split goes to every CTA of the cluster
-        push_f32x2(cluster_addr(smem_u32(&s_xml[split][g][0]), tid & 63), M, Lsum,
-                   cluster_addr(smem_u32(&s_push), tid & 63));
-      }
+    for (int w = 0; w < kStreamWarps; ++w) {
+      const float sc = mw[w] > -INFINITY ? ex2_approx(mw[w] - M) : 0.f;
+      const float4 v = *reinterpret_cast<const float4*>(wo + (w * kMaxG + g) * kWoStride + d0);
+      Lsum = fmaf(wml[(w * kMaxG + g) * 2 + 1], sc, Lsum);
+      acc.x = fmaf(v.x, sc, acc.x); acc.y = fmaf(v.y, sc, acc.y);
+      acc.z = fmaf(v.z, sc, acc.z); acc.w = fmaf(v.w, sc, acc.w);
     }
+    const int own = d0 >> lg_dpc;  // dpc is a multiple of eight: the four dimensions have the same owner
+    push_f32x4(cluster_addr(smem_u32(s_xpart + (split * kMaxG + g) * dpc + (d0 - own * dpc)), own), acc,
+               cluster_addr(smem_u32(&s_push), own));
+    if (lane < nsplit)  // the (max, sum) pair of this split goes to every CTA of the cluster
+      push_f32x2(cluster_addr(smem_u32(&s_xml[split][g][0]), lane), M, Lsum, cluster_addr(smem_u32(&s_push), lane));
   }
   // (B) everything pushed to this CTA has arrived when its byte count is complete.  No cluster
   // barrier: a CTA waits for its own data only, and nothing else of a peer touches its shared memory.
@@ -817,27 +825,37 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
 
   // ---- (6) finish: reduce the splits for this CTA's output slice (local data only from here on,
   // so no CTA has to wait for another before it leaves)
+  // A split after another in one thread, the sixteen of a cluster took 2200 cycles, most of them for fetching 250 instructions
+  // that run once per launch; with four threads to an element it is a quarter of the code and of the chain.
   const int lu = layer * a.units + unit;
-  for (int item = tid; item < n_items; item += kThreads) {
+  constexpr int kMine = 4;   // splits of a thread at most: elements get fewer threads only where there are few splits
+  const int sub = tid & ((1 << lg_sub) - 1);
+  for (int item = tid >> lg_sub; item < n_items; item += kThreads >> lg_sub) {   // (a warp's items are in range all or none)
     const int g = item >> lg_dpc, dl = item & (dpc - 1), d = split * dpc + dl;
     const int hq = hq0 + g;
     const unsigned long long best = s_bestall[g];
-    float ms[S::kClu], ls[S::kClu], xs[S::kClu], M = -INFINITY;
+    float ms[kMine], ls[kMine], xs[kMine], M = -INFINITY;
 #pragma unroll
-    for (int s = 0; s < S::kClu; ++s) {  // all loads first
+    for (int k = 0; k < kMine; ++k) {  // all loads first
+      const int s = (k << lg_sub) + sub;
       const bool on = s < nsplit;
-      ms[s] = on ? s_xml[s][g][0] : -INFINITY;
-      ls[s] = on ? s_xml[s][g][1] : 0.f;
-      xs[s] = on ? s_xpart[(s * kMaxG + g) * dpc + dl] : 0.f;
-      M = fmaxf(M, ms[s]);
+      ms[k] = on ? s_xml[s][g][0] : -INFINITY;
+      ls[k] = on ? s_xml[s][g][1] : 0.f;
+      xs[k] = on ? s_xpart[(s * kMaxG + g) * dpc + dl] : 0.f;
+      M = fmaxf(M, ms[k]);
     }
+    if (lg_sub > 0) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 1));
+    if (lg_sub > 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 2));
     float Lsum = 0.f, acc = 0.f;
 #pragma unroll
-    for (int s = 0; s < S::kClu; ++s) {
-      const float sc = ms[s] > -INFINITY ? ex2_approx(ms[s] - M) : 0.f;
-      Lsum = fmaf(ls[s], sc, Lsum);
-      acc = fmaf(xs[s], sc, acc);
+    for (int k = 0; k < kMine; ++k) {
+      const float sc = ms[k] > -INFINITY ? ex2_approx(ms[k] - M) : 0.f;
+      Lsum = fmaf(ls[k], sc, Lsum);
+      acc = fmaf(xs[k], sc, acc);
     }
+    if (lg_sub > 0) { Lsum += __shfl_xor_sync(0xffffffffu, Lsum, 1); acc += __shfl_xor_sync(0xffffffffu, acc, 1); }
+    if (lg_sub > 1) { Lsum += __shfl_xor_sync(0xffffffffu, Lsum, 2); acc += __shfl_xor_sync(0xffffffffu, acc, 2); }
+    if (sub != 0) continue;
     if (single) {
       if constexpr (RECAL) {
         recal_store(a, P, hq, d, acc, M, Lsum);
