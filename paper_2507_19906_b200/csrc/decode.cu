@@ -72,11 +72,18 @@ using ShapeNarrow = Shape<3, 32, 4, 1>;          // more than that: 48 KB, four 
 constexpr int kWoStride = kD + 4;  // row stride of the per-warp partial outputs: heads land in distinct banks
 constexpr long long kWaitLimitCycles = 2000000000ll;  // about a second: a wait this long has failed
 
-// Byte offset of 16-byte chunk `chunk` (0..15) of row `row` inside the K or V part of a
-// slot: two column halves, each a [rows][128 bytes] plane in the 128-byte swizzle TMA writes.
+// The K or the V part of a slot, as the copies leave it: the two halves of the columns as planes of 128-byte lines in the
+// 128-byte swizzle, over the whole slot where one copy brings it (64 rows), else a pair of planes for every 16 rows.
+struct Planes {
+  uint32_t block, half;   // bytes from a 16-row block to the next, and from the first half of a block to its second
+};
 template <class S>
-__device__ __forceinline__ uint32_t plane_off(int row, int chunk) {
-  return (uint32_t)((chunk >> 3) * S::kPlaneBytes + row * 128 + (((chunk & 7) ^ (row & 7)) << 4));
+__device__ __forceinline__ Planes planes_of(bool whole) {
+  return whole ? Planes{kBlkRows * 128, S::kPlaneBytes} : Planes{2 * kBlkRows * 128, kBlkRows * 128};
+}
+// Byte offset of 16-byte chunk `chunk` (0..15) of row `row` (0..15) of a block.
+__device__ __forceinline__ uint32_t block_off(const Planes& p, int row, int chunk) {
+  return (uint32_t)(chunk >> 3) * p.half + (uint32_t)(row * 128 + (((chunk & 7) ^ (row & 7)) << 4));
 }
 
 __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t x) {
@@ -150,12 +157,13 @@ __device__ __forceinline__ bool mbar_wait_sit_out(uint32_t bar, uint32_t parity,
   }
   return true;
 }
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1,
-                                            int c2, uint64_t pol) {
+// Rows from row on of a unit, both halves of the head dimension.
+__device__ __forceinline__ void tma_load_rows(uint32_t dst, const CUtensorMap* map, uint32_t bar, int row, int unit,
+                                              uint64_t pol) {
   asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint "
-      "[%0], [%1, {%3, %4, %5}], [%2], %6;"
-      ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "l"(pol)
+      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint "
+      "[%0], [%1, {%3, %4, %5, %3}], [%2], %6;"
+      ::"r"(dst), "l"(map), "r"(bar), "r"(0), "r"(row), "r"(unit), "l"(pol)
       : "memory");
 }
 
@@ -428,8 +436,9 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
   // finish, is done here: a single warp runs a dependent chain of scalar instructions at a few
   // cycles each, and at this kernel's scale a hundred of them behind the wait are a measurable
   // part of a launch (0.4 us each for the similarity loads and for the O_c loads, measured).
-  constexpr int kPairsPerPass = kThreads / 4;
-  const int pairs = n_c * a.G;
+  // (the stream warps': the producer has the first fills to send off)
+  constexpr int kPairsPerPass = kStreamWarps * 8;
+  const int pairs = warp == kStreamWarps ? 0 : n_c * a.G;
   const int sub4 = tid & 3;
   const int pi0 = tid >> 2;
   const int pg0 = pi0 < pairs ? pi0 % a.G : 0, pc0 = c_begin + (pi0 < pairs ? pi0 / a.G : 0);
@@ -452,7 +461,7 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
   // One ring fill into slot sb % kSlots: calibration queries first where they go through the ring, then kSlotRows rows of
-  // K and V.  Whole slots of 64 rows take four 64-row boxes; slots of 32 rows and the ragged last one take 16-row boxes
+  // K and V.  Whole slots of 64 rows take a 64-row box each; slots of 32 rows and the ragged last one take 16-row boxes
   // for the row groups that hold valid rows, so a split never pulls more than 15 rows of its neighbour.  Only a 16-row
   // box can reach past row kv_len: the V map of those boxes ends at kv_len, so such V rows arrive as zeros (a zero
   // probability times whatever lies in the caller's memory could still be a NaN); the K rows
@@ -476,19 +485,15 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
     const int nrows = min(kSlotRows, r1 - row0);
     if (kSlotRows == kWideRows && nrows == kSlotRows) {
       mbar_expect_tx(bar, kSlotBytes);
-      tma_load_3d(dst, &TM.k64, bar, 0, row0, unit, pol_stream);
-      tma_load_3d(dst + kPlaneBytes, &TM.k64, bar, 64, row0, unit, pol_stream);
-      tma_load_3d(dst + 2 * kPlaneBytes, &TM.v64, bar, 0, row0, unit, pol_stream);
-      tma_load_3d(dst + 3 * kPlaneBytes, &TM.v64, bar, 64, row0, unit, pol_stream);
+      tma_load_rows(dst, &TM.k64, bar, row0, unit, pol_stream);
+      tma_load_rows(dst + 2 * kPlaneBytes, &TM.v64, bar, row0, unit, pol_stream);
     } else {
       const int nb = (nrows + kBlkRows - 1) / kBlkRows;
       mbar_expect_tx(bar, (uint32_t)nb * 4u * kBlkRows * 128u);
       for (int j = 0; j < nb; ++j) {
-        const uint32_t dj = dst + j * kBlkRows * 128;
-        tma_load_3d(dj, &TM.k16, bar, 0, row0 + j * kBlkRows, unit, pol_stream);
-        tma_load_3d(dj + kPlaneBytes, &TM.k16, bar, 64, row0 + j * kBlkRows, unit, pol_stream);
-        tma_load_3d(dj + 2 * kPlaneBytes, &TM.v16, bar, 0, row0 + j * kBlkRows, unit, pol_stream);
-        tma_load_3d(dj + 3 * kPlaneBytes, &TM.v16, bar, 64, row0 + j * kBlkRows, unit, pol_stream);
+        const uint32_t dj = dst + j * 2 * kBlkRows * 128;
+        tma_load_rows(dj, &TM.k16, bar, row0 + j * kBlkRows, unit, pol_stream);
+        tma_load_rows(dj + 2 * kPlaneBytes, &TM.v16, bar, row0 + j * kBlkRows, unit, pol_stream);
       }
     }
   };
@@ -652,21 +657,22 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
       if (kOne && sb < n_cf) {
         if (!RECAL && ok && mbar_wait(smem_u32(&s_qfull), 0, abort_flag, a.status, 0x400u)) rho_slot(s, sb, sub);
       } else if (ok && row_base < r1) {
-        const uint32_t sK = ring + s * kSlotBytes;
+        const Planes pl = planes_of<S>(kSlotRows == kWideRows && r1 - r0 - (sb - n_cf) * kSlotRows >= kSlotRows);
+        const uint32_t sK = ring + s * kSlotBytes + sub * pl.block;   // this warp's block
         const uint32_t sV = sK + 2 * kPlaneBytes;
         // D1: the warp that meets row kv_len takes it from k_new / v_new (the cache row has not
         // been written yet: what arrived for it is stale) and appends it to the cache
         if (a.has_new && a.kv_len >= row_base && a.kv_len < row_base + kBlkRows) {
           const int chunk = lane & 15;
-          const int rs = a.kv_len - (r0 + (sb - n_cf) * kSlotRows);  // row inside the slot
+          const int rs = a.kv_len - row_base;  // row inside the block
           const unsigned char* src = (const unsigned char*)(lane < 16 ? P.k_new : P.v_new) +
                                      (size_t)unit * kRowBytes + chunk * 16;
           const uint4 v = *reinterpret_cast<const uint4*>(src);
           unsigned char* dstg = (unsigned char*)(lane < 16 ? P.K : P.V) +
                                 ((size_t)unit * a.cap + a.kv_len) * kRowBytes + chunk * 16;
           *reinterpret_cast<uint4*>(dstg) = v;
-          *reinterpret_cast<uint4*>(ring_ptr + s * kSlotBytes + (lane < 16 ? 0 : 2 * kPlaneBytes) +
-                                    plane_off<S>(rs, chunk)) = v;
+          *reinterpret_cast<uint4*>(ring_ptr + s * kSlotBytes + sub * pl.block + (lane < 16 ? 0 : 2 * kPlaneBytes) +
+                                    block_off(pl, rs, chunk)) = v;
           __syncwarp();
         }
         // S^T: two accumulators (even and odd k-steps) halve the dependent chain
@@ -674,7 +680,7 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
 #pragma unroll
         for (int kk = 0; kk < kD / 16; ++kk) {
           uint32_t a0, a1, a2, a3;
-          ldmatrix_x4(sK + plane_off<S>(sub * kBlkRows + (lane & 7) + (mid & 1) * 8, kk * 2 + (mid >> 1)), a0, a1, a2, a3);
+          ldmatrix_x4(sK + block_off(pl, (lane & 7) + (mid & 1) * 8, kk * 2 + (mid >> 1)), a0, a1, a2, a3);
           if (kk & 1) mma_bf16_16816(sb2, a0, a1, a2, a3, qa[kk][0], qa[kk][1]);
           else mma_bf16_16816(sa, a0, a1, a2, a3, qa[kk][0], qa[kk][1]);
         }
@@ -704,7 +710,7 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
 #pragma unroll
         for (int n = 0; n < kD / 16; ++n) {
           uint32_t a0, a1, a2, a3;
-          ldmatrix_x4_trans(sV + plane_off<S>(sub * kBlkRows + (lane & 7) + (mid >> 1) * 8, n * 2 + (mid & 1)), a0, a1, a2, a3);
+          ldmatrix_x4_trans(sV + block_off(pl, (lane & 7) + (mid >> 1) * 8, n * 2 + (mid & 1)), a0, a1, a2, a3);
           mma_bf16_16816(o[n], a0, a1, a2, a3, pb0, pb1);
         }
       }
@@ -947,14 +953,14 @@ bool make_decode_maps(const DecodeCommon& c, const DecodeLayerPtrs& L, DecodeLay
     const Entry& e = table[i];
     if (e.K == L.K && e.V == L.V && e.cap == c.cap && e.units == c.units && e.K != nullptr) {
       *out = e.maps;
-      return make_tensor_map_bf16(&out->v16, L.V, 3, dims_v16, strides, box16);
+      return make_tile_map_bf16(&out->v16, L.V, 3, dims_v16, strides, box16);
     }
   }
   const uint64_t dims[2] = {(uint64_t)c.cap, (uint64_t)c.units};
-  if (!(make_tensor_map_bf16(&out->k64, L.K, 3, dims, strides, box64) &&
-        make_tensor_map_bf16(&out->v64, L.V, 3, dims, strides, box64) &&
-        make_tensor_map_bf16(&out->k16, L.K, 3, dims, strides, box16) &&
-        make_tensor_map_bf16(&out->v16, L.V, 3, dims_v16, strides, box16)))
+  if (!(make_tile_map_bf16(&out->k64, L.K, 3, dims, strides, box64) &&
+        make_tile_map_bf16(&out->v64, L.V, 3, dims, strides, box64) &&
+        make_tile_map_bf16(&out->k16, L.K, 3, dims, strides, box16) &&
+        make_tile_map_bf16(&out->v16, L.V, 3, dims_v16, strides, box16)))
     return false;
   Entry& e = table[next];
   next = (next + 1) % kEntries;

@@ -22,13 +22,12 @@ PFN_cuTensorMapEncodeTiled_v12000 resolve_encode() {
   return fn;
 }
 
-}  // namespace
-
-bool make_tensor_map_bf16(CUtensorMap* out, const void* base, int rank, const uint64_t* dims_from_1,
-                          const uint64_t* strides_from_1, const uint32_t* box_from_1) {
+// `halves`: the two halves of the head dimension as a last dimension of their own, both in the box.
+bool encode_map(CUtensorMap* out, const void* base, int rank, const uint64_t* dims_from_1, const uint64_t* strides_from_1,
+                const uint32_t* box_from_1, bool halves) {
   auto encode = resolve_encode();
-  if (!encode || rank < 2 || rank > 5) return false;
-  cuuint64_t dims[5] = {(cuuint64_t)kD, 1, 1, 1, 1};
+  if (!encode || rank < 2 || rank + (halves ? 1 : 0) > 5) return false;
+  cuuint64_t dims[5] = {(cuuint64_t)(halves ? tc::kHalfCols : kD), 1, 1, 1, 1};
   cuuint64_t strides[4] = {0, 0, 0, 0};
   cuuint32_t box[5] = {(cuuint32_t)tc::kHalfCols, 1, 1, 1, 1};
   cuuint32_t estr[5] = {1, 1, 1, 1, 1};
@@ -37,6 +36,12 @@ bool make_tensor_map_bf16(CUtensorMap* out, const void* base, int rank, const ui
     strides[i - 1] = strides_from_1[i - 1];
     box[i] = box_from_1[i - 1];
     if (box[i] < 1 || box[i] > 256 || dims[i] < 1 || (strides[i - 1] & 15u)) return false;
+  }
+  if (halves) {
+    dims[rank] = 2;
+    strides[rank - 1] = tc::kLineBytes;
+    box[rank] = 2;
+    ++rank;
   }
   auto run = [&] {
     return encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), dims, strides, box, estr,
@@ -50,6 +55,18 @@ bool make_tensor_map_bf16(CUtensorMap* out, const void* base, int rank, const ui
     if (cudaGetDevice(&dev) == cudaSuccess && cudaSetDevice(dev) == cudaSuccess) r = run();
   }
   return r == CUDA_SUCCESS;
+}
+
+}  // namespace
+
+bool make_tensor_map_bf16(CUtensorMap* out, const void* base, int rank, const uint64_t* dims_from_1,
+                          const uint64_t* strides_from_1, const uint32_t* box_from_1) {
+  return encode_map(out, base, rank, dims_from_1, strides_from_1, box_from_1, false);
+}
+
+bool make_tile_map_bf16(CUtensorMap* out, const void* base, int rank, const uint64_t* dims_from_1,
+                        const uint64_t* strides_from_1, const uint32_t* box_from_1) {
+  return encode_map(out, base, rank, dims_from_1, strides_from_1, box_from_1, true);
 }
 
 }  // namespace calidrop
