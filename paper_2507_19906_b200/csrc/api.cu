@@ -154,14 +154,15 @@ DecodeCommon plan_decode(const calidrop_params* p, const DecodeWs& w, int n_laye
   // The splits of a unit form one thread-block cluster of 1, 2, 4, 8 or 16 CTAs, or several clusters that meet through the
   // workspace.  What a choice costs, in microseconds: the clusters that the device does not hold at once queue for a
   // second round (eight CTAs: 15 clusters on a B200, whose processor clusters differ in size; 16 units on clusters of
-  // eight took two rounds); a round is a fixed chain (4.4) and the longest slice, at 5.8 ns per row of one CTA or at the
-  // rate of the memory if that is less; the meeting of several clusters costs 4, that of sixteen CTAs 1.4 more than of
-  // eight.  Measured per launch: 4 units x 4333 rows 7.4 (8 CTAs) and 7.0 (16), x 2100 rows 6.2 and 6.8, x 15000 rows
-  // 15.1 and 11.0; 8 units x 20000 rows on 16 clusters of eight 29.5.
+  // eight took two rounds); a round is a fixed chain (4.3) and the longest slice, at 4.4 ns per row of one CTA or at the
+  // rate of the memory if that is less; the meeting of several clusters costs 2.9, clusters of eight 0.25 and of sixteen 0.6
+  // more than smaller ones.  Measured per launch, in a stream: 4 units x 300 rows 4.63 (4 CTAs) and 4.65 (8), x 700 rows 4.61 (8) and
+  // 4.76 (16), x 1300 rows 5.15 and 4.75, x 2100 rows 5.72 and 4.93, x 4333 rows 6.93 and 5.94; 2 units x 15500 rows 8.99 (one
+  // cluster of 16) and 9.76 (three), x 40000 rows 16.3 and 12.5; 8 units x 20000 rows on 16 clusters of eight 28.1.
   const int units_total = a.units * n_layers;
   int want = decode_nsplit(units_total, n_kv);
   if (want > w.max_split) want = w.max_split;
-  const double memory = (double)units_total * n_kv * kRowBytes * 2 / 6.3e6;
+  const double memory = (double)units_total * n_kv * kRowBytes * 2 / 8.5e6;   // (a part is prefetched beside the launch ahead)
   double best = 0.0;
   a.nsplit = a.nclu = 1;
   for (int ns = 1; ns <= (recal ? 8 : 16) && ns <= want; ns *= 2) {
@@ -169,8 +170,8 @@ DecodeCommon plan_decode(const calidrop_params* p, const DecodeWs& w, int n_laye
     for (int nc = 1; resident > 0 && nc <= 8 && ns * nc <= want; ++nc) {
       const int rounds = (units_total * nc + resident - 1) / resident;
       const double rows = (double)((n_kv + ns * nc - 1) / (ns * nc));
-      const double slice = rows * 5.8e-3, share = memory / rounds;
-      const double t = rounds * (4.4 + (slice > share ? slice : share)) + (nc > 1 ? 4.0 : 0.0) + (ns > 8 ? 1.4 : 0.0);
+      const double slice = rows * 4.4e-3, share = memory / rounds;
+      const double t = rounds * (4.3 + (slice > share ? slice : share)) + (nc > 1 ? 2.9 : 0.0) + (ns > 8 ? 0.6 : ns > 4 ? 0.25 : 0.0);
       if ((ns == 1 && nc == 1) || t < best) { best = t; a.nsplit = ns; a.nclu = nc; }
     }
   }
