@@ -154,21 +154,6 @@ __device__ __forceinline__ void tmem_wait(uint32_t (&r)[N]) {
                  : "memory");
   }
 }
-// Whether a phase has completed, without waiting.
-__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n"
-      ".reg .pred p;\n"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      "selp.u32 %0, 1, 0, p;\n"
-      "}\n"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
 template <bool kSized>
 __global__ void __launch_bounds__(kThreads, 1)
 compress_cluster_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap qc_map,
@@ -501,38 +486,24 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_
     };
     int buf = 0;
     uint32_t t_ph = 0;
-    // n accumulators of phase S or V in turn, N columns of each: the next one is on its way to the registers while `fold`
-    // works on the current one, unless its product is late
+    // n accumulators of phase S or V in turn, N columns of each.  (With the next one on its way to the registers while `fold`
+    // works on the current one, in loops of two steps, the calls took longer: 8 units x 8192 keys 35.6 us instead of 33.5,
+    // 8 x 2048 17.0 instead of 16.6.  Four warps a scheduler hide the wait, and the code is half as long.)
     auto drain = [&](auto n_tag, int n, uint32_t taddr, auto&& fold) __attribute__((always_inline)) {
       constexpr int N = decltype(n_tag)::value;
-      uint32_t ra[N], rb[N];
-      auto issue = [&](uint32_t (&r)[N]) __attribute__((always_inline)) {
+#pragma unroll 1
+      for (int i = 0; i < n; ++i) {
+        uint32_t r[N];
+        mbar_wait_far(&ctl, t_full(buf), t_ph, 73u);
         __syncwarp();
         tc_fence_after_sync();
         tmem_issue(taddr + (uint32_t)(buf * 128), r);
-      };
-      auto step = [&](uint32_t (&cur)[N], uint32_t (&nxt)[N], int i) __attribute__((always_inline)) {
-        tmem_wait(cur);
+        tmem_wait(r);
         tc_fence_before_sync();
         __syncwarp();
         if (lane == 0) mbar_arrive(t_empty(buf));
         if (++buf == kAccBufs) { buf = 0; t_ph ^= 1u; }
-        const bool ahead = i + 1 < n && __all_sync(0xffffffffu, mbar_test(t_full(buf), t_ph));
-        if (ahead) issue(nxt);
-        fold(cur, i);
-        if (!ahead && i + 1 < n) {
-          mbar_wait_far(&ctl, t_full(buf), t_ph, 73u);
-          issue(nxt);
-        }
-      };
-      if (n > 0) {
-        mbar_wait_far(&ctl, t_full(buf), t_ph, 73u);
-        issue(ra);
-      }
-#pragma unroll 1
-      for (int i = 0; i < n; i += 2) {
-        step(ra, rb, i);
-        if (i + 1 < n) step(rb, ra, i + 1);
+        fold(r, i);
       }
     };
 
@@ -544,7 +515,6 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_
       const int lim = a.n_cand + row % a.W;                  // the last key the row may see (causal inside the window)
       const bool any = (quad * 32 & (rows - 1)) < a.GW;      // a warp without a row only hands the buffers on
       float2 ml = make_float2(-1e30f, 0.f);
-      // (the accumulator of the next tile is on its way to the registers while the exponentials of this one run)
       auto run = [&](auto n_tag) __attribute__((always_inline)) {
         constexpr int N = decltype(n_tag)::value;
         auto fold = [&](uint32_t (&r)[N], int i) __attribute__((always_inline)) {
@@ -984,20 +954,18 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_
         constexpr int N = decltype(n_tag)::value;
         const int first = copy_c * N;
         const uint32_t taddr = lane_addr + (uint32_t)(grp * 32);
-        uint32_t ra[N], rb[N];
         int b = 0;
         uint32_t b_ph = 0;
-        auto issue = [&](uint32_t (&r)[N], int nb) __attribute__((always_inline)) {
+#pragma unroll 1
+        for (int t = 0; t < nC; ++t) {
+          uint32_t sv[N];
+          mbar_wait_far(&ctl, s_full(b), b_ph, 78u);
           __syncwarp();
           tc_fence_after_sync();
-          tmem_issue(taddr + (uint32_t)(nb * 128 + first), r);
-        };
-        auto step = [&](uint32_t (&sv)[N], uint32_t (&nxt)[N], int t) __attribute__((always_inline)) {
+          tmem_issue(taddr + (uint32_t)(b * 128 + first), sv);
           tmem_wait(sv);
           const uint32_t dst = taddr + (uint32_t)(b * 128), bar_p = p_full(b);
           if (++b == kCalBufs) { b = 0; b_ph ^= 1u; }
-          const bool ahead = t + 1 < nC && __all_sync(0xffffffffu, mbar_test(s_full(b), b_ph));
-          if (ahead) issue(nxt, b);
           const uint32_t w = mask_s[t * 4 + grp] >> first;
 #pragma unroll
           for (int e = 0; e < N; e += 2) {
@@ -1027,19 +995,6 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_
           tc_fence_before_sync();
           __syncwarp();
           if (lane == 0) mbar_arrive(bar_p);
-          if (!ahead && t + 1 < nC) {
-            mbar_wait_far(&ctl, s_full(b), b_ph, 78u);
-            issue(nxt, b);
-          }
-        };
-        if (nC > 0) {
-          mbar_wait_far(&ctl, s_full(0), 0, 78u);
-          issue(ra, 0);
-        }
-#pragma unroll 1
-        for (int t = 0; t < nC; t += 2) {
-          step(ra, rb, t);
-          if (t + 1 < nC) step(rb, ra, t + 1);
         }
       };
       if (!any_c) {
