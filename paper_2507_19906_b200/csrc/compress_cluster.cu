@@ -213,19 +213,24 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_
   const int half = a.pool >> 1;
   const bool quarter = a.tiles_per_cta <= kQuarterTiles;
   const uint32_t hist_bytes = (uint32_t)(n_clu * kThr * 512);
-  int ld_s = 0, ld_n = 0;      // producer: ring position, loads issued
+  int ld_s = 0, ld_n = 0, ld_k = 0;   // producer: ring position, loads issued, K tiles of phase C among them
   uint32_t ld_ph = 1;
   // load n of the CTA: the tiles of phase S upwards, of phase V downwards (the last ones are the recent ones), then K
-  // and V of phase C in turn
+  // and V of phase C, K three tiles ahead: its S has a buffer by then, and a V slot is held until its P.V is done (in turn,
+  // K(t+3) waited behind V(t+2) for P.V(t))
   const int n_loads = nS + nV + 2 * nC;
   auto load_next = [&]() -> bool {
     int tile = tile0 + ld_n;
     const CUtensorMap* map = &k_map;
     uint32_t bar = full_k(ld_s);
     if (ld_n >= nS + nV) {
-      const int t = ld_n - nS - nV;
-      tile = tile0 + (t >> 1);
-      if (t & 1) { map = &v_map; bar = full_v(ld_s); }
+      if (ld_k < min(nC, ld_n - nS - nV - ld_k + kCalBufs)) {
+        tile = tile0 + ld_k++;
+      } else {
+        tile = tile0 + ld_n - nS - nV - ld_k;
+        map = &v_map;
+        bar = full_v(ld_s);
+      }
     } else if (ld_n >= nS) {
       tile = tile0 + nV - 1 - (ld_n - nS);
     }
@@ -426,7 +431,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_
         }
         __syncwarp();
         k_ph ^= 1u << s;
-        s = (s + 2) % a.stages;   // (the V tile of the pair is the other issuer's)
+        s = (s + (t < kCalBufs - 1 ? 1 : 2)) % a.stages;   // (the V tiles between are the other issuer's)
         if (++b == kCalBufs) { b = 0; b_ph ^= 1u; }
       }
     }
@@ -435,7 +440,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_
     const uint32_t idesc_o = umma_idesc(128, 128, false, true);
     const uint64_t dv0 = smem_desc_sw128(ring, kTileBytes / 2, 1024u);
     const bool leader = elect_one();
-    const int n0 = nS + nV + 1;   // the ring's position of the first V tile
+    const int n0 = nS + nV + min(nC, kCalBufs);   // the ring's position of the first V tile
     int s = n0 % a.stages, b = 0;
     uint32_t v_ph = 0, b_ph = 0;
     bool ok = true;
@@ -461,7 +466,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_
       }
       __syncwarp();
       v_ph ^= 1u << s;
-      s = (s + 2) % a.stages;
+      s = (s + (t + kCalBufs < nC ? 2 : 1)) % a.stages;
       if (++b == kCalBufs) { b = 0; b_ph ^= 1u; }
     }
   } else if (warp >= kGatherWarp) {
@@ -1064,16 +1069,13 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_
       const uint2 cq = reinterpret_cast<const uint2*>(a.Q_obs + ((size_t)hq0 * a.W + wrow) * kD)[lane];
       float l = lane < n_clu ? __ldcg(a.l_part + slot0 + (size_t)lane * a.cal_rows) : 0.f;
       float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 1
-      for (int p0 = 0; p0 < n_clu; p0 += 8) {
-        float4 v[8];
+      float4 v[kMaxClu];
 #pragma unroll
-        for (int p = 0; p < 8; ++p)
-          v[p] = p0 + p < n_clu ? __ldcg(reinterpret_cast<const float4*>(a.o_part + (slot0 + (size_t)(p0 + p) * a.cal_rows) * kD) + lane)
-                                : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int p = 0; p < kMaxClu; ++p)
+        v[p] = p < n_clu ? __ldcg(reinterpret_cast<const float4*>(a.o_part + (slot0 + (size_t)p * a.cal_rows) * kD) + lane)
+                         : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int p = 0; p < 8; ++p) { acc.x += v[p].x; acc.y += v[p].y; acc.z += v[p].z; acc.w += v[p].w; }
-      }
+      for (int p = 0; p < kMaxClu; ++p) { acc.x += v[p].x; acc.y += v[p].y; acc.z += v[p].z; acc.w += v[p].w; }
       l = warp_sum(l);
       float4 out = make_float4(0.f, 0.f, 0.f, 0.f);
       float lse = -INFINITY;
