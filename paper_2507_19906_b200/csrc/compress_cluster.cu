@@ -22,8 +22,8 @@
 // the exponentials, one per logit and phase (see exp2.cuh), and the warps' issue slots beside them: 1250 cycles a tile and
 // phase for 1024 exponential-unit cycles, whatever share of them is on the FMA pipe.  The code is kept small on purpose
 // (loops not unrolled, waits out of line): most of it runs once per launch, and 260 KB of it took 20 us
-// where 145 KB take 17.  Five to six kernels -> this one, us: 8 units x 2048 keys x 32 rows 28.3 -> 17.4, 8 x 8192 x 128 45.0 ->
-// 35.6, 16 x 5003 x 120 with the caller's row LSE and a calibration size 42.8 -> 30.6.
+// where 110 KB take 16.6.  Five to six kernels -> this one, us: 8 units x 2048 keys x 32 rows 28.3 -> 16.7, 8 x 8192 x 128 45.0 ->
+// 32.2, 16 x 5003 x 120 with the caller's row LSE and a calibration size 42.8 -> 27.3.
 #include <algorithm>
 #include <atomic>
 #include <type_traits>
@@ -1201,12 +1201,12 @@ cudaError_t launch_kernel(const ClusterArgs& a, const ClusterPlan& p, int units,
 }
 
 // The fewest tiles per CTA with which every unit has its cluster at once; false where the kernel does not cover the
-// shape or the separate kernels are the faster way.  A call costs, in microseconds, about 15.5 and 0.97 for each tile of a
-// CTA and phase here, and 33 and 1.2 for each tile of an SM and pass there, where all 148 SMs have a share; here those
-// that no cluster fits on are idle.  Measured, us, separate and here: 8 units x 1100 keys x 128 rows 32.0 and 18.1, x 8192
-// 43.8 and 35.0, x 16384 61.9 and 53.9, x 24576 73.5 and 72.2, x 32768 83 and 91; 2 units x 32768 53 and 60; 16 x 8192 60.4
-// and 47.1, x 24576 104 and 107; 32 x 2048 46.2 and 28.1, x 16384 126 and 111; with the caller's row LSE 64 x 4096 68.1 and 54.1, x 12288
-// 135 and 125, and, with a ring of three tiles, x 16384 163 and 172.
+// shape or the separate kernels are the faster way.  A call costs, in microseconds, about 13 and 1.9 for each tile of a CTA
+// here, 0.68 more for one with statistics, and 37.5 and 1.08 for each tile of an SM and pass there, where all 148 SMs have
+// a share; here those that no cluster fits on are idle.  Measured, us, separate and here: 8 units x 1100 keys x 128 rows 32.0
+// and 18, x 8192 44 and 32, x 16384 62 and 47, x 32768 84 and 81; 2 units x 24000 56 and 43, x 32768 53 and 52; 16 x 16384 81 and 73,
+// x 32768 125 and 126; 32 x 2048 46 and 26, x 20000 146 and 129; with the caller's row LSE 8 x 32768 65 and 63, 16 x 24576 80 and 76,
+// 64 x 12288 135 and 122 and, with a ring of three tiles, x 16384 163 and 172.
 bool plan_cluster(const CompressGeom& g, bool stats, ClusterPlan* p) {
   if (g.keep_all || g.n_cand < 1 || g.G * g.W > kMaxRows || g.pool >> 1 > kHaloMax) return false;
   if (g.sized && g.n_calib == 0) return false;
@@ -1218,8 +1218,8 @@ bool plan_cluster(const CompressGeom& g, bool stats, ClusterPlan* p) {
   for (int t = (n_tiles + kMaxClu - 1) / kMaxClu; t <= kMaxTiles; ++t) {
     const int n_clu = (n_tiles + t - 1) / t;
     if (g.units > resident_clusters(n_clu) || (size_t)g.units * n_clu > parts) continue;
-    const double here = 0.97 * t, there = 1.2 * g.units * n_tiles / 148.0;
-    return (stats ? 3 : 2) * (here - there) < 33.0 - 15.5 && lay_out(g, stats, t, p);
+    const double here = 13.0 + (stats ? 2.58 : 1.9) * t, there = 37.5 + (stats ? 3.24 : 2.16) * g.units * n_tiles / 148.0;
+    return here < there && lay_out(g, stats, t, p);
   }
   return false;
 }
