@@ -268,7 +268,7 @@ int calidrop_compress(const calidrop_params* p, const void* Q_obs, const void* K
                       g.L, g.n_kept, g.cap, g.units};
   if (tc_path) {   // short prompts: the whole step in one kernel
     bool taken = false;
-    cudaError_t ec = launch_compress_cluster(g, ws, Q_obs, K, V, lse_obs, wsp, kept_idx, O_c, LSE_c, C_q, ga, &taken, st);
+    cudaError_t ec = launch_compress_cluster(g, ws, Q_obs, K, V, lse_obs, wsp, kept_idx, O_c, LSE_c, C_q, ga, false, &taken, st);
     if (ec != cudaSuccess) return cuda_fail(ec);
     if (taken) return CALIDROP_OK;
   }
@@ -328,6 +328,15 @@ int calidrop_calibrate(const calidrop_params* p, const void* Q_obs, const void* 
   cudaStream_t st = (cudaStream_t)stream;
   char* wsp = (char*)workspace;
   const bool tc_path = score_tc_supported(g), calib_tc = tc_path && calib_tc_supported(g);
+  const GatherArgs ga{(const uint4*)K, (const uint4*)V, kept_idx, (uint4*)K_kept, (uint4*)V_kept,
+                      g.L, g.n_kept, g.cap, g.units};
+  if (tc_path) {   // short prompts: one kernel
+    bool taken = false;
+    cudaError_t ec = launch_compress_cluster(g, ws, Q_obs, K, V, lse_obs, wsp, const_cast<int32_t*>(kept_idx), O_c, LSE_c, C_q,
+                                             ga, true, &taken, st);
+    if (ec != cudaSuccess) return cuda_fail(ec);
+    if (taken) return CALIDROP_OK;
+  }
   // the error word is cleared by the call's first tensor-core kernel, where it has one
   const bool stats_tc = tc_path && !lse_obs;
   cudaError_t e = stats_tc || calib_tc ? cudaSuccess : cudaMemsetAsync(wsp + ws.status, 0, 4, st);
@@ -346,8 +355,6 @@ int calidrop_calibrate(const calidrop_params* p, const void* Q_obs, const void* 
     e = launch_gather(g, K, V, kept_idx, K_kept, V_kept, st);
     if (e != cudaSuccess) return cuda_fail(e);
   }
-  const GatherArgs ga{(const uint4*)K, (const uint4*)V, kept_idx, (uint4*)K_kept, (uint4*)V_kept,
-                      g.L, g.n_kept, g.cap, g.units};
   e = calib_tc ? launch_calib_tc(g, ws, Q_obs, K, V, row_lse, wsp, O_c, LSE_c, C_q, ga, !stats_tc, st)
                : launch_calib_direct(g, ws, Q_obs, K, V, wsp, O_c, LSE_c, C_q, st);
   if (e != cudaSuccess) return cuda_fail(e);

@@ -7,6 +7,7 @@
 //      cluster into the row LSE (left out when the caller supplies it)
 //   V  votes: S^T = K Q^T with the keys on the lanes, the vote of a key is a per-thread sum over the rows
 //   select: pooling and an exact radix select over the cluster; the votes never leave the CTA but for the outputs
+//   (for a caller's kept list, calidrop_calibrate, V and the selection fall away)
 //   C  calibration: S = Q_c K^T again, probabilities of the evicted keys as the A operand of O += P V
 //   reduce: every CTA finishes a share of the calibration rows from the partial O that all left in the workspace; one warp copies the
 //      retained rows meanwhile
@@ -154,7 +155,8 @@ __device__ __forceinline__ void tmem_wait(uint32_t (&r)[N]) {
                  : "memory");
   }
 }
-template <bool kSized>
+// kGiven: the kept list is the caller's; V and the selection fall away.
+template <bool kSized, bool kGiven>
 __global__ void __launch_bounds__(kThreads, 1)
 compress_cluster_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap qc_map,
                         const __grid_constant__ CUtensorMap k_map, const __grid_constant__ CUtensorMap v_map,
@@ -178,7 +180,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_
   const int tile0 = rank * a.tiles_per_cta, c0 = tile0 * kTileKeys;
   const int nt = min(a.tiles_per_cta, a.n_tiles - tile0);            // at least one
   const int n_own = max(0, min(nt * kTileKeys, a.n_cand - c0));      // candidates of this CTA
-  const int nS = a.row_lse ? 0 : nt, nV = (n_own + kTileKeys - 1) / kTileKeys, nC = nV;
+  const int nC = (n_own + kTileKeys - 1) / kTileKeys, nV = kGiven ? 0 : nC, nS = a.row_lse ? 0 : nt;
 
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   unsigned char* const smem_al = smem_raw + (smem_base - smem_u32(smem_raw));
@@ -350,7 +352,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_
       while (ok && ld_n < nS + nV) ok = load_next();
       if (nC > 0 && ok) {
         // the calibration rows replace the window rows once the last S^T is done
-        ok = mbar_wait_far(&ctl, q_empty, 0, 62u);
+        ok = nS + nV == 0 || mbar_wait_far(&ctl, q_empty, 0, 62u);
         if (ok) {
           mbar_arrive_expect_tx(q_full, ((uint32_t)(2 * a.cal_rows) << a.lg_rep_c) * kLineBytes);
 #pragma unroll 1
@@ -401,7 +403,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_
       if (++buf == kAccBufs) { buf = 0; t_ph ^= 1u; }
     }
     if (nC > 0 && ok) {
-      ok = mbar_wait_far(&ctl, q_full, 1, 66u);
+      ok = mbar_wait_far(&ctl, q_full, nS + nV > 0 ? 1u : 0u, 66u);
       // every accumulator of phase V has been read out: buf and t_ph are where the next job of that kind would go
 #pragma unroll 1
       for (int b = 0; b < kAccBufs; ++b) {
@@ -471,9 +473,11 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_
     }
   } else if (warp >= kGatherWarp) {
     // ------------------------------------------------------------ compaction of the retained rows: from the selection on
-    asm volatile("barrier.cta.sync 3, %0;" ::"n"(kConsumers + 32) : "memory");
-    if (lane < n_clu) arrive_peer(peer_addr(x_kept, lane));
-    if (mbar_wait_cluster(&ctl, x_kept, 0, 72u)) compact_rows();
+    if (!kGiven) {
+      asm volatile("barrier.cta.sync 3, %0;" ::"n"(kConsumers + 32) : "memory");
+      if (lane < n_clu) arrive_peer(peer_addr(x_kept, lane));
+    }
+    if (kGiven || mbar_wait_cluster(&ctl, x_kept, 0, 72u)) compact_rows();
     __syncwarp();
   } else {
     // ------------------------------------------------------------ consumers
@@ -612,6 +616,21 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_
     }
     block_sync();
 
+    if constexpr (kGiven) {
+      // the listed rows of this CTA, and those that are no candidates, are not calibrated
+      if (nS == 0) peers_up();
+      for (int i = tid; i < nt * 4; i += kConsumers) {
+        const int rest = n_own - i * 32;
+        mask_s[i] = rest >= 32 ? 0u : rest <= 0 ? 0xffffffffu : 0xffffffffu << rest;
+      }
+      block_sync();
+      const int32_t* const list = a.kept_idx + (size_t)unit * a.n_kept;
+      for (int i = tid; i < a.n_kept; i += kConsumers) {
+        const int at = list[i] - c0;   // (a caller's list may hold anything)
+        if (at >= 0 && at < nt * kTileKeys) atomicOr(mask_s + (at >> 5), 1u << (at & 31));
+      }
+      block_sync();
+    } else {
     // ---- V: votes of this CTA's keys.  Up to kQuarterTiles tiles the four groups share a tile, a quarter of the rows
     // each, and the parts meet in shared memory; beyond, a group takes every fourth tile alone.
 #pragma unroll 1
@@ -946,6 +965,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_
     // the compacting warp tells the cluster: its release waits until the list has reached the L2, a thousand cycles
     asm volatile("barrier.cta.arrive 3, %0;" ::"n"(kConsumers + 32) : "memory");
     block_sync();
+    }
 
     // ---- C: probabilities of the evicted keys (see calib_tc.cu); copies of the rows as in S
     const int rows_c = 128 >> a.lg_rep_c, row_c = r128 & (rows_c - 1), copy_c = r128 >> (7 - a.lg_rep_c);
@@ -1089,7 +1109,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_
       if (lane == 0) a.LSE_c[dst] = lse;
       reinterpret_cast<uint2*>(a.C_q + dst * kD)[lane] = cq;
     }
-    if (mbar_wait_cluster(&ctl, x_kept, 0, 81u)) compact_rows();
+    if (kGiven || mbar_wait_cluster(&ctl, x_kept, 0, 81u)) compact_rows();
   }
 
   // ---------------------------------------------------------------- teardown (every path)
@@ -1149,16 +1169,16 @@ void launch_config(int n_clu, int units, int smem, cudaStream_t st, cudaLaunchCo
   cfg.numAttrs = 2;
 }
 
-template <bool kSized>
+template <bool kSized, bool kGiven>
 cudaError_t setup() {
   static OncePerDevice granted, wide;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = grant_smem(compress_cluster_kernel<kSized>, kSmemMax, granted);
+  if (e == cudaSuccess) e = grant_smem(compress_cluster_kernel<kSized, kGiven>, kSmemMax, granted);
   if (e != cudaSuccess) return e;
   const bool slot = dev >= 0 && dev < 64;
   if (slot && wide[dev].load(std::memory_order_acquire)) return cudaSuccess;
-  e = cudaFuncSetAttribute(compress_cluster_kernel<kSized>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  e = cudaFuncSetAttribute(compress_cluster_kernel<kSized, kGiven>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e == cudaSuccess && slot) wide[dev].store(true, std::memory_order_release);
   return e;
 }
@@ -1170,13 +1190,13 @@ int resident_clusters(int n_clu) {
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
   int n = known[dev][n_clu].load(std::memory_order_acquire);
   if (n == 0) {
-    if (setup<false>() != cudaSuccess) return 0;
+    if (setup<false, false>() != cudaSuccess) return 0;
     int active = 0;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
     launch_config(n_clu, 1, kSmemMax, nullptr, cfg, attr);
     cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&active, compress_cluster_kernel<false>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&active, compress_cluster_kernel<false, false>, &cfg) != cudaSuccess) {
       cudaGetLastError();   // no such cluster on this device
       active = 0;
     }
@@ -1186,15 +1206,15 @@ int resident_clusters(int n_clu) {
   return n - 1;
 }
 
-template <bool kSized>
+template <bool kSized, bool kGiven>
 cudaError_t launch_kernel(const ClusterArgs& a, const ClusterPlan& p, int units, const CUtensorMap& qm, const CUtensorMap& qcm,
                           const CUtensorMap& km, const CUtensorMap& vm, cudaStream_t st) {
-  cudaError_t e = setup<kSized>();
+  cudaError_t e = setup<kSized, kGiven>();
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
   launch_config(p.n_clu, units, p.smem, st, cfg, attr);
-  e = cudaLaunchKernelEx(&cfg, compress_cluster_kernel<kSized>, qm, qcm, km, vm, a);
+  e = cudaLaunchKernelEx(&cfg, compress_cluster_kernel<kSized, kGiven>, qm, qcm, km, vm, a);
   if (e != cudaSuccess) return e;
   count_launch(1);
   return cudaGetLastError();
@@ -1206,8 +1226,9 @@ cudaError_t launch_kernel(const ClusterArgs& a, const ClusterPlan& p, int units,
 // a share; here those that no cluster fits on are idle.  Measured, us, separate and here: 8 units x 1100 keys x 128 rows 32.0
 // and 18, x 8192 44 and 32, x 16384 62 and 47, x 32768 84 and 81; 2 units x 24000 56 and 43, x 32768 53 and 52; 16 x 16384 81 and 73,
 // x 32768 125 and 126; 32 x 2048 46 and 26, x 20000 146 and 129; with the caller's row LSE 8 x 32768 65 and 63, 16 x 24576 80 and 76,
-// 64 x 12288 135 and 122 and, with a ring of three tiles, x 16384 163 and 172.
-bool plan_cluster(const CompressGeom& g, bool stats, ClusterPlan* p) {
+// 64 x 12288 135 and 122 and, with a ring of three tiles, x 16384 163 and 172.  For a given kept list 8 x 1000 24 and 12, x 8192 31 and
+// 21, x 45000 77 and 66, 2 x 24000 41 and 28, 64 x 8192 100 and 77; with the caller's row LSE 8 x 8192 22 and 14, 16 x 32768 65 and 54.
+bool plan_cluster(const CompressGeom& g, bool stats, bool given, ClusterPlan* p) {
   if (g.keep_all || g.n_cand < 1 || g.G * g.W > kMaxRows || g.pool >> 1 > kHaloMax) return false;
   if (g.sized && g.n_calib == 0) return false;
   const int n_tiles = (g.L + kTileKeys - 1) / kTileKeys;
@@ -1218,7 +1239,9 @@ bool plan_cluster(const CompressGeom& g, bool stats, ClusterPlan* p) {
   for (int t = (n_tiles + kMaxClu - 1) / kMaxClu; t <= kMaxTiles; ++t) {
     const int n_clu = (n_tiles + t - 1) / t;
     if (g.units > resident_clusters(n_clu) || (size_t)g.units * n_clu > parts) continue;
-    const double here = 13.0 + (stats ? 2.58 : 1.9) * t, there = 37.5 + (stats ? 3.24 : 2.16) * g.units * n_tiles / 148.0;
+    const double tiles = g.units * n_tiles / 148.0;
+    const double here = given ? (stats ? 10.5 + 1.55 * t : 8.7 + 0.95 * t) : 13.0 + (stats ? 2.58 : 1.9) * t;
+    const double there = given ? (stats ? 30.0 + 2.3 * tiles : 19.0 + 1.75 * tiles) : 37.5 + (stats ? 3.24 : 2.16) * tiles;
     return here < there && lay_out(g, stats, t, p);
   }
   return false;
@@ -1226,12 +1249,13 @@ bool plan_cluster(const CompressGeom& g, bool stats, ClusterPlan* p) {
 
 }  // namespace
 
-// The whole step in one launch; *taken is false (and nothing launched) where the separate kernels are to be used.
+// The whole step in one launch, or (`given`) the calibration and compaction for the kept list in kept_idx; *taken is false (and
+// nothing launched) where the separate kernels are to be used.
 cudaError_t launch_compress_cluster(const CompressGeom& g, const CompressWs& ws, const void* Q_obs, const void* K, const void* V,
                                     const float* row_lse, char* wsp, int32_t* kept_idx, float* O_c, float* LSE_c, void* C_q,
-                                    const GatherArgs& gather, bool* taken, cudaStream_t st) {
+                                    const GatherArgs& gather, bool given, bool* taken, cudaStream_t st) {
   ClusterPlan p;
-  *taken = plan_cluster(g, row_lse == nullptr, &p);
+  *taken = plan_cluster(g, row_lse == nullptr, given, &p);
   if (!*taken) return cudaSuccess;
   ClusterArgs a{};
   a.Hq = g.Hq; a.G = g.G; a.W = g.W; a.L = g.L; a.n_cand = g.n_cand; a.n_cal = g.n_cal;
@@ -1270,8 +1294,9 @@ cudaError_t launch_compress_cluster(const CompressGeom& g, const CompressWs& ws,
       !make_tensor_map_bf16(&qcm, (const char*)Q_obs + (size_t)(g.W - g.n_cal) * 256, 4, cd, cs, cb) ||
       !make_tensor_map_bf16(&km, K, 3, kd, ks, kb) || !make_tensor_map_bf16(&vm, V, 3, kd, ks, kb))
     return cudaErrorInvalidValue;
-  return g.sized ? launch_kernel<true>(a, p, g.units, qm, qcm, km, vm, st)
-                 : launch_kernel<false>(a, p, g.units, qm, qcm, km, vm, st);
+  if (given) return launch_kernel<false, true>(a, p, g.units, qm, qcm, km, vm, st);
+  return g.sized ? launch_kernel<true, false>(a, p, g.units, qm, qcm, km, vm, st)
+                 : launch_kernel<false, false>(a, p, g.units, qm, qcm, km, vm, st);
 }
 
 }  // namespace calidrop

@@ -121,10 +121,11 @@ struct GatherArgs {
 cudaError_t launch_calib_tc(const CompressGeom& g, const CompressWs& ws, const void* Q_obs, const void* K,
                             const void* V, const float* row_lse, char* wsp, float* O_c, float* LSE_c, void* C_q,
                             const GatherArgs& gather, bool first, cudaStream_t st);
-// compress_cluster.cu: the whole step in one kernel, where a unit is small enough for a cluster
+// compress_cluster.cu: the whole step (or, given a kept list, what follows the selection) in one kernel, where a unit is
+// small enough for a cluster
 cudaError_t launch_compress_cluster(const CompressGeom& g, const CompressWs& ws, const void* Q_obs, const void* K, const void* V,
                                     const float* row_lse, char* wsp, int32_t* kept_idx, float* O_c, float* LSE_c, void* C_q,
-                                    const GatherArgs& gather, bool* taken, cudaStream_t st);
+                                    const GatherArgs& gather, bool given, bool* taken, cudaStream_t st);
 #ifdef __CUDACC__
 // Rows [16 bx, 16 bx + 16) of unit `unit`: 16 lanes x 16 bytes per row, 256 threads.
 __device__ __forceinline__ void gather_rows16(const GatherArgs& a, int bx, int unit, int tid) {

@@ -372,6 +372,30 @@ def test_compress_in_one_kernel(cuda_lib, B, Hq, Hkv, L, W, pool, budget, n_cal,
         assert_close_lse(st.LSE_c.cpu().numpy(), orc.LSE_c, "LSE_c")
         assert_close_out(st.O_c.cpu().numpy(), orc.O_c, "O_c")
 
+@pytest.mark.parametrize("B,Hq,Hkv,L,W,pool,budget,n_cal", [c[:8] for c in ONE_KERNEL if c[8] == 0 and c[9] == 1])
+@pytest.mark.parametrize("supply_lse", [False, True])
+def test_calibrate_in_one_kernel(cuda_lib, B, Hq, Hkv, L, W, pool, budget, n_cal, supply_lse):
+    """The calibration for a given kept list takes the same cluster kernel without its selection: for the list that the whole
+    step chose, the same rows and the same calibration state (the same sums in the same order)."""
+    from paper_2507_19906_b200 import binding as cd
+    cfg = wl.small_config(B=B, Hq=Hq, Hkv=Hkv, L=L, window=W, pool=pool, budget=budget, steps=1, n_sink=2,
+                          n_heavy=max(1, L // 50))
+    Q, K, V = (to_dev(x) for x in _inputs(cfg))
+    p = cd.make_params(B=B, Hq=Hq, Hkv=Hkv, L=L, window=W, pool=pool, budget=budget, n_cal=n_cal, cap=budget)
+    st, got = cd.alloc_layer_state(p), cd.alloc_layer_state(p)
+    cd.calidrop_compress(p, Q, K, V, None, st.kept_idx, st.K_kept, st.V_kept, st.O_c, st.LSE_c, st.C_q, st.ws_compress)
+    off = cd.calidrop_compress_workspace_layout(p).row_lse_offset
+    lse = st.ws_compress[off:off + 4 * B * Hq * W].view(torch.float32).clone() if supply_lse else None
+    before = cd.calidrop_launch_count()
+    cd.calidrop_calibrate(p, Q, K, V, lse, st.kept_idx, got.K_kept, got.V_kept, got.O_c, got.LSE_c, got.C_q, got.ws_compress)
+    torch.cuda.synchronize()
+    assert cd.calidrop_launch_count() - before == 1
+    lay = cd.calidrop_compress_workspace_layout(p)
+    assert int(got.ws_compress[lay.status_offset:lay.status_offset + 4].view(torch.int32).item()) == 0
+    for name in ("K_kept", "V_kept", "C_q"):
+        assert torch.equal(getattr(got, name), getattr(st, name)), name
+    assert torch.allclose(got.LSE_c, st.LSE_c, rtol=0, atol=1e-5) and torch.allclose(got.O_c, st.O_c, rtol=1e-5, atol=1e-6)
+
 def test_supplied_row_lse_matches_self_computed(cuda_lib):
     cfg = wl.small_config(B=1, Hq=4, Hkv=2, L=400, window=16, pool=7, budget=64)
     Q, K, V = _inputs(cfg)
