@@ -315,23 +315,23 @@ def test_calibration_size(cuda_lib, calib_size):
 
 
 ONE_KERNEL = [
-    # B, Hq, Hkv, L, W, pool, budget, n_cal, calib_size, kernels (1: the cluster kernel; else the separate ones)
-    (1, 1, 1, 136, 8, 7, 40, 1, 0, 1),           # two CTAs, the second has window rows only
-    (1, 2, 1, 128 * 3 + 33, 32, 1, 70, 32, 0, 1),   # 64 window rows (two copies of them on the lanes), one candidate in the last tile
-    (1, 5, 1, 2048, 8, 9, 200, 8, 0, 1),         # sixteen CTAs of a tile, 40 rows, a pool without a kernel of its own
-    (2, 5, 1, 2300, 24, 129, 300, 24, 500, 1),   # 120 rows, the widest pool that the kernel takes, a calibration size
-    (1, 4, 1, 900, 32, 5, 899, 32, 0, 1),        # a single evicted candidate, 128 calibration rows
-    (3, 8, 8, 1300, 16, 7, 17, 1, 3, 1),         # 24 units, 16 rows; one candidate kept, three calibrated
-    (1, 100, 100, 300, 8, 7, 50, 8, 0, 1),       # one CTA to a unit
-    (1, 100, 100, 128 * 17 + 5, 8, 5, 60, 2, 40, 1),   # ... of 18 tiles: the groups take tiles of their own in the votes
-    (1, 3, 1, 900, 64, 7, 200, 3, 0, 5),         # 192 rows: the separate kernels, the row LSE combined by the votes
-    (1, 100, 100, 900, 128, 131, 300, 2, 0, 5),  # a pool wider than the halo
+    # B, Hq, Hkv, L, W, pool, budget, n_cal, calib_size, whether the cluster kernel takes it
+    (1, 1, 1, 136, 8, 7, 40, 1, 0, True),           # two CTAs, the second has window rows only
+    (1, 2, 1, 128 * 3 + 33, 32, 1, 70, 32, 0, True),   # 64 window rows (two copies of them on the lanes), one candidate in the last tile
+    (1, 5, 1, 2048, 8, 9, 200, 8, 0, True),         # sixteen CTAs of a tile, 40 rows, a pool without a kernel of its own
+    (2, 5, 1, 2300, 24, 129, 300, 24, 500, True),   # 120 rows, the widest pool that the kernel takes, a calibration size
+    (1, 4, 1, 900, 32, 5, 899, 32, 0, True),        # a single evicted candidate, 128 calibration rows
+    (3, 8, 8, 1300, 16, 7, 17, 1, 3, True),         # 24 units, 16 rows; one candidate kept, three calibrated
+    (1, 100, 100, 300, 8, 7, 50, 8, 0, True),       # one CTA to a unit
+    (1, 100, 100, 128 * 17 + 5, 8, 5, 60, 2, 40, True),   # ... of 18 tiles: the groups take tiles of their own in the votes
+    (1, 3, 1, 900, 64, 7, 200, 3, 0, False),         # 192 rows: the separate kernels, the row LSE combined by the votes
+    (1, 100, 100, 900, 128, 131, 300, 2, 0, False),  # a pool wider than the halo
 ]
 
 
-@pytest.mark.parametrize("B,Hq,Hkv,L,W,pool,budget,n_cal,calib_size,kernels", ONE_KERNEL)
+@pytest.mark.parametrize("B,Hq,Hkv,L,W,pool,budget,n_cal,calib_size,one_kernel", ONE_KERNEL)
 @pytest.mark.parametrize("octaves", [None, 0, 24, -40])
-def test_compress_in_one_kernel(cuda_lib, B, Hq, Hkv, L, W, pool, budget, n_cal, calib_size, kernels, octaves):
+def test_compress_in_one_kernel(cuda_lib, B, Hq, Hkv, L, W, pool, budget, n_cal, calib_size, one_kernel, octaves):
     """Units that a cluster holds take one kernel.  With `octaves` the caller supplies the row LSE, less that many factors of
     two: the votes then lie inside, above and below the range that the first selection pass resolves.  Rounding the
     shifted row LSE moves a vote by 2^-18 of itself at most (|lse| below 64), the same for all keys of a row."""
@@ -351,8 +351,7 @@ def test_compress_in_one_kernel(cuda_lib, B, Hq, Hkv, L, W, pool, budget, n_cal,
     before = cd.calidrop_launch_count()
     cd.calidrop_compress(p, dQ, dK, dV, lse, st.kept_idx, st.K_kept, st.V_kept, st.O_c, st.LSE_c, st.C_q, st.ws_compress)
     torch.cuda.synchronize()
-    launched = cd.calidrop_launch_count() - before
-    assert launched == kernels - (octaves is not None and kernels > 1)
+    assert (cd.calidrop_launch_count() - before == 1) == one_kernel
     lay = cd.calidrop_compress_workspace_layout(p)
     assert int(st.ws_compress[lay.status_offset:lay.status_offset + 4].view(torch.int32).item()) == 0
     ws = lambda off, ref: st.ws_compress[off:off + 4 * ref.size].view(torch.float32).cpu().numpy().reshape(ref.shape)
@@ -372,7 +371,7 @@ def test_compress_in_one_kernel(cuda_lib, B, Hq, Hkv, L, W, pool, budget, n_cal,
         assert_close_lse(st.LSE_c.cpu().numpy(), orc.LSE_c, "LSE_c")
         assert_close_out(st.O_c.cpu().numpy(), orc.O_c, "O_c")
 
-@pytest.mark.parametrize("B,Hq,Hkv,L,W,pool,budget,n_cal", [c[:8] for c in ONE_KERNEL if c[8] == 0 and c[9] == 1])
+@pytest.mark.parametrize("B,Hq,Hkv,L,W,pool,budget,n_cal", [c[:8] for c in ONE_KERNEL if c[8] == 0 and c[9]])
 @pytest.mark.parametrize("supply_lse", [False, True])
 def test_calibrate_in_one_kernel(cuda_lib, B, Hq, Hkv, L, W, pool, budget, n_cal, supply_lse):
     """The calibration for a given kept list takes the same cluster kernel without its selection: for the list that the whole
