@@ -117,6 +117,33 @@ __device__ __forceinline__ bool mbar_wait_cluster(Ctl* ctl, uint32_t bar, uint32
   return true;
 }
 
+// Elements 4 lane .. 4 lane + 3 of a row's partial O over n keys, for a row with copies whose copies added up to NaN: a copy has
+// zeros for the other copies' keys, and zero times an infinite value of V is NaN where the row itself has a probability above zero.
+// Only products that are not finite decide such an element (`l`, the row's sum, tells whether a probability can be one); none
+// found, it stays as it is.  Out of line: finite inputs never get here, and the instruction fetch of code beside the loop costs all.
+__device__ __noinline__ float4 refold_nonfinite(float4 o, const __nv_bfloat16* q, const __nv_bfloat16* K, const __nv_bfloat16* V,
+                                                int n, const uint32_t* mask, float scale2, float nlse2, float l, int lane) {
+  if (isnan(l)) return o;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int t = 0; t < n; ++t) {
+    const __nv_bfloat16* vp = V + (size_t)t * kD + 4 * lane;
+    const float4 v = make_float4(__bfloat162float(vp[0]), __bfloat162float(vp[1]), __bfloat162float(vp[2]), __bfloat162float(vp[3]));
+    if (isfinite(v.x) && isfinite(v.y) && isfinite(v.z) && isfinite(v.w) && isfinite(l)) continue;
+    float p = 0.f;
+    if (!((mask[t >> 5] >> (t & 31)) & 1u)) {
+      float s = 0.f;
+      for (int d = 0; d < kD; ++d) s = fmaf(__bfloat162float(q[d]), __bfloat162float(K[(size_t)t * kD + d]), s);
+      p = __bfloat162float(__float2bfloat16(exp2f(fmaf(s, scale2, nlse2))));
+    }
+    acc.x = fmaf(p, v.x, acc.x);
+    acc.y = fmaf(p, v.y, acc.y);
+    acc.z = fmaf(p, v.z, acc.z);
+    acc.w = fmaf(p, v.w, acc.w);
+  }
+  return make_float4(isfinite(acc.x) ? o.x : acc.x, isfinite(acc.y) ? o.y : acc.y, isfinite(acc.z) ? o.z : acc.z,
+                     isfinite(acc.w) ? o.w : acc.w);
+}
+
 // Columns of this thread's lane: the load, and its completion (see tmem_ld32_issue).
 template <int N>
 __device__ __forceinline__ void tmem_issue(uint32_t taddr, uint32_t (&r)[N]) {
@@ -1065,6 +1092,17 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_
         for (int c = 1; c < 1 << a.lg_rep_c; ++c) {
           const float4 u = *reinterpret_cast<const float4*>(obuf + (c * rows_c + row) * kOStride + 4 * lane);
           v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
+        }
+        if (a.lg_rep_c > 0 && (isnan(v.x) || isnan(v.y) || isnan(v.z) || isnan(v.w))) {
+          const int wrow = row / a.n_cal * a.W + a.W - a.n_cal + row % a.n_cal;
+          float l = 0.f;
+          for (int c = 0; c < 1 << a.lg_rep_c; ++c)
+            for (int q = 0; q < kGroups; ++q) l += l_s[q][c * rows_c + row];
+          const size_t first = ((size_t)unit * a.L + c0) * kD;
+          v = refold_nonfinite(v, a.Q_obs + ((size_t)hq0 * a.W + wrow) * kD,
+                               reinterpret_cast<const __nv_bfloat16*>(a.gather.K) + first,
+                               reinterpret_cast<const __nv_bfloat16*>(a.gather.V) + first, min(nC * kTileKeys, a.L - c0), mask_s,
+                               a.scale2, nlse2_s[wrow], l, lane);
         }
         __stcg(reinterpret_cast<float4*>(a.o_part + slot * kD) + i, v);
       }

@@ -395,6 +395,49 @@ def test_calibrate_in_one_kernel(cuda_lib, B, Hq, Hkv, L, W, pool, budget, n_cal
         assert torch.equal(getattr(got, name), getattr(st, name)), name
     assert torch.allclose(got.LSE_c, st.LSE_c, rtol=0, atol=1e-5) and torch.allclose(got.O_c, st.O_c, rtol=1e-5, atol=1e-6)
 
+
+@pytest.mark.parametrize("G,n_cal,octave", [(1, 1, 0), (2, 16, 0), (3, 16, 0), (4, 16, 0), (8, 16, 0), (2, 16, 200)])
+def test_infinite_value_of_an_evicted_row_stays_infinite(cuda_lib, G, n_cal, octave):
+    """The calibration rows of a small unit lie on the lanes two or four times, each copy with a part of the keys: an infinite
+    value of V makes its column of O_c infinite (NaN where the probability is zero) and leaves every other element as it was."""
+    from paper_2507_19906_b200 import binding as cd
+    L, W, budget = 700, 16, 100
+    cfg = wl.small_config(B=1, Hq=G, Hkv=1, L=L, window=W, pool=5, budget=budget, steps=1, n_sink=2, n_heavy=14)
+    Q, K, V = (to_dev(x) for x in _inputs(cfg))
+    p = cd.make_params(B=1, Hq=G, Hkv=1, L=L, window=W, pool=5, budget=budget, n_cal=n_cal, cap=budget)
+    lse = None
+
+    def run(V):
+        st = cd.alloc_layer_state(p)
+        before = cd.calidrop_launch_count()
+        cd.calidrop_compress(p, Q, K, V, lse, st.kept_idx, st.K_kept, st.V_kept, st.O_c, st.LSE_c, st.C_q, st.ws_compress)
+        torch.cuda.synchronize()
+        assert cd.calidrop_launch_count() - before == 1
+        off = cd.calidrop_compress_workspace_layout(p).row_lse_offset
+        return st, st.ws_compress[off:off + 4 * G * W].view(torch.float32).clone()
+
+    st, row_lse = run(V)
+    if octave:   # the first row's probabilities are all zero
+        lse = row_lse.clone()
+        lse[W - 1] += octave
+        lse = lse.view(1, G, W)
+        st, _ = run(V)
+    kept = set(st.kept_idx.flatten().tolist())
+    evicted = [t for t in range(L - W) if t not in kept]
+    for t in (evicted[0], evicted[len(evicted) // 2], evicted[-1]):
+        Vi = V.clone()
+        Vi[0, 0, t, 77] = -float("inf")
+        got, _ = run(Vi)
+        assert torch.equal(got.kept_idx, st.kept_idx) and torch.equal(got.LSE_c, st.LSE_c)
+        col = got.O_c[0, :, :, 77].flatten()
+        zero = torch.zeros_like(col, dtype=torch.bool)
+        if octave:
+            zero[n_cal - 1] = True
+        assert torch.all(torch.isneginf(col[~zero])), t
+        other = torch.arange(128, device="cuda") != 77
+        assert torch.equal(got.O_c[..., other], st.O_c[..., other]), t
+
+
 def test_supplied_row_lse_matches_self_computed(cuda_lib):
     cfg = wl.small_config(B=1, Hq=4, Hkv=2, L=400, window=16, pool=7, budget=64)
     Q, K, V = _inputs(cfg)
