@@ -175,7 +175,9 @@ DecodeCommon plan_decode(const calidrop_params* p, const DecodeWs& w, int n_laye
       if ((ns == 1 && nc == 1) || t < best) { best = t; a.nsplit = ns; a.nclu = nc; }
     }
   }
-  a.rows_per_split = (n_kv + a.nsplit * a.nclu - 1) / (a.nsplit * a.nclu);
+  // Slices begin at multiples of the 16 rows that a warp takes at a time and a copy brings: the longest one has as many of them
+  // either way, and none brings rows of its neighbour (probability zero, but zero times an infinite value is NaN).
+  a.rows_per_split = ((n_kv + a.nsplit * a.nclu - 1) / (a.nsplit * a.nclu) + 15) / 16 * 16;
   a.scale2 = scale2_of(p);
   a.theta1 = p->theta1; a.theta2 = p->theta2; a.always_apply = p->theta2 <= -1.0f;
   // The workspace is laid out array by array with the layer index outermost inside each

@@ -438,6 +438,37 @@ def test_infinite_value_of_an_evicted_row_stays_infinite(cuda_lib, G, n_cal, oct
         assert torch.equal(got.O_c[..., other], st.O_c[..., other]), t
 
 
+@pytest.mark.parametrize("Hkv,G,n", [(1, 2, 1997), (2, 8, 529), (8, 4, 1000), (1, 1, 33)])
+def test_decode_with_an_infinite_value_in_any_row(cuda_lib, Hkv, G, n):
+    """An infinite value of V in one row makes its column of the output infinite and touches no other, at whatever distance
+    from the ends of the slices that a unit is cut into: no CTA may multiply a neighbour's rows by zero."""
+    from paper_2507_19906_b200 import binding as cd
+    g = torch.Generator(device="cuda").manual_seed(n)
+    rn = lambda *sh: torch.randn(sh, generator=g, device="cuda")
+    p = cd.make_params(B=1, Hq=G * Hkv, Hkv=Hkv, L=n + 64, window=16, pool=7, budget=n, n_cal=4, cap=n, theta2=-1.0)
+    st = cd.alloc_layer_state(p)
+    for t in (st.K_kept, st.V_kept, st.C_q, st.O_c, st.LSE_c):
+        t.copy_(rn(*t.shape))
+    q = rn(1, G * Hkv, 128).to(torch.bfloat16)
+    lse, flags = torch.zeros((1, G * Hkv), device="cuda"), torch.zeros((1, G * Hkv), dtype=torch.uint8, device="cuda")
+
+    def run():
+        out = torch.zeros((1, G * Hkv, 128), dtype=torch.bfloat16, device="cuda")
+        cd.calidrop_decode(p, q, None, None, st.K_kept, st.V_kept, n, st.O_c, st.LSE_c, st.C_q, out, lse, flags, st.ws_decode)
+        return out
+
+    clean = run()
+    other = torch.arange(128, device="cuda") != 77
+    ok = torch.ones((), dtype=torch.bool, device="cuda")
+    for t in range(n):
+        was = st.V_kept[0, :, t, 77].clone()
+        st.V_kept[0, :, t, 77] = float("inf")
+        out = run()
+        ok &= torch.all(torch.isposinf(out[..., 77])) & torch.all(out[..., other] == clean[..., other])
+        st.V_kept[0, :, t, 77] = was
+    assert bool(ok)
+
+
 def test_supplied_row_lse_matches_self_computed(cuda_lib):
     cfg = wl.small_config(B=1, Hq=4, Hkv=2, L=400, window=16, pool=7, budget=64)
     Q, K, V = _inputs(cfg)
