@@ -652,27 +652,30 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
     bool rho_done = false;
     for (int sb = group; sb < n_sb; sb += 2) {
       const int s = sb % kSlots, k = sb / kSlots;
-      const bool ok = mbar_wait(smem_u32(&s_full[s][k & 1]), (k >> 1) & 1, abort_flag, a.status, 0x200u + sb);
       const int row_base = r0 + (sb - n_cf) * kSlotRows + sub * kBlkRows;
+      // D1: the warp that meets row kv_len takes it from k_new / v_new, on their way while the slot is.  (Rows of calibration
+      // queries have a row_base of -16 at most.)
+      const bool new_row = a.has_new && a.kv_len >= row_base && a.kv_len < row_base + kBlkRows;
+      uint4 v_new;
+      if (new_row)
+        v_new = *reinterpret_cast<const uint4*>((const unsigned char*)(lane < 16 ? P.k_new : P.v_new) +
+                                                (size_t)unit * kRowBytes + (lane & 15) * 16);
+      const bool ok = mbar_wait(smem_u32(&s_full[s][k & 1]), (k >> 1) & 1, abort_flag, a.status, 0x200u + sb);
       if (kOne && sb < n_cf) {
         if (!RECAL && ok && mbar_wait(smem_u32(&s_qfull), 0, abort_flag, a.status, 0x400u)) rho_slot(s, sb, sub);
       } else if (ok && row_base < r1) {
         const Planes pl = planes_of<S>(kSlotRows == kWideRows && r1 - r0 - (sb - n_cf) * kSlotRows >= kSlotRows);
         const uint32_t sK = ring + s * kSlotBytes + sub * pl.block;   // this warp's block
         const uint32_t sV = sK + 2 * kPlaneBytes;
-        // D1: the warp that meets row kv_len takes it from k_new / v_new (the cache row has not
-        // been written yet: what arrived for it is stale) and appends it to the cache
-        if (a.has_new && a.kv_len >= row_base && a.kv_len < row_base + kBlkRows) {
+        // ... and appends it to the cache (whose row has not been written yet: what arrived for it is stale)
+        if (new_row) {
           const int chunk = lane & 15;
           const int rs = a.kv_len - row_base;  // row inside the block
-          const unsigned char* src = (const unsigned char*)(lane < 16 ? P.k_new : P.v_new) +
-                                     (size_t)unit * kRowBytes + chunk * 16;
-          const uint4 v = *reinterpret_cast<const uint4*>(src);
           unsigned char* dstg = (unsigned char*)(lane < 16 ? P.K : P.V) +
                                 ((size_t)unit * a.cap + a.kv_len) * kRowBytes + chunk * 16;
-          *reinterpret_cast<uint4*>(dstg) = v;
+          *reinterpret_cast<uint4*>(dstg) = v_new;
           *reinterpret_cast<uint4*>(ring_ptr + s * kSlotBytes + sub * pl.block + (lane < 16 ? 0 : 2 * kPlaneBytes) +
-                                    block_off(pl, rs, chunk)) = v;
+                                    block_off(pl, rs, chunk)) = v_new;
           __syncwarp();
         }
         // S^T: two accumulators (even and odd k-steps) halve the dependent chain
