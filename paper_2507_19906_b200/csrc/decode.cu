@@ -653,8 +653,8 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
     for (int sb = group; sb < n_sb; sb += 2) {
       const int s = sb % kSlots, k = sb / kSlots;
       const int row_base = r0 + (sb - n_cf) * kSlotRows + sub * kBlkRows;
-      // D1: the warp that meets row kv_len takes it from k_new / v_new, on their way while the slot is.  (Rows of calibration
-      // queries have a row_base of -16 at most.)
+      // D1: the warp that meets row kv_len takes it from k_new / v_new, on their way while the slot is.  (Loaded once the slot had
+      // arrived, 8 units x 700 rows took 4.89 instead of 4.71 us.  Rows of calibration queries have a row_base of -16 at most.)
       const bool new_row = a.has_new && a.kv_len >= row_base && a.kv_len < row_base + kBlkRows;
       uint4 v_new;
       if (new_row)
