@@ -162,8 +162,8 @@ size_t accum_scores_workspace_bytes(int B, int Hq, int L);
 cudaError_t launch_accum_scores(int B, int Hq, int Hkv, int L, float scale2, const void* Q_full, const void* K,
                                 char* wsp, float* scores, cudaStream_t st);
 // decode.cu
-// Fills the TMA views of one layer; false when the driver refuses the encoding.
-bool make_decode_maps(const DecodeCommon& c, const DecodeLayerPtrs& L, DecodeLayerMaps* out);
+// Fills the TMA views of one layer, of a decode step or of a recomputation; false when the driver refuses the encoding.
+bool make_decode_maps(const DecodeCommon& c, const DecodeLayerPtrs& L, bool recal, DecodeLayerMaps* out);
 cudaError_t launch_decode(const DecodeArgsT<1>& a, cudaStream_t st);
 cudaError_t launch_decode(const DecodeArgsT<kDecodeMaxLayers>& a, cudaStream_t st);
 // The same stream over the evicted KV (K, V of the layer = the compacted evicted rows), rewriting

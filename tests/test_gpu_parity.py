@@ -1098,6 +1098,33 @@ def test_recalibrate_launch_shapes_against_fp64(cuda_lib, units, G, n_evict, lay
         assert torch.equal(got[:, :, ::2], was[:, :, ::2])
 
 
+@pytest.mark.parametrize("units,n", [(2, 2000), (160, 300)])
+def test_decode_and_recalibrate_over_the_same_buffers(cuda_lib, units, n):
+    """A recomputation brings its rows by other copies than a decode step: each has its own descriptors, also where the two read
+    the same buffers with the same capacity, in whatever order.  Without a calibration applied they compute the same sums."""
+    cd = cuda_lib
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    rn = lambda *sh: torch.randn(sh, generator=gen, device="cuda")
+    p = cd.make_params(B=1, Hq=units, Hkv=units, n_cal=1, cap=n, theta2=2.0)
+    q, C_q = rn(1, units, 128).to(torch.bfloat16), rn(1, units, 1, 128).to(torch.bfloat16)
+    K, V = (rn(1, units, n, 128).to(torch.bfloat16) for _ in range(2))
+    O_c, LSE_c = rn(1, units, 1, 128), rn(1, units, 1)
+    out, lse = torch.empty((1, units, 128), dtype=torch.bfloat16, device="cuda"), torch.empty((1, units), device="cuda")
+    ws = torch.zeros((cd.calidrop_decode_workspace_bytes(p, n),), dtype=torch.uint8, device="cuda")
+    s = torch.einsum("ud,utd->ut", q[0].double(), K[0].double()) / 128 ** 0.5
+    want = torch.einsum("ut,utd->ud", torch.softmax(s, -1), V[0].double())
+    for _ in range(2):
+        out.zero_(), lse.zero_(), O_c.zero_(), LSE_c.zero_()
+        cd.calidrop_decode(p, q, None, None, K, V, n, O_c, LSE_c, C_q, out, lse, None, ws)
+        cd.calidrop_recalibrate(p, q, K, V, n, 0, O_c, LSE_c, C_q, ws)
+        off = cd.calidrop_decode_workspace_status_offset(p)
+        assert int(ws[off:off + 4].view(torch.int32).item()) == 0
+        for got in (out[0].double(), O_c[0, :, 0].double()):
+            assert (got - want).abs().max() < 2e-2 and (got - want).abs().mean() < 2e-3
+        for got in (lse[0], LSE_c[0, :, 0]):
+            assert (got.double() - torch.logsumexp(s, -1)).abs().max() < 1e-3
+
+
 @pytest.mark.parametrize("B,Hq,Hkv,L,W,budget,n_cal,slot", [
     (1, 4, 2, 600, 16, 80, 1, 0),          # the paper's single calibration query
     (2, 8, 2, 1500, 32, 256, 4, 2),        # G = 4, one of four rows rewritten
