@@ -117,31 +117,67 @@ __device__ __forceinline__ bool mbar_wait_cluster(Ctl* ctl, uint32_t bar, uint32
   return true;
 }
 
+__device__ __forceinline__ bool nonfinite_bf16x4(uint2 x) {
+  return (x.x & 0x7f80u) == 0x7f80u || (x.x & 0x7f800000u) == 0x7f800000u || (x.y & 0x7f80u) == 0x7f80u ||
+         (x.y & 0x7f800000u) == 0x7f800000u;
+}
 // Elements 4 lane .. 4 lane + 3 of a row's partial O over n keys, for a row with copies whose copies added up to NaN: a copy has
 // zeros for the other copies' keys, and zero times an infinite value of V is NaN where the row itself has a probability above zero.
 // Only products that are not finite decide such an element (`l`, the row's sum, tells whether a probability can be one); none
-// found, it stays as it is.  Out of line: finite inputs never get here, and the instruction fetch of code beside the loop costs all.
+// found, it stays as it is.  A whole warp works on a row, four elements a lane, until all of its NaN are settled.  Out of line:
+// finite inputs never get here, and the instruction fetch of code beside the loop costs all.  (Every lane for itself, with a
+// product of 128 terms for each key that it met, a call of 8 units x 8192 keys x 64 calibration rows whose values were all infinite
+// took 11.2 ms; a key per lane 1.5, bound by the uncoalesced loads; now 0.8, and 0.05 where both signs meet.)
 __device__ __noinline__ float4 refold_nonfinite(float4 o, const __nv_bfloat16* q, const __nv_bfloat16* K, const __nv_bfloat16* V,
                                                 int n, const uint32_t* mask, float scale2, float nlse2, float l, int lane) {
+  constexpr int kKeys = 8;   // at a time
   if (isnan(l)) return o;
+  const bool all = !isfinite(l);
+  const uint2 q4 = reinterpret_cast<const uint2*>(q)[lane];
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int t = 0; t < n; ++t) {
-    const __nv_bfloat16* vp = V + (size_t)t * kD + 4 * lane;
-    const float4 v = make_float4(__bfloat162float(vp[0]), __bfloat162float(vp[1]), __bfloat162float(vp[2]), __bfloat162float(vp[3]));
-    if (isfinite(v.x) && isfinite(v.y) && isfinite(v.z) && isfinite(v.w) && isfinite(l)) continue;
-    float p = 0.f;
-    if (!((mask[t >> 5] >> (t & 31)) & 1u)) {
-      float s = 0.f;
-      for (int d = 0; d < kD; ++d) s = fmaf(__bfloat162float(q[d]), __bfloat162float(K[(size_t)t * kD + d]), s);
-      p = __bfloat162float(__float2bfloat16(exp2f(fmaf(s, scale2, nlse2))));
+#pragma unroll 1
+  for (int t0 = 0; t0 < n; t0 += kKeys) {
+    uint2 v[kKeys], k[kKeys];
+    bool any = false;
+#pragma unroll
+    for (int j = 0; j < kKeys; ++j) {
+      const size_t at = (size_t)min(t0 + j, n - 1) * (kD / 4) + lane;
+      v[j] = reinterpret_cast<const uint2*>(V)[at];
+      k[j] = reinterpret_cast<const uint2*>(K)[at];
     }
-    acc.x = fmaf(p, v.x, acc.x);
-    acc.y = fmaf(p, v.y, acc.y);
-    acc.z = fmaf(p, v.z, acc.z);
-    acc.w = fmaf(p, v.w, acc.w);
+#pragma unroll
+    for (int j = 0; j < kKeys; ++j) any = any || nonfinite_bf16x4(v[j]);
+    if (!__any_sync(0xffffffffu, all || any)) continue;
+    float s[kKeys], mine = 0.f;   // mine: of key lane % kKeys
+#pragma unroll
+    for (int j = 0; j < kKeys; ++j) {
+      s[j] = fmaf(bf16_hi(q4.x), bf16_hi(k[j].x), bf16_lo(q4.x) * bf16_lo(k[j].x));
+      s[j] = fmaf(bf16_hi(q4.y), bf16_hi(k[j].y), fmaf(bf16_lo(q4.y), bf16_lo(k[j].y), s[j]));
+    }
+#pragma unroll
+    for (int o2 = 16; o2 > 0; o2 >>= 1)
+#pragma unroll
+      for (int j = 0; j < kKeys; ++j) s[j] += __shfl_xor_sync(0xffffffffu, s[j], o2);
+#pragma unroll
+    for (int j = 0; j < kKeys; ++j) mine = lane % kKeys == j ? s[j] : mine;
+    const int t = min(t0 + lane % kKeys, n - 1);
+    const float p = (mask[t >> 5] >> (t & 31)) & 1u ? 0.f : __bfloat162float(__float2bfloat16(exp2f(fmaf(mine, scale2, nlse2))));
+#pragma unroll
+    for (int j = 0; j < kKeys; ++j) {
+      const float pj = __shfl_sync(0xffffffffu, p, j);
+      if (t0 + j < n && (all || nonfinite_bf16x4(v[j]))) {
+        acc.x = fmaf(pj, bf16_lo(v[j].x), acc.x);
+        acc.y = fmaf(pj, bf16_hi(v[j].x), acc.y);
+        acc.z = fmaf(pj, bf16_lo(v[j].y), acc.z);
+        acc.w = fmaf(pj, bf16_hi(v[j].y), acc.w);
+      }
+    }
+    const bool settled = (isnan(acc.x) || !isnan(o.x)) && (isnan(acc.y) || !isnan(o.y)) && (isnan(acc.z) || !isnan(o.z)) &&
+                         (isnan(acc.w) || !isnan(o.w));
+    if (__all_sync(0xffffffffu, settled)) break;
   }
-  return make_float4(isfinite(acc.x) ? o.x : acc.x, isfinite(acc.y) ? o.y : acc.y, isfinite(acc.z) ? o.z : acc.z,
-                     isfinite(acc.w) ? o.w : acc.w);
+  return make_float4(isnan(o.x) && !isfinite(acc.x) ? acc.x : o.x, isnan(o.y) && !isfinite(acc.y) ? acc.y : o.y,
+                     isnan(o.z) && !isfinite(acc.z) ? acc.z : o.z, isnan(o.w) && !isfinite(acc.w) ? acc.w : o.w);
 }
 
 // Columns of this thread's lane: the load, and its completion (see tmem_ld32_issue).
@@ -1093,7 +1129,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_
           const float4 u = *reinterpret_cast<const float4*>(obuf + (c * rows_c + row) * kOStride + 4 * lane);
           v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
         }
-        if (a.lg_rep_c > 0 && (isnan(v.x) || isnan(v.y) || isnan(v.z) || isnan(v.w))) {
+        if (a.lg_rep_c > 0 && __any_sync(0xffffffffu, isnan(v.x) || isnan(v.y) || isnan(v.z) || isnan(v.w))) {   // (a warp to a row)
           const int wrow = row / a.n_cal * a.W + a.W - a.n_cal + row % a.n_cal;
           float l = 0.f;
           for (int c = 0; c < 1 << a.lg_rep_c; ++c)

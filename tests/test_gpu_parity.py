@@ -438,6 +438,48 @@ def test_infinite_value_of_an_evicted_row_stays_infinite(cuda_lib, G, n_cal, oct
         assert torch.equal(got.O_c[..., other], st.O_c[..., other]), t
 
 
+def test_infinite_values_of_all_evicted_rows(cuda_lib):
+    """As above with an infinite value in every evicted row: of one sign the column of O_c is infinite, of both it is NaN, the
+    other columns are as they were.  Settling the elements takes a bounded time (with a product of 128 terms per thread and
+    key it took 11 ms where a call of finite values takes 0.04; now 0.8)."""
+    cd = cuda_lib
+    units, G, W, L, budget = 8, 8, 8, 8192, 108
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    rn = lambda *sh: torch.randn(sh, generator=gen, device="cuda").to(torch.bfloat16)
+    Q, K, V = rn(1, units * G, W, 128), rn(1, units, L, 128), rn(1, units, L, 128)
+    p = cd.make_params(B=1, Hq=units * G, Hkv=units, L=L, window=W, pool=5, budget=budget, n_cal=W, cap=budget)
+
+    def run(V):
+        st = cd.alloc_layer_state(p)
+        e = [torch.cuda.Event(enable_timing=True) for _ in range(4)]
+        before = cd.calidrop_launch_count()
+        for i in range(4):
+            e[i].record()
+            if i < 3:
+                cd.calidrop_compress(p, Q, K, V, None, st.kept_idx, st.K_kept, st.V_kept, st.O_c, st.LSE_c, st.C_q, st.ws_compress)
+        torch.cuda.synchronize()
+        assert cd.calidrop_launch_count() - before == 3
+        off = cd.calidrop_compress_workspace_layout(p).status_offset
+        assert int(st.ws_compress[off:off + 4].view(torch.int32).item()) == 0
+        return st, min(e[i].elapsed_time(e[i + 1]) for i in range(3))
+
+    st, _ = run(V)
+    evicted = torch.ones((units, L), dtype=torch.bool, device="cuda")
+    evicted[:, L - W:] = False
+    evicted.scatter_(1, st.kept_idx[0].long(), False)
+    other = torch.arange(128, device="cuda") != 77
+    for alternate in (False, True):
+        Vi = V.clone()
+        Vi[0, :, :, 77][evicted] = float("inf")
+        if alternate:
+            Vi[0, :, 1::2, 77] *= -1
+        got, ms = run(Vi)
+        assert torch.equal(got.kept_idx, st.kept_idx) and torch.equal(got.LSE_c, st.LSE_c)
+        assert torch.all(torch.isnan(got.O_c[..., 77]) if alternate else torch.isposinf(got.O_c[..., 77]))
+        assert torch.equal(got.O_c[..., other], st.O_c[..., other])
+        assert ms < 4.0, ms
+
+
 @pytest.mark.parametrize("Hkv,G,n", [(1, 2, 1997), (2, 8, 529), (8, 4, 1000), (1, 1, 33)])
 def test_decode_with_an_infinite_value_in_any_row(cuda_lib, Hkv, G, n):
     """An infinite value of V in one row makes its column of the output infinite and touches no other, at whatever distance
