@@ -10,7 +10,7 @@
 //   (for a caller's kept list, calidrop_calibrate, V and the selection fall away)
 //   C  calibration: S = Q_c K^T again, probabilities of the evicted keys as the A operand of O += P V
 //   reduce: every CTA finishes a share of the calibration rows from the partial O that all left in the workspace; one warp copies the
-//      retained rows meanwhile
+//      retained rows meanwhile (up to kCopyRows a CTA: more of them take a kernel on all SMs behind this one)
 // K is streamed once per phase through one TMA ring (from L2 after the first time), so the keys of a CTA are not limited
 // by its shared memory, and the loads of phase C run during the selection.  What the CTAs of a cluster tell each
 // other is PUSHED with asynchronous stores that report their bytes to an mbarrier of the receiver; only the partial O, which is
@@ -59,6 +59,10 @@ constexpr int kTileBytes = kKvTileBytes;   // 32 KB
 constexpr int kOStride = kD + 4;           // row stride of the partial O in shared memory: no bank conflicts
 constexpr int kQuarterTiles = 16;          // up to this many tiles the four groups share a tile's votes
 constexpr int kHistCopies = 8;
+// Retained rows of a CTA that this kernel compacts itself.  Beyond, the SMs without a CTA of it are missed, and a kernel of their own
+// behind it compacts the rows, us: 100 units x 4000 keys, 3200 of them kept, 159 -> 133; 8 x 30000, 24000 kept, 113 -> 91; 1 x
+// 30000, 12000 kept, 51 -> 46; 40 x 8000, 1600 kept (533 a CTA) 71.6 and 72.2; 8 x 8192, 1638 kept (164 a CTA) 29.5 and 30.9.
+constexpr int kCopyRows = 512;
 constexpr int kSmemMax = 221 * 1024;       // dynamic; the static arrays take less than 6 KB
 
 struct ClusterArgs {
@@ -67,6 +71,7 @@ struct ClusterArgs {
   int lg_rep, lg_rep_c;   // copies of the window rows / calibration rows on the 128 lanes
   int n_pad;              // phase V: columns of an accumulator, 32, 64 or 128
   int pool, k_sel, n_kept, n_calib, bitmap_words;
+  int n_copy;             // retained rows that this kernel compacts: all of them or none
   int stage_off, keys_off, mask_off;   // bytes from the scratch area's start
   float scale2;
   const float* row_lse;   // the caller's, or null
@@ -372,7 +377,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_
   // to one warp from the selection on, to the consumers when they are done.  (By the one warp alone, 512 rows a CTA
   // took 8 us longer than everything else.)
   auto compact_rows = [&]() {
-    const int per = (a.n_kept + n_clu - 1) / n_clu, i0 = min(a.n_kept, rank * per), i1 = min(a.n_kept, i0 + per);
+    const int per = (a.n_copy + n_clu - 1) / n_clu, i0 = min(a.n_copy, rank * per), i1 = min(a.n_copy, i0 + per);
     const int32_t* list = a.kept_idx + (size_t)unit * a.n_kept;
     constexpr int kRows = 4;
     const int sub = lane >> 4, chunk = lane & 15;
@@ -1205,6 +1210,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_
 
 struct ClusterPlan {
   int tiles_per_cta, n_clu, stages, stage_off, keys_off, mask_off, smem;
+  bool copy_behind;   // the retained rows are compacted by a kernel of their own
 };
 
 int round_up(int x, int to) { return (x + to - 1) / to * to; }
@@ -1302,6 +1308,7 @@ cudaError_t launch_kernel(const ClusterArgs& a, const ClusterPlan& p, int units,
 // x 32768 125 and 126; 32 x 2048 46 and 26, x 20000 146 and 129; with the caller's row LSE 8 x 32768 65 and 63, 16 x 24576 80 and 76,
 // 64 x 12288 135 and 122 and, with a ring of three tiles, x 16384 163 and 172.  For a given kept list 8 x 1000 24 and 12, x 8192 31 and
 // 21, x 45000 77 and 66, 2 x 24000 41 and 28, 64 x 8192 100 and 77; with the caller's row LSE 8 x 8192 22 and 14, 16 x 32768 65 and 54.
+// (The compaction costs both ways alike, but for 3 us where it is a kernel behind this one.)
 bool plan_cluster(const CompressGeom& g, bool stats, bool given, ClusterPlan* p) {
   if (g.keep_all || g.n_cand < 1 || g.G * g.W > kMaxRows || g.pool >> 1 > kHaloMax) return false;
   if (g.sized && g.n_calib == 0) return false;
@@ -1316,14 +1323,15 @@ bool plan_cluster(const CompressGeom& g, bool stats, bool given, ClusterPlan* p)
     const double tiles = g.units * n_tiles / 148.0;
     const double here = given ? (stats ? 10.5 + 1.55 * t : 8.7 + 0.95 * t) : 13.0 + (stats ? 2.58 : 1.9) * t;
     const double there = given ? (stats ? 30.0 + 2.3 * tiles : 19.0 + 1.75 * tiles) : 37.5 + (stats ? 3.24 : 2.16) * tiles;
-    return here < there && lay_out(g, stats, t, p);
+    p->copy_behind = g.n_kept > kCopyRows * n_clu;
+    return here + (p->copy_behind ? 3.0 : 0.0) < there && lay_out(g, stats, t, p);
   }
   return false;
 }
 
 }  // namespace
 
-// The whole step in one launch, or (`given`) the calibration and compaction for the kept list in kept_idx; *taken is false (and
+// The whole step in one launch (two with many retained rows), or (`given`) the calibration and compaction for the kept list in kept_idx; *taken is false (and
 // nothing launched) where the separate kernels are to be used.
 cudaError_t launch_compress_cluster(const CompressGeom& g, const CompressWs& ws, const void* Q_obs, const void* K, const void* V,
                                     const float* row_lse, char* wsp, int32_t* kept_idx, float* O_c, float* LSE_c, void* C_q,
@@ -1368,9 +1376,12 @@ cudaError_t launch_compress_cluster(const CompressGeom& g, const CompressWs& ws,
       !make_tensor_map_bf16(&qcm, (const char*)Q_obs + (size_t)(g.W - g.n_cal) * 256, 4, cd, cs, cb) ||
       !make_tensor_map_bf16(&km, K, 3, kd, ks, kb) || !make_tensor_map_bf16(&vm, V, 3, kd, ks, kb))
     return cudaErrorInvalidValue;
-  if (given) return launch_kernel<false, true>(a, p, g.units, qm, qcm, km, vm, st);
-  return g.sized ? launch_kernel<true, false>(a, p, g.units, qm, qcm, km, vm, st)
-                 : launch_kernel<false, false>(a, p, g.units, qm, qcm, km, vm, st);
+  a.n_copy = p.copy_behind ? 0 : g.n_kept;
+  cudaError_t e = given     ? launch_kernel<false, true>(a, p, g.units, qm, qcm, km, vm, st)
+                  : g.sized ? launch_kernel<true, false>(a, p, g.units, qm, qcm, km, vm, st)
+                            : launch_kernel<false, false>(a, p, g.units, qm, qcm, km, vm, st);
+  if (e == cudaSuccess && p.copy_behind) e = launch_gather(g, K, V, kept_idx, gather.K_out, gather.V_out, st);
+  return e;
 }
 
 }  // namespace calidrop

@@ -396,6 +396,32 @@ def test_calibrate_in_one_kernel(cuda_lib, B, Hq, Hkv, L, W, pool, budget, n_cal
     assert torch.allclose(got.LSE_c, st.LSE_c, rtol=0, atol=1e-5) and torch.allclose(got.O_c, st.O_c, rtol=1e-5, atol=1e-6)
 
 
+@pytest.mark.parametrize("units,L,W,budget,launches", [
+    (100, 900, 8, 512, 1),      # one CTA to a unit: as many rows as the cluster kernel compacts itself
+    (100, 900, 8, 513, 2),      # ... one more
+    (60, 1500, 16, 1484, 2),    # two CTAs, sixteen evicted rows
+    (60, 1500, 16, 1024, 1),
+])
+def test_compaction_of_many_rows_behind_the_cluster_kernel(cuda_lib, units, L, W, budget, launches):
+    """Beyond 512 retained rows a CTA, a kernel of their own compacts them, for a chosen and for a given kept list."""
+    from paper_2507_19906_b200 import binding as cd
+    cfg = wl.small_config(B=1, Hq=units, Hkv=units, L=L, window=W, pool=5, budget=budget, steps=1, n_sink=2, n_heavy=20)
+    Q, K, V = _inputs(cfg)
+    before = cd.calidrop_launch_count()
+    g = gpu_compress(Q, K, V, window=W, pool=5, budget=budget, n_cal=2, cap=budget + 3, keep_inputs=True)
+    assert cd.calidrop_launch_count() - before == launches
+    compare_compress(g, Q, K, V, window=W, pool=5, budget=budget, n_cal=2)
+    got = cd.alloc_layer_state(g.p)
+    before = cd.calidrop_launch_count()
+    cd.calidrop_calibrate(g.p, to_dev(Q), g.dK, g.dV, None, g.st.kept_idx, got.K_kept, got.V_kept, got.O_c, got.LSE_c, got.C_q,
+                          got.ws_compress)
+    torch.cuda.synchronize()
+    assert cd.calidrop_launch_count() - before == launches
+    assert torch.equal(got.K_kept[:, :, :budget], g.st.K_kept[:, :, :budget])
+    assert torch.equal(got.V_kept[:, :, :budget], g.st.V_kept[:, :, :budget])
+    assert torch.allclose(got.LSE_c, g.st.LSE_c, rtol=0, atol=1e-5) and torch.allclose(got.O_c, g.st.O_c, rtol=1e-5, atol=1e-6)
+
+
 @pytest.mark.parametrize("G,n_cal,octave", [(1, 1, 0), (2, 16, 0), (3, 16, 0), (4, 16, 0), (8, 16, 0), (2, 16, 200)])
 def test_infinite_value_of_an_evicted_row_stays_infinite(cuda_lib, G, n_cal, octave):
     """The calibration rows of a small unit lie on the lanes two or four times, each copy with a part of the keys: an infinite
