@@ -179,6 +179,7 @@ DecodeCommon plan_decode(const calidrop_params* p, const DecodeWs& w, int n_laye
   // either way, and none brings rows of its neighbour (probability zero, but zero times an infinite value is NaN).  Eight layers
   // of 4 units x 4333 rows 51.7 -> 49.2 us in all, 8 x 1300 rows 5.38 -> 5.09 us a launch.
   a.rows_per_split = ((n_kv + a.nsplit * a.nclu - 1) / (a.nsplit * a.nclu) + 15) / 16 * 16;
+  a.half_copies = a.rows_per_split <= kDecodeHalfCopyRows;
   a.scale2 = scale2_of(p);
   a.theta1 = p->theta1; a.theta2 = p->theta2; a.always_apply = p->theta2 <= -1.0f;
   // The workspace is laid out array by array with the layer index outermost inside each
@@ -489,7 +490,7 @@ int calidrop_recalibrate(const calidrop_params* p, const void* q, const void* K_
   args.c.recal_slot = slot;
   args.layer[0] = DecodeLayerPtrs{q, nullptr, nullptr, const_cast<void*>(K_evict), const_cast<void*>(V_evict), O_c,
                                   LSE_c, C_q, nullptr, nullptr, nullptr};
-  if (!make_decode_maps(args.c, args.layer[0], true, &args.maps[0])) return CALIDROP_CUDA_ERROR;
+  if (!make_decode_maps(args.c, args.layer[0], &args.maps[0])) return CALIDROP_CUDA_ERROR;
   cudaError_t e = launch_recalibrate(args, (cudaStream_t)stream);
   return e == cudaSuccess ? CALIDROP_OK : cuda_fail(e);
 }
@@ -540,7 +541,7 @@ int calidrop_decode_batched(const calidrop_params* p, int32_t n_layers, const ca
     const calidrop_decode_layer& L = layers[0];
     args.layer[0] = DecodeLayerPtrs{L.q, L.k_new, L.v_new, L.K_kept, L.V_kept, L.O_c, L.LSE_c, L.C_q,
                                     L.out, L.lse_out, L.flags};
-    if (!make_decode_maps(a, args.layer[0], false, &args.maps[0])) return CALIDROP_CUDA_ERROR;
+    if (!make_decode_maps(a, args.layer[0], &args.maps[0])) return CALIDROP_CUDA_ERROR;
     e = launch_decode(args, (cudaStream_t)stream);
   } else {
     static thread_local DecodeArgsT<kDecodeMaxLayers> args;
@@ -549,7 +550,7 @@ int calidrop_decode_batched(const calidrop_params* p, int32_t n_layers, const ca
       const calidrop_decode_layer& L = layers[i];
       args.layer[i] = DecodeLayerPtrs{L.q, L.k_new, L.v_new, L.K_kept, L.V_kept, L.O_c, L.LSE_c, L.C_q,
                                       L.out, L.lse_out, L.flags};
-      if (!make_decode_maps(a, args.layer[i], false, &args.maps[i])) return CALIDROP_CUDA_ERROR;
+      if (!make_decode_maps(a, args.layer[i], &args.maps[i])) return CALIDROP_CUDA_ERROR;
     }
     e = launch_decode(args, (cudaStream_t)stream);
   }

@@ -157,21 +157,13 @@ __device__ __forceinline__ bool mbar_wait_sit_out(uint32_t bar, uint32_t parity,
   }
   return true;
 }
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1,
-                                            int c2, uint64_t pol) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint "
-      "[%0], [%1, {%3, %4, %5}], [%2], %6;"
-      ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "l"(pol)
-      : "memory");
-}
-// Rows from row on of a unit, both halves of the head dimension.
+// Rows from row on of a unit: both halves of the head dimension, or half `h` alone where the map's box has one.
 __device__ __forceinline__ void tma_load_rows(uint32_t dst, const CUtensorMap* map, uint32_t bar, int row, int unit,
-                                              uint64_t pol) {
+                                              uint64_t pol, int h = 0) {
   asm volatile(
       "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint "
-      "[%0], [%1, {%3, %4, %5, %3}], [%2], %6;"
-      ::"r"(dst), "l"(map), "r"(bar), "r"(0), "r"(row), "r"(unit), "l"(pol)
+      "[%0], [%1, {%3, %4, %5, %7}], [%2], %6;"
+      ::"r"(dst), "l"(map), "r"(bar), "r"(0), "r"(row), "r"(unit), "l"(pol), "r"(h)
       : "memory");
 }
 
@@ -493,15 +485,10 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
     const int nrows = min(kSlotRows, r1 - row0);
     if (kSlotRows == kWideRows && nrows == kSlotRows) {
       mbar_expect_tx(bar, kSlotBytes);
-      if constexpr (RECAL) {   // (see make_decode_maps)
-        for (int h = 0; h < 2; ++h)
-          tma_load_3d(dst + h * kPlaneBytes, &TM.k64, bar, h * tc::kHalfCols, row0, unit, pol_stream);
-        for (int h = 0; h < 2; ++h)
-          tma_load_3d(dst + (2 + h) * kPlaneBytes, &TM.v64, bar, h * tc::kHalfCols, row0, unit, pol_stream);
-      } else {
-        tma_load_rows(dst, &TM.k64, bar, row0, unit, pol_stream);
-        tma_load_rows(dst + 2 * kPlaneBytes, &TM.v64, bar, row0, unit, pol_stream);
-      }
+      tma_load_rows(dst, &TM.k64, bar, row0, unit, pol_stream);
+      if (a.half_copies) tma_load_rows(dst + kPlaneBytes, &TM.k64, bar, row0, unit, pol_stream, 1);   // (see DecodeCommon)
+      tma_load_rows(dst + 2 * kPlaneBytes, &TM.v64, bar, row0, unit, pol_stream);
+      if (a.half_copies) tma_load_rows(dst + 3 * kPlaneBytes, &TM.v64, bar, row0, unit, pol_stream, 1);
     } else {
       const int nb = (nrows + kBlkRows - 1) / kBlkRows;
       mbar_expect_tx(bar, (uint32_t)nb * 4u * kBlkRows * 128u);
@@ -952,19 +939,15 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
 
 }  // namespace
 
-bool make_decode_maps(const DecodeCommon& c, const DecodeLayerPtrs& L, bool recal, DecodeLayerMaps* out) {
+bool make_decode_maps(const DecodeCommon& c, const DecodeLayerPtrs& L, DecodeLayerMaps* out) {
   // Three of the four maps cover all `cap` rows of the cache, whatever kv_len is, so one encoding
   // serves every step on a cache: a small per-thread table keyed by everything the encoding depends
-  // on (the two base addresses, the capacity, the number of units, the kind) returns them on the following
+  // on (the two base addresses, the capacity, the number of units, the kind of copies) returns them on the following
   // calls (encoding all four on every call cost more host time than the kernel runs).  An entry can
   // never be stale: equal keys encode equal maps.  The fourth, V in 16-row boxes, is the only one
   // through which rows at or beyond kv_len can reach a product; it ends at kv_len, so the TMA unit
   // delivers zeros for those rows, and is encoded per call.
-  // A whole slot of a decode step is one copy of K and one of V: less to issue where a launch is short, and faster from L2
-  // (8 units x 20000 rows 18.2 us a launch, with a copy per half of the head dimension 19.4).  A recomputation, whose rows come from
-  // HBM while the compaction ahead of it is still being written back, takes a copy per half: a pass of compaction, recomputation
-  // and decode over 32 units x 30720 rows 257.0 -> 255.1 us.
-  struct Entry { const void* K; const void* V; int cap, units; bool recal; DecodeLayerMaps maps; };
+  struct Entry { const void* K; const void* V; int cap, units, half_copies; DecodeLayerMaps maps; };
   constexpr int kEntries = 64;
   static thread_local Entry table[kEntries];
   static thread_local int next = 0;
@@ -973,20 +956,21 @@ bool make_decode_maps(const DecodeCommon& c, const DecodeLayerPtrs& L, bool reca
   const uint64_t dims_v16[2] = {(uint64_t)(c.kv_len > 0 ? c.kv_len : 1), (uint64_t)c.units};
   for (int i = 0; i < kEntries; ++i) {
     const Entry& e = table[i];
-    if (e.K == L.K && e.V == L.V && e.cap == c.cap && e.units == c.units && e.recal == recal && e.K != nullptr) {
+    if (e.K == L.K && e.V == L.V && e.cap == c.cap && e.units == c.units && e.half_copies == c.half_copies && e.K != nullptr) {
       *out = e.maps;
-      return make_tile_map_bf16(&out->v16, L.V, 3, dims_v16, strides, box16);
+      return make_tile_map_bf16(&out->v16, L.V, 3, dims_v16, strides, box16, 2);
     }
   }
   const uint64_t dims[2] = {(uint64_t)c.cap, (uint64_t)c.units};
-  const auto make64 = recal ? make_tensor_map_bf16 : make_tile_map_bf16;
-  if (!(make64(&out->k64, L.K, 3, dims, strides, box64) && make64(&out->v64, L.V, 3, dims, strides, box64) &&
-        make_tile_map_bf16(&out->k16, L.K, 3, dims, strides, box16) &&
-        make_tile_map_bf16(&out->v16, L.V, 3, dims_v16, strides, box16)))
+  const int halves = c.half_copies ? 1 : 2;
+  if (!(make_tile_map_bf16(&out->k64, L.K, 3, dims, strides, box64, halves) &&
+        make_tile_map_bf16(&out->v64, L.V, 3, dims, strides, box64, halves) &&
+        make_tile_map_bf16(&out->k16, L.K, 3, dims, strides, box16, 2) &&
+        make_tile_map_bf16(&out->v16, L.V, 3, dims_v16, strides, box16, 2)))
     return false;
   Entry& e = table[next];
   next = (next + 1) % kEntries;
-  e.K = L.K; e.V = L.V; e.cap = c.cap; e.units = c.units; e.recal = recal; e.maps = *out;
+  e.K = L.K; e.V = L.V; e.cap = c.cap; e.units = c.units; e.half_copies = c.half_copies; e.maps = *out;
   return true;
 }
 

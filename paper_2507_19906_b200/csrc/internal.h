@@ -48,8 +48,8 @@ struct DecodeLayerPtrs {
 };
 
 // TMA views of one layer's retained cache, [unit][row][128] bf16 with 128-byte swizzle: boxes of
-// 64 rows for whole ring slots and of 16 rows for the ragged end of a split.  k64, v64 and k16 span
-// the cache's capacity; v16 ends at row kv_len (rows beyond it arrive as zeros).
+// 64 rows for whole ring slots (k64 and v64: of 64 columns or, without half_copies, of whole rows) and of 16 rows for the ragged end of
+// a split.  k64, v64 and k16 span the cache's capacity; v16 ends at row kv_len (rows beyond it arrive as zeros).
 struct alignas(64) DecodeLayerMaps {
   CUtensorMap k64, v64, k16, v16;
 };
@@ -57,6 +57,7 @@ struct alignas(64) DecodeLayerMaps {
 constexpr int kCalibGroups = 4;  // softmax warpgroups of the calibration kernel: row-sum partials per slot
 constexpr int kDecodeMaxLayers = 32;
 constexpr int kDecodeMaxSplit = 64;
+constexpr int kDecodeHalfCopyRows = 576;   // rows of a slice (see DecodeCommon)
 constexpr int kDecodeTargetCtas = 148;  // one CTA of a launch on each of the 148 SMs
 
 struct DecodeCommon {
@@ -64,6 +65,11 @@ struct DecodeCommon {
   int units, n_layers, rows_per_split;
   int nsplit;  // CTAs per cluster (1, 2, 4, 8 or 16): the splits combined through distributed shared memory
   int nclu;    // clusters per (layer, unit); more than one only when few units share a long cache
+  // Whole ring slots are brought by a copy for each half of the head dimension instead of one for both.  Slices of up to nine slots
+  // take them: alone either way is as fast (32 units x 2049 rows 7.18 and 7.16 us a launch, 12 layers in turn 8.19 both), behind a
+  // recomputation and ahead of a compaction the halves are faster (the pass of the three over 32 units x 32768 rows 258.0 -> 254.9
+  // us).  One copy is faster in longer slices: 32 x 4100 rows 9.8 and 9.9, 8 x 12000 11.6 and 12.3, 32 x 30720 81.5 and 82.1.
+  int half_copies;
   float scale2, theta1, theta2;
   int always_apply;
   // workspace arrays, used only when nclu > 1: per-cluster partials and the arrival counters
@@ -162,8 +168,8 @@ size_t accum_scores_workspace_bytes(int B, int Hq, int L);
 cudaError_t launch_accum_scores(int B, int Hq, int Hkv, int L, float scale2, const void* Q_full, const void* K,
                                 char* wsp, float* scores, cudaStream_t st);
 // decode.cu
-// Fills the TMA views of one layer, of a decode step or of a recomputation; false when the driver refuses the encoding.
-bool make_decode_maps(const DecodeCommon& c, const DecodeLayerPtrs& L, bool recal, DecodeLayerMaps* out);
+// Fills the TMA views of one layer; false when the driver refuses the encoding.
+bool make_decode_maps(const DecodeCommon& c, const DecodeLayerPtrs& L, DecodeLayerMaps* out);
 cudaError_t launch_decode(const DecodeArgsT<1>& a, cudaStream_t st);
 cudaError_t launch_decode(const DecodeArgsT<kDecodeMaxLayers>& a, cudaStream_t st);
 // The same stream over the evicted KV (K, V of the layer = the compacted evicted rows), rewriting

@@ -314,9 +314,9 @@ __device__ __forceinline__ uint64_t kmajor_desc(uint32_t tile_base, uint32_t hal
 // second one on (the head dimension is implied); strides in bytes.  Returns false on failure.
 bool make_tensor_map_bf16(CUtensorMap* out, const void* base, int rank, const uint64_t* dims_from_1,
                           const uint64_t* strides_from_1, const uint32_t* box_from_1);
-// The same tensor with the halves of the head dimension as a last dimension, both in the box: one copy, with coordinates 0
-// in the first and the last dimension, brings whole rows, the two halves behind one another.
+// The same tensor with the halves of the head dimension as a last dimension, `halves` (1 or 2) of them in the box: with two, one
+// copy from coordinate 0 in the first and the last dimension brings whole rows, the two halves behind one another.
 bool make_tile_map_bf16(CUtensorMap* out, const void* base, int rank, const uint64_t* dims_from_1,
-                        const uint64_t* strides_from_1, const uint32_t* box_from_1);
+                        const uint64_t* strides_from_1, const uint32_t* box_from_1, int halves);
 
 }  // namespace calidrop

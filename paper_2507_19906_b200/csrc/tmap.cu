@@ -22,9 +22,9 @@ PFN_cuTensorMapEncodeTiled_v12000 resolve_encode() {
   return fn;
 }
 
-// `halves`: the two halves of the head dimension as a last dimension of their own, both in the box.
+// `halves`: the two halves of the head dimension as a last dimension of their own, so many in the box (0: no such dimension).
 bool encode_map(CUtensorMap* out, const void* base, int rank, const uint64_t* dims_from_1, const uint64_t* strides_from_1,
-                const uint32_t* box_from_1, bool halves) {
+                const uint32_t* box_from_1, int halves) {
   auto encode = resolve_encode();
   if (!encode || rank < 2 || rank + (halves ? 1 : 0) > 5) return false;
   cuuint64_t dims[5] = {(cuuint64_t)(halves ? tc::kHalfCols : kD), 1, 1, 1, 1};
@@ -40,7 +40,7 @@ bool encode_map(CUtensorMap* out, const void* base, int rank, const uint64_t* di
   if (halves) {
     dims[rank] = 2;
     strides[rank - 1] = tc::kLineBytes;
-    box[rank] = 2;
+    box[rank] = (cuuint32_t)halves;
     ++rank;
   }
   auto run = [&] {
@@ -61,12 +61,12 @@ bool encode_map(CUtensorMap* out, const void* base, int rank, const uint64_t* di
 
 bool make_tensor_map_bf16(CUtensorMap* out, const void* base, int rank, const uint64_t* dims_from_1,
                           const uint64_t* strides_from_1, const uint32_t* box_from_1) {
-  return encode_map(out, base, rank, dims_from_1, strides_from_1, box_from_1, false);
+  return encode_map(out, base, rank, dims_from_1, strides_from_1, box_from_1, 0);
 }
 
 bool make_tile_map_bf16(CUtensorMap* out, const void* base, int rank, const uint64_t* dims_from_1,
-                        const uint64_t* strides_from_1, const uint32_t* box_from_1) {
-  return encode_map(out, base, rank, dims_from_1, strides_from_1, box_from_1, true);
+                        const uint64_t* strides_from_1, const uint32_t* box_from_1, int halves) {
+  return encode_map(out, base, rank, dims_from_1, strides_from_1, box_from_1, halves);
 }
 
 }  // namespace calidrop

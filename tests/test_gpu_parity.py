@@ -1166,31 +1166,37 @@ def test_recalibrate_launch_shapes_against_fp64(cuda_lib, units, G, n_evict, lay
         assert torch.equal(got[:, :, ::2], was[:, :, ::2])
 
 
-@pytest.mark.parametrize("units,n", [(2, 2000), (160, 300)])
-def test_decode_and_recalibrate_over_the_same_buffers(cuda_lib, units, n):
-    """A recomputation brings its rows by other copies than a decode step: each has its own descriptors, also where the two read
-    the same buffers with the same capacity, in whatever order.  Without a calibration applied they compute the same sums."""
+@pytest.mark.parametrize("units,lengths", [
+    (160, (900, 576, 900, 577, 300, 592)),   # a CTA to a unit: slices of up to 576 rows come by a copy per half, longer ones by one
+    (4, (16000, 2000, 16000)),               # clusters
+])
+def test_slices_of_changing_length_over_the_same_buffers(cuda_lib, units, lengths):
+    """Short and long slices are brought by different copies, each with descriptors of its own, also where steps and recomputations
+    of either kind read the same buffers with the same capacity in turn.  Without a calibration applied both compute attention."""
     cd = cuda_lib
-    gen = torch.Generator(device="cuda").manual_seed(n)
+    gen = torch.Generator(device="cuda").manual_seed(units)
     rn = lambda *sh: torch.randn(sh, generator=gen, device="cuda")
-    p = cd.make_params(B=1, Hq=units, Hkv=units, n_cal=1, cap=n, theta2=2.0)
+    cap = max(lengths)
+    p = cd.make_params(B=1, Hq=units, Hkv=units, n_cal=1, cap=cap, theta2=2.0)
     q, C_q = rn(1, units, 128).to(torch.bfloat16), rn(1, units, 1, 128).to(torch.bfloat16)
-    K, V = (rn(1, units, n, 128).to(torch.bfloat16) for _ in range(2))
+    K, V = (rn(1, units, cap, 128).to(torch.bfloat16) for _ in range(2))
     O_c, LSE_c = rn(1, units, 1, 128), rn(1, units, 1)
     out, lse = torch.empty((1, units, 128), dtype=torch.bfloat16, device="cuda"), torch.empty((1, units), device="cuda")
-    ws = torch.zeros((cd.calidrop_decode_workspace_bytes(p, n),), dtype=torch.uint8, device="cuda")
+    ws = torch.zeros((cd.calidrop_decode_workspace_bytes(p, cap),), dtype=torch.uint8, device="cuda")
     s = torch.einsum("ud,utd->ut", q[0].double(), K[0].double()) / 128 ** 0.5
-    want = torch.einsum("ut,utd->ud", torch.softmax(s, -1), V[0].double())
-    for _ in range(2):
+    off = cd.calidrop_decode_workspace_status_offset(p)
+    for n in lengths:
+        want, want_lse = torch.einsum("ut,utd->ud", torch.softmax(s[:, :n], -1), V[0, :, :n].double()), torch.logsumexp(s[:, :n], -1)
         out.zero_(), lse.zero_(), O_c.zero_(), LSE_c.zero_()
         cd.calidrop_decode(p, q, None, None, K, V, n, O_c, LSE_c, C_q, out, lse, None, ws)
-        cd.calidrop_recalibrate(p, q, K, V, n, 0, O_c, LSE_c, C_q, ws)
-        off = cd.calidrop_decode_workspace_status_offset(p)
+        results = [(out[0], lse[0])]
+        if n == cap:   # the same buffers as evicted rows
+            cd.calidrop_recalibrate(p, q, K, V, n, 0, O_c, LSE_c, C_q, ws)
+            results.append((O_c[0, :, 0], LSE_c[0, :, 0]))
         assert int(ws[off:off + 4].view(torch.int32).item()) == 0
-        for got in (out[0].double(), O_c[0, :, 0].double()):
-            assert (got - want).abs().max() < 2e-2 and (got - want).abs().mean() < 2e-3
-        for got in (lse[0], LSE_c[0, :, 0]):
-            assert (got.double() - torch.logsumexp(s, -1)).abs().max() < 1e-3
+        for o, l in results:
+            assert (o.double() - want).abs().max() < 2e-2 and (o.double() - want).abs().mean() < 2e-3, n
+            assert (l.double() - want_lse).abs().max() < 1e-3, n
 
 
 @pytest.mark.parametrize("B,Hq,Hkv,L,W,budget,n_cal,slot", [
