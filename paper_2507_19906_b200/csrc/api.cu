@@ -144,6 +144,11 @@ DecodeWs make_decode_ws(const calidrop_params* p) {
   return w;
 }
 
+// Rows of the longest slice of a unit on `ctas` CTAs.  Slices begin at multiples of the 16 rows that a warp takes at a time and a
+// copy brings: the longest one has as many of them either way, and none brings rows of its neighbour (probability zero, but zero
+// times an infinite value is NaN).  Eight layers of 4 units x 4333 rows 51.7 -> 49.2 us in all, 8 x 1300 rows 5.38 -> 5.09 us a launch.
+int slice_rows(int n_kv, int ctas) { return ((n_kv + ctas - 1) / ctas + 15) / 16 * 16; }
+
 // Split plan and workspace carving of one decode-kernel launch over `cap_rows`-row caches.
 DecodeCommon plan_decode(const calidrop_params* p, const DecodeWs& w, int n_layers, int kv_len, int n_kv,
                          bool has_new, int cap_rows, bool recal, void* workspace) {
@@ -158,7 +163,9 @@ DecodeCommon plan_decode(const calidrop_params* p, const DecodeWs& w, int n_laye
   // rate of the memory if that is less; the meeting of several clusters costs 2.9, clusters of eight 0.25 and of sixteen 0.6
   // more than smaller ones.  Measured per launch, in a stream: 4 units x 300 rows 4.63 (4 CTAs) and 4.65 (8), x 700 rows 4.61 (8) and
   // 4.76 (16), x 1300 rows 5.15 and 4.75, x 2100 rows 5.72 and 4.93, x 4333 rows 6.93 and 5.94; 2 units x 15500 rows 8.99 (one
-  // cluster of 16) and 9.76 (three), x 40000 rows 16.3 and 12.5; 8 units x 20000 rows on 16 clusters of eight 28.1.
+  // cluster of 16) and 9.76 (three), x 40000 rows 16.3 and 12.5; 8 units x 20000 rows on 16 clusters of eight 28.1.  (A slice costs what
+  // is launched, whole blocks of 16 rows: by the unrounded length 4 units x 1200 rows took 8 CTAs and 4.88 us instead of 16 and
+  // 4.68, 7 x 2700 8 and 5.90 instead of 16 and 5.34, 15 x 1040 4 and 5.68 instead of 8 and 5.39, 1 x 12450 64 and 15.5 instead of 16 and 8.3.)
   const int units_total = a.units * n_layers;
   int want = decode_nsplit(units_total, n_kv);
   if (want > w.max_split) want = w.max_split;
@@ -169,16 +176,13 @@ DecodeCommon plan_decode(const calidrop_params* p, const DecodeWs& w, int n_laye
     const int resident = want > 1 ? decode_resident_clusters(ns) : 1;
     for (int nc = 1; resident > 0 && nc <= 8 && ns * nc <= want; ++nc) {
       const int rounds = (units_total * nc + resident - 1) / resident;
-      const double rows = (double)((n_kv + ns * nc - 1) / (ns * nc));
+      const double rows = (double)slice_rows(n_kv, ns * nc);
       const double slice = rows * 4.4e-3, share = memory / rounds;
       const double t = rounds * (4.3 + (slice > share ? slice : share)) + (nc > 1 ? 2.9 : 0.0) + (ns > 8 ? 0.6 : ns > 4 ? 0.25 : 0.0);
       if ((ns == 1 && nc == 1) || t < best) { best = t; a.nsplit = ns; a.nclu = nc; }
     }
   }
-  // Slices begin at multiples of the 16 rows that a warp takes at a time and a copy brings: the longest one has as many of them
-  // either way, and none brings rows of its neighbour (probability zero, but zero times an infinite value is NaN).  Eight layers
-  // of 4 units x 4333 rows 51.7 -> 49.2 us in all, 8 x 1300 rows 5.38 -> 5.09 us a launch.
-  a.rows_per_split = ((n_kv + a.nsplit * a.nclu - 1) / (a.nsplit * a.nclu) + 15) / 16 * 16;
+  a.rows_per_split = slice_rows(n_kv, a.nsplit * a.nclu);
   a.half_copies = a.rows_per_split <= kDecodeHalfCopyRows;
   a.scale2 = scale2_of(p);
   a.theta1 = p->theta1; a.theta2 = p->theta2; a.always_apply = p->theta2 <= -1.0f;

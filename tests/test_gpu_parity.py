@@ -956,6 +956,9 @@ def test_decode_ignores_cache_rows_beyond_kv_len(cuda_lib, B, Hq, Hkv, kv0, step
     (1, 2, 8, 9001, 64, (16, 1, 1)),      # ... 64, in two layers
     (1, 2, 8, 17000, 64, (8, 5, 1)),      # several clusters of eight
     (16, 1, 4, 2100, 8, (4, 1, 1)),       # more clusters of eight than the GPU holds at once
+    (4, 1, 4, 1199, 8, (16, 1, 1)),       # slices of 75 rows are launched as 80, of 150 as 160
+    (12, 1, 4, 649, 8, (8, 1, 1)),        # ... of 82 as 96, of 163 as 176
+    (1, 1, 8, 12449, 16, (16, 1, 1)),     # ... of 195 (on 64 CTAs) as 208
 ])
 def test_decode_launch_shapes_against_fp32(cuda_lib, units, layers, G, kv, n_cal, layout):
     """Every shape that the launch rules choose between, at its edges, against the same step in fp32: outputs are bf16
