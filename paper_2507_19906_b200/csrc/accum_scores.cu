@@ -35,7 +35,6 @@ constexpr int kGroups = 4;
 constexpr int kProducerWarp = kGroups * 4;
 constexpr int kMmaWarp = kGroups * 4 + 1;
 constexpr int kThreads = kGroups * 128 + 64;
-constexpr int kSms = 148;
 constexpr int kRows = 128, kCols = 256;             // an item's rows, a job's columns
 constexpr int kABytes = kRows * 256, kBBytes = kCols * 256;
 constexpr int kStages = 2;

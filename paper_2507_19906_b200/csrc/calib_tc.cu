@@ -48,7 +48,6 @@ constexpr uint32_t kColO = kBufs * 128;
 constexpr int kStages = kBufs;             // K ring and V ring: slot t % 3 feeds buffer t % 3
 constexpr int kTileBytes = kKvTileBytes;   // 32 KB
 constexpr int kSmemBytes = (1 + 2 * kStages) * kTileBytes + 1024;  // Q_c block, K ring, V ring
-constexpr int kSms = 148;
 
 struct CalibArgs {
   int Hq, G, W, L, n_cand, n_cal;

@@ -1301,14 +1301,16 @@ cudaError_t launch_kernel(const ClusterArgs& a, const ClusterPlan& p, int units,
 }
 
 // The fewest tiles per CTA with which every unit has its cluster at once; false where the kernel does not cover the
-// shape or the separate kernels are the faster way.  A call costs, in microseconds, about 13 and 1.9 for each tile of a CTA
-// here, 0.68 more for one with statistics, and 37.5 and 1.08 for each tile of an SM and pass there, where all 148 SMs have
-// a share; here those that no cluster fits on are idle.  Measured, us, separate and here: 8 units x 1100 keys x 128 rows 32.0
-// and 18, x 8192 44 and 32, x 16384 62 and 47, x 32768 84 and 81; 2 units x 24000 56 and 43, x 32768 53 and 52; 16 x 16384 81 and 73,
-// x 32768 125 and 126; 32 x 2048 46 and 26, x 20000 146 and 129; with the caller's row LSE 8 x 32768 65 and 63, 16 x 24576 80 and 76,
-// 64 x 12288 135 and 122 and, with a ring of three tiles, x 16384 163 and 172.  For a given kept list 8 x 1000 24 and 12, x 8192 31 and
-// 21, x 45000 77 and 66, 2 x 24000 41 and 28, 64 x 8192 100 and 77; with the caller's row LSE 8 x 8192 22 and 14, 16 x 32768 65 and 54.
-// (The compaction costs both ways alike, but for 3 us where it is a kernel behind this one.)
+// shape or the separate kernels are the faster way.  What a call costs, in microseconds: here a chain and each tile of a CTA, there
+// a chain, each tile of an SM, where all SMs have a share (here those that no cluster fits on are idle), and the selection of a long
+// unit; the compaction costs both alike, but for 3 where it is a kernel behind this one.  The constants for the separate kernels are
+// those with which the fewest of 333 calls, drawn wide and timed both ways on inputs in L2 and not, took the slower way; the margin of
+// 4 % is from 300 more, of which one is still slower here (80 units x 2745 keys 66.4 and 69.8; 66.8 and 67.4 from memory).  (Constants fitted
+// to 30 shapes, without a margin, took 80 x 3109 x 128 rows with the caller's row LSE, 59 here and 54 there, and 4 x 56877 for a given list,
+// 92 and 81.)  Measured, us, separate and here: 8 units x 1100 keys x 128 rows 32.0 and 18, x 8192 44 and 32, x 16384 62 and
+// 47, x 32768 84 and 81; 2 units x 24000 56 and 43; 16 x 16384 81 and 73; 32 x 2048 46 and 26, x 20000 146 and 129; with the caller's
+// row LSE 16 x 24576 80 and 76, 64 x 12288 135 and 122.  For a given kept list 8 x 1000 24 and 12, x 8192 31 and 21, x 45000 77 and
+// 66, 2 x 24000 41 and 28, 64 x 8192 100 and 77; with the caller's row LSE 8 x 8192 22 and 14, 16 x 32768 65 and 54.
 bool plan_cluster(const CompressGeom& g, bool stats, bool given, ClusterPlan* p) {
   if (g.keep_all || g.n_cand < 1 || g.G * g.W > kMaxRows || g.pool >> 1 > kHaloMax) return false;
   if (g.sized && g.n_calib == 0) return false;
@@ -1320,19 +1322,19 @@ bool plan_cluster(const CompressGeom& g, bool stats, bool given, ClusterPlan* p)
   for (int t = (n_tiles + kMaxClu - 1) / kMaxClu; t <= kMaxTiles; ++t) {
     const int n_clu = (n_tiles + t - 1) / t;
     if (g.units > resident_clusters(n_clu) || (size_t)g.units * n_clu > parts) continue;
-    const double tiles = g.units * n_tiles / 148.0;
+    const double tiles = (double)g.units * n_tiles / kSms;
     const double here = given ? (stats ? 10.5 + 1.55 * t : 8.7 + 0.95 * t) : 13.0 + (stats ? 2.58 : 1.9) * t;
-    const double there = given ? (stats ? 30.0 + 2.3 * tiles : 19.0 + 1.75 * tiles) : 37.5 + (stats ? 3.24 : 2.16) * tiles;
+    const double there = given ? 25.0 + (stats ? 2.72 : 1.2) * tiles : 35.0 + (stats ? 3.6 : 1.76) * tiles + g.L * 1.5e-4;
     p->copy_behind = g.n_kept > kCopyRows * n_clu;
-    return here + (p->copy_behind ? 3.0 : 0.0) < there && lay_out(g, stats, t, p);
+    return 1.04 * (here + (p->copy_behind ? 3.0 : 0.0)) < there && lay_out(g, stats, t, p);
   }
   return false;
 }
 
 }  // namespace
 
-// The whole step in one launch (two with many retained rows), or (`given`) the calibration and compaction for the kept list in kept_idx; *taken is false (and
-// nothing launched) where the separate kernels are to be used.
+// The whole step in one launch (two with many retained rows), or (`given`) the calibration and compaction for the kept list in
+// kept_idx; *taken is false (and nothing launched) where the separate kernels are to be used.
 cudaError_t launch_compress_cluster(const CompressGeom& g, const CompressWs& ws, const void* Q_obs, const void* K, const void* V,
                                     const float* row_lse, char* wsp, int32_t* kept_idx, float* O_c, float* LSE_c, void* C_q,
                                     const GatherArgs& gather, bool given, bool* taken, cudaStream_t st) {

@@ -58,7 +58,8 @@ constexpr int kCalibGroups = 4;  // softmax warpgroups of the calibration kernel
 constexpr int kDecodeMaxLayers = 32;
 constexpr int kDecodeMaxSplit = 64;
 constexpr int kDecodeHalfCopyRows = 576;   // rows of a slice (see DecodeCommon)
-constexpr int kDecodeTargetCtas = 148;  // one CTA of a launch on each of the 148 SMs
+constexpr int kSms = 148;                // of a B200
+constexpr int kDecodeTargetCtas = kSms;  // one CTA of a launch on each SM
 
 struct DecodeCommon {
   int B, Hq, Hkv, G, n_cal, cap, kv_len, n_kv, has_new;

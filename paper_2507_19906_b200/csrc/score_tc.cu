@@ -43,7 +43,6 @@ constexpr int kThreads = kGroups * 128 + 64;
 constexpr int kTmemCols = 512;  // two accumulators of 256 columns or four of 128
 constexpr int kMaxBufs = 4;
 constexpr int kMaxRows = 512;   // G * W handled by the tiles
-constexpr int kSms = 148;
 
 // Where the partial statistics of a row lie: those of the CTAs whose tile range overlaps the row's virtual unit.
 struct StatParts {

@@ -409,7 +409,7 @@ cudaError_t launch_any(const SelectArgs& a, int units, cudaStream_t st) {
   auto clusters = [&](int chunk) { return (a.L + chunk - 1) / chunk; };
   auto fits = [&](int rows) {
     const int c = clusters(512 * rows);
-    return c <= kPortableClu && (long long)c * units <= 2 * 148;
+    return c <= kPortableClu && (long long)c * units <= 2 * kSms;
   };
   if (fits(4)) return Launch<512, 4, kSized, kPortableClu>::run(a, units, st);
   if (fits(8)) return Launch<512, 8, kSized, kPortableClu>::run(a, units, st);

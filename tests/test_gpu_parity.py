@@ -371,6 +371,28 @@ def test_compress_in_one_kernel(cuda_lib, B, Hq, Hkv, L, W, pool, budget, n_cal,
         assert_close_lse(st.LSE_c.cpu().numpy(), orc.LSE_c, "LSE_c")
         assert_close_out(st.O_c.cpu().numpy(), orc.O_c, "O_c")
 
+@pytest.mark.parametrize("units,G,W,L,supply_lse,one_kernel", [
+    (8, 4, 32, 8192, False, True),
+    (8, 4, 32, 8192, True, True),
+    (80, 4, 32, 3109, True, False),    # one CTA a unit: half of the SMs would be idle
+    (80, 4, 32, 3109, False, True),
+    (48, 5, 16, 8838, True, False),    # two CTAs a unit
+])
+def test_route_of_a_compress_call(cuda_lib, units, G, W, L, supply_lse, one_kernel):
+    """The cluster kernel is taken where it was measured to be faster than the separate kernels."""
+    cd = cuda_lib
+    gen = torch.Generator(device="cuda").manual_seed(L)
+    rn = lambda *sh: torch.randn(sh, generator=gen, device="cuda").to(torch.bfloat16)
+    Q, K, V = rn(1, units * G, W, 128), rn(1, units, L, 128), rn(1, units, L, 128)
+    lse = torch.full((1, units * G, W), 9.0, device="cuda") if supply_lse else None
+    p = cd.make_params(B=1, Hq=units * G, Hkv=units, L=L, window=W, pool=7, budget=200, n_cal=1, cap=200)
+    st = cd.alloc_layer_state(p)
+    before = cd.calidrop_launch_count()
+    cd.calidrop_compress(p, Q, K, V, lse, st.kept_idx, st.K_kept, st.V_kept, st.O_c, st.LSE_c, st.C_q, st.ws_compress)
+    torch.cuda.synchronize()
+    assert (cd.calidrop_launch_count() - before == 1) == one_kernel
+
+
 @pytest.mark.parametrize("B,Hq,Hkv,L,W,pool,budget,n_cal", [c[:8] for c in ONE_KERNEL if c[8] == 0 and c[9]])
 @pytest.mark.parametrize("supply_lse", [False, True])
 def test_calibrate_in_one_kernel(cuda_lib, B, Hq, Hkv, L, W, pool, budget, n_cal, supply_lse):
