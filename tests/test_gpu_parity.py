@@ -81,28 +81,32 @@ def test_single_cta_selection_for_very_long_prompts(cuda_lib):
     decode_steps_compare(g, ref, q, kn, vn, steps=2)
 
 
-@pytest.mark.parametrize("units,G,W,L", [
-    (3, 1, 8, 300),        # combined by the votes: 32 threads share a row, two statistics tiles
-    (2, 8, 64, 700),       # ... 512 rows in two virtual units, a thread each
-    (40, 4, 16, 1500),     # ... CTAs whose range spans two units
-    (1, 4, 32, 20000),     # too many partials for it: a kernel of its own
-    (300, 1, 8, 140),      # ... CTAs of more than two units
-    (1, 4, 32, 20225),     # one unit: 80 tiles on a CTA each, 81 slots of four partials
-    (1, 4, 64, 32768),     # ... 129 slots of two
-    (1, 1, 8, 32768),      # ... of four
-    (1, 2, 16, 65536),     # ... two tiles a CTA
+@pytest.mark.parametrize("units,G,W,L,own_kernel", [
+    (3, 1, 8, 300, False),        # combined by the votes: 32 threads share a row, two statistics tiles
+    (2, 8, 64, 700, False),       # ... 512 rows in two virtual units, a thread each
+    (40, 4, 16, 1500, False),     # ... CTAs whose range spans two units
+    (1, 4, 32, 20000, True),      # too many partials for it: a kernel of its own
+    (300, 1, 8, 140, True),       # ... CTAs of more than two units
+    (1, 4, 32, 20225, True),      # one unit: 80 tiles on a CTA each, 81 slots of four partials
+    (1, 4, 64, 32768, True),      # ... 129 slots of two
+    (1, 1, 8, 32768, True),       # ... of four
+    (1, 2, 16, 65536, True),      # ... two tiles a CTA
 ])
-def test_row_lse_of_the_statistics(cuda_lib, units, G, W, L):
+def test_row_lse_of_the_statistics(cuda_lib, units, G, W, L, own_kernel):
     """Row LSE that a compress call leaves in its workspace, against fp64.  A logit is a sum of 128 exact products in
-    fp32: an error of 128 * 2^-24 of a sum of magnitudes below 13 at the most, 1e-4."""
+    fp32: an error of 128 * 2^-24 of a sum of magnitudes below 13 at the most, 1e-4.  (A pool wider than the cluster kernel's
+    halo keeps the calls on the separate kernels.)"""
     cd = cuda_lib
     gen = torch.Generator(device="cuda").manual_seed(L)
     rn = lambda *sh: torch.randn(sh, generator=gen, device="cuda").to(torch.bfloat16)
     Q, K, V = rn(1, units * G, W, 128), rn(1, units, L, 128), rn(1, units, L, 128)
-    p = cd.make_params(B=1, Hq=units * G, Hkv=units, L=L, window=W, pool=5, budget=W + 20, n_cal=1, cap=W + 20)
+    p = cd.make_params(B=1, Hq=units * G, Hkv=units, L=L, window=W, pool=131, budget=W + 20, n_cal=1, cap=W + 20)
     st = cd.alloc_layer_state(p)
+    before = cd.calidrop_launch_count()
     cd.calidrop_compress(p, Q, K, V, None, st.kept_idx, st.K_kept, st.V_kept, st.O_c, st.LSE_c, st.C_q, st.ws_compress)
     torch.cuda.synchronize()
+    # statistics, (row LSE,) votes, selection, calibration, its reduction with the compaction
+    assert cd.calidrop_launch_count() - before == (6 if own_kernel else 5)
     off = cd.calidrop_compress_workspace_layout(p).row_lse_offset
     got = st.ws_compress[off:off + units * G * W * 4].view(torch.float32).view(units, G * W)
     s = torch.einsum("urd,utd->urt", Q.view(units, G * W, 128).double(), K[0].double()) / 128 ** 0.5
@@ -112,12 +116,13 @@ def test_row_lse_of_the_statistics(cuda_lib, units, G, W, L):
 
 
 @pytest.mark.parametrize("gap_one,gap_rest", [(78, 78), (78, 140), (140, 140)])
-def test_calibration_of_evicted_rows_with_almost_no_attention(cuda_lib, gap_one, gap_rest):
+@pytest.mark.parametrize("G,W,one_kernel", [(2, 16, True), (4, 40, False)])
+def test_calibration_of_evicted_rows_with_almost_no_attention(cuda_lib, gap_one, gap_rest, G, W, one_kernel):
     """The kept rows lead the evicted ones by `gap` nats, one row per kv head by another gap.  A probability below 2^-126
     is 0 and adds nothing; where all of them are, the row has no calibration: O_c = 0, LSE_c = -inf, not applied.  The
     one row at 78 nats is e^-82 of the softmax, far from the rest at e^-144."""
     cd = cuda_lib
-    units, G, W, L, n_heavy = 2, 2, 16, 3000, 64
+    units, L, n_heavy = 2, 3000, 64
     gen = torch.Generator(device="cuda").manual_seed(gap_one + gap_rest)
     rn = lambda *sh: torch.randn(sh, generator=gen, device="cuda")
     e = rn(units, 128).sign()
@@ -133,7 +138,9 @@ def test_calibration_of_evicted_rows_with_almost_no_attention(cuda_lib, gap_one,
     budget = W + n_heavy
     p = cd.make_params(B=1, Hq=units * G, Hkv=units, L=L, window=W, pool=1, budget=budget, n_cal=W, cap=budget, theta2=-1.0)
     st = cd.alloc_layer_state(p)
+    before = cd.calidrop_launch_count()
     cd.calidrop_compress(p, Q, K, V, None, st.kept_idx, st.K_kept, st.V_kept, st.O_c, st.LSE_c, st.C_q, st.ws_compress)
+    assert (cd.calidrop_launch_count() - before == 1) == one_kernel
     assert torch.equal(st.kept_idx[0, :, :n_heavy].long(), at[:n_heavy].sort().values.expand(units, -1))
     out = torch.empty((1, units * G, 128), dtype=torch.bfloat16, device="cuda")
     flags = torch.empty((1, units * G), dtype=torch.uint8, device="cuda")
@@ -152,13 +159,14 @@ def test_calibration_of_evicted_rows_with_almost_no_attention(cuda_lib, gap_one,
     assert (flags & 1).all()
 
 
-def test_votes_with_a_row_lse_far_below_the_logits(cuda_lib):
+@pytest.mark.parametrize("G,W,one_kernel", [(4, 8, True), (4, 40, False)])
+def test_votes_with_a_row_lse_far_below_the_logits(cuda_lib, G, W, one_kernel):
     """A caller's row LSE is not validated: one row's that is 200 nats too low makes every vote overflow to infinity,
     whichever of the 32 columns the row is, and the lowest candidates win."""
     cd = cuda_lib
     gen = torch.Generator(device="cuda").manual_seed(5)
     rn = lambda *sh: torch.randn(sh, generator=gen, device="cuda").to(torch.bfloat16)
-    L, W, G, budget = 900, 8, 4, 60
+    L, budget = 900, 60
     Q, K, V = rn(1, G, W, 128), rn(1, 1, L, 128), rn(1, 1, L, 128)
     p = cd.make_params(B=1, Hq=G, Hkv=1, L=L, window=W, pool=1, budget=budget, n_cal=1, cap=budget)
     st = cd.alloc_layer_state(p)
@@ -166,20 +174,23 @@ def test_votes_with_a_row_lse_far_below_the_logits(cuda_lib):
     for row in range(G * W):
         lse = torch.full((G * W,), 7.0, device="cuda")
         lse[row] = -200.0
+        before = cd.calidrop_launch_count()
         cd.calidrop_compress(p, Q, K, V, lse.view(1, G, W), st.kept_idx, st.K_kept, st.V_kept, st.O_c, st.LSE_c, st.C_q,
                              st.ws_compress)
+        assert (cd.calidrop_launch_count() - before == 1) == one_kernel
         votes = st.ws_compress[off:off + 4 * (L - W)].view(torch.float32)
         assert torch.all(votes == float("inf")), row
         assert torch.equal(st.kept_idx[0, 0, :budget - W].long(), torch.arange(budget - W, device="cuda"))
 
 
-def test_nan_inputs_leave_a_nan_wherever_they_lie(cuda_lib):
+@pytest.mark.parametrize("G,W,one_kernel", [(4, 8, True), (4, 40, False)])
+def test_nan_inputs_leave_a_nan_wherever_they_lie(cuda_lib, G, W, one_kernel):
     """One NaN in a key or query row reaches every result that depends on it, at every position inside the 32 logits that
     a thread works on at a time: row LSE, votes, accumulated scores; a calibration over such a key is none."""
     cd = cuda_lib
     gen = torch.Generator(device="cuda").manual_seed(9)
     rn = lambda *sh: torch.randn(sh, generator=gen, device="cuda").to(torch.bfloat16)
-    L, W, G, budget = 300, 8, 4, 60
+    L, budget = 300, 60
     Q, K, V, Q_full = rn(1, G, W, 128), rn(1, 1, L, 128), rn(1, 1, L, 128), rn(1, G, L, 128)
     p = cd.make_params(B=1, Hq=G, Hkv=1, L=L, window=W, pool=1, budget=budget, n_cal=W, cap=budget)
     st = cd.alloc_layer_state(p)
@@ -194,7 +205,9 @@ def test_nan_inputs_leave_a_nan_wherever_they_lie(cuda_lib):
         Kt, Qt = K.clone(), Q.clone()
         Kt[0, 0, 32 + t, 5] = float("nan")
         Qt.view(G * W, 128)[t, 5] = float("nan")
+        before = cd.calidrop_launch_count()
         cd.calidrop_compress(p, Q, Kt, V, None, st.kept_idx, *outs)
+        assert (cd.calidrop_launch_count() - before == 1) == one_kernel
         assert torch.all(torch.isnan(get(lay.row_lse_offset, G * W))), t
         cd.calidrop_compress(p, Qt, K, V, lse, st.kept_idx, *outs)
         assert torch.all(torch.isnan(get(lay.vote_offset, L - W))), t
@@ -269,11 +282,16 @@ def test_selection_on_clusters_of_more_than_eight(cuda_lib, units, L, tail, pool
 
 
 @pytest.mark.parametrize("calib_size", [1, 40, 300, 10 ** 6, -1])
-def test_calibration_size(cuda_lib, calib_size):
+@pytest.mark.parametrize("B,Hq,Hkv,L,W,budget,n_cal,one_kernel", [
+    (2, 8, 2, 1500, 16, 200, 16, True),
+    (1, 8, 2, 1500, 64, 200, 16, False),      # 256 window rows: the separate kernels
+    (1, 150, 150, 400, 16, 200, 4, False),    # more units than the device holds clusters
+])
+def test_calibration_size(cuda_lib, calib_size, B, Hq, Hkv, L, W, budget, n_cal, one_kernel):
     """Section 4.4's calibration size m: only the m evicted rows of highest pooled vote are calibrated
     (and offloaded); m >= the number evicted is Algorithm 1 as printed, -1 switches the calibration off."""
     from paper_2507_19906_b200 import binding as cd
-    B, Hq, Hkv, L, W, pool, budget, n_cal = 2, 8, 2, 1500, 16, 7, 200, 16
+    pool = 7
     cfg = wl.small_config(B=B, Hq=Hq, Hkv=Hkv, L=L, window=W, pool=pool, budget=budget, steps=3, n_sink=2, n_heavy=40)
     Q, K, V = _inputs(cfg)
     m = None if calib_size == 10 ** 6 else max(calib_size, 0)
@@ -282,9 +300,11 @@ def test_calibration_size(cuda_lib, calib_size):
                        calib_size=calib_size)
     st = cd.alloc_layer_state(p)
     dQ, dK, dV = to_dev(Q), to_dev(K), to_dev(V)
+    before = cd.calidrop_launch_count()
     cd.calidrop_compress(p, dQ, dK, dV, None, st.kept_idx, st.K_kept, st.V_kept, st.O_c, st.LSE_c, st.C_q,
                          st.ws_compress)
     torch.cuda.synchronize()
+    assert (cd.calidrop_launch_count() - before == 1) == (one_kernel and calib_size != -1)
     np.testing.assert_array_equal(st.kept_idx.cpu().numpy(), orc.kept_idx)      # no near-tie in this input
     np.testing.assert_array_equal(to_bits(st.C_q), orc.C_q)
     assert_close_lse(st.LSE_c.cpu().numpy(), orc.LSE_c, "LSE_c")
@@ -361,15 +381,80 @@ def test_compress_in_one_kernel(cuda_lib, B, Hq, Hkv, L, W, pool, budget, n_cal,
     if octaves is None:
         np.testing.assert_allclose(ws(lay.row_lse_offset, orc.row_lse), orc.row_lse, atol=2e-5)
     kept = st.kept_idx.cpu().numpy()
-    swaps = check_kept_sets(kept, orc)
+    check_kept_sets(kept, orc)
     np.testing.assert_array_equal(to_bits(st.C_q), orc.C_q)
     for b in range(B):
         for h in range(Hkv):
             np.testing.assert_array_equal(to_bits(st.K_kept)[b, h], K[b, h][kept[b, h]])
             np.testing.assert_array_equal(to_bits(st.V_kept)[b, h], V[b, h][kept[b, h]])
-    if swaps == 0:   # (neither depends on the shift)
-        assert_close_lse(st.LSE_c.cpu().numpy(), orc.LSE_c, "LSE_c")
-        assert_close_out(st.O_c.cpu().numpy(), orc.O_c, "O_c")
+    # the selection is that of the kernel's own pooled votes to the last bit, and the calibration state is that of the rows
+    # it leaves (the shift of the row LSE does not enter)
+    check_selection_and_calibration(p, st, dQ, dK, dV, ws(lay.pooled_offset, orc.pooled))
+
+
+def check_selection_and_calibration(p, st, dQ, dK, dV, pooled):
+    """Kept list and calibrated rows of a call against a stable sort of the pooled votes it left in its workspace, the calibration
+    state against fp64 over those rows."""
+    from paper_2507_19906_b200 import binding as cd
+    B, Hkv, G, L, W, n_cal = p.B, p.Hkv, p.Hq // p.Hkv, p.L, p.window, p.n_cal
+    k_sel, n_cand = p.budget - W, L - W
+    m = n_cand - k_sel if p.calib_size == 0 else min(p.calib_size, n_cand - k_sel)
+    order = np.argsort(-pooled.reshape(B * Hkv, n_cand), axis=-1, kind="stable")
+    kept, calib = np.sort(order[:, :k_sel], -1), np.sort(order[:, k_sel:k_sel + m], -1)
+    got = st.kept_idx.cpu().numpy().reshape(B * Hkv, p.budget)
+    np.testing.assert_array_equal(got[:, :k_sel], kept)
+    np.testing.assert_array_equal(got[:, k_sel:], np.broadcast_to(np.arange(n_cand, L), (B * Hkv, W)))
+    ev_idx = torch.empty((B, Hkv, m), dtype=torch.int32, device="cuda")
+    K_e, V_e = (torch.empty((B, Hkv, m, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    cd.calidrop_gather_evicted(p, dK, dV, st.kept_idx, ev_idx, K_e, V_e, st.ws_compress)
+    np.testing.assert_array_equal(ev_idx.cpu().numpy().reshape(B * Hkv, m), calib)
+    q = dQ[:, :, W - n_cal:].reshape(B * Hkv, G * n_cal, 128).double()
+    for u in range(B * Hkv):
+        s = q[u] @ K_e.view(-1, m, 128)[u].double().T / 128 ** 0.5
+        want_lse, want = torch.logsumexp(s, -1), torch.softmax(s, -1) @ V_e.view(-1, m, 128)[u].double()
+        assert_close_lse(st.LSE_c.view(B * Hkv, -1)[u].cpu().numpy(), want_lse.cpu().numpy(), "LSE_c")
+        assert_close_out(st.O_c.view(B * Hkv, -1, 128)[u].cpu().numpy(), want.cpu().numpy(), "O_c")
+
+
+@pytest.mark.parametrize("units,L,W,G,pool", [
+    (1, 2056, 8, 4, 1),         # CTAs of one or two tiles
+    (3, 6000, 16, 8, 1),        # 128 window rows
+    (100, 128 * 18 + 9, 8, 2, 1),   # one CTA of more than sixteen tiles to a unit
+    (60, 128 * 40 - 3, 8, 2, 1),    # ... two
+    (5, 3000, 8, 4, 3),         # pooled: runs of equal sums
+])
+@pytest.mark.parametrize("mid,low", [(0.5, 0.25), (0.5, -10.0)])
+@pytest.mark.parametrize("sized", [False, True])
+def test_ties_in_one_kernel(cuda_lib, units, L, W, G, pool, mid, low, sized):
+    """Keys of three kinds, equal to the bit and so in their votes: the cut of the kept list lies inside the second kind, in the
+    middle of the prompt, that of a calibration size inside the third, whose votes are in the range of the first selection pass
+    or far below it."""
+    cd = cuda_lib
+    gen = torch.Generator(device="cuda").manual_seed(L + sized)
+    rn = lambda *sh: torch.randn(sh, generator=gen, device="cuda")
+    n_cand = L - W
+    u = rn(units, 128).sign()
+    Q = (u[:, None, None] * 0.5 + 0.1 * rn(units, G, W, 128)).reshape(1, units * G, W, 128).to(torch.bfloat16)
+    kind = torch.rand((units, n_cand), generator=gen, device="cuda")
+    kind = (kind > 0.1).long() + (kind > 0.4).long()                  # a tenth, three tenths, the rest
+    level = torch.tensor([0.8, mid, low], device="cuda") / 2
+    K = torch.cat([(level[kind][..., None] * u[:, None]), 0.1 * rn(units, W, 128)], 1).to(torch.bfloat16)[None].contiguous()
+    V = rn(1, units, L, 128).to(torch.bfloat16)
+    budget = W + n_cand // 4
+    m = n_cand // 2 if sized else 0
+    p = cd.make_params(B=1, Hq=units * G, Hkv=units, L=L, window=W, pool=pool, budget=budget, n_cal=2, cap=budget, calib_size=m)
+    st = cd.alloc_layer_state(p)
+    before = cd.calidrop_launch_count()
+    cd.calidrop_compress(p, Q, K, V, None, st.kept_idx, st.K_kept, st.V_kept, st.O_c, st.LSE_c, st.C_q, st.ws_compress)
+    torch.cuda.synchronize()
+    assert cd.calidrop_launch_count() - before <= 2   # (the second one compacts many rows)
+    off = cd.calidrop_compress_workspace_layout(p).pooled_offset
+    pooled = st.ws_compress[off:off + 4 * units * n_cand].view(torch.float32).cpu().numpy().reshape(units, n_cand)
+    if pool == 1:
+        for row in pooled:
+            assert len(np.unique(row)) == 3
+    check_selection_and_calibration(p, st, Q, K, V, pooled)
+
 
 @pytest.mark.parametrize("units,G,W,L,supply_lse,one_kernel", [
     (8, 4, 32, 8192, False, True),
@@ -1554,13 +1639,14 @@ for G, s in states.items():
     subprocess.run([sys.executable, "-c", code], cwd=root, check=True, timeout=300)
 
 
-def test_calls_enqueued_back_to_back_give_the_results_of_calls_run_one_at_a_time(cuda_lib):
+@pytest.mark.parametrize("Hq,one_kernel", [(8, True), (10, False)])
+def test_calls_enqueued_back_to_back_give_the_results_of_calls_run_one_at_a_time(cuda_lib, Hq, one_kernel):
     """The kernels of a compress call start beside the end of their predecessors (programmatic dependent
     launch) and a decode launch prefetches ahead of its dependency wait: a stream of calls with no
     synchronisation between them, on one shared workspace, must leave exactly what the same calls leave
     when each is waited for."""
     cd = cuda_lib
-    B, Hq, Hkv, L, W, pool, budget, n_cal = 2, 8, 2, 2300, 32, 7, 256, 32
+    B, Hkv, L, W, pool, budget, n_cal = 2, 2, 2300, 32, 7, 256, 32
     cfgs = [wl.small_config(B=B, Hq=Hq, Hkv=Hkv, L=L, window=W, pool=pool, budget=budget, steps=3, n_heavy=24,
                             seed=s) for s in (5, 6)]
     inputs = [tuple(to_dev(x) for x in _inputs(c)) for c in cfgs]
@@ -1575,8 +1661,10 @@ def test_calls_enqueued_back_to_back_give_the_results_of_calls_run_one_at_a_time
         outs = []
         for rnd in range(3):
             for i, (st, (dQ, dK, dV)) in enumerate(zip(states, inputs)):
+                before = cd.calidrop_launch_count()
                 cd.calidrop_compress(p, dQ, dK, dV, None, st.kept_idx, st.K_kept, st.V_kept, st.O_c, st.LSE_c, st.C_q,
                                      st.ws_compress)
+                assert (cd.calidrop_launch_count() - before == 1) == one_kernel
                 if sync:
                     torch.cuda.synchronize()
                 q, kn, vn = dec[i]
