@@ -183,7 +183,7 @@ DecodeCommon plan_decode(const calidrop_params* p, const DecodeWs& w, int n_laye
     }
   }
   a.rows_per_split = slice_rows(n_kv, a.nsplit * a.nclu);
-  a.half_copies = a.rows_per_split <= kDecodeHalfCopyRows;
+  a.half_copies = a.rows_per_split >= kDecodeHalfCopyMin && a.rows_per_split <= kDecodeHalfCopyMax;
   a.scale2 = scale2_of(p);
   a.theta1 = p->theta1; a.theta2 = p->theta2; a.always_apply = p->theta2 <= -1.0f;
   // The workspace is laid out array by array with the layer index outermost inside each

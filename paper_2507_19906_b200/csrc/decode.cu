@@ -54,10 +54,11 @@ constexpr int kBlkRows = 16;                        // rows of one warp's MMA bl
 constexpr int kWideRows = 64;                       // rows of the boxes of whole slots in the wide shape
 // The shape of a CTA: ring slots of kRows rows, each consumed by kRows / 16 warps, kWarps stream warps in two groups on
 // alternate slots, kCtas CTAs per SM.
-template <int kSlots_, int kRows_, int kCtas_, int kClu_>
+template <int kSlots_, int kRows_, int kCtas_, int kClu_, bool kHalf_ = false>
 struct Shape {
   static constexpr int kSlots = kSlots_, kRows = kRows_, kCtas = kCtas_;
   static constexpr int kClu = kClu_;                // the most CTAs of a cluster
+  static constexpr bool kHalf = kHalf_;             // whole slots by a copy per half of the columns (see DecodeCommon)
   static constexpr int kSubs = kRows / kBlkRows;    // warps per slot
   static constexpr int kStreamWarps = 2 * kSubs;
   static constexpr int kThreads = (kStreamWarps + 1) * 32;   // the last warp is the producer
@@ -65,10 +66,13 @@ struct Shape {
   static constexpr int kSlotBytes = 4 * kPlaneBytes;         // K low / K high / V low / V high column halves
   static constexpr int kSmemBytes = kSlots * kSlotBytes + 1024;   // + slack for the 1024-byte alignment
 };
-using ShapeWide = Shape<6, kWideRows, 1, 8>;     // a launch with one CTA per SM at most: 192 KB
-using ShapeCluster16 = Shape<6, kWideRows, 1, 16>;  // few units with a longer cache (see plan_decode)
-using ShapePair = Shape<3, kWideRows, 2, 1>;     // a launch with up to two CTAs per SM: 96 KB
-using ShapeNarrow = Shape<3, 32, 4, 1>;          // more than that: 48 KB, four CTAs per SM
+template <bool kHalf>
+using ShapeWide = Shape<6, kWideRows, 1, 8, kHalf>;     // a launch with one CTA per SM at most: 192 KB
+template <bool kHalf>
+using ShapeCluster16 = Shape<6, kWideRows, 1, 16, kHalf>;  // few units with a longer cache (see plan_decode)
+template <bool kHalf>
+using ShapePair = Shape<3, kWideRows, 2, 1, kHalf>;     // a launch with up to two CTAs per SM: 96 KB
+using ShapeNarrow = Shape<3, 32, 4, 1>;                 // more than that: 48 KB, four CTAs per SM
 constexpr int kWoStride = kD + 4;  // row stride of the per-warp partial outputs: heads land in distinct banks
 constexpr long long kWaitLimitCycles = 2000000000ll;  // about a second: a wait this long has failed
 
@@ -461,9 +465,10 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
   // One ring fill into slot sb % kSlots: calibration queries first where they go through the ring, then kSlotRows rows of
-  // K and V.  Whole slots of 64 rows take a 64-row box each; slots of 32 rows and the ragged last one take 16-row boxes
-  // for the row groups that hold valid rows, so a split never pulls more than 15 rows of its neighbour.  Only a 16-row
-  // box can reach past row kv_len: the V map of those boxes ends at kv_len, so such V rows arrive as zeros (a zero
+  // K and V.  Whole slots of 64 rows take a 64-row box each, or one for each half of the columns; slots of 32 rows and the ragged
+  // last one take 16-row boxes for the row groups that hold valid rows.  Slices begin at multiples of 16 rows, so none of these
+  // brings rows of a neighbour, and the results rely on that (a probability of zero times an infinite value of V is NaN).  Only a
+  // 16-row box can reach past row kv_len: the V map of those boxes ends at kv_len, so such V rows arrive as zeros (a zero
   // probability times whatever lies in the caller's memory could still be a NaN); the K rows
   // arrive as they lie in memory and their scores are masked.
   auto fill = [&](int sb) {
@@ -485,10 +490,11 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
     const int nrows = min(kSlotRows, r1 - row0);
     if (kSlotRows == kWideRows && nrows == kSlotRows) {
       mbar_expect_tx(bar, kSlotBytes);
+      const bool halves = RECAL ? a.half_copies != 0 : S::kHalf;   // (see DecodeCommon)
       tma_load_rows(dst, &TM.k64, bar, row0, unit, pol_stream);
-      if (a.half_copies) tma_load_rows(dst + kPlaneBytes, &TM.k64, bar, row0, unit, pol_stream, 1);   // (see DecodeCommon)
+      if (halves) tma_load_rows(dst + kPlaneBytes, &TM.k64, bar, row0, unit, pol_stream, 1);
       tma_load_rows(dst + 2 * kPlaneBytes, &TM.v64, bar, row0, unit, pol_stream);
-      if (a.half_copies) tma_load_rows(dst + 3 * kPlaneBytes, &TM.v64, bar, row0, unit, pol_stream, 1);
+      if (halves) tma_load_rows(dst + 3 * kPlaneBytes, &TM.v64, bar, row0, unit, pol_stream, 1);
     } else {
       const int nb = (nrows + kBlkRows - 1) / kBlkRows;
       mbar_expect_tx(bar, (uint32_t)nb * 4u * kBlkRows * 128u);
@@ -553,9 +559,9 @@ decode_kernel(const __grid_constant__ DecodeArgsT<NL> args) {
       for (int sb = 0; sb < min(n_sb, kSlots); ++sb) fill(sb);
     __syncwarp();
   }
-  // The similarities are finished by the producer warp at once and by a stream warp after its first
-  // slot, whose data is already there when the query arrives.  The stream warps then hand their updates of s_best to the
-  // producer warp through a CTA barrier, and that one, which has time, pushes them to the CTAs of the cluster.
+  // A stream warp finishes its similarities after its first slot, whose data is already there when the query arrives.  The stream
+  // warps then hand their updates of s_best to the producer warp through a CTA barrier, and that one, which has no similarities and
+  // time, pushes them to the CTAs of the cluster.
   auto rho_rest = [&]() {
     if (kOne) return;
     rho_finish(pi0, pg0, pc0, rl);
@@ -1021,15 +1027,22 @@ cudaError_t launch_decode_s(const DecodeArgsT<NL>& a, cudaStream_t st) {
 // through registers 88.9, four of four warps 73, with the calibration queries through the ring 60 (48 for the bytes).
 constexpr int kNarrowRows = 1024;
 
-template <int NL, bool RECAL>
-cudaError_t launch_decode_t(const DecodeArgsT<NL>& a, cudaStream_t st) {
+template <int NL, bool RECAL, bool kHalf>
+cudaError_t launch_decode_h(const DecodeArgsT<NL>& a, cudaStream_t st) {
   switch (decode_ctas_per_sm(a.c)) {
     case 4: return launch_decode_s<NL, RECAL, ShapeNarrow>(a, st);
-    case 2: return launch_decode_s<NL, RECAL, ShapePair>(a, st);
+    case 2: return launch_decode_s<NL, RECAL, ShapePair<kHalf>>(a, st);
   }
   if constexpr (!RECAL)
-    if (a.c.nsplit > 8) return launch_decode_s<NL, RECAL, ShapeCluster16>(a, st);
-  return launch_decode_s<NL, RECAL, ShapeWide>(a, st);
+    if (a.c.nsplit > 8) return launch_decode_s<NL, RECAL, ShapeCluster16<kHalf>>(a, st);
+  return launch_decode_s<NL, RECAL, ShapeWide<kHalf>>(a, st);
+}
+
+template <int NL, bool RECAL>
+cudaError_t launch_decode_t(const DecodeArgsT<NL>& a, cudaStream_t st) {
+  if constexpr (!RECAL)
+    if (a.c.half_copies) return launch_decode_h<NL, RECAL, true>(a, st);
+  return launch_decode_h<NL, RECAL, false>(a, st);
 }
 
 }  // namespace
@@ -1053,11 +1066,11 @@ int decode_resident_clusters(int ctas) {
   if (n == 0) {
     // (the kernels of one shape differ in their arguments only)
     int active = 0;
-    if (setup_decode<1, false, ShapeCluster16>(dev) != cudaSuccess) return 0;
+    if (setup_decode<1, false, ShapeCluster16<false>>(dev) != cudaSuccess) return 0;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(ctas);
-    cfg.blockDim = dim3(ShapeCluster16::kThreads);
-    cfg.dynamicSmemBytes = ShapeCluster16::kSmemBytes;
+    cfg.blockDim = dim3(ShapeCluster16<false>::kThreads);
+    cfg.dynamicSmemBytes = ShapeCluster16<false>::kSmemBytes;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = ctas;
@@ -1065,7 +1078,7 @@ int decode_resident_clusters(int ctas) {
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&active, decode_kernel<1, false, ShapeCluster16>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&active, decode_kernel<1, false, ShapeCluster16<false>>, &cfg) != cudaSuccess) {
       cudaGetLastError();   // no such cluster on this device
       active = 0;
     }

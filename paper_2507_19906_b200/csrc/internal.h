@@ -57,7 +57,7 @@ struct alignas(64) DecodeLayerMaps {
 constexpr int kCalibGroups = 4;  // softmax warpgroups of the calibration kernel: row-sum partials per slot
 constexpr int kDecodeMaxLayers = 32;
 constexpr int kDecodeMaxSplit = 64;
-constexpr int kDecodeHalfCopyRows = 576;   // rows of a slice (see DecodeCommon)
+constexpr int kDecodeHalfCopyMin = 64, kDecodeHalfCopyMax = 576;   // rows of a slice (see DecodeCommon)
 constexpr int kSms = 148;                // of a B200
 constexpr int kDecodeTargetCtas = kSms;  // one CTA of a launch on each SM
 
@@ -66,10 +66,12 @@ struct DecodeCommon {
   int units, n_layers, rows_per_split;
   int nsplit;  // CTAs per cluster (1, 2, 4, 8 or 16): the splits combined through distributed shared memory
   int nclu;    // clusters per (layer, unit); more than one only when few units share a long cache
-  // Whole ring slots are brought by a copy for each half of the head dimension instead of one for both.  Slices of up to nine slots
-  // take them: alone either way is as fast (32 units x 2049 rows 7.18 and 7.16 us a launch, 12 layers in turn 8.19 both), behind a
-  // recomputation and ahead of a compaction the halves are faster (the pass of the three over 32 units x 32768 rows 258.0 -> 254.9
-  // us).  One copy is faster in longer slices: 32 x 4100 rows 9.8 and 9.9, 8 x 12000 11.6 and 12.3, 32 x 30720 81.5 and 82.1.
+  // Whole ring slots are brought by a copy for each half of the head dimension instead of one for both.  Slices of one to nine slots
+  // take them: alone either way is as fast (32 units x 2049 rows 7.18 and 7.16 us a launch, 12 layers in turn 8.19 both), between a
+  // recomputation and a compaction the halves are faster (the pass of the three over 32 units x 32768 rows, mean over 24 placements
+  // of its buffers, 252.7 -> 250.4 us; 249.5 before the halves were one copy).  One copy is faster in longer slices: 32 x 4100 rows
+  // 9.8 and 9.9, 8 x 12000 11.6 and 12.3, 32 x 30720 81.5 and 82.1.  Decode has a kernel for each: with both in one, 8 x 20000 rows
+  // took 18.6 instead of 18.2 us and 8 x 129 rows, which have no whole slot, 4.19 instead of 4.16.
   int half_copies;
   float scale2, theta1, theta2;
   int always_apply;
