@@ -24,7 +24,7 @@
 // phase for 1024 exponential-unit cycles, whatever share of them is on the FMA pipe.  The code is kept small on purpose
 // (loops not unrolled, waits out of line): most of it runs once per launch, and 260 KB of it took 20 us
 // where 110 KB take 16.6.  Five to six kernels -> this one, us: 8 units x 2048 keys x 32 rows 28.3 -> 16.7, 8 x 8192 x 128 45.0 ->
-// 32.2, 16 x 5003 x 120 with the caller's row LSE and a calibration size 42.8 -> 27.3.
+// 32.2, 16 x 5003 x 120 with the caller's row LSE and a calibration size 42.8 -> 28.5.
 #include <algorithm>
 #include <atomic>
 #include <type_traits>
