@@ -131,7 +131,7 @@ cudaError_t launch_calib_tc(const CompressGeom& g, const CompressWs& ws, const v
                             const void* V, const float* row_lse, char* wsp, float* O_c, float* LSE_c, void* C_q,
                             const GatherArgs& gather, bool first, cudaStream_t st);
 // compress_cluster.cu: the whole step (or, given a kept list, what follows the selection) in one kernel, where a unit is
-// small enough for a cluster
+// small enough for a cluster; many retained rows are compacted by a second one
 cudaError_t launch_compress_cluster(const CompressGeom& g, const CompressWs& ws, const void* Q_obs, const void* K, const void* V,
                                     const float* row_lse, char* wsp, int32_t* kept_idx, float* O_c, float* LSE_c, void* C_q,
                                     const GatherArgs& gather, bool given, bool* taken, cudaStream_t st);
